@@ -127,8 +127,11 @@ gbmc_status gbmc_set_sweep_launch(gbmc_ctx *ctx, int32_t mode);
  * copy on chip; the population stays in the int8 layout in device memory and
  * is converted on load and store), for 2D ferromagnets with L in {16, 32, 64,
  * 128, 256} and 3D lattices (ferromagnet or +-J) with L = 8 or 16; other lattices of the
- * same call take the BYTES kernel. AUTO (default): BITS for a supported lattice
- * class unless gbmc_autotune timed BYTES faster for it. The mode also picks the
+ * same call take the BYTES kernel. AUTO (default): one bit per spin for every
+ * lattice, BITS for the classes above and, for any other L, a kernel that holds
+ * each colour plane as one stream of bits and sweeps several copies per thread
+ * (profiled as "sweep_stream"; a grid launch whatever gbmc_set_sweep_launch says),
+ * unless gbmc_autotune timed BYTES faster for the class. The mode also picks the
  * strip-resident sweeps of large int8 2D ferromagnets (gbmc_set_sweep_launch):
  * BYTES runs them on the int8 strips; AUTO and BITS, where the bit-packed strip
  * kernel fits (L % 1024 == 0, at most SM count / 8 copies), pack the
@@ -300,8 +303,8 @@ gbmc_status observables(gbmc_ctx *ctx, const gbmc_lattice *lat, int32_t *E_dev, 
  * (up to 32768) copies of the lattice, swept as one instance (n_sweeps sweeps
  * at beta, the lattice itself is left unchanged), then the fastest of them
  * once more as a persistent launch, and the fastest is recorded for the
- * lattice class (dim, model, L) for the rest of the process; for the classes
- * the bit-sliced kernel supports it is timed too (kernel). Untuned classes
+ * lattice class (dim, model, L) for the rest of the process; the kernel that
+ * holds one bit per spin for the class is timed too (kernel). Untuned classes
  * use threads per copy = the power of two covering a quarter of a colour's
  * words (8..256; about four words per thread and half-sweep) in 256-thread
  * blocks. Every shape gives bit-identical results: the random words depend

@@ -54,7 +54,7 @@ enum ProfKind {
     PK_INIT, PK_COUPLINGS, PK_SWEEP_RES, PK_HALFSWEEP, PK_OBS, PK_PA_WEIGHTS, PK_PA_REDUCE,
     PK_PA_DRAWS, PK_PA_PLACE, PK_PA_RECORD, PK_PA_RESET, PK_SWEEP_TILES, PK_SCHEDULE, PK_PA_FUSED,
     PK_BP_HALFSWEEP, PK_SWEEP_DCB, PK_SWEEP_MSC, PK_SW, PK_BP_STRIPS, PK_SWEEP_STRIPS, PK_PT_EXCHANGE, PK_SWEEP_BITS,
-    PK_BP_PACK, PK_SWEEP_DCB_BITS, PK_SWEEP_DCB_RES, PK_COUNT
+    PK_BP_PACK, PK_SWEEP_DCB_BITS, PK_SWEEP_DCB_RES, PK_SWEEP_STREAM, PK_COUNT
 };
 const char* const kProfNames[PK_COUNT] = {"init_spins", "couplings", "sweep_resident", "halfsweep_global",
                                           "observables", "pa_weights", "pa_reduce", "pa_draws", "pa_place",
@@ -62,7 +62,7 @@ const char* const kProfNames[PK_COUNT] = {"init_spins", "couplings", "sweep_resi
                                           "bitpack_halfsweep", "sweep_dcb", "sweep_msc", "swendsen_wang",
                                           "bitpack_strips", "sweep_strips", "pt_exchange", "sweep_bits",
                                           "bitpack_convert", "sweep_dcb_bits",
-                                          "sweep_dcb_resident"};
+                                          "sweep_dcb_resident", "sweep_stream"};
 
 // Device words of a context: 8 flags and counters, then the progress
 // counters of strip-resident sweeps (one per CTA, one CTA per SM).
@@ -165,6 +165,7 @@ struct gbmc_lattice {
     uint8_t* jbits;    // +-J bond planes [inst][3][N]
     uint8_t* jsplit;   // the same bonds per colour plane [inst][2][6][N/2] (L % 8 == 0)
     uint32_t* jb3;     // the same bonds as bit words of the bit-sliced 3D sweeps [inst][2][6][L^3 / 64]
+    uint32_t* stab;    // tables of the bit-stream sweeps: masks [5][PW], then +-J bond words [inst][2][6][PW]
     uint32_t* packed;  // bit-packed copy of the configuration for the strip-resident bit sweeps (int8 layout)
     int8_t* alt;       // second configuration buffer of the tiled large-lattice sweeps
     uint32_t* dcb_scratch;    // tile edges and progress counters of the resident double checkerboard
@@ -368,6 +369,10 @@ SweepJob base_job(const gbmc_lattice* l, const Tuning& tu) {
     J.jbits = l->jbits;
     J.jsplit = l->jsplit;
     J.jb3 = l->jb3;
+    if (l->stab) {
+        J.smask = l->stab;
+        J.sbond = l->d.model == GBMC_EA_PMJ ? l->stab + stream_mask_words((uint32_t)l->N) : nullptr;
+    }
     J.seed = l->d.seed;
     J.L = (uint32_t)l->d.L;
     J.N = (uint32_t)l->N;
@@ -466,18 +471,50 @@ bool job_takes_bits(const SweepLaunch& P, const SweepJob& J, const Tuning& tu, i
     return kernel == GBMC_KERNEL_BITS || tu.bits;
 }
 
+// Whether the bit-stream kernel takes a job the bit-sliced kernel does not: any
+// resident lattice, in AUTO mode only (BITS leaves what the bit-sliced kernel
+// does not support to the byte-plane kernel).
+bool job_takes_stream(const SweepJob& J, const Tuning& tu, int kernel) {
+    return kernel == GBMC_KERNEL_AUTO && tu.bits && J.smask;
+}
+
+// Whether the jobs of P that the bit-sliced kernel would take (AUTO mode) are so
+// few that the bit-stream kernel is faster: it spreads a copy's words over up to
+// four threads each and a whole block, where the bit-sliced kernel gives every
+// copy to one warp, p words per lane one after the other. The line lies at half a
+// warp per scheduler and word of a lane. Measured, 10 sweeps of R copies, us
+// (bit-sliced -> bit-stream): 2D L = 16 R = 1200 15.2 -> 10.8, R = 5000 19.9 -> 22.2;
+// L = 64 R = 1 31.5 -> 10.7, R = 600 31.6 -> 25.9, R = 1200 47.1 -> 51.2; L = 128 R = 1
+// 119 -> 31, R = 1200 168 -> 145; L = 256 R = 1 471 -> 79; 3D L = 8 R = 1200 18.1 ->
+// 15.1, R = 2500 23.6 -> 29.5; L = 16 R = 600 37.2 -> 30.1, R = 1200 53.3 -> 59.4.
+bool bits_jobs_small(const SweepLaunch& P, const std::vector<Tuning>& tu, int kernel, int sm_count) {
+    if (kernel != GBMC_KERNEL_AUTO) return false;
+    double warps = 0.0;
+    for (int j = 0; j < P.njobs; ++j) {
+        const SweepJob& J = P.jobs[j];
+        if (!job_takes_bits(P, J, tu[j], kernel)) continue;
+        if (!J.smask) return false;
+        warps += (double)J.n_inst * J.R * (J.N / 64u) / 32.0 / std::max(1.0, J.N / 2048.0 * (J.N / 2048.0));
+    }
+    return warps <= 0.53 * 4.0 * sm_count;
+}
+
 // Enqueues the sweep launches of P's jobs: the jobs the bit-sliced kernel
-// takes in one launch of it, the others in one byte-plane resident launch.
-// force_kernel: -1 takes the context's kernel mode.
+// takes in one launch of it, those the bit-stream kernel takes in one of that,
+// the others in one byte-plane resident launch. force_kernel: -1 takes the
+// context's kernel mode.
 gbmc_status launch_jobs(gbmc_ctx* ctx, const SweepLaunch& P0, const std::vector<Tuning>& tu,
                         int force_persistent = -1, int force_kernel = -1) {
     const int kernel = force_kernel >= 0 ? force_kernel : ctx->sweep_kernel;
-    SweepLaunch B = P0, Y = P0;
-    B.njobs = Y.njobs = 0;
+    SweepLaunch B = P0, S = P0, Y = P0;
+    B.njobs = S.njobs = Y.njobs = 0;
     std::vector<Tuning> ty;
+    const bool small = bits_jobs_small(P0, tu, kernel, ctx->sm_count);
     for (int j = 0; j < P0.njobs; ++j) {
-        if (job_takes_bits(P0, P0.jobs[j], tu[j], kernel)) {
+        if (!small && job_takes_bits(P0, P0.jobs[j], tu[j], kernel)) {
             B.jobs[B.njobs++] = P0.jobs[j];
+        } else if (job_takes_stream(P0.jobs[j], tu[j], kernel)) {
+            S.jobs[S.njobs++] = P0.jobs[j];
         } else {
             Y.jobs[Y.njobs++] = P0.jobs[j];
             ty.push_back(tu[j]);
@@ -486,6 +523,10 @@ gbmc_status launch_jobs(gbmc_ctx* ctx, const SweepLaunch& P0, const std::vector<
     if (B.njobs) {
         ProfScope ps_(ctx, PK_SWEEP_BITS);
         CUDA_TRY(launch_sweep_bits(B, ctx->stream));
+    }
+    if (S.njobs) {
+        ProfScope ps_(ctx, PK_SWEEP_STREAM);
+        CUDA_TRY(launch_sweep_stream(S, ctx->sm_count, ctx->stream));
     }
     if (Y.njobs == 0) return GBMC_OK;
     return launch_bytes(ctx, Y, ty, force_persistent);
@@ -755,6 +796,16 @@ gbmc_status lattice_init(gbmc_ctx* ctx, const gbmc_lattice_desc* d, void* spins_
             CUDA_TRY(launch_bits3_bonds(l->jbits, l->jb3, (uint32_t)d->L, d->n_instances, ctx->stream));
         }
     }
+    if (d->layout == GBMC_INT8 && tune(l).resident) {
+        const size_t words = stream_mask_words((uint32_t)N) + (l->jbits ? stream_bond_words((uint32_t)N) * d->n_instances : 0);
+        cudaError_t e = cudaMalloc(&l->stab, words * 4);
+        if (e != cudaSuccess) {
+            lattice_free(l);
+            return fail(GBMC_ERR_OOM, "cudaMalloc(bit-stream tables): %s", cudaGetErrorString(e));
+        }
+        CUDA_TRY(launch_stream_tables(l->jbits, l->stab, l->jbits ? l->stab + stream_mask_words((uint32_t)N) : nullptr,
+                                      d->dim, (uint32_t)d->L, d->n_instances, ctx->stream));
+    }
     {
         ProfScope ps_(ctx, PK_INIT);
         if (d->layout == GBMC_BITPACK)
@@ -775,6 +826,7 @@ gbmc_status lattice_free(gbmc_lattice* l) {
     if (l->jbits) cudaFree(l->jbits);
     if (l->jsplit) cudaFree(l->jsplit);
     if (l->jb3) cudaFree(l->jb3);
+    if (l->stab) cudaFree(l->stab);
     if (l->packed) cudaFree(l->packed);
     if (l->dcb_scratch) cudaFree(l->dcb_scratch);
     if (l->alt) cudaFree(l->alt);
@@ -2357,9 +2409,11 @@ gbmc_status gbmc_autotune(gbmc_ctx* ctx, const gbmc_lattice* l, double beta, uin
                 best_shape.persistent = true;
             }
         }
-        // the bit-sliced kernel, where it supports the lattice
-        if (st == GBMC_OK && bits_supported(l->d.dim, l->d.L) && (l->d.model != GBMC_EA_PMJ || l->jb3)) {
-            st = time_launches(ctx, P, tv, 0, e0, e1, &ms, GBMC_KERNEL_BITS);
+        // the bit-sliced kernel, where it supports the lattice, else the bit-stream kernel
+        const bool bits = bits_supported(l->d.dim, l->d.L) && (l->d.model != GBMC_EA_PMJ || l->jb3);
+        if (st == GBMC_OK && (bits || l->stab)) {
+            tv[0].bits = true;
+            st = time_launches(ctx, P, tv, 0, e0, e1, &ms, bits ? GBMC_KERNEL_BITS : GBMC_KERNEL_AUTO);
             if (st == GBMC_OK) {
                 ++n_cand;
                 if (ms < best) {

@@ -32,6 +32,7 @@
 //    lanes l -/+ 4.
 #include "bits.cuh"
 #include "check.cuh"
+#include "copies.cuh"
 #include "device.cuh"
 #include "internal.h"
 
@@ -60,30 +61,6 @@ __device__ __forceinline__ void copy_thresholds(const SweepJob& J, uint64_t slot
         T4 = J.thr[0];
         T8 = J.thr[1];
         T12 = J.thr[2];
-    }
-}
-
-// Energy and magnetisation of one copy after the last sweep (or of every
-// sweep when a series is asked for): lane 0 writes them and, for annealing
-// runs, adds them to the population's histogram, range and exact sums.
-__device__ __forceinline__ void record_copy(const SweepJob& J, uint64_t slot, uint32_t inst, uint32_t s, bool sweep,
-                                            bool last, int E, int M) {
-    const uint64_t ncopies = (uint64_t)J.n_inst * J.R;
-    if (J.Eser && sweep) J.Eser[(uint64_t)s * ncopies + slot] = E;
-    if (J.Mser && sweep) J.Mser[(uint64_t)s * ncopies + slot] = M;
-    if (!last) return;
-    if (J.E) J.E[slot] = E;
-    if (J.M) J.M[slot] = M;
-    if (J.hist) {
-        atomicAdd(&J.hist[(uint64_t)inst * J.nbins + (uint32_t)((E - J.e_lo) >> 2)], 1u);
-        atomicMin(&J.emin[inst], E);
-        atomicMax(&J.emax[inst], E);
-        unsigned long long* su = J.sums + (uint64_t)inst * 4;
-        const long long el = E, ml = M;
-        atomicAdd(&su[0], (unsigned long long)el);
-        atomicAdd(&su[1], (unsigned long long)(el * el));
-        atomicAdd(&su[2], (unsigned long long)(ml < 0 ? -ml : ml));
-        atomicAdd(&su[3], (unsigned long long)(ml * ml));
     }
 }
 
@@ -242,7 +219,8 @@ __global__ void __launch_bounds__(128) k_sweep_bits2(const __grid_constant__ Swe
                 U += __shfl_xor_sync(0xffffffffu, U, o);
                 D += __shfl_xor_sync(0xffffffffu, D, o);
             }
-            if (active && li == 0) record_copy(J, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
+            if (ROWS) record_copies(J, active && li == 0, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
+            else if (li == 0) record_copy(J, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
         }
     }
 
@@ -373,7 +351,7 @@ __global__ void __launch_bounds__(128) k_sweep_bits3(const __grid_constant__ Swe
                 D += __shfl_xor_sync(0xffffffffu, D, o);
             }
             // E = 2 (unsatisfied bonds of the colour-0 sites) - 3 N
-            if (active && z == 0) record_copy(J, slot, inst, s, sweep, last, 2 * U - 3 * (int)N, (int)N - 2 * D);
+            record_copies(J, active && z == 0, slot, inst, s, sweep, last, 2 * U - 3 * (int)N, (int)N - 2 * D);
         }
     }
 

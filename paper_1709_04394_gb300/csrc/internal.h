@@ -44,6 +44,10 @@ struct SweepJob {
     const uint32_t* nlive;    // variable populations: [n_inst] live copies (the first ones); null: R
     const uint32_t* jb3;      // +-J bonds of the bit-sliced 3D L = 8 sweep: [n_inst][2][6][8] words, bit 1
                               // where J = -1; null for J = 1
+    const uint32_t* smask;    // bit-stream sweeps: per-word masks [5][PW] of the lattice class (stream.cu)
+    const uint32_t* sbond;    // bit-stream sweeps: +-J bond words [n_inst][2][6][PW]; null for J = 1
+    uint32_t team;            // bit-stream sweeps: threads per team (rpc: groups of copies per team,
+                              // ctas_per_inst: groups per instance)
 };
 
 struct SweepLaunch {
@@ -175,6 +179,15 @@ cudaError_t launch_sweep_bits(const SweepLaunch& P, cudaStream_t s);
 // bits3_bond_words(L) words per instance.
 size_t bits3_bond_words(uint32_t L);
 cudaError_t launch_bits3_bonds(const uint8_t* jbits, uint32_t* jb3, uint32_t L, uint32_t n_inst, cudaStream_t s);
+
+// Bit-stream resident sweeps (stream.cu): any even L, the same results. Tables:
+// stream_mask_words(N) words per lattice class and, for +-J lattices,
+// stream_bond_words(N) words per instance.
+size_t stream_mask_words(uint32_t N);
+size_t stream_bond_words(uint32_t N);
+cudaError_t launch_stream_tables(const uint8_t* jbits, uint32_t* smask, uint32_t* sbond, int dim, uint32_t L,
+                                 uint32_t n_inst, cudaStream_t s);
+cudaError_t launch_sweep_stream(const SweepLaunch& P, int sm_count, cudaStream_t s);
 
 // Multi-spin-coded sweeps (2D ferromagnet, L % 16 == 0): jobs with rpc = 32 G
 // replicas per CTA; G in 1..4 groups of 32.

@@ -1,0 +1,718 @@
+// stream.cu -- checkerboard Metropolis sweeps (Sec. 3.1, Eq. (8)) of copies held
+// bit-sliced on chip for every even L, several copies per thread.
+//
+// A colour plane is one cyclic stream of its H = N / 2 sites in colour-rank
+// order (bit k & 31 of word k >> 5; s = L / 2 ranks per row, A = s L per slab of
+// a 3D lattice), whatever L is. The neighbours of the 32 sites of a word are
+// then windows of the other plane's stream at offsets -s, +s (y), -A, +A (z) and
+// single-bit shifts (x), with the row and slab ends taken from windows at
+// +-(s - 1) and +-(A - s) under per-word masks (k_stream_tables). Reads run up
+// to 31 bits past the end of the stream, so each plane keeps its first bits
+// again behind its last one (stream_extend).
+//
+// A thread updates the same word of C copies (C = 4, 2 or 1) of one instance
+// together. Window positions, masks and +-J bond words are worked out once for
+// the C copies, their words lie side by side in shared memory (one 128-bit load
+// for C = 4), and the Philox calls of the copies run in lockstep: they share
+// the counter q, hence the products of round 0 and of round 1's second word
+// (2 of 18 wide multiplies per call) and every round's key.
+//
+// Bound: the integer pipes together. Measured on sm_103a with independent
+// instructions and eight warps per scheduler, a three-input xor or a compare
+// takes 2.1 cycles of a scheduler, a wide 32 x 32 -> 64-bit multiply 4.3, and a mix
+// of both 2.1 per logic instruction + 2.2 per multiply: the two do not overlap. A
+// Philox call (4 sites) is 18 xors, 16.5 to 18 multiplies and 8 (2D) or 12 (3D)
+// threshold compares, about 95 to 105 cycles; the kernel runs at 107 to 109 (2D).
+// Replacing the carry compares by predicates, or moving them to the float adder,
+// left that unchanged. Site updates per ns before (byte planes; per-site loop where
+// L % 8 != 0) and after, theta = 10 sweeps per load: 2D L = 24 610 -> 1399, L = 96
+// 843 -> 1363, L = 10 286 -> 1090; 3D +-J L = 4 240 -> 1299, L = 10 248 -> 1268, L = 12
+// 240 -> 1194, L = 32 540 -> 1291. (L = 16, 32, 64 in 2D and L = 8, 16 in 3D stay on
+// bitsweep.cu, whose fixed sizes need no windows: 1475 / 1512 and 1323 / 1337 there
+// against 1437 / 1486 and 1317 / 1328 here.)
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <utility>
+
+#include "bits.cuh"
+#include "check.cuh"
+#include "copies.cuh"
+#include "device.cuh"
+#include "internal.h"
+
+namespace gbmc {
+
+namespace {
+
+constexpr uint32_t kStreamThreads = 128;      // threads per block with one-warp teams
+constexpr size_t kStreamSmem = 227 * 1024;   // shared memory of an SM
+constexpr uint32_t kStreamTeamWords = 3072;  // a one-warp team's share of shared memory, at most
+// largest block: 64 registers a thread for C = 1 (1024 threads), 128 for C = 2, 255 for C = 4
+constexpr uint32_t stream_max_threads(int C) { return C == 4 ? 256u : C == 2 ? 512u : 1024u; }
+
+// Philox calls of one copy in lockstep: with fewer copies per thread more calls of
+// the same copy keep as many independent chains in flight. Measured (site updates
+// per ns, 2D L = 96 / 3D +-J L = 10, large populations): C = 1: 1, 4, 8 calls 1143 /
+// 919, 1209 / 946, 1209 / 957; C = 2: 1, 2, 4 calls 1282 / 1097, 1230 / 1136, 1333 /
+// 1163; C = 4: 1 call (loop unrolled twice), 2 calls 1309 / 1270, 1296 / 1223.
+constexpr int stream_calls(int C) { return C == 4 ? 1 : 8 / C; }
+
+// C words (one per copy) loaded and stored together.
+template <int C>
+struct alignas(4 * C) Words {
+    uint32_t v[C];
+};
+
+struct StreamShape {
+    uint32_t L, s, A, H, PW, PWX;
+    uint32_t mh, h;  // valid bits of the last word: mask and count (1..32)
+};
+
+template <int DIM>
+__device__ __forceinline__ StreamShape stream_shape(uint32_t L, uint32_t N) {
+    StreamShape g;
+    g.L = L;
+    g.s = L >> 1;
+    g.A = DIM == 3 ? g.s * L : 0u;
+    g.H = N >> 1;
+    g.PW = (g.H + 31u) >> 5;
+    g.PWX = g.PW + 1u;
+    g.h = ((g.H - 1u) & 31u) + 1u;
+    g.mh = 0xFFFFFFFFu >> (32u - g.h);
+    return g;
+}
+
+// 32 bits of a stream from bit p: the two words that hold them.
+template <int C>
+struct Window {
+    Words<C> a, b;
+    uint32_t sh;
+    __device__ __forceinline__ void load(const Words<C>* pl, uint32_t p, uint32_t n_words) {
+        const uint32_t i = p >> 5;
+        a = pl[GBMC_IDX(i, n_words)];
+        b = pl[GBMC_IDX(i + 1u, n_words)];
+        sh = p & 31u;
+    }
+    // the window from bit p (at<0>) or p + 1 (at<1>: shift 1..32, 32 gives the upper word)
+    template <int PLUS>
+    __device__ __forceinline__ uint32_t at(int c) const {
+        return PLUS ? __funnelshift_rc(a.v[c], b.v[c], sh + 1u) : __funnelshift_r(a.v[c], b.v[c], sh);
+    }
+};
+
+__device__ __forceinline__ uint32_t sel(uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); }
+
+// Unsatisfied-bond masks of word w of colour c: d[k][copy], k in the order
+// (same-j x neighbour, other x neighbour, y - 1, y + 1, z - 1, z + 1).
+template <int DIM, bool EA, int C>
+__device__ __forceinline__ void stream_unsat(const StreamShape& g, const Words<C>* oth, const Words<C>& own, uint32_t w,
+                                             uint32_t colour, const uint32_t* __restrict__ mask,
+                                             const uint32_t* __restrict__ bond, uint32_t d[2 * DIM][C]) {
+    const uint32_t k0 = w << 5;
+    const uint32_t odd = __ldg(mask + w) ^ (colour ? 0xFFFFFFFFu : 0u);
+    const uint32_t edge = __ldg(mask + (1u + colour) * g.PW + w);
+    uint32_t j[2 * DIM];
+#pragma unroll
+    for (int k = 0; k < 2 * DIM; ++k) j[k] = EA ? __ldg(bond + k * g.PW + w) : 0u;
+    Window<C> up, dn;  // from k - s, and from k + s - 1
+    const uint32_t pu = k0 >= g.s ? k0 - g.s : k0 + g.H - g.s;
+    uint32_t pd = k0 + g.s - 1u;
+    if (pd >= g.H) pd -= g.H;
+    up.load(oth, pu, g.PWX);
+    dn.load(oth, pd, g.PWX);
+    {
+        const Words<C> same = oth[GBMC_IDX(w, g.PWX)];
+        const Words<C> prv = oth[w ? w - 1u : 0u];  // bit 0 of word 0 starts a row: its edge window is taken
+        const Words<C> nxt = oth[GBMC_IDX(w + 1u, g.PWX)];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            // the x neighbour not sharing j: j + 1 for odd x, j - 1 for even x; at
+            // the row's end the first (k - (s - 1)), resp. last (k + s - 1) site of the row
+            const uint32_t to_next = sel(edge, up.template at<1>(c), __funnelshift_r(same.v[c], nxt.v[c], 1));
+            const uint32_t to_prev = sel(edge, dn.template at<0>(c), __funnelshift_l(prv.v[c], same.v[c], 1));
+            d[0][c] = own.v[c] ^ same.v[c] ^ j[0];
+            d[1][c] = own.v[c] ^ sel(odd, to_next, to_prev) ^ j[1];
+        }
+    }
+    if constexpr (DIM == 2) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            d[2][c] = own.v[c] ^ up.template at<0>(c) ^ j[2];
+            d[3][c] = own.v[c] ^ dn.template at<1>(c) ^ j[3];
+        }
+    } else {
+        const uint32_t y0 = __ldg(mask + 3u * g.PW + w), yl = __ldg(mask + 4u * g.PW + w);
+        Window<C> a, b;
+        uint32_t p = k0 + g.A - g.s;
+        if (p >= g.H) p -= g.H;
+        a.load(oth, p, g.PWX);  // y = 0: row L - 1 of the slab
+        b.load(oth, k0 + g.s >= g.A ? k0 + g.s - g.A : k0 + g.s + g.H - g.A, g.PWX);  // y = L - 1: row 0
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            d[2][c] = own.v[c] ^ sel(y0, a.template at<0>(c), up.template at<0>(c)) ^ j[2];
+            d[3][c] = own.v[c] ^ sel(yl, b.template at<0>(c), dn.template at<1>(c)) ^ j[3];
+        }
+        p = k0 + g.A;
+        if (p >= g.H) p -= g.H;
+        a.load(oth, k0 >= g.A ? k0 - g.A : k0 + g.H - g.A, g.PWX);
+        b.load(oth, p, g.PWX);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            d[4][c] = own.v[c] ^ a.template at<0>(c) ^ j[4];
+            d[5][c] = own.v[c] ^ b.template at<0>(c) ^ j[5];
+        }
+    }
+}
+
+// Philox constants of one copy: round 1 before the q-dependent words.
+struct CopyKey {
+    uint32_t b1, u1, v1;
+};
+
+// Thread teams: one warp each, or the whole block for copies too large for a warp's share.
+__device__ __forceinline__ void team_sync(bool warp) {
+    if (warp) __syncwarp();
+    else __syncthreads();
+}
+
+// First bits of each plane again behind its last one.
+template <int C>
+__device__ __forceinline__ void stream_extend(uint32_t* plane, uint32_t n, const StreamShape& g, uint32_t tl,
+                                              uint32_t T) {
+    for (uint32_t i = tl; i < n * C; i += T) {
+        uint32_t* p = plane + (i / C) * g.PWX * C + i % C;
+        const uint32_t tail = p[(g.PW - 1u) * C] & g.mh;
+        const uint64_t e = tail | ((uint64_t)(g.PW == 1u ? tail : p[0]) << g.h);
+        p[(g.PW - 1u) * C] = (uint32_t)e;
+        p[g.PW * C] = (uint32_t)(e >> 32);
+    }
+}
+
+// A team of T threads (a warp, or the block) sweeps G groups of C copies;
+// item i of its n_groups * PW words is word i % PW of group i / PW. S = 4 (C = 1
+// only): four threads per word, each the eight sites of one byte of it (two
+// Philox calls), for launches too small to give every scheduler two warps.
+template <int DIM, bool EA, int C, int S, bool PT>
+__global__ void __launch_bounds__(stream_max_threads(C)) k_sweep_stream(const __grid_constant__ SweepLaunch P,
+                                                                        uint32_t smem_words) {
+    extern __shared__ __align__(16) uint32_t smw[];
+    int jid = 0;
+    while (jid + 1 < P.njobs && blockIdx.x >= P.cta_begin[jid + 1]) ++jid;
+    const SweepJob& J = P.jobs[jid];
+    const uint32_t T = J.team, G = J.rpc;
+    const bool warp = T == 32u;
+    const uint32_t tib = warp ? threadIdx.x >> 5 : 0u, tl = warp ? threadIdx.x & 31u : threadIdx.x;
+    const uint32_t ng = J.ctas_per_inst;  // groups per instance
+    const uint32_t n_all = J.n_inst * ng;
+    const uint64_t first = ((uint64_t)(blockIdx.x - P.cta_begin[jid]) * (blockDim.x / T) + tib) * G;
+    if (first >= n_all) return;  // the whole team; teams share no barrier
+    const uint32_t n = min(G, n_all - (uint32_t)first);
+    const StreamShape g = stream_shape<DIM>(J.L, J.N);
+    // shared memory of the team: planes [colour][group][word][copy], then per
+    // group [instance, first replica, active copies] and per copy [U, D], the
+    // replica it is read from and (tempering) its thresholds
+    uint32_t* const sm = smw + tib * smem_words;
+    const uint32_t plane = G * g.PWX * C;
+    uint32_t* const meta = sm + 2u * plane;
+    int* const acc = reinterpret_cast<int*>(meta + 3u * G);
+    uint32_t* const sfrom = meta + 3u * G + 2u * G * C;
+    uint32_t* const sthr = sfrom + G * C;
+    uint32_t any = 0;
+    for (uint32_t gi = tl; gi < n; gi += T) {
+        const uint32_t grp = (uint32_t)first + gi, inst = grp / ng, r0 = (grp - inst * ng) * C;
+        // variable populations: only the first nlive[inst] slots hold replicas
+        const uint32_t live = J.nlive ? J.nlive[inst] : J.R;
+        const uint32_t na = r0 < live ? min((uint32_t)C, live - r0) : 0u;
+        meta[3u * gi] = inst;
+        meta[3u * gi + 1u] = r0;
+        meta[3u * gi + 2u] = na;
+        any |= na;
+        for (uint32_t c = 0; c < C; ++c) {
+            acc[2u * (gi * C + c)] = acc[2u * (gi * C + c) + 1u] = 0;
+            if (c < na) sfrom[gi * C + c] = J.parent ? J.parent[(uint64_t)inst * J.R + r0 + c] : r0 + c;
+            if (PT && c < na) {
+                const uint32_t* th = J.thr_temp + 3ull * J.temp_of[(uint64_t)inst * J.R + r0 + c];
+                for (uint32_t k = 0; k < 3; ++k) sthr[3u * (gi * C + c) + k] = th[k];
+            } else if (PT) {
+                for (uint32_t k = 0; k < 3; ++k) sthr[3u * (gi * C + c) + k] = 0u;
+            }
+        }
+    }
+    if (warp ? !__any_sync(0xFFFFFFFFu, any != 0u) : !__syncthreads_or(any != 0u)) return;
+    team_sync(warp);
+
+    const uint32_t* mask = J.smask;
+    const uint8_t* odd_b = reinterpret_cast<const uint8_t*>(mask);
+    // ---- load: 16 sites in row-major order are 8 pairs (even x, odd x) = byte ch
+    // of the streams of even-x and of odd-x sites; a site of the even-x stream
+    // has colour 0 where its row's colour-0 sites have even x (odd mask bit 0) ----
+    const uint32_t nch = (J.N + 15u) >> 4;
+    const bool wide = (J.N & 15u) == 0u;
+    // four chunks per thread in flight
+    for (uint32_t i0 = tl; i0 < n * C * nch; i0 += 4u * T) {
+        uint4 v[4];
+        uint32_t at[4], chunk[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t i = i0 + k * T, cp = i / nch, ch = i - cp * nch, gi = cp / C, c = cp % C;
+            at[k] = 0xFFFFFFFFu;
+            if (i >= n * C * nch || c >= meta[3u * gi + 2u]) continue;
+            const uint64_t from = (uint64_t)meta[3u * gi] * J.R + sfrom[cp];
+            const int8_t* src = J.src + GBMC_IDX(from, (uint64_t)J.n_inst * J.R) * J.N + 16u * ch;
+            if (wide) {
+                v[k] = *reinterpret_cast<const uint4*>(src);
+            } else {  // copies start on 4-byte boundaries (N % 4 == 0), the last chunk is short
+                const uint32_t* s4 = reinterpret_cast<const uint32_t*>(src);
+                const uint32_t left = J.N - 16u * ch;
+                v[k].x = s4[0];
+                v[k].y = left > 4u ? s4[1] : 0u;
+                v[k].z = left > 8u ? s4[2] : 0u;
+                v[k].w = left > 12u ? s4[3] : 0u;
+            }
+            at[k] = ((GBMC_IDX(gi * g.PWX + (ch >> 2), G * g.PWX)) * C + c) * 4u + (ch & 3u);
+            chunk[k] = ch;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (at[k] == 0xFFFFFFFFu) continue;
+            uint32_t e0, o0, e1, o1;
+            pack8(v[k].x, v[k].y, e0, o0);
+            pack8(v[k].z, v[k].w, e1, o1);
+            const uint32_t ev = e0 | (e1 << 4), od = o0 | (o1 << 4), m = odd_b[chunk[k]];
+            uint8_t* p0 = reinterpret_cast<uint8_t*>(sm) + at[k];
+            p0[0] = (uint8_t)sel(m, od, ev);
+            p0[4u * plane] = (uint8_t)sel(m, ev, od);
+        }
+    }
+    team_sync(warp);
+    stream_extend<C>(sm, n, g, tl, T);
+    stream_extend<C>(sm + plane, n, g, tl, T);
+    team_sync(warp);
+
+    const uint32_t k0 = (uint32_t)J.seed, k1 = (uint32_t)(J.seed >> 32);
+    const bool want_final = J.E || J.M || J.hist;
+    const uint32_t items = n * g.PW, nsw = J.nsweeps;
+    static_assert(S == 1 || (S == 4 && C == 1), "");
+    constexpr int NQ = S == 4 ? 2 : stream_calls(C);
+    const uint32_t NB = 2u * DIM * g.PW;  // bond words per instance and colour
+    for (uint32_t s = 0; s <= nsw; ++s) {
+        if (s == nsw && nsw != 0) break;  // s == nsw: measurement-only pass when nothing is swept
+        const bool sweep = s < nsw;
+        for (uint32_t colour = 0; sweep && colour < 2; ++colour) {
+            for (uint32_t is = tl; is < items * S; is += T) {
+                const uint32_t i = is / S, part = is % S;
+                const uint32_t gi = G == 1u ? 0u : i / g.PW, w = i - gi * g.PW;
+                const uint32_t inst = meta[3u * gi], r0 = meta[3u * gi + 1u];
+                Words<C>* own = reinterpret_cast<Words<C>*>(sm + colour * plane + gi * g.PWX * C);
+                const Words<C>* oth = reinterpret_cast<const Words<C>*>(sm + (colour ^ 1u) * plane + gi * g.PWX * C);
+                Words<C> nw = own[w];
+                uint32_t ge[C], ea[C], eb[C];  // dE <= 0; dE = 4; dE = 8 (3D)
+                {
+                    uint32_t d[2 * DIM][C];
+                    stream_unsat<DIM, EA, C>(g, oth, nw, w, colour, mask,
+                                             EA ? J.sbond + ((uint64_t)inst * 2u + colour) * NB : nullptr, d);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        if constexpr (DIM == 2) {
+                            const uint32_t s1 = d[0][c] ^ d[1][c], c1 = d[0][c] & d[1][c];
+                            const uint32_t s2 = d[2][c] ^ d[3][c], c2 = d[2][c] & d[3][c];
+                            ge[c] = c1 | c2 | (s1 & s2);      // two or more unsatisfied bonds
+                            ea[c] = (s1 ^ s2) & ~ge[c];       // one
+                            eb[c] = 0u;
+                        } else {
+                            const uint32_t s1 = d[0][c] ^ d[1][c] ^ d[2][c], c1 = maj3(d[0][c], d[1][c], d[2][c]);
+                            const uint32_t s2 = d[3][c] ^ d[4][c] ^ d[5][c], c2 = maj3(d[3][c], d[4][c], d[5][c]);
+                            const uint32_t a0 = s1 ^ s2, t = s1 & s2;
+                            const uint32_t a1 = c1 ^ c2 ^ t, a2 = maj3(c1, c2, t);
+                            ge[c] = a2 | (a1 & a0);           // three or more
+                            ea[c] = a1 & ~(a0 | a2);          // two
+                            eb[c] = a0 & ~(a1 | a2);          // one
+                        }
+                    }
+                }
+                CopyKey ck[C];
+                uint32_t T4[C], T8[C], T12[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    uint32_t hi, lo, uh, ul;
+                    mulhilo_wide(kPhiloxM1, r0 + c, hi, lo);
+                    mulhilo_wide(kPhiloxM0, hi ^ (J.t0 + s) ^ k0, uh, ul);
+                    ck[c].b1 = lo ^ (k0 + kPhiloxW0);
+                    ck[c].u1 = uh ^ (k1 + kPhiloxW1);
+                    ck[c].v1 = ul;
+                    T4[c] = PT ? sthr[3u * (gi * C + c)] : J.thr[0];
+                    T8[c] = PT ? sthr[3u * (gi * C + c) + 1u] : J.thr[1];
+                    T12[c] = PT ? sthr[3u * (gi * C + c) + 2u] : J.thr[2];
+                }
+                const uint32_t x0 = c3_word(kPurposeMetro, colour, J.inst_base + inst) ^ k1;
+                uint32_t r4[C], r8[C], r12[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) r4[c] = r8[c] = r12[c] = 0u;
+#pragma unroll 2
+                for (uint32_t k = 0; k < 8u / S; k += NQ) {
+                    const uint32_t q = 8u * w + 2u * part + k;  // part: 0 unless S = 4
+                    uint4 v[NQ][C];
+#pragma unroll
+                    for (int m = 0; m < NQ; ++m) {
+                        uint32_t x, y, h1, l1;  // the same for every copy
+                        mulhilo_wide(kPhiloxM0, q + m, x, y);
+                        mulhilo_wide(kPhiloxM1, x ^ x0, h1, l1);
+#pragma unroll
+                        for (int c = 0; c < C; ++c) v[m][c] = make_uint4(h1 ^ ck[c].b1, l1, ck[c].u1 ^ y, ck[c].v1);
+                    }
+                    uint32_t ka = k0 + 2u * kPhiloxW0, kb = k1 + 2u * kPhiloxW1;
+#pragma unroll
+                    for (int round = 2; round < 10; ++round) {
+#pragma unroll
+                        for (int m = 0; m < NQ; ++m)
+#pragma unroll
+                            for (int c = 0; c < C; ++c) {
+                                uint4& u = v[m][c];
+                                uint32_t hi0, lo0, hi1, lo1;
+                                mulhilo_wide(kPhiloxM0, u.x, hi0, lo0);
+                                mulhilo_wide(kPhiloxM1, u.z, hi1, lo1);
+                                u = make_uint4(hi1 ^ u.y ^ ka, lo1, hi0 ^ u.w ^ kb, lo0);
+                            }
+                        ka += kPhiloxW0;
+                        kb += kPhiloxW1;
+                    }
+#pragma unroll
+                    for (int m = 0; m < NQ; ++m)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const uint4 u = v[m][c];
+                            if constexpr (DIM == 2) {
+                                accept_bits(r4[c], r8[c], T4[c], T8[c], u.x);
+                                accept_bits(r4[c], r8[c], T4[c], T8[c], u.y);
+                                accept_bits(r4[c], r8[c], T4[c], T8[c], u.z);
+                                accept_bits(r4[c], r8[c], T4[c], T8[c], u.w);
+                            } else {
+                                accept_bits3(r4[c], r8[c], r12[c], T4[c], T8[c], T12[c], u.x);
+                                accept_bits3(r4[c], r8[c], r12[c], T4[c], T8[c], T12[c], u.y);
+                                accept_bits3(r4[c], r8[c], r12[c], T4[c], T8[c], T12[c], u.z);
+                                accept_bits3(r4[c], r8[c], r12[c], T4[c], T8[c], T12[c], u.w);
+                            }
+                        }
+                }
+                if constexpr (S == 4) {
+                    const uint32_t sh = 8u * part, gb = ge[0] >> sh, ab = ea[0] >> sh, bb = eb[0] >> sh;
+                    const uint32_t a4 = __brev(r4[0]) >> 24, a8 = __brev(r8[0]) >> 24, a12 = __brev(r12[0]) >> 24;
+                    const uint32_t f = DIM == 2 ? gb | (ab & a4) | (~(gb | ab) & a8)
+                                                : gb | (ab & a4) | (bb & a8) | (~(gb | ab | bb) & a12);
+                    uint8_t* ob = reinterpret_cast<uint8_t*>(own) + part;
+                    const uint8_t nb = (uint8_t)((nw.v[0] >> sh) ^ f);
+                    ob[4u * w] = nb;  // the other bytes of the word belong to the neighbouring threads
+                    if (g.h == 32u && w == 0u) ob[4u * g.PW] = nb;
+                } else {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        uint32_t f;
+                        if constexpr (DIM == 2)
+                            f = ge[c] | (ea[c] & __brev(r4[c])) | (~(ge[c] | ea[c]) & __brev(r8[c]));
+                        else
+                            f = ge[c] | (ea[c] & __brev(r4[c])) | (eb[c] & __brev(r8[c])) |
+                                (~(ge[c] | ea[c] | eb[c]) & __brev(r12[c]));
+                        nw.v[c] ^= f;
+                    }
+                    own[w] = nw;
+                    if (g.h == 32u && w == 0u) own[g.PW] = nw;  // whole words: the extension is word 0 again
+                }
+            }
+            team_sync(warp);
+            if (g.h != 32u) {
+                stream_extend<C>(sm + colour * plane, n, g, tl, T);
+                team_sync(warp);
+            }
+        }
+        const bool last = sweep ? s + 1 == nsw : true;
+        if ((J.Eser && sweep) || (J.Mser && sweep) || (last && want_final)) {
+            // every bond has one colour-0 end: E = 2 (unsatisfied bonds of the colour-0 sites) - DIM N
+            for (uint32_t i0 = 0; i0 < items; i0 += T) {
+                const uint32_t i = i0 + tl;
+                int U[C], D[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) U[c] = D[c] = 0;
+                uint32_t gi = 0;
+                if (i < items) {
+                    gi = G == 1u ? 0u : i / g.PW;
+                    const uint32_t w = i - gi * g.PW, valid = w + 1u == g.PW ? g.mh : 0xFFFFFFFFu;
+                    const Words<C>* p0 = reinterpret_cast<const Words<C>*>(sm + gi * g.PWX * C);
+                    const Words<C>* p1 = reinterpret_cast<const Words<C>*>(sm + plane + gi * g.PWX * C);
+                    const Words<C> w0 = p0[w], w1 = p1[w];
+                    uint32_t d[2 * DIM][C];
+                    stream_unsat<DIM, EA, C>(g, p1, w0, w, 0u, mask,
+                                             EA ? J.sbond + (uint64_t)meta[3u * gi] * 2u * NB : nullptr, d);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+#pragma unroll
+                        for (int k = 0; k < 2 * DIM; ++k) U[c] += __popc(d[k][c] & valid);
+                        D[c] = __popc(w0.v[c] & valid) + __popc(w1.v[c] & valid);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    if (G == 1u) {  // one group: the warp's sum first
+                        const int u = __reduce_add_sync(0xFFFFFFFFu, U[c]), dd = __reduce_add_sync(0xFFFFFFFFu, D[c]);
+                        if ((threadIdx.x & 31u) == 0u) {
+                            atomicAdd(acc + 2 * c, u);
+                            atomicAdd(acc + 2 * c + 1, dd);
+                        }
+                    } else if (i < items) {
+                        atomicAdd(acc + 2u * (gi * C + c), U[c]);
+                        atomicAdd(acc + 2u * (gi * C + c) + 1u, D[c]);
+                    }
+                }
+            }
+            team_sync(warp);
+            for (uint32_t i0 = 0; i0 < n * C; i0 += T) {  // whole warps (record_copies)
+                const uint32_t i = i0 + tl, gi = i < n * C ? i / C : 0u, c = i % C, inst = meta[3u * gi];
+                const bool has = i < n * C && c < meta[3u * gi + 2u];
+                record_copies(J, has, (uint64_t)inst * J.R + meta[3u * gi + 1u] + c, inst, s, sweep, last,
+                              has ? 2 * acc[2u * i] - DIM * (int)J.N : 0, has ? (int)J.N - 2 * acc[2u * i + 1u] : 0);
+                if (i < n * C) acc[2u * i] = acc[2u * i + 1u] = 0;
+            }
+            team_sync(warp);
+        }
+    }
+
+    // ---- store ----
+    if (nsw > 0 || J.dst != J.src || J.parent) {
+        for (uint32_t i = tl; i < n * C * nch; i += T) {
+            const uint32_t cp = i / nch, ch = i - cp * nch, gi = cp / C, c = cp % C;
+            if (c >= meta[3u * gi + 2u]) continue;
+            const uint8_t* p0 =
+                reinterpret_cast<const uint8_t*>(sm + (GBMC_IDX(gi * g.PWX + (ch >> 2), G * g.PWX)) * C + c) + (ch & 3u);
+            const uint32_t a = p0[0], b = p0[4u * plane], m = odd_b[ch];
+            const uint32_t ev = sel(m, b, a), od = sel(m, a, b);
+            const uint2 lo = unpack8(ev & 15u, od & 15u), hi = unpack8(ev >> 4, od >> 4);
+            const uint64_t slot = (uint64_t)meta[3u * gi] * J.R + meta[3u * gi + 1u] + c;
+            int8_t* dst = J.dst + slot * J.N + 16u * ch;
+            if (wide) {
+                *reinterpret_cast<uint4*>(dst) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+            } else {
+                uint32_t* d4 = reinterpret_cast<uint32_t*>(dst);
+                const uint32_t left = J.N - 16u * ch;
+                d4[0] = lo.x;
+                if (left > 4u) d4[1] = lo.y;
+                if (left > 8u) d4[2] = hi.x;
+                if (left > 12u) d4[3] = hi.y;
+            }
+        }
+    }
+}
+
+// Per-word masks of a lattice class, [5][PW]: the sites whose colour-0 row starts
+// at odd x; the row ends whose x neighbour wraps around, for colour 0 and for
+// colour 1; the sites with y = 0; those with y = L - 1. Bits past the stream's
+// end are 0. With +-J bonds, per instance [2][6][PW] bond words: bit 1 where the
+// bond from the colour-c site to its k-th neighbour (order of stream_unsat) has
+// J = -1 (jbits: [inst][mu][site] bytes, 1 where the forward bond has J = -1).
+__global__ void k_stream_tables(const uint8_t* jbits, uint32_t* smask, uint32_t* sbond, uint32_t dim, uint32_t L,
+                                uint32_t N, uint32_t n_inst) {
+    const uint32_t s = L >> 1, H = N >> 1, PW = (H + 31u) >> 5;
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (i < 5u * PW) {
+        const uint32_t t = (uint32_t)i / PW, w = (uint32_t)i % PW;
+        uint32_t word = 0;
+        for (uint32_t b = 0; b < 32u && 32u * w + b < H; ++b) {
+            const uint32_t k = 32u * w + b, row = k / s, j = k - row * s;
+            const uint32_t y = row % L, z = dim == 3 ? row / L : 0u;  // 2D: row < L
+            const uint32_t o = (y + z) & 1u;
+            bool on;
+            switch (t) {
+                case 0: on = o; break;
+                case 1: on = o ? j == s - 1u : j == 0u; break;
+                case 2: on = o ? j == 0u : j == s - 1u; break;
+                case 3: on = y == 0u; break;
+                default: on = y == L - 1u; break;
+            }
+            word |= (on ? 1u : 0u) << b;
+        }
+        smask[i] = word;
+    }
+    if (sbond && i < 12ull * n_inst * PW) {
+        const uint32_t w = (uint32_t)(i % PW), k = (uint32_t)(i / PW % 6u), c = (uint32_t)(i / (6u * PW) % 2u);
+        const uint8_t* jx = jbits + i / (12ull * PW) * 3u * N;
+        const uint8_t *jy = jx + N, *jz = jx + 2u * N;
+        uint32_t word = 0;
+        for (uint32_t b = 0; b < 32u && 32u * w + b < H; ++b) {
+            const uint32_t kk = 32u * w + b, row = kk / s, y = row % L, z = row / L;
+            const uint32_t o = (y + z + c) & 1u, x = 2u * (kk - row * s) + o, site = row * L + x;
+            const uint32_t xm = row * L + (x ? x - 1u : L - 1u);
+            uint32_t bond;
+            switch (k) {
+                case 0: bond = o ? jx[xm] : jx[site]; break;
+                case 1: bond = o ? jx[site] : jx[xm]; break;
+                case 2: bond = jy[(z * L + (y ? y - 1u : L - 1u)) * L + x]; break;
+                case 3: bond = jy[site]; break;
+                case 4: bond = jz[((z ? z - 1u : L - 1u) * L + y) * L + x]; break;
+                default: bond = jz[site]; break;
+            }
+            word |= (bond ? 1u : 0u) << b;
+        }
+        sbond[i] = word;
+    }
+}
+
+// Words of a team's shared memory for G groups of C copies.
+uint32_t stream_smem_words(uint32_t N, uint32_t G, uint32_t C, bool pt) {
+    const uint32_t PWX = (N / 2u + 31u) / 32u + 1u;
+    return (2u * G * PWX * C + 3u * G + 3u * G * C + (pt ? 3u * G * C : 0u) + 3u) & ~3u;
+}
+
+// How a launch spreads its jobs: C copies per thread, and per job teams of T
+// threads (32: four one-warp teams per block; else the block) with G groups of C
+// copies each. The estimate is in cycles of a scheduler per half-sweep: a pass of
+// a warp over its words issues for `pass` cycles (the multiply and logic pipes)
+// but takes `lat` by itself, so a scheduler with w warps at work spends
+// max(pass, lat / w) per pass; on top of the average comes the longest team, for
+// what the last teams leave idle.
+struct StreamPlan {
+    int C = 1, split = 1;
+    uint32_t threads = kStreamThreads;
+    uint32_t T[kMaxJobs] = {}, G[kMaxJobs] = {};
+    double cost = 1e300;
+};
+
+StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_count) {
+    // measured: 2D L = 64 with 10^5 copies (pass), L = 36 and 68 with one warp per scheduler (lat)
+    const double pass = C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 980.0 : 420.0;
+    const double lat = C == 4 ? 9000.0 : C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0;
+    const double by_regs = C == 4 ? 5.0 : 8.0;  // warps per scheduler the registers allow
+    const double schedulers = 4.0 * sm_count;
+    StreamPlan S;
+    S.C = C;
+    S.split = split;
+    double total = 0.0, longest = 0.0;
+    for (int j = 0; j < P.njobs; ++j) {
+        const SweepJob& J = P.jobs[j];
+        const uint32_t PW = (J.N / 2u + 31u) / 32u * (uint32_t)split;  // items of a copy
+        const double groups = (double)J.n_inst * ((J.R + C - 1u) / C);
+        double best = 1e300, best_sum = 0.0, best_len = 0.0;
+        auto consider = [&](uint32_t T, uint32_t G) {
+            const double p = (double)((G * PW + T - 1u) / T);
+            const double share = std::ceil(groups / G) * (T / 32u) / schedulers;
+            const uint32_t warps = T == 32u ? kStreamThreads / 32u : T / 32u;
+            const size_t smem = (size_t)stream_smem_words(J.N, G, C, pt) * 4u * (T == 32u ? warps : 1u);
+            const double fit = std::floor((double)kStreamSmem / smem) * warps / 4.0;
+            const double w = std::max(1.0, std::min(share, std::min(by_regs, fit)));
+            const double step = std::max(pass, lat / w) + (T == 32u ? 0.0 : 60.0);
+            const double sum = p * share * step, len = p * step;
+            if (sum + len < best * 0.98) {
+                best = sum + len;
+                best_sum = sum;
+                best_len = len;
+                S.T[j] = T;
+                S.G[j] = G;
+            }
+        };
+        // one-warp teams; larger copies, and a single lattice with too few copies
+        // to give every scheduler work, take whole blocks
+        for (uint32_t G = 1; G <= 32u && stream_smem_words(J.N, G, C, pt) <= kStreamTeamWords; ++G) consider(32u, G);
+        if (P.njobs == 1)
+            for (uint32_t T = 64u; T <= stream_max_threads(C) && T < PW + 32u; T += 32u) consider(T, 1u);
+        if (S.T[j] == 0u) consider(kStreamThreads, 1u);
+        total += best_sum;
+        longest = std::max(longest, best_len);
+    }
+    if (P.njobs == 1 && S.T[0] != 32u) S.threads = S.T[0];
+    S.cost = total + longest;
+    return S;
+}
+
+template <int DIM, bool EA, int C, int SP, bool PT>
+cudaError_t launch_stream(const SweepLaunch& P0, const StreamPlan& S, cudaStream_t st) {
+    SweepLaunch P = P0;
+    uint64_t total = 0;
+    size_t smem = 0;
+    uint32_t warp_words = 0;
+    for (int j = 0; j < P.njobs; ++j) {
+        SweepJob& J = P.jobs[j];
+        J.ctas_per_inst = (J.R + C - 1u) / C;  // groups per instance
+        J.team = S.T[j];
+        J.rpc = S.G[j];
+        const uint64_t groups = (uint64_t)J.n_inst * J.ctas_per_inst;
+        if (groups > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+        if (J.team == 32u) warp_words = std::max(warp_words, stream_smem_words(J.N, J.rpc, C, PT));
+        else smem = std::max(smem, (size_t)stream_smem_words(J.N, 1u, C, PT) * 4u);
+        const uint64_t teams = (groups + J.rpc - 1u) / J.rpc, per_block = S.threads / J.team;
+        P.cta_begin[j] = (uint32_t)total;
+        total += (teams + per_block - 1u) / per_block;
+        if (total > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    }
+    smem = std::max(smem, (size_t)warp_words * 4u * (S.threads / 32u));
+    P.cta_begin[P.njobs] = (uint32_t)total;
+    P.total = (uint32_t)total;
+    if (total == 0) return cudaSuccess;
+    auto kern = k_sweep_stream<DIM, EA, C, SP, PT>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kern<<<(uint32_t)total, S.threads, smem, st>>>(P, warp_words);
+    count_launch();
+    return cudaGetLastError();
+}
+
+template <int DIM, bool EA>
+cudaError_t launch_stream_c(const SweepLaunch& P, const StreamPlan& S, bool pt, cudaStream_t st) {
+    if (S.C == 4) return pt ? launch_stream<DIM, EA, 4, 1, true>(P, S, st) : launch_stream<DIM, EA, 4, 1, false>(P, S, st);
+    if (S.C == 2) return pt ? launch_stream<DIM, EA, 2, 1, true>(P, S, st) : launch_stream<DIM, EA, 2, 1, false>(P, S, st);
+    if (S.split == 4)
+        return pt ? launch_stream<DIM, EA, 1, 4, true>(P, S, st) : launch_stream<DIM, EA, 1, 4, false>(P, S, st);
+    return pt ? launch_stream<DIM, EA, 1, 1, true>(P, S, st) : launch_stream<DIM, EA, 1, 1, false>(P, S, st);
+}
+
+}  // namespace
+
+size_t stream_mask_words(uint32_t N) { return 5ull * ((N / 2u + 31u) / 32u); }
+size_t stream_bond_words(uint32_t N) { return 12ull * ((N / 2u + 31u) / 32u); }
+
+cudaError_t launch_stream_tables(const uint8_t* jbits, uint32_t* smask, uint32_t* sbond, int dim, uint32_t L,
+                                 uint32_t n_inst, cudaStream_t s) {
+    const uint32_t N = L * L * (dim == 3 ? L : 1u);
+    uint64_t n = stream_mask_words(N);
+    if (sbond && stream_bond_words(N) * n_inst > n) n = stream_bond_words(N) * n_inst;
+    k_stream_tables<<<(uint32_t)((n + 127u) / 128u), 128, 0, s>>>(jbits, smask, sbond, (uint32_t)dim, L, N, n_inst);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_stream(const SweepLaunch& P0, int sm_count, cudaStream_t s) {
+    SweepLaunch P = P0;
+    // largest copies first: their blocks are dispatched first, shortening the tail
+    for (int a = 1; a < P.njobs; ++a)
+        for (int b = a; b > 0 && P.jobs[b].N > P.jobs[b - 1].N; --b) std::swap(P.jobs[b], P.jobs[b - 1]);
+    bool pt = false;
+    for (int j = 0; j < P.njobs; ++j) {
+        if (!P.jobs[j].smask || (P.ea && !P.jobs[j].sbond)) return cudaErrorInvalidValue;
+        pt = pt || P.jobs[j].temp_of != nullptr;
+    }
+    // the plan depends only on these numbers; a run's launches repeat the last ones
+    struct Key {
+        uint32_t head[4], job[kMaxJobs][3];
+    };
+    static thread_local Key last = {};
+    static thread_local StreamPlan S;
+    Key key = {};
+    key.head[0] = (uint32_t)P.njobs, key.head[1] = (uint32_t)sm_count, key.head[2] = pt, key.head[3] = (uint32_t)P.dim;
+    for (int j = 0; j < P.njobs; ++j)
+        key.job[j][0] = P.jobs[j].N, key.job[j][1] = P.jobs[j].R, key.job[j][2] = P.jobs[j].n_inst;
+    if (std::memcmp(&key, &last, sizeof(key)) != 0) {
+        S = stream_plan(P, 1, 4, pt, sm_count);
+        for (int C = 4; C >= 1; C >>= 1) {
+            // a group's planes at most 36 KB, so that an SM holds six blocks
+            if (C > 1 && stream_smem_words(P.jobs[0].N, 1u, (uint32_t)C, pt) * 4u > 36u * 1024u) continue;
+            const StreamPlan t = stream_plan(P, C, 1, pt, sm_count);
+            if (t.cost < S.cost) S = t;
+        }
+        last = key;
+    }
+    if (P.dim == 2 && !P.ea) return launch_stream_c<2, false>(P, S, pt, s);
+    if (P.dim == 3 && !P.ea) return launch_stream_c<3, false>(P, S, pt, s);
+    if (P.dim == 3 && P.ea) return launch_stream_c<3, true>(P, S, pt, s);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace gbmc
