@@ -76,6 +76,8 @@ cudaError_t launch_jbits_to_int8(const uint8_t* jbits, int8_t* out, uint32_t N, 
                                  cudaStream_t s);
 cudaError_t launch_observables(const int8_t* spins, const uint8_t* jbits, int dim, uint32_t L,
                                uint32_t n_inst, uint32_t R, int32_t* E, int32_t* M, cudaStream_t s);
+// a[i] = b[i] = 0, i < n; either may be null.
+cudaError_t launch_zero2(int32_t* a, int32_t* b, uint64_t n, cudaStream_t s);
 
 // Bit-packed 2D ferromagnet layout (one bit per spin, per-colour planes).
 cudaError_t launch_bp_init(uint32_t* P, uint32_t L, uint64_t copies, uint32_t R, uint32_t inst_base, uint64_t seed,
