@@ -110,9 +110,15 @@ gbmc_status gbmc_set_resample_mode(gbmc_ctx *ctx, int32_t fused);
  * all sweeps of a metropolis_sweeps call without E/M series as one cooperative
  * launch, each thread block keeping a strip of rows in shared memory and
  * trading its first and last rows with its neighbours through global memory
- * after every half-sweep (bounded waits; GBMC_ERR_TIMEOUT if one runs out);
- * GRID uses the per-launch kernels (halo tiles of up to 4 sweeps, resp. one
- * launch per half-sweep). Double-checkerboard sweeps with bit-sliced tiles
+ * after every half-sweep (bounded waits; GBMC_ERR_TIMEOUT if one runs out).
+ * Other lattices too large for shared memory (any even L, 3D too), calls with
+ * E/M series, and few large copies that would fit: AUTO and PERSISTENT convert
+ * the configuration to tagged bit words in a library buffer (N / 4 bytes per copy,
+ * kept with the lattice), run all sweeps of the call, series included, as one
+ * cooperative launch with the same bounded waits, and convert it back, unless the
+ * call is only a sweep or two. GRID uses the per-launch kernels (halo tiles of up
+ * to 4 sweeps, resp. one launch per half-sweep), and so does the BYTES kernel mode
+ * where its strips do not apply. Double-checkerboard sweeps with bit-sliced tiles
  * (metropolis_sweeps_dcb): PERSISTENT runs every round of a call in one
  * launch whenever all tile pairs fit on the device at once, GRID one launch
  * per coarse colour and round, AUTO the first for small k (k <= 3 with tiles

@@ -54,7 +54,7 @@ enum ProfKind {
     PK_INIT, PK_COUPLINGS, PK_SWEEP_RES, PK_HALFSWEEP, PK_OBS, PK_PA_WEIGHTS, PK_PA_REDUCE,
     PK_PA_DRAWS, PK_PA_PLACE, PK_PA_RECORD, PK_PA_RESET, PK_SWEEP_TILES, PK_SCHEDULE, PK_PA_FUSED,
     PK_BP_HALFSWEEP, PK_SWEEP_DCB, PK_SWEEP_MSC, PK_SW, PK_BP_STRIPS, PK_SWEEP_STRIPS, PK_PT_EXCHANGE, PK_SWEEP_BITS,
-    PK_BP_PACK, PK_SWEEP_DCB_BITS, PK_SWEEP_DCB_RES, PK_SWEEP_STREAM, PK_COUNT
+    PK_BP_PACK, PK_SWEEP_DCB_BITS, PK_SWEEP_DCB_RES, PK_SWEEP_STREAM, PK_STREAM_STRIPS, PK_COUNT
 };
 const char* const kProfNames[PK_COUNT] = {"init_spins", "couplings", "sweep_resident", "halfsweep_global",
                                           "observables", "pa_weights", "pa_reduce", "pa_draws", "pa_place",
@@ -62,7 +62,7 @@ const char* const kProfNames[PK_COUNT] = {"init_spins", "couplings", "sweep_resi
                                           "bitpack_halfsweep", "sweep_dcb", "sweep_msc", "swendsen_wang",
                                           "bitpack_strips", "sweep_strips", "pt_exchange", "sweep_bits",
                                           "bitpack_convert", "sweep_dcb_bits",
-                                          "sweep_dcb_resident", "sweep_stream"};
+                                          "sweep_dcb_resident", "sweep_stream", "stream_strips"};
 
 // Device words of a context: 8 flags and counters, then the progress
 // counters of strip-resident sweeps (one per CTA, one CTA per SM).
@@ -167,6 +167,7 @@ struct gbmc_lattice {
     uint32_t* jb3;     // the same bonds as bit words of the bit-sliced 3D sweeps [inst][2][6][L^3 / 64]
     uint32_t* stab;    // tables of the bit-stream sweeps: masks [5][PW], then +-J bond words [inst][2][6][PW]
     uint32_t* packed;  // bit-packed copy of the configuration for the strip-resident bit sweeps (int8 layout)
+    uint64_t* tagged;  // the same beside tags, for the sweeps of streamstrips.cu (either layout)
     int8_t* alt;       // second configuration buffer of the tiled large-lattice sweeps
     uint32_t* dcb_scratch;    // tile edges and progress counters of the resident double checkerboard
     size_t dcb_scratch_bytes;
@@ -796,7 +797,7 @@ gbmc_status lattice_init(gbmc_ctx* ctx, const gbmc_lattice_desc* d, void* spins_
             CUDA_TRY(launch_bits3_bonds(l->jbits, l->jb3, (uint32_t)d->L, d->n_instances, ctx->stream));
         }
     }
-    if (d->layout == GBMC_INT8 && tune(l).resident) {
+    if (d->layout == GBMC_INT8 && (d->dim == 3 || tune(l).resident)) {
         const size_t words = stream_mask_words((uint32_t)N) + (l->jbits ? stream_bond_words((uint32_t)N) * d->n_instances : 0);
         cudaError_t e = cudaMalloc(&l->stab, words * 4);
         if (e != cudaSuccess) {
@@ -828,6 +829,7 @@ gbmc_status lattice_free(gbmc_lattice* l) {
     if (l->jb3) cudaFree(l->jb3);
     if (l->stab) cudaFree(l->stab);
     if (l->packed) cudaFree(l->packed);
+    if (l->tagged) cudaFree(l->tagged);
     if (l->dcb_scratch) cudaFree(l->dcb_scratch);
     if (l->alt) cudaFree(l->alt);
     if (l->sw_bonds) cudaFree(l->sw_bonds);
@@ -915,6 +917,82 @@ gbmc_status lattice_couplings_out(gbmc_ctx* ctx, const gbmc_lattice* l, int8_t* 
     return GBMC_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Whether a call's sweeps run as one cooperative launch over bit planes in global
+// memory (streamstrips.cu), with a conversion before and after (about 6 us). Lattices
+// too large for shared memory: unless the call is so short that a launch per
+// half-sweep (4.1 us) costs less; those that fit, when they are so few and so large
+// that a block per copy leaves most of the device idle. Measured, us per call:
+// L = 520 n = 2 17.0 -> 16.5, n = 4 32.9 -> 22.6, n = 50 412 -> 162; L = 1000 n = 2
+// 17.0 -> 19.3, n = 50 412 -> 208, with E and M of every sweep 4894 -> 197; L = 4000
+// n = 2 90.6 -> 49.7, n = 50 2256 -> 754; 3D +-J L = 48 n = 50 412 -> 260; one copy of
+// L = 256 (a block: 79 us per 10 sweeps) n = 10 79 -> 35, of L = 128 n = 50 154 -> 123;
+// bit-packed L = 448 n = 2 17.0 -> 16.5, n = 50 412 -> 162.
+bool takes_stream_strips(const gbmc_ctx* ctx, const gbmc_lattice* l, const Tuning& tu, uint32_t n_sweeps, bool series) {
+    if (ctx->launch_mode == GBMC_LAUNCH_GRID || !ctx->coop || n_sweeps > 0x3FFFFFFFu) return false;
+    if (n_sweeps < 2 || (l->d.dim == 2 && l->d.L < 64)) return false;
+    if (l->d.layout == GBMC_BITPACK) return l->ncopies <= (uint64_t)ctx->sm_count / 8;
+    if (ctx->sweep_kernel == GBMC_KERNEL_BYTES || (l->d.dim == 3 && !l->stab)) return false;
+    if (!tu.resident) return series || n_sweeps >= 3 || l->N * l->ncopies >= 1u << 21;
+    if (ctx->sweep_kernel != GBMC_KERNEL_AUTO || !tu.bits) return false;
+    // words per plane, less where other copies keep their multiprocessors busy
+    const double words = l->N / 64.0 * (1.0 - (double)l->ncopies / ctx->sm_count);
+    return 4 * l->ncopies <= (uint64_t)ctx->sm_count && words >= 250.0 && n_sweeps >= (words >= 512.0 ? 4u : 8u);
+}
+
+gbmc_status stream_strips_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint32_t n_sweeps, int32_t* E_series,
+                                 int32_t* M_series) {
+    uint32_t thr[3];
+    thresholds(beta, thr);
+    StreamStrips S;
+    std::memset(&S, 0, sizeof(S));
+    if (l->d.dim == 3) {
+        S.mask = l->stab;
+        S.bond = l->jbits ? l->stab + stream_mask_words((uint32_t)l->N) : nullptr;
+    }
+    const uint64_t words = l->ncopies * stream_plane_words((uint32_t)l->N);
+    if (!l->tagged) {
+        cudaError_t e = cudaMalloc(&l->tagged, words * 8);
+        if (e != cudaSuccess) return fail(GBMC_ERR_OOM, "cudaMalloc(packed copy): %s", cudaGetErrorString(e));
+    }
+    auto convert = [&](bool pack) -> cudaError_t {
+        ProfScope ps_(ctx, PK_BP_PACK);
+        if (l->d.layout == GBMC_BITPACK) return launch_stream_words((uint32_t*)l->cur, l->tagged, words, pack, ctx->stream);
+        return launch_stream_convert(l->cur, l->tagged, S.mask, l->d.dim, (uint32_t)l->d.L, l->ncopies, pack, ctx->stream);
+    };
+    CUDA_TRY(convert(true));
+    S.P = l->tagged;
+    S.err = ctx->words + 1;
+    S.Eser = E_series;
+    S.Mser = M_series;
+    S.budget = ctx->budget;
+    S.seed = l->d.seed;
+    S.L = (uint32_t)l->d.L;
+    S.N = (uint32_t)l->N;
+    S.R = l->d.n_replicas;
+    S.inst_base = l->d.instance_base;
+    S.t0 = l->t;
+    S.n_half = 2 * n_sweeps;
+    S.T4 = thr[0];
+    S.T8 = thr[1];
+    S.T12 = thr[2];
+    S.phantom = ctx->phantom;
+    {
+        ProfScope ps_(ctx, PK_STREAM_STRIPS);
+        CUDA_TRY(launch_stream_strips(S, l->d.dim, l->ncopies, ctx->sm_count, ctx->stream));
+    }
+    CUDA_TRY(convert(false));
+    l->t += n_sweeps;
+    return GBMC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 gbmc_status metropolis_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint32_t n_sweeps, int32_t* E_series,
                               int32_t* M_series) {
     if (!ctx || !l) return fail(GBMC_ERR_ARG, "NULL argument");
@@ -956,6 +1034,8 @@ gbmc_status metropolis_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint3
             l->t += n_sweeps;
             return GBMC_OK;
         }
+        if (takes_stream_strips(ctx, l, Tuning{}, n_sweeps, E_series || M_series))
+            return stream_strips_sweeps(ctx, l, beta, n_sweeps, E_series, M_series);
         for (uint32_t s = 0; s < n_sweeps; ++s) {
             for (uint32_t colour = 0; colour < 2; ++colour) {
                 ProfScope ps_(ctx, PK_BP_HALFSWEEP);
@@ -1024,6 +1104,8 @@ gbmc_status metropolis_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint3
             return GBMC_OK;
         }
     }
+    if (takes_stream_strips(ctx, l, tu, n_sweeps, E_series || M_series))
+        return stream_strips_sweeps(ctx, l, beta, n_sweeps, E_series, M_series);
     // strips of rows resident in shared memory for the whole call (large 2D ferromagnets, no E/M series)
     uint32_t sGc = 0, srmax = 0, sthreads = 0;
     size_t ssmem = 0;

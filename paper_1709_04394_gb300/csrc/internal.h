@@ -191,6 +191,30 @@ cudaError_t launch_stream_tables(const uint8_t* jbits, uint32_t* smask, uint32_t
                                  uint32_t n_inst, cudaStream_t s);
 cudaError_t launch_sweep_stream(const SweepLaunch& P, int sm_count, cudaStream_t s);
 
+// Large lattices, one bit per spin, every half-sweep of a call in one cooperative
+// launch (streamstrips.cu; 2D: L >= 64). P: per copy two planes of
+// stream_plane_words(N) / 2 words beside their tags, as written by the conversions;
+// mask, bond: the tables of launch_stream_tables (mask in 3D only, bond: null for
+// J = 1). Eser / Mser: null or [n_half / 2][ncopies]. A wait that outlasts `budget`
+// cycles raises *err. Gc, edge, copy0, ncopies are set by the launch.
+struct StreamStrips {
+    uint64_t* P;
+    const uint32_t* mask;
+    const uint32_t* bond;
+    unsigned int* err;
+    int32_t* Eser;
+    int32_t* Mser;
+    long long budget;
+    uint64_t seed, ncopies;
+    uint32_t L, N, R, inst_base, t0, n_half, T4, T8, T12, phantom;
+    uint32_t Gc, edge, copy0;
+};
+size_t stream_plane_words(uint32_t N);
+cudaError_t launch_stream_convert(int8_t* spins, uint64_t* P, const uint32_t* mask, int dim, uint32_t L, uint64_t copies,
+                                  bool pack, cudaStream_t s);
+cudaError_t launch_stream_words(uint32_t* words, uint64_t* P, uint64_t n, bool pack, cudaStream_t s);
+cudaError_t launch_stream_strips(const StreamStrips& P, int dim, uint64_t copies, int sm_count, cudaStream_t s);
+
 // Multi-spin-coded sweeps (2D ferromagnet, L % 16 == 0): jobs with rpc = 32 G
 // replicas per CTA; G in 1..4 groups of 32.
 size_t msc_smem_bytes(uint32_t N, uint32_t G);
