@@ -41,12 +41,15 @@ __device__ __forceinline__ void record_copy(const SweepJob& J, uint64_t slot, ui
 __device__ __forceinline__ void record_copies(const SweepJob& J, bool has, uint64_t slot, uint32_t inst, uint32_t s,
                                               bool sweep, bool last, int E, int M) {
     constexpr uint32_t kAll = 0xFFFFFFFFu;
+    if (!(last && J.hist)) {
+        if (has) record_copy(J, slot, inst, s, sweep, last, E, M);
+        return;
+    }
     const uint32_t mask = __ballot_sync(kAll, has);
     if (!mask) return;
     const uint32_t leader = (uint32_t)__ffs(mask) - 1u;
     const uint32_t inst0 = __shfl_sync(kAll, inst, leader);
-    const bool one = __all_sync(kAll, !has || inst == inst0) != 0;
-    if (!(last && J.hist) || !one) {
+    if (!__all_sync(kAll, !has || inst == inst0)) {
         if (has) record_copy(J, slot, inst, s, sweep, last, E, M);
         return;
     }

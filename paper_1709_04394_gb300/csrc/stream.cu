@@ -48,8 +48,10 @@ namespace {
 constexpr uint32_t kStreamThreads = 128;      // threads per block with one-warp teams
 constexpr size_t kStreamSmem = 227 * 1024;   // shared memory of an SM
 constexpr uint32_t kStreamTeamWords = 3072;  // a one-warp team's share of shared memory, at most
-// largest block: 64 registers a thread for C = 1 (1024 threads), 128 for C = 2, 255 for C = 4
-constexpr uint32_t stream_max_threads(int C) { return C == 4 ? 256u : C == 2 ? 512u : 1024u; }
+// largest block, and blocks per SM the registers have to leave room for: 64 registers
+// a thread for C = 1 and 2 (128 for S = 4), 96 for C = 4
+constexpr uint32_t stream_max_threads(int C, int S) { return C == 4 ? 128u : C == 2 || S == 4 ? 512u : 1024u; }
+constexpr uint32_t stream_min_blocks(int C) { return C == 4 ? 5u : C == 2 ? 2u : 1u; }
 
 // Philox calls of one copy in lockstep: with fewer copies per thread more calls of
 // the same copy keep as many independent chains in flight. Measured (site updates
@@ -103,26 +105,84 @@ struct Window {
 
 __device__ __forceinline__ uint32_t sel(uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); }
 
+// What the update of word w reads besides spins: masks for colour 0 (odd, edge) and
+// colour 1, and the windows' positions. EAGER: worked out by set() and kept (a
+// thread with one word for the whole launch); else where they are used.
+template <int DIM, bool EAGER>
+struct Place {
+    uint32_t w;
+    const uint32_t* mask;
+    uint32_t kept[EAGER ? (DIM == 3 ? 11 : 5) : 1];
+    __device__ __forceinline__ uint32_t mask_word(const StreamShape& g, uint32_t k) const {
+        return __ldg(mask + k * g.PW + w);
+    }
+    __device__ __forceinline__ uint32_t position(const StreamShape& g, int k) const {
+        const uint32_t k0 = w << 5;
+        auto wrap = [&](uint32_t p) { return p >= g.H ? p - g.H : p; };
+        switch (k) {
+            case 0: return k0 >= g.s ? k0 - g.s : k0 + g.H - g.s;                  // from k - s
+            case 1: return wrap(k0 + g.s - 1u);                                    // from k + s - 1
+            case 2: return wrap(k0 + g.A - g.s);                                   // 3D, y = 0: row L - 1 of the slab
+            case 3: return k0 + g.s >= g.A ? k0 + g.s - g.A : k0 + g.s + g.H - g.A;  // y = L - 1: row 0
+            case 4: return k0 >= g.A ? k0 - g.A : k0 + g.H - g.A;                  // z - 1
+            default: return wrap(k0 + g.A);                                        // z + 1
+        }
+    }
+    __device__ __forceinline__ void set(const StreamShape& g, uint32_t word, const uint32_t* m) {
+        w = word;
+        mask = m;
+        if constexpr (EAGER) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) kept[k] = mask_word(g, k);
+#pragma unroll
+            for (int k = 0; k < (DIM == 3 ? 6 : 2); ++k) kept[3 + k] = position(g, k);
+            if constexpr (DIM == 3) {
+                kept[9] = mask_word(g, 3u);
+                kept[10] = mask_word(g, 4u);
+            }
+        }
+    }
+    __device__ __forceinline__ uint32_t odd(const StreamShape& g, uint32_t colour) const {
+        const uint32_t o = EAGER ? kept[0] : mask_word(g, 0u);
+        return colour ? ~o : o;
+    }
+    __device__ __forceinline__ uint32_t edge(const StreamShape& g, uint32_t colour) const {
+        if constexpr (EAGER) return colour ? kept[2] : kept[1];
+        return mask_word(g, 1u + colour);
+    }
+    template <int K>
+    __device__ __forceinline__ uint32_t at(const StreamShape& g) const {
+        if constexpr (EAGER) return kept[3 + K];
+        return position(g, K);
+    }
+    __device__ __forceinline__ uint32_t first_row(const StreamShape& g) const {
+        if constexpr (EAGER && DIM == 3) return kept[9];
+        return mask_word(g, 3u);
+    }
+    __device__ __forceinline__ uint32_t last_row(const StreamShape& g) const {
+        if constexpr (EAGER && DIM == 3) return kept[10];
+        return mask_word(g, 4u);
+    }
+};
+
 // Unsatisfied-bond masks of word w of colour c: d[k][copy], k in the order
-// (same-j x neighbour, other x neighbour, y - 1, y + 1, z - 1, z + 1).
-template <int DIM, bool EA, int C>
-__device__ __forceinline__ void stream_unsat(const StreamShape& g, const Words<C>* oth, const Words<C>& own, uint32_t w,
-                                             uint32_t colour, const uint32_t* __restrict__ mask,
-                                             const uint32_t* __restrict__ bond, uint32_t d[2 * DIM][C]) {
-    const uint32_t k0 = w << 5;
-    const uint32_t odd = __ldg(mask + w) ^ (colour ? 0xFFFFFFFFu : 0u);
-    const uint32_t edge = __ldg(mask + (1u + colour) * g.PW + w);
+// (same-j x neighbour, other x neighbour, y - 1, y + 1, z - 1, z + 1), and the
+// other plane's word w (same).
+template <int DIM, bool EA, int C, bool EAGER>
+__device__ __forceinline__ void stream_unsat(const StreamShape& g, const Words<C>* oth, const Words<C>& own,
+                                             const Place<DIM, EAGER>& at, uint32_t colour,
+                                             const uint32_t* __restrict__ bond,
+                                             uint32_t d[2 * DIM][C], Words<C>& same) {
+    const uint32_t w = at.w;
+    const uint32_t odd = at.odd(g, colour), edge = at.edge(g, colour);
     uint32_t j[2 * DIM];
 #pragma unroll
     for (int k = 0; k < 2 * DIM; ++k) j[k] = EA ? __ldg(bond + k * g.PW + w) : 0u;
-    Window<C> up, dn;  // from k - s, and from k + s - 1
-    const uint32_t pu = k0 >= g.s ? k0 - g.s : k0 + g.H - g.s;
-    uint32_t pd = k0 + g.s - 1u;
-    if (pd >= g.H) pd -= g.H;
-    up.load(oth, pu, g.PWX);
-    dn.load(oth, pd, g.PWX);
+    Window<C> up, dn;
+    up.load(oth, at.template at<0>(g), g.PWX);
+    dn.load(oth, at.template at<1>(g), g.PWX);
+    same = oth[GBMC_IDX(w, g.PWX)];
     {
-        const Words<C> same = oth[GBMC_IDX(w, g.PWX)];
         const Words<C> prv = oth[w ? w - 1u : 0u];  // bit 0 of word 0 starts a row: its edge window is taken
         const Words<C> nxt = oth[GBMC_IDX(w + 1u, g.PWX)];
 #pragma unroll
@@ -142,21 +202,17 @@ __device__ __forceinline__ void stream_unsat(const StreamShape& g, const Words<C
             d[3][c] = own.v[c] ^ dn.template at<1>(c) ^ j[3];
         }
     } else {
-        const uint32_t y0 = __ldg(mask + 3u * g.PW + w), yl = __ldg(mask + 4u * g.PW + w);
+        const uint32_t y0 = at.first_row(g), yl = at.last_row(g);
         Window<C> a, b;
-        uint32_t p = k0 + g.A - g.s;
-        if (p >= g.H) p -= g.H;
-        a.load(oth, p, g.PWX);  // y = 0: row L - 1 of the slab
-        b.load(oth, k0 + g.s >= g.A ? k0 + g.s - g.A : k0 + g.s + g.H - g.A, g.PWX);  // y = L - 1: row 0
+        a.load(oth, at.template at<2>(g), g.PWX);  // y = 0: row L - 1 of the slab
+        b.load(oth, at.template at<3>(g), g.PWX);  // y = L - 1: row 0
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             d[2][c] = own.v[c] ^ sel(y0, a.template at<0>(c), up.template at<0>(c)) ^ j[2];
             d[3][c] = own.v[c] ^ sel(yl, b.template at<0>(c), dn.template at<1>(c)) ^ j[3];
         }
-        p = k0 + g.A;
-        if (p >= g.H) p -= g.H;
-        a.load(oth, k0 >= g.A ? k0 - g.A : k0 + g.H - g.A, g.PWX);
-        b.load(oth, p, g.PWX);
+        a.load(oth, at.template at<4>(g), g.PWX);
+        b.load(oth, at.template at<5>(g), g.PWX);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             d[4][c] = own.v[c] ^ a.template at<0>(c) ^ j[4];
@@ -194,8 +250,8 @@ __device__ __forceinline__ void stream_extend(uint32_t* plane, uint32_t n, const
 // only): four threads per word, each the eight sites of one byte of it (two
 // Philox calls), for launches too small to give every scheduler two warps.
 template <int DIM, bool EA, int C, int S, bool PT>
-__global__ void __launch_bounds__(stream_max_threads(C)) k_sweep_stream(const __grid_constant__ SweepLaunch P,
-                                                                        uint32_t smem_words) {
+__global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C))
+    k_sweep_stream(const __grid_constant__ SweepLaunch P, uint32_t smem_words) {
     extern __shared__ __align__(16) uint32_t smw[];
     int jid = 0;
     while (jid + 1 < P.njobs && blockIdx.x >= P.cta_begin[jid + 1]) ++jid;
@@ -296,22 +352,85 @@ __global__ void __launch_bounds__(stream_max_threads(C)) k_sweep_stream(const __
     static_assert(S == 1 || (S == 4 && C == 1), "");
     constexpr int NQ = S == 4 ? 2 : stream_calls(C);
     const uint32_t NB = 2u * DIM * g.PW;  // bond words per instance and colour
+    // item is -> group, copies and place; worked out once where a thread has one
+    // item at most (small populations, where the chain of a half-sweep is what counts)
+    uint32_t gi = 0, part = 0, inst = 0, r0 = 0;
+    Place<DIM, S == 4> at;
+    auto locate = [&](uint32_t is) {
+        const uint32_t i = is / S;
+        part = is % S;
+        gi = G == 1u ? 0u : i / g.PW;
+        inst = meta[3u * gi];
+        r0 = meta[3u * gi + 1u];
+        at.set(g, i - gi * g.PW, mask);
+    };
+    const bool once = S == 4 && items * S <= T;
+    if (once && tl < items * S) locate(tl);
+    // adds an item's unsatisfied bonds (of colour-0 sites, d) and down spins to its
+    // copies' sums: at once, or in registers first where all items are one group's
+    int U[C], D[C];
+    auto tally = [&](const uint32_t (&d)[2 * DIM][C], const Words<C>& p0, const Words<C>& p1, uint32_t mine) {
+        const uint32_t valid = at.w + 1u == g.PW ? g.mh & mine : mine;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            int u = 0;
+#pragma unroll
+            for (int k = 0; k < 2 * DIM; ++k) u += __popc(d[k][c] & valid);
+            const int dn = __popc(p0.v[c] & valid) + __popc(p1.v[c] & valid);
+            if (G == 1u) {
+                U[c] += u;
+                D[c] += dn;
+            } else {
+                atomicAdd(acc + 2u * (gi * C + c), u);
+                atomicAdd(acc + 2u * (gi * C + c) + 1u, dn);
+            }
+        }
+    };
+    auto flush = [&]() {  // whole warps
+        if (G != 1u) return;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int u = __reduce_add_sync(0xFFFFFFFFu, U[c]), dn = __reduce_add_sync(0xFFFFFFFFu, D[c]);
+            if ((threadIdx.x & 31u) == 0u) {
+                atomicAdd(acc + 2 * c, u);
+                atomicAdd(acc + 2 * c + 1, dn);
+            }
+        }
+    };
+    auto record = [&](uint32_t s, bool sweep, bool last) {
+        for (uint32_t i0 = 0; i0 < n * C; i0 += T) {  // whole warps (record_copies)
+            const uint32_t i = i0 + tl, gr = i < n * C ? i / C : 0u, c = i % C, ins = meta[3u * gr];
+            const bool has = i < n * C && c < meta[3u * gr + 2u];
+            // every bond has one colour-0 end: E = 2 (unsatisfied bonds of the colour-0 sites) - DIM N
+            record_copies(J, has, (uint64_t)ins * J.R + meta[3u * gr + 1u] + c, ins, s, sweep, last,
+                          has ? 2 * acc[2u * i] - DIM * (int)J.N : 0, has ? (int)J.N - 2 * acc[2u * i + 1u] : 0);
+            if (i < n * C) acc[2u * i] = acc[2u * i + 1u] = 0;
+        }
+    };
+#pragma unroll
+    for (int c = 0; c < C; ++c) U[c] = D[c] = 0;
+    const bool series = J.Eser || J.Mser;
     for (uint32_t s = 0; s <= nsw; ++s) {
         if (s == nsw && nsw != 0) break;  // s == nsw: measurement-only pass when nothing is swept
         const bool sweep = s < nsw;
         for (uint32_t colour = 0; sweep && colour < 2; ++colour) {
+            // a series' E and M after sweep s - 1 come from the words this update reads
+            // (one copy per thread; with more the tallies cost more registers than the
+            // pass of their own below costs time)
+            const bool measure = C == 1 && series && colour == 0u && s > 0u;
             for (uint32_t is = tl; is < items * S; is += T) {
-                const uint32_t i = is / S, part = is % S;
-                const uint32_t gi = G == 1u ? 0u : i / g.PW, w = i - gi * g.PW;
-                const uint32_t inst = meta[3u * gi], r0 = meta[3u * gi + 1u];
+                if (!once) locate(is);
+                const uint32_t w = at.w;
                 Words<C>* own = reinterpret_cast<Words<C>*>(sm + colour * plane + gi * g.PWX * C);
                 const Words<C>* oth = reinterpret_cast<const Words<C>*>(sm + (colour ^ 1u) * plane + gi * g.PWX * C);
                 Words<C> nw = own[w];
                 uint32_t ge[C], ea[C], eb[C];  // dE <= 0; dE = 4; dE = 8 (3D)
                 {
                     uint32_t d[2 * DIM][C];
-                    stream_unsat<DIM, EA, C>(g, oth, nw, w, colour, mask,
-                                             EA ? J.sbond + ((uint64_t)inst * 2u + colour) * NB : nullptr, d);
+                    Words<C> same;
+                    stream_unsat<DIM, EA, C>(g, oth, nw, at, colour,
+                                             EA ? J.sbond + ((uint64_t)inst * 2u + colour) * NB : nullptr, d, same);
+                    if (measure) tally(d, nw, same, S == 4 ? 0xFFu << (8u * part) : 0xFFFFFFFFu);
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
                         if constexpr (DIM == 2) {
@@ -419,59 +538,38 @@ __global__ void __launch_bounds__(stream_max_threads(C)) k_sweep_stream(const __
                     if (g.h == 32u && w == 0u) own[g.PW] = nw;  // whole words: the extension is word 0 again
                 }
             }
+            if (measure) flush();
             team_sync(warp);
             if (g.h != 32u) {
                 stream_extend<C>(sm + colour * plane, n, g, tl, T);
                 team_sync(warp);
             }
-        }
-        const bool last = sweep ? s + 1 == nsw : true;
-        if ((J.Eser && sweep) || (J.Mser && sweep) || (last && want_final)) {
-            // every bond has one colour-0 end: E = 2 (unsatisfied bonds of the colour-0 sites) - DIM N
-            for (uint32_t i0 = 0; i0 < items; i0 += T) {
-                const uint32_t i = i0 + tl;
-                int U[C], D[C];
+            if (measure) {
+                record(s - 1u, true, false);  // the sums' next use is a half-sweep, and its sync, away
 #pragma unroll
                 for (int c = 0; c < C; ++c) U[c] = D[c] = 0;
-                uint32_t gi = 0;
-                if (i < items) {
-                    gi = G == 1u ? 0u : i / g.PW;
-                    const uint32_t w = i - gi * g.PW, valid = w + 1u == g.PW ? g.mh : 0xFFFFFFFFu;
-                    const Words<C>* p0 = reinterpret_cast<const Words<C>*>(sm + gi * g.PWX * C);
-                    const Words<C>* p1 = reinterpret_cast<const Words<C>*>(sm + plane + gi * g.PWX * C);
-                    const Words<C> w0 = p0[w], w1 = p1[w];
-                    uint32_t d[2 * DIM][C];
-                    stream_unsat<DIM, EA, C>(g, p1, w0, w, 0u, mask,
-                                             EA ? J.sbond + (uint64_t)meta[3u * gi] * 2u * NB : nullptr, d);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-#pragma unroll
-                        for (int k = 0; k < 2 * DIM; ++k) U[c] += __popc(d[k][c] & valid);
-                        D[c] = __popc(w0.v[c] & valid) + __popc(w1.v[c] & valid);
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    if (G == 1u) {  // one group: the warp's sum first
-                        const int u = __reduce_add_sync(0xFFFFFFFFu, U[c]), dd = __reduce_add_sync(0xFFFFFFFFu, D[c]);
-                        if ((threadIdx.x & 31u) == 0u) {
-                            atomicAdd(acc + 2 * c, u);
-                            atomicAdd(acc + 2 * c + 1, dd);
-                        }
-                    } else if (i < items) {
-                        atomicAdd(acc + 2u * (gi * C + c), U[c]);
-                        atomicAdd(acc + 2u * (gi * C + c) + 1u, D[c]);
-                    }
-                }
             }
+        }
+        const bool last = sweep ? s + 1u == nsw : true;
+        if ((last && want_final) || (series && sweep && (last || C > 1))) {
+            for (uint32_t i = tl; i < items; i += T) {
+                const uint32_t gr = G == 1u ? 0u : i / g.PW;
+                const Words<C>* p0 = reinterpret_cast<const Words<C>*>(sm + gr * g.PWX * C);
+                const Words<C>* p1 = reinterpret_cast<const Words<C>*>(sm + plane + gr * g.PWX * C);
+                gi = gr;
+                at.set(g, i - gr * g.PW, mask);
+                const Words<C> w0 = p0[at.w];
+                uint32_t d[2 * DIM][C];
+                Words<C> w1;
+                stream_unsat<DIM, EA, C>(g, p1, w0, at, 0u, EA ? J.sbond + (uint64_t)meta[3u * gr] * 2u * NB : nullptr, d,
+                                         w1);
+                tally(d, w0, w1, 0xFFFFFFFFu);
+            }
+            flush();
             team_sync(warp);
-            for (uint32_t i0 = 0; i0 < n * C; i0 += T) {  // whole warps (record_copies)
-                const uint32_t i = i0 + tl, gi = i < n * C ? i / C : 0u, c = i % C, inst = meta[3u * gi];
-                const bool has = i < n * C && c < meta[3u * gi + 2u];
-                record_copies(J, has, (uint64_t)inst * J.R + meta[3u * gi + 1u] + c, inst, s, sweep, last,
-                              has ? 2 * acc[2u * i] - DIM * (int)J.N : 0, has ? (int)J.N - 2 * acc[2u * i + 1u] : 0);
-                if (i < n * C) acc[2u * i] = acc[2u * i + 1u] = 0;
-            }
+            record(s, sweep, last);
+#pragma unroll
+            for (int c = 0; c < C; ++c) U[c] = D[c] = 0;
             team_sync(warp);
         }
     }
@@ -611,7 +709,7 @@ StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_c
         // to give every scheduler work, take whole blocks
         for (uint32_t G = 1; G <= 32u && stream_smem_words(J.N, G, C, pt) <= kStreamTeamWords; ++G) consider(32u, G);
         if (P.njobs == 1)
-            for (uint32_t T = 64u; T <= stream_max_threads(C) && T < PW + 32u; T += 32u) consider(T, 1u);
+            for (uint32_t T = 64u; T <= stream_max_threads(C, split) && T < PW + 32u; T += 32u) consider(T, 1u);
         if (S.T[j] == 0u) consider(kStreamThreads, 1u);
         total += best_sum;
         longest = std::max(longest, best_len);

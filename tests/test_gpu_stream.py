@@ -28,7 +28,6 @@ def _kinds(ctx, fn):
     (2, 2, FM, 1, 3, 0.4, 4),       # a plane of 2 sites
     (2, 4, FM, 2, 5, 0.44, 4),
     (2, 6, FM, 1, 7, 0.3, 4),
-    (2, 8, FM, 1, 130, 0.44, 3),    # a plane of one whole word
     (2, 10, FM, 1, 9, 0.44, 4),
     (2, 18, FM, 2, 5, 0.5, 3),
     (2, 24, FM, 1, 3, 0.0, 2),      # beta = 0: every site flips
@@ -76,6 +75,7 @@ def test_stream_sweeps_match_oracle(ctx, dim, L, model, I, R, beta, n):
 
 
 @pytest.mark.parametrize("dim,L,model,I,R", [
+    (2, 8, FM, 1, 20011),     # a plane of one whole word
     (2, 12, FM, 1, 70001),    # four copies per thread, 3 words per plane
     (2, 24, FM, 1, 34603),
     (2, 24, FM, 1, 9001),     # two
