@@ -2565,23 +2565,12 @@ gbmc_status mlp_train(gbmc_ctx* ctx, float* params, const float* X, const float*
     if (batch == 0 || batch > kMlpMaxBatch) return fail(GBMC_ERR_ARG, "batch must be 1..%u", kMlpMaxBatch);
     CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
-    float* work = nullptr;  // grad, m, v
-    CUDA_TRY(cudaMallocAsync((void**)&work, 3 * kMlpParams * sizeof(float) + 16, s));
-    float* g = work;
-    float* m = work + kMlpParams;
-    float* v = work + 2 * kMlpParams;
+    float* work = nullptr;  // Adam's moments m, v
+    CUDA_TRY(cudaMallocAsync((void**)&work, 2 * kMlpParams * sizeof(float), s));
     gbmc_status st = GBMC_OK;
-    cudaError_t e = cudaMemsetAsync(m, 0, 2 * kMlpParams * sizeof(float), s);
-    uint32_t k = 0;
-    const uint32_t nb = (n + batch - 1) / batch;
-    for (uint32_t ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
-        for (uint32_t bi = 0; bi < nb && e == cudaSuccess; ++bi) {
-            const uint32_t b0 = bi * batch, B = (n - b0) < batch ? (n - b0) : batch;
-            float* lp = loss_out ? loss_out + (uint64_t)ep * nb + bi : work + 3 * kMlpParams;
-            e = launch_mlp_grad(params, X + (uint64_t)b0 * kMlpIn, T + b0, B, g, lp, s);
-            if (e == cudaSuccess) e = launch_mlp_adam(params, g, m, v, ++k, lr, s);
-        }
-    }
+    cudaError_t e = cudaMemsetAsync(work, 0, 2 * kMlpParams * sizeof(float), s);
+    if (e == cudaSuccess)
+        e = launch_mlp_train(params, work, work + kMlpParams, X, T, n, epochs, batch, lr, loss_out, s);
     if (e != cudaSuccess) st = fail(GBMC_ERR_CUDA, "mlp_train: %s", cudaGetErrorString(e));
     cudaFreeAsync(work, s);
     return st;

@@ -335,6 +335,10 @@ constexpr uint32_t kMlpMaxBatch = 128;
 cudaError_t launch_mlp_forward(const float* p, const float* X, uint32_t B, float* Y, cudaStream_t s);
 cudaError_t launch_mlp_grad(const float* p, const float* X, const float* T, uint32_t B, float* g, float* loss,
                             cudaStream_t s);
+// Training of mlp_train: m, v the Adam moments (zeroed by the caller), losses null or
+// one per step.
+cudaError_t launch_mlp_train(float* p, float* m, float* v, const float* X, const float* T, uint32_t n, uint32_t epochs,
+                             uint32_t batch, float lr, float* losses, cudaStream_t s);
 cudaError_t launch_mlp_adam(float* p, const float* g, float* m, float* v, uint32_t k, float lr, cudaStream_t s);
 
 // ---- adaptive annealing steps: overlap bisection and MLP proposals ----
