@@ -87,9 +87,10 @@ gbmc_status gbmc_destroy(gbmc_ctx *ctx);
 
 /* Resampling path of population annealing: fused = 1 (default when the device
  * supports cooperative launches) runs the weights, ln Q / prefix sums,
- * multinomial draws and child placement of one lattice in ONE cooperative
- * launch with grid-wide barriers; fused = 0 uses one launch per phase. Both
- * give identical results. */
+ * multinomial draws and child placement in ONE launch: populations of up to
+ * some ten thousand copies of all lattices together, a cluster of blocks each;
+ * larger ones a cooperative launch with grid-wide barriers per lattice.
+ * fused = 0 uses one launch per phase. All give identical results. */
 gbmc_status gbmc_set_resample_mode(gbmc_ctx *ctx, int32_t fused);
 
 /* Launch form of the shared-memory sweep kernel (Sec. 3.1 checkerboard sweeps
@@ -148,7 +149,7 @@ gbmc_status gbmc_set_sweep_launch(gbmc_ctx *ctx, int32_t mode);
 enum { GBMC_KERNEL_AUTO = 0, GBMC_KERNEL_BYTES = 1, GBMC_KERNEL_BITS = 2 };
 gbmc_status gbmc_set_sweep_kernel(gbmc_ctx *ctx, int32_t kernel);
 /* Test aid for the bounded waits: each grid barrier of the fused resampling
- * waits for `phantom_arrivals` CTAs more than the launch has, and each
+ * (with phantom arrivals, every population's resampling takes that form) waits for `phantom_arrivals` CTAs more than the launch has, and each
  * neighbour wait of the strip-resident sweeps for that many half-sweeps more
  * (so with 1 a wait can only end by running out of its budget); waits give up
  * after `budget_cycles` SM cycles (default 2e9). A wait that runs out makes the

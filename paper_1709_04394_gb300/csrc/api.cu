@@ -1819,9 +1819,18 @@ gbmc_status pa_populations(const gbmc_pa* pa, uint32_t* n) {
 // with `stepping` set (its next beta already appended to pl.betas).
 static gbmc_status pa_enqueue_common(gbmc_pa* pa) {
     cudaStream_t s = pa->ctx->stream;
+    PaLattice small[kMaxJobs];
+    double* small_lnZ[kMaxJobs];
+    uint32_t n_small = 0;
     for (auto& pl : pa->lats) {
         if (!pl.stepping) continue;
         PaLattice P = pa_params(pa, pl, pl.steps);
+        // (a phantom arrival belongs to the grid barrier's test)
+        if (pa->ctx->fused && !pa->ctx->phantom && resample_in_clusters(P)) {
+            small[n_small] = P;
+            small_lnZ[n_small++] = pl.lnZ;
+            continue;
+        }
         if (pa->ctx->fused) {
             GridBarrier B{pa->ctx->words, pa->ctx->words + 1, pa->ctx->budget, pa->ctx->phantom};
             ProfScope ps_(pa->ctx, PK_PA_FUSED);
@@ -1845,6 +1854,10 @@ static gbmc_status pa_enqueue_common(gbmc_pa* pa) {
             ProfScope ps_(pa->ctx, PK_PA_PLACE);
             CUDA_TRY(launch_pa_place(P, s));
         }
+    }
+    if (n_small) {
+        ProfScope ps_(pa->ctx, PK_PA_FUSED);
+        CUDA_TRY(launch_pa_resample_clusters(small, small_lnZ, n_small, s));
     }
     gbmc_status st = pa_sweep_launch(pa, false);
     if (st != GBMC_OK) return st;

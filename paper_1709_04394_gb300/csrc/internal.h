@@ -300,6 +300,10 @@ struct GridBarrier {
 
 cudaError_t launch_pa_resample_fused(const PaLattice& P, double* lnZ, const GridBarrier& B, int n_sms,
                                      cudaStream_t s);
+// Whole resampling of every population of up to kMaxJobs lattices in one launch, where each
+// lattice passes resample_in_clusters.
+bool resample_in_clusters(const PaLattice& P);
+cudaError_t launch_pa_resample_clusters(const PaLattice* jobs, double* const* lnZ, uint32_t njobs, cudaStream_t s);
 cudaError_t launch_pa_weights(const PaLattice& P, cudaStream_t s);
 cudaError_t launch_pa_reduce(const PaLattice& P, double* lnZ, int first_step, cudaStream_t s);
 cudaError_t launch_pa_draws(const PaLattice& P, cudaStream_t s);

@@ -23,7 +23,14 @@
 // plus one with probability frac(tau_j), tau_j = R0 W_j / C, decided in
 // integers -- every phase only looks at the R_{i-1} live replicas, ln Q uses
 // R_{i-1}, and the placement writes R_i (at most the capacity P.R).
+//
+// The phases run in one launch: small and medium populations each in a cluster of blocks
+// (k_pa_resample_clusters), larger ones over the whole grid (k_pa_resample_fused); the
+// separate kernels are for captured runs and on request.
 #include <climits>
+#include <cstring>
+
+#include <cooperative_groups.h>
 
 #include "../../include/gbmc.h"
 #include "check.cuh"
@@ -31,6 +38,8 @@
 #include "internal.h"
 
 namespace gbmc {
+
+namespace cg = cooperative_groups;
 
 constexpr int kScanThreads = 512;
 constexpr int kPerThread = kScanChunk / kScanThreads;  // 4
@@ -48,6 +57,15 @@ __device__ __forceinline__ unsigned long long resample_u64(const PaLattice& P, u
         make_uint4(k >> 1, P.step, r, c3_word(kPurposeResample, 0u, P.inst_base + inst)),
         (uint32_t)P.seed, (uint32_t)(P.seed >> 32));
     return (k & 1u) ? (((unsigned long long)w.w << 32) | w.z) : (((unsigned long long)w.y << 32) | w.x);
+}
+
+// Draws 2 p and 2 p + 1.
+__device__ __forceinline__ void resample_u64_pair(const PaLattice& P, uint32_t inst, uint32_t p,
+                                                  unsigned long long (&U)[2]) {
+    const uint4 w = philox4x32_10(make_uint4(p, P.step, 0u, c3_word(kPurposeResample, 0u, P.inst_base + inst)),
+                                  (uint32_t)P.seed, (uint32_t)(P.seed >> 32));
+    U[0] = ((unsigned long long)w.y << 32) | w.x;
+    U[1] = ((unsigned long long)w.w << 32) | w.z;
 }
 
 // ---- the five phases, as block-level device functions ----
@@ -80,11 +98,8 @@ __device__ __forceinline__ void phase_weights(const PaLattice& P, uint32_t inst,
     if (threadIdx.x == 0) P.ctot[(uint64_t)inst * P.nchunks + chunk] = total;
 }
 
-// ln Q of one population (fixed-order fp64 tree), ln Z += ln Q, exclusive
-// scan of its chunk totals, reset of the accumulators for the next sweep.
-__device__ __forceinline__ void phase_reduce(const PaLattice& P, uint32_t inst, double* lnZ, double* lnQ_out,
-                                             double* sd, unsigned long long* su) {
-    const int32_t emin = P.emin[inst], emax = P.emax[inst];
+// This thread's share of sum_E h(E) exp(-dbeta (E - Emin)); clears the histogram.
+__device__ __forceinline__ double hist_weight(const PaLattice& P, uint32_t inst, int32_t emin, int32_t emax) {
     uint32_t* h = P.hist + (uint64_t)inst * P.nbins;
     double acc = 0.0;
     if (emin <= emax) {  // an empty population (variable sizes) has no range
@@ -95,7 +110,22 @@ __device__ __forceinline__ void phase_reduce(const PaLattice& P, uint32_t inst, 
             h[b] = 0u;
         }
     }
-    acc = warp_sum(acc);
+    return acc;
+}
+
+__device__ __forceinline__ void reset_accumulators(const PaLattice& P, uint32_t inst) {
+    P.emin[inst] = INT_MAX;
+    P.emax[inst] = INT_MIN;
+    unsigned long long* sums = P.sums + (uint64_t)inst * 4;
+    sums[0] = sums[1] = sums[2] = sums[3] = 0ull;
+}
+
+// ln Q of one population (fixed-order fp64 tree), ln Z += ln Q, exclusive
+// scan of its chunk totals, reset of the accumulators for the next sweep.
+__device__ __forceinline__ void phase_reduce(const PaLattice& P, uint32_t inst, double* lnZ, double* lnQ_out,
+                                             double* sd, unsigned long long* su) {
+    const int32_t emin = P.emin[inst], emax = P.emax[inst];
+    double acc = warp_sum(hist_weight(P, inst, emin, emax));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     if (lane == 0) sd[warp] = acc;
     __syncthreads();
@@ -122,10 +152,7 @@ __device__ __forceinline__ void phase_reduce(const PaLattice& P, uint32_t inst, 
     }
     if (threadIdx.x == 0) {
         cp[P.nchunks] = carry;
-        P.emin[inst] = INT_MAX;
-        P.emax[inst] = INT_MIN;
-        unsigned long long* sums = P.sums + (uint64_t)inst * 4;
-        sums[0] = sums[1] = sums[2] = sums[3] = 0ull;
+        reset_accumulators(P, inst);
     }
     __syncthreads();
 }
@@ -159,6 +186,14 @@ __device__ __forceinline__ void phase_draw(const PaLattice& P, uint64_t g) {
 // Nearest-integer copies of replica g (global over the lattice's populations):
 // n_j = floor(R0 W_j / C) + [floor(U64_j C / 2^64) < (R0 W_j mod C)], C = sum W.
 // R0 W_j <= capacity 2^s <= 2^63 and C <= R_{i-1} 2^s <= 2^63 by the choice of s.
+__device__ __forceinline__ uint32_t nearest_copies(const PaLattice& P, uint32_t inst, uint32_t j,
+                                                   unsigned long long W, unsigned long long C) {
+    const unsigned long long num = (unsigned long long)P.R0 * W;
+    const unsigned long long n0 = num / C, rem = num - n0 * C;
+    const unsigned long long x = __umul64hi(resample_u64(P, inst, j), C);
+    return (uint32_t)n0 + (x < rem ? 1u : 0u);
+}
+
 __device__ __forceinline__ void phase_nearest(const PaLattice& P, uint64_t g) {
     const uint32_t inst = (uint32_t)(g / P.R), j = (uint32_t)(g - (uint64_t)inst * P.R);
     if (j >= live_prev(P, inst)) return;
@@ -166,11 +201,33 @@ __device__ __forceinline__ void phase_nearest(const PaLattice& P, uint64_t g) {
     // W_j from the inclusive in-chunk sums (E_min was already reset by ln Q's phase)
     const unsigned long long W = __ldcg(P.cloc + base + j) - ((j % kScanChunk) ? __ldcg(P.cloc + base + j - 1) : 0ull);
     const unsigned long long C = __ldcg(P.cpre + (uint64_t)inst * (P.nchunks + 1) + P.nchunks);
-    const unsigned long long num = (unsigned long long)P.R0 * W;
-    const unsigned long long n0 = num / C, rem = num - n0 * C;
-    const unsigned long long x = __umul64hi(resample_u64(P, inst, j), C);
-    P.counts[base + j] = (uint32_t)n0 + (x < rem ? 1u : 0u);
+    P.counts[base + j] = nearest_copies(P, inst, j, W, C);
 }
+
+// a / n rounded to nearest for a small integer n, y = 1 / n rounded to nearest, 2^-900 <= |a|,
+// in three operations of fp64 (whose rate is 1/64 of fp32's) instead of a division's ten or more.
+// q = a y is within 1.5 units in the last place of a / n, so e = a - n q is exact, a / n =
+// q + e / n, and e y differs from e / n by less than 2^-52 units; but a / n is no tie of the
+// rounding (n odd: n times a 54-bit odd number does not fit 53 bits; powers of two divide
+// out) and lies at least 1 / (2 n) units from one.
+__device__ __forceinline__ double div_small(double a, double n, double y) {
+    const double q = __dmul_rn(a, y);
+    return __fma_rn(__fma_rn(-n, q, a), y, q);
+}
+constexpr double kDivSmallest = 0x1p-900;
+
+// n and 1 / n, up to the counts that a mean of 500 reaches (a few sigma of 22 above it).
+struct Inverses {
+    static constexpr uint32_t kMost = 767;
+    double2 v[kMost + 1];
+    constexpr Inverses() : v() {
+        for (uint32_t n = 1; n <= kMost; ++n) {
+            v[n].x = (double)n;
+            v[n].y = 1.0 / (double)n;
+        }
+    }
+};
+__constant__ constexpr Inverses kInverses;
 
 // e^{-x}, x >= 0, in a fixed sequence of correctly rounded fp64 operations
 // (so host and device agree bit for bit): Cody and Waite's reduction x = k ln2
@@ -184,8 +241,13 @@ __device__ __forceinline__ double exp_neg_ieee(double x) {
     const double r = __dsub_rn(__dsub_rn(x, __dmul_rn(k, 0.693147180559890330187045037746429443359375)),
                                __dmul_rn(k, 5.4979230187083711552420206887059365096458314e-14));
     double s = 1.0;
+    if (fabs(r) >= kDivSmallest) {
+#pragma unroll
+        for (int n = 20; n >= 1; --n) s = __dsub_rn(1.0, __dmul_rn(div_small(r, (double)n, 1.0 / n), s));
+    } else {  // a step this small rounds away: s = 1 either way, in the sequence's own words
 #pragma unroll 1
-    for (int n = 20; n >= 1; --n) s = __dsub_rn(1.0, __dmul_rn(__ddiv_rn(r, (double)n), s));
+        for (int n = 20; n >= 1; --n) s = __dsub_rn(1.0, __dmul_rn(__ddiv_rn(r, (double)n), s));
+    }
     return ldexp(s, -(int)k);
 }
 
@@ -198,35 +260,51 @@ __device__ __forceinline__ uint32_t poisson_count(double tau, unsigned long long
     const double u = __dmul_rn(__ull2double_rn(U >> 11), 1.1102230246251565404236316680908203125e-16);
     double p = exp_neg_ieee(tau), F = p;
     uint32_t n = 0;
-    while (u >= F && n < 100000u) {
+    // None of the values compared is negative: they compare as their bits do, and n > tau as
+    // n > floor(tau), both off the fp64 unit. A replica with a mean in the hundreds makes this
+    // loop the kernel's longest chain; its five fp64 operations replace some 17 (17 populations of 4170
+    // with such replicas: 420 -> 215 us a step).
+    const uint32_t mode = (uint32_t)floor(tau);
+    const long long ub = __double_as_longlong(u);
+    const bool small = tau >= kDivSmallest;
+    while (ub >= __double_as_longlong(F) && n < 100000u) {
         n += 1;
-        p = __dmul_rn(p, __ddiv_rn(tau, (double)n));
+        double q;
+        if (small && n <= Inverses::kMost) {
+            const double2 d = kInverses.v[n];
+            q = div_small(tau, d.x, d.y);
+        } else {
+            q = __ddiv_rn(tau, (double)n);
+        }
+        p = __dmul_rn(p, q);
         const double Fn = __dadd_rn(F, p);
-        if (Fn == F && (double)n > tau) break;
+        if (__double_as_longlong(Fn) == __double_as_longlong(F) && n > mode) break;
         F = Fn;
     }
     return n;
 }
 
-// Poisson copies of replica g: Poisson(tau_j), tau_j = R0 W_j / C in fp64; a
+// Poisson copies of replica j: Poisson(tau_j), tau_j = R0 W_j / C in fp64; a
 // mean above 500 as the sum of m = ceil(tau / 500) Poisson(tau / m) pieces,
 // piece p from the replica's resampling word with counter field r = p.
+__device__ __forceinline__ uint32_t poisson_copies(const PaLattice& P, uint32_t inst, uint32_t j,
+                                                   unsigned long long W, unsigned long long C) {
+    const double tau = __ddiv_rn(__ull2double_rn((unsigned long long)P.R0 * W), __ull2double_rn(C));
+    if (tau <= 500.0) return poisson_count(tau, resample_u64(P, inst, j));
+    uint32_t n = 0;
+    const uint32_t m = (uint32_t)ceil(__ddiv_rn(tau, 500.0));
+    const double part = __ddiv_rn(tau, (double)m);
+    for (uint32_t p = 0; p < m; ++p) n += poisson_count(part, resample_u64(P, inst, j, p));
+    return n;
+}
+
 __device__ __forceinline__ void phase_poisson(const PaLattice& P, uint64_t g) {
     const uint32_t inst = (uint32_t)(g / P.R), j = (uint32_t)(g - (uint64_t)inst * P.R);
     if (j >= live_prev(P, inst)) return;
     const uint64_t base = (uint64_t)inst * P.R;
     const unsigned long long W = __ldcg(P.cloc + base + j) - ((j % kScanChunk) ? __ldcg(P.cloc + base + j - 1) : 0ull);
     const unsigned long long C = __ldcg(P.cpre + (uint64_t)inst * (P.nchunks + 1) + P.nchunks);
-    const double tau = __ddiv_rn(__ull2double_rn((unsigned long long)P.R0 * W), __ull2double_rn(C));
-    uint32_t n = 0;
-    if (tau <= 500.0) {
-        n = poisson_count(tau, resample_u64(P, inst, j));
-    } else {
-        const uint32_t m = (uint32_t)ceil(__ddiv_rn(tau, 500.0));
-        const double part = __ddiv_rn(tau, (double)m);
-        for (uint32_t p = 0; p < m; ++p) n += poisson_count(part, resample_u64(P, inst, j, p));
-    }
-    P.counts[base + j] = n;
+    P.counts[base + j] = poisson_copies(P, inst, j, W, C);
 }
 
 // Exclusive scan of the counts within one chunk, chunk total.
@@ -253,6 +331,26 @@ __device__ __forceinline__ void phase_count_scan(const PaLattice& P, uint32_t in
     if (threadIdx.x == 0) P.ntot[(uint64_t)inst * P.nchunks + chunk] = total;
 }
 
+// R_i of a variable population.
+__device__ __forceinline__ void record_population(const PaLattice& P, uint32_t inst, uint64_t total) {
+    if (total > P.R || total == 0) {  // outgrown its capacity, or died out
+        atomicExch(P.overflow, 1u);
+        if (total > P.R) total = P.R;
+    }
+    P.nnext[inst] = (uint32_t)total;
+}
+
+// Parent j fills the slots [S, S + n).
+__device__ __forceinline__ void place_children(const PaLattice& P, uint64_t base, uint64_t S, uint32_t n, uint32_t j) {
+    for (uint32_t m = 0; m < n; ++m) {
+        if (S + m >= P.R) {
+            atomicExch(P.overflow, 1u);
+            break;
+        }
+        P.parent[base + GBMC_IDX(S + m, P.R)] = j;
+    }
+}
+
 // Parent j fills slots [S_j, S_j + n_j); counts are cleared for the next step.
 // Variable populations: slots at or beyond the capacity are not written (the
 // overflow flag is raised instead) and the last chunk's CTA records R_i.
@@ -268,26 +366,14 @@ __device__ __forceinline__ void phase_place(const PaLattice& P, uint32_t inst, u
     __syncthreads();
     const uint32_t pre = *prefix;
     if (P.nnext && threadIdx.x == 0 && chunk + 1 == P.nchunks) {
-        uint64_t total = (uint64_t)pre + __ldcg(P.ntot + (uint64_t)inst * P.nchunks + chunk);
-        if (total > P.R || total == 0) {  // outgrown its capacity, or died out
-            atomicExch(P.overflow, 1u);
-            if (total > P.R) total = P.R;
-        }
-        P.nnext[inst] = (uint32_t)total;
+        record_population(P, inst, (uint64_t)pre + __ldcg(P.ntot + (uint64_t)inst * P.nchunks + chunk));
     }
     for (uint32_t i = threadIdx.x; i < kScanChunk; i += blockDim.x) {
         const uint32_t j = chunk * kScanChunk + i;
         if (j >= live) break;
         const uint32_t n = __ldcg(P.counts + base + j);
         if (n) {
-            const uint64_t S = (uint64_t)pre + __ldcg(P.sloc + base + j);
-            for (uint32_t m = 0; m < n; ++m) {
-                if (S + m >= P.R) {
-                    atomicExch(P.overflow, 1u);
-                    break;
-                }
-                P.parent[base + GBMC_IDX(S + m, P.R)] = j;
-            }
+            place_children(P, base, (uint64_t)pre + __ldcg(P.sloc + base + j), n, j);
             P.counts[base + j] = 0u;
         }
     }
@@ -446,6 +532,242 @@ cudaError_t launch_pa_resample_fused(const PaLattice& P, double* lnZ, const Grid
                                     0, s);
     count_launch();
     return e;
+}
+
+// ---- small and medium populations: one cluster of blocks per population ----
+//
+// The weights, draws, counts and placement of one population in the shared memory of
+// C - 1 worker blocks, each with a contiguous slice of the replicas; what they exchange
+// are the slices' totals, and the waits between the phases are the cluster's hardware
+// barrier. Every worker goes through all draws and keeps those that fall into its slice:
+// a generator call costs less than a search in another block's memory (five reads and
+// an atomic there: 14 us for 20 000 draws over 15 workers, going through all 8 us). The last
+// block of the cluster works out ln Q meanwhile (its fp64 sum and logarithm take as long as
+// the draws) and clears the accumulators. The populations of all lattices stepping go
+// in one launch. Same integers, and the same fp64 sum for ln Q, as k_pa_resample_fused.
+//
+// Bound: latency -- a few thousand replicas' chains of dependent loads.
+// With the launch's own 5 us: 10 us for 500 copies, 14 us for 5000, 15 us for 8 x 5000, where
+// the grid-wide kernel with its five barriers over L2 takes 21, 27 and 29 us.
+
+constexpr uint32_t kMaxWorkers = 15;
+
+struct ResampleClusters {
+    PaLattice jobs[kMaxJobs];
+    double* lnZ[kMaxJobs];
+    uint32_t first[kMaxJobs + 1];  // job j's clusters: [first[j], first[j + 1])
+    uint32_t slice;                // replicas a worker can hold (even)
+};
+
+// ln Q, ln Z and the reset of the accumulators, around the workers' three waits.
+__device__ __forceinline__ void cluster_lnq(const PaLattice& P, uint32_t inst, double* lnZ, double* sd) {
+    const int32_t emin = P.emin[inst], emax = P.emax[inst];
+    const uint32_t live = live_prev(P, inst);
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive();
+    const double acc = hist_weight(P, inst, emin, emax);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    // a warp without a bin holds zeros
+    const bool any = emin <= emax && (uint32_t)(emax - emin) >> 2 >= (threadIdx.x & ~31u);
+    const double w = any ? warp_sum(acc) : 0.0;
+    if (lane == 0) sd[warp] = w;
+    __syncthreads();
+    cluster.barrier_wait();  // all blocks have started
+    cluster.barrier_arrive();
+    if (warp == 0) {
+        const double v = warp_sum(lane < nwarps ? sd[lane] : 0.0);
+        if (lane == 0) {
+            const double log_R = P.nprev ? log((double)live) : P.log_R;
+            const double lnQ = -P.dbeta * (double)emin + log(v) - log_R;
+            lnZ[P.n_inst + inst] = lnQ;
+            lnZ[inst] += lnQ;
+        }
+        __syncwarp();
+    }
+    cluster.barrier_wait();  // every worker has read E_min
+    cluster.barrier_arrive();
+    if (threadIdx.x == 0) reset_accumulators(P, inst);
+    __syncwarp();
+    cluster.barrier_wait();  // the counts' totals
+}
+
+__global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const __grid_constant__ ResampleClusters A) {
+    extern __shared__ __align__(16) unsigned long long dyn[];
+    __shared__ unsigned long long tot[kMaxWorkers], pre[kMaxWorkers + 1];
+    __shared__ uint32_t ntot[kMaxWorkers];
+    __shared__ unsigned long long sh64[32];
+    __shared__ uint32_t sh32[32];
+    __shared__ double sd[32];
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t rank = cluster.block_rank(), K = cluster.num_blocks() - 1u, cid = blockIdx.x / (K + 1u);
+    uint32_t job = 0;
+    while (cid >= A.first[job + 1]) ++job;
+    const PaLattice& P = A.jobs[job];
+    const uint32_t inst = cid - A.first[job];
+    if (rank == K) {
+        cluster_lnq(P, inst, A.lnZ[job], sd);
+        return;
+    }
+    cluster.barrier_arrive();
+    unsigned long long* cum = dyn;                                   // [slice] inclusive sums of the slice
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(dyn + A.slice);      // [slice]
+    unsigned long long* mine = dyn + A.slice + A.slice / 2u + 64u * (threadIdx.x / 32u);  // [64] per warp: draws kept
+
+    // the slice [j0, j0 + n), `per` consecutive replicas per thread
+    const uint64_t base = (uint64_t)inst * P.R;
+    const uint32_t live = live_prev(P, inst);
+    const uint32_t width = (live + K - 1u) / K;
+    const uint32_t j0 = min(live, rank * width), n = min(live - j0, width);
+    const uint32_t per = (width + kScanThreads - 1u) / kScanThreads;
+    const uint32_t i0 = min(n, threadIdx.x * per), i1 = min(n, i0 + per);
+    {
+        const int32_t emin = P.emin[inst];
+        unsigned long long run = 0;
+        const int32_t* E = P.E + base + j0;
+        for (uint32_t i = i0; i < i1; i += 4u) {  // four replicas' loads in flight
+            uint32_t bin[4];
+            unsigned long long w[4];
+#pragma unroll
+            for (uint32_t k = 0; k < 4u; ++k) bin[k] = (uint32_t)(E[min(i + k, i1 - 1u)] - emin) >> 2;
+#pragma unroll
+            for (uint32_t k = 0; k < 4u; ++k) w[k] = P.wint[GBMC_IDX(bin[k], P.nbins)];
+#pragma unroll
+            for (uint32_t k = 0; k < 4u; ++k)
+                if (i + k < i1) {
+                    run += w[k];
+                    cum[i + k] = run;
+                    cnt[i + k] = 0u;
+                }
+        }
+        unsigned long long total;
+        const unsigned long long excl = block_inclusive_scan<unsigned long long>(run, sh64, &total) - run;
+        for (uint32_t i = i0; i < i1; ++i) cum[i] += excl;
+        cluster.barrier_wait();  // all blocks have started: their shared memory may be written
+        if (threadIdx.x < K) *cluster.map_shared_rank(&tot[rank], threadIdx.x) = total;
+    }
+    cluster.sync();
+
+    if (threadIdx.x < 32u) {
+        const unsigned long long v = threadIdx.x < K ? tot[threadIdx.x] : 0ull;
+        const unsigned long long incl = warp_inclusive_scan(v);
+        if (threadIdx.x < K) pre[threadIdx.x + 1u] = incl;
+        if (threadIdx.x == 0) pre[0] = 0ull;
+    }
+    __syncthreads();
+    const unsigned long long C = pre[K];
+    if (!P.nearest) {
+        // draws 2 p and 2 p + 1 share a generator call; a warp gathers those of its slice
+        // and looks them up 32 at a time
+        const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+        const unsigned long long lo = pre[rank], span = pre[rank + 1u] - lo;
+        const uint32_t top = n ? 1u << (31 - __clz(n)) : 0u;
+        uint32_t kept = 0;
+        auto look_up = [&](uint32_t first, uint32_t count) {
+            __syncwarp();
+            if (lane < count) {
+                const unsigned long long xr = mine[first + lane];
+                uint32_t pos = 0;  // the sums that do not exceed x
+                for (uint32_t step = top; step; step >>= 1)
+                    if (pos + step <= n && cum[pos + step - 1u] <= xr) pos += step;
+                atomicAdd(cnt + pos, 1u);
+            }
+            __syncwarp();
+        };
+        for (uint32_t p0 = threadIdx.x - lane; 2u * p0 < live; p0 += kScanThreads) {
+            unsigned long long U[2];
+            resample_u64_pair(P, inst, p0 + lane, U);
+#pragma unroll
+            for (uint32_t e = 0; e < 2u; ++e) {
+                const unsigned long long xr = __umul64hi(U[e], C) - lo;
+                const bool hit = 2u * (p0 + lane) + e < live && xr < span;
+                const uint32_t hits = __ballot_sync(~0u, hit);
+                if (hit) mine[kept + __popc(hits & below)] = xr;
+                kept += __popc(hits);
+                if (kept >= 32u) {
+                    kept -= 32u;
+                    look_up(kept, 32u);
+                }
+            }
+        }
+        look_up(0u, kept);
+        __syncthreads();
+    } else {
+        for (uint32_t i = threadIdx.x; i < n; i += kScanThreads) {
+            const unsigned long long W = cum[i] - (i ? cum[i - 1u] : 0ull);
+            cnt[i] = P.nearest == 2 ? poisson_copies(P, inst, j0 + i, W, C) : nearest_copies(P, inst, j0 + i, W, C);
+        }
+        __syncthreads();
+    }
+
+    uint32_t run = 0, total;
+    for (uint32_t i = i0; i < i1; ++i) run += cnt[i];
+    uint32_t S32 = block_inclusive_scan<uint32_t>(run, sh32, &total) - run;
+    if (threadIdx.x < K) *cluster.map_shared_rank(&ntot[rank], threadIdx.x) = total;
+    cluster.sync();
+    uint32_t before = 0;
+    for (uint32_t c = 0; c < rank; ++c) before += ntot[c];
+    if (P.nnext && threadIdx.x == 0 && rank + 1u == K) record_population(P, inst, (uint64_t)before + total);
+    for (uint32_t i = i0; i < i1; ++i) {
+        place_children(P, base, (uint64_t)before + S32, cnt[i], j0 + i);
+        S32 += cnt[i];
+    }
+}
+
+// The largest populations that a cluster resamples faster than the grid-wide kernel, whose
+// blocks are all of the chip's (us, one population, clusters : grid). Multinomial 20 000
+// copies 22 : 29, 40 000 33 : 30. Nearest integer 80 000 24 : 28. Poisson, bound by fp64 in a
+// cluster's few multiprocessors, 5000 27 : 49, 10 000 44 : 52, 20 000 77 : 54.
+bool resample_in_clusters(const PaLattice& P) {
+    return P.R <= (P.nearest == 2 ? 8192u : P.nearest ? 65536u : 24576u);
+}
+
+cudaError_t launch_pa_resample_clusters(const PaLattice* jobs, double* const* lnZ, uint32_t njobs, cudaStream_t s) {
+    static_assert(sizeof(ResampleClusters) <= 4000, "kernel parameters");
+    ResampleClusters A;
+    std::memset(&A, 0, sizeof(A));
+    uint32_t R = 1;
+    for (uint32_t j = 0; j < njobs; ++j) {
+        A.jobs[j] = jobs[j];
+        A.lnZ[j] = lnZ[j];
+        A.first[j + 1] = A.first[j] + jobs[j].n_inst;
+        R = jobs[j].R > R ? jobs[j].R : R;
+    }
+    for (uint32_t j = njobs; j < (uint32_t)kMaxJobs; ++j) A.first[j + 1] = A.first[j];
+    // Blocks per cluster: 8; 16 for larger populations while there are few of them, as only a
+    // few clusters of 16 find room at once (multinomial, us for 16 : 8 : 4 blocks: one population
+    // of 5000 14 : 15 : 18, of 20 000 22 : 26 : 44; 32 of 5000 32 : 18 : 20).
+    uint32_t blocks = R > 2048u && A.first[njobs] <= 4u ? 16u : 8u;
+    cudaError_t e = cudaSuccess;
+    for (;; blocks = 8u) {
+        const uint32_t K = blocks - 1u;
+        A.slice = ((R + K - 1u) / K + 1u) & ~1u;
+        const size_t bytes = (size_t)A.slice * 12u + kScanThreads / 32 * 64 * 8;
+        cudaLaunchConfig_t cfg = {};
+        cfg.blockDim = dim3(kScanThreads);
+        cfg.gridDim = dim3(blocks * A.first[njobs]);
+        cfg.dynamicSmemBytes = bytes;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = blocks;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaFuncSetAttribute(k_pa_resample_clusters, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        if (blocks > 8u) {  // beyond the portable size: where the device can place it
+            e = cudaFuncSetAttribute(k_pa_resample_clusters, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            int clusters = 0;
+            if (e != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&clusters, k_pa_resample_clusters, &cfg) != cudaSuccess || clusters < 1) {
+                cudaGetLastError();
+                continue;
+            }
+        }
+        e = cudaLaunchKernelEx(&cfg, k_pa_resample_clusters, A);
+        count_launch();
+        return e;
+    }
 }
 
 // Record of one step for every population of a lattice, after its sweeps.
