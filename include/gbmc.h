@@ -521,6 +521,8 @@ gbmc_status pa_state_load(gbmc_ctx *ctx, gbmc_pa *pa, const void *host, size_t b
 /* r = 0) is <= ceil(exp(-(beta_{k+1}-beta_k)(E_a-E_b)) 2^32) - 1 (host fp64). */
 /* Swaps exchange temperature labels (two maps), not configurations. The     */
 /* lattice (int8, shared-memory resident) belongs to the run until pt_free.  */
+/* pt_step runs many rounds in one launch where that is faster (AUTO kernel    */
+/* mode; profiled as pt_rounds), else one sweep and one exchange launch each.  */
 /* ------------------------------------------------------------------------ */
 gbmc_status pt_create(gbmc_ctx *ctx, gbmc_lattice *lat, const double *betas /* host [n_replicas] */,
                       uint32_t theta, gbmc_pt **out);

@@ -54,7 +54,7 @@ enum ProfKind {
     PK_INIT, PK_COUPLINGS, PK_SWEEP_RES, PK_HALFSWEEP, PK_OBS, PK_PA_WEIGHTS, PK_PA_REDUCE,
     PK_PA_DRAWS, PK_PA_PLACE, PK_PA_RECORD, PK_PA_RESET, PK_SWEEP_TILES, PK_SCHEDULE, PK_PA_FUSED,
     PK_BP_HALFSWEEP, PK_SWEEP_DCB, PK_SWEEP_MSC, PK_SW, PK_BP_STRIPS, PK_SWEEP_STRIPS, PK_PT_EXCHANGE, PK_SWEEP_BITS,
-    PK_BP_PACK, PK_SWEEP_DCB_BITS, PK_SWEEP_DCB_RES, PK_SWEEP_STREAM, PK_STREAM_STRIPS, PK_COUNT
+    PK_BP_PACK, PK_SWEEP_DCB_BITS, PK_SWEEP_DCB_RES, PK_SWEEP_STREAM, PK_STREAM_STRIPS, PK_PT_ROUNDS, PK_COUNT
 };
 const char* const kProfNames[PK_COUNT] = {"init_spins", "couplings", "sweep_resident", "halfsweep_global",
                                           "observables", "pa_weights", "pa_reduce", "pa_draws", "pa_place",
@@ -62,7 +62,7 @@ const char* const kProfNames[PK_COUNT] = {"init_spins", "couplings", "sweep_resi
                                           "bitpack_halfsweep", "sweep_dcb", "sweep_msc", "swendsen_wang",
                                           "bitpack_strips", "sweep_strips", "pt_exchange", "sweep_bits",
                                           "bitpack_convert", "sweep_dcb_bits",
-                                          "sweep_dcb_resident", "sweep_stream", "stream_strips"};
+                                          "sweep_dcb_resident", "sweep_stream", "stream_strips", "pt_rounds"};
 
 // Device words of a context: 8 flags and counters, then the progress
 // counters of strip-resident sweeps (one per CTA, one CTA per SM).
@@ -2673,8 +2673,8 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
     CUDA_TRY(cudaSetDevice(ctx->device));
     gbmc_lattice* l = pt->lat;
     if ((uint64_t)l->t + (uint64_t)n_steps * pt->theta > 0xFFFFFFFFull) return fail(GBMC_ERR_ARG, "sweep counter would wrap");
-    for (uint32_t n = 0; n < n_steps; ++n) {
-        const Tuning tu = tune(l);
+    const Tuning tu = tune(l);
+    for (uint32_t n = 0; n < n_steps;) {
         SweepJob J = base_job(l, tu);
         J.nsweeps = pt->theta;
         J.E = pt->E;
@@ -2688,9 +2688,6 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
         P.dim = l->d.dim;
         P.ea = l->d.model == GBMC_EA_PMJ;
         P.swar = (l->d.L % 8) == 0;
-        gbmc_status st = launch_jobs(ctx, P, std::vector<Tuning>{tu});
-        if (st != GBMC_OK) return st;
-        l->t += pt->theta;
         PtExchange X;
         X.E = pt->E;
         X.rep_of = pt->rep_of;
@@ -2702,9 +2699,23 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
         X.M = pt->M;
         X.n_inst = l->d.n_instances;
         X.inst_base = l->d.instance_base;
-        X.round = pt->round++;
-        ProfScope ps_(ctx, PK_PT_EXCHANGE);
-        CUDA_TRY(launch_pt_exchange(X, ctx->stream));
+        X.round = pt->round;
+        // a launch of rounds is kept to some ten milliseconds: 2^34 site updates, 2^13 sweeps
+        const double sweeps = std::max(1u, pt->theta), updates = (double)l->N * (double)l->ncopies * sweeps;
+        X.rounds = (uint32_t)std::max(1.0, std::min({(double)(n_steps - n), 17179869184.0 / updates, 8192.0 / sweeps}));
+        if (ctx->sweep_kernel == GBMC_KERNEL_AUTO && tu.bits && tempering_in_rounds(P, ctx->sm_count)) {
+            ProfScope ps_(ctx, PK_PT_ROUNDS);
+            CUDA_TRY(launch_tempering_rounds(P, X, ctx->sm_count, ctx->stream));
+        } else {
+            X.rounds = 1;
+            gbmc_status st = launch_jobs(ctx, P, std::vector<Tuning>{tu});
+            if (st != GBMC_OK) return st;
+            ProfScope ps_(ctx, PK_PT_EXCHANGE);
+            CUDA_TRY(launch_pt_exchange(X, ctx->stream));
+        }
+        l->t += pt->theta * X.rounds;
+        pt->round += X.rounds;
+        n += X.rounds;
     }
     return GBMC_OK;
 }

@@ -1,12 +1,26 @@
 // copies.cuh -- what the bit-sliced resident sweep kernels (bitsweep.cu,
-// stream.cu) write per copy after its sweeps.
+// stream.cu) do with a copy after its sweeps: write its energy and magnetisation,
+// decide its exchanges in parallel tempering.
 #pragma once
 #include <climits>
 #include <cstdint>
 
+#include "device.cuh"
 #include "internal.h"
 
 namespace gbmc {
+
+// Whether the configurations at temperatures k and k + 1 of instance `inst`, with
+// energies Ea and Eb, are exchanged in round `round`.
+__device__ __forceinline__ bool pt_accept(const PtExchange& X, uint32_t inst, uint32_t k, int32_t Ea, int32_t Eb,
+                                          uint32_t round) {
+    if (Eb >= Ea) return true;
+    const uint32_t m = (uint32_t)(Ea - Eb) >> 2;
+    const long long thr = X.tab[(uint64_t)k * (X.M + 1) + (m <= X.M ? m : X.M)];
+    const uint4 w = philox4x32_10(make_uint4(k >> 2, round, 0u, (4u << 28) | (X.inst_base + inst)), (uint32_t)X.seed,
+                                  (uint32_t)(X.seed >> 32));
+    return (long long)word_of(w, k & 3u) <= thr;
+}
 
 // Energy and magnetisation of one copy after the last sweep (or of every
 // sweep when a series is asked for): lane 0 writes them and, for annealing

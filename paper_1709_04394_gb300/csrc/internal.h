@@ -321,8 +321,13 @@ struct PtExchange {
     const long long* tab;      // [T-1][M+1] threshold of pair k at energy gap 4m (-1: never)
     uint64_t seed;
     uint32_t T, M, n_inst, inst_base, round;
+    uint32_t rounds;           // tempering_in_rounds: rounds of the launch, from `round`
 };
 cudaError_t launch_pt_exchange(const PtExchange& X, cudaStream_t s);
+// Rounds of sweeps (J.nsweeps each) and exchanges in one launch (stream.cu), and whether
+// that is the faster way for P's one job.
+bool tempering_in_rounds(const SweepLaunch& P, int sm_count);
+cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, int sm_count, cudaStream_t s);
 
 // ---- schedule MLP (6 -> 64 -> 64 -> 1) ----
 constexpr int kMlpIn = 6;

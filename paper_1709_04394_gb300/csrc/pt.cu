@@ -7,6 +7,10 @@
 // word k&3, t = n, r = 0) is <= the host-computed threshold of the energy gap
 // E_a - E_b = 4m. Swaps exchange temperature labels (rep_of / temp_of), not
 // configurations, as the paper recommends for shared memory.
+//
+// One launch per round, after the round's sweep launch; where that is faster, whole
+// rounds run in one launch instead (stream.cu, tempering_in_rounds).
+#include "copies.cuh"
 #include "device.cuh"
 #include "internal.h"
 
@@ -19,16 +23,7 @@ __global__ void k_pt_exchange(const __grid_constant__ PtExchange X) {
     const int32_t* E = X.E + (uint64_t)inst * X.T;
     for (uint32_t k = 2 * threadIdx.x + (X.round & 1u); k + 1 < X.T; k += 2 * blockDim.x) {
         const uint32_t a = rep[k], b = rep[k + 1];
-        const int32_t Ea = E[a], Eb = E[b];
-        bool accept = Eb >= Ea;
-        if (!accept) {
-            const uint32_t m = (uint32_t)(Ea - Eb) >> 2;
-            const long long thr = X.tab[(uint64_t)k * (X.M + 1) + (m <= X.M ? m : X.M)];
-            const uint4 w = philox4x32_10(make_uint4(k >> 2, X.round, 0u, (4u << 28) | (X.inst_base + inst)),
-                                          (uint32_t)X.seed, (uint32_t)(X.seed >> 32));
-            const uint32_t u = word_of(w, k & 3u);
-            accept = (long long)u <= thr;
-        }
+        const bool accept = pt_accept(X, inst, k, E[a], E[b], X.round);
         if (accept) {
             rep[k] = b;
             rep[k + 1] = a;

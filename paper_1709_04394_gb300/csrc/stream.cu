@@ -35,6 +35,8 @@
 #include <cstring>
 #include <utility>
 
+#include <cooperative_groups.h>
+
 #include "bits.cuh"
 #include "check.cuh"
 #include "copies.cuh"
@@ -43,14 +45,20 @@
 
 namespace gbmc {
 
+namespace cg = cooperative_groups;
+
 namespace {
 
 constexpr uint32_t kStreamThreads = 128;      // threads per block with one-warp teams
 constexpr size_t kStreamSmem = 227 * 1024;   // shared memory of an SM
 constexpr uint32_t kStreamTeamWords = 3072;  // a one-warp team's share of shared memory, at most
+// temperatures of the copies of a launch (kRounds: exchanged, too, round after round)
+enum { kOneTemp = 0, kPerCopy = 1, kRounds = 2 };
 // largest block, and blocks per SM the registers have to leave room for: 64 registers
-// a thread for C = 1 and 2 (128 for S = 4), 96 for C = 4
-constexpr uint32_t stream_max_threads(int C, int S) { return C == 4 ? 128u : C == 2 || S == 4 ? 512u : 1024u; }
+// a thread for C = 1 and 2 (128 for S = 4 and for C = 1 in rounds), 96 for C = 4
+constexpr uint32_t stream_max_threads(int C, int S, int PT = kOneTemp) {
+    return C == 4 ? 128u : C == 2 || S == 4 || PT == kRounds ? 512u : 1024u;
+}
 constexpr uint32_t stream_min_blocks(int C) { return C == 4 ? 5u : C == 2 ? 2u : 1u; }
 
 // Philox calls of one copy in lockstep: with fewer copies per thread more calls of
@@ -166,18 +174,15 @@ struct Place {
 };
 
 // Unsatisfied-bond masks of word w of colour c: d[k][copy], k in the order
-// (same-j x neighbour, other x neighbour, y - 1, y + 1, z - 1, z + 1), and the
-// other plane's word w (same).
-template <int DIM, bool EA, int C, bool EAGER>
+// (same-j x neighbour, other x neighbour, y - 1, y + 1, z - 1, z + 1), j the bond
+// words in that order, and the other plane's word w (same).
+template <int DIM, int C, bool EAGER>
 __device__ __forceinline__ void stream_unsat(const StreamShape& g, const Words<C>* oth, const Words<C>& own,
                                              const Place<DIM, EAGER>& at, uint32_t colour,
-                                             const uint32_t* __restrict__ bond,
+                                             const uint32_t (&j)[2 * DIM],
                                              uint32_t d[2 * DIM][C], Words<C>& same) {
     const uint32_t w = at.w;
     const uint32_t odd = at.odd(g, colour), edge = at.edge(g, colour);
-    uint32_t j[2 * DIM];
-#pragma unroll
-    for (int k = 0; k < 2 * DIM; ++k) j[k] = EA ? __ldg(bond + k * g.PW + w) : 0u;
     Window<C> up, dn;
     up.load(oth, at.template at<0>(g), g.PWX);
     dn.load(oth, at.template at<1>(g), g.PWX);
@@ -249,9 +254,16 @@ __device__ __forceinline__ void stream_extend(uint32_t* plane, uint32_t n, const
 // item i of its n_groups * PW words is word i % PW of group i / PW. S = 4 (C = 1
 // only): four threads per word, each the eight sites of one byte of it (two
 // Philox calls), for launches too small to give every scheduler two warps.
-template <int DIM, bool EA, int C, int S, bool PT>
-__global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C))
-    k_sweep_stream(const __grid_constant__ SweepLaunch P, uint32_t smem_words) {
+//
+// PT = kRounds: X.rounds rounds of parallel tempering. The copies of an instance are
+// divided over the blocks of one cluster and stay there; after a round's sweeps every
+// block receives all their energies, works out all exchanges for itself and takes its
+// copies' new thresholds. Against a sweep and an exchange launch per round: 3D +-J L = 8,
+// 128 x 32 copies, 10 sweeps per round 34 -> 27 us per round, 1 x 32 copies 28
+// -> 10.
+template <int DIM, bool EA, int C, int S, int PT>
+__global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_blocks(C))
+    k_sweep_stream(const __grid_constant__ SweepLaunch P, const __grid_constant__ PtExchange X, uint32_t smem_words) {
     extern __shared__ __align__(16) uint32_t smw[];
     int jid = 0;
     while (jid + 1 < P.njobs && blockIdx.x >= P.cta_begin[jid + 1]) ++jid;
@@ -261,9 +273,17 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
     const uint32_t tib = warp ? threadIdx.x >> 5 : 0u, tl = warp ? threadIdx.x & 31u : threadIdx.x;
     const uint32_t ng = J.ctas_per_inst;  // groups per instance
     const uint32_t n_all = J.n_inst * ng;
-    const uint64_t first = ((uint64_t)(blockIdx.x - P.cta_begin[jid]) * (blockDim.x / T) + tib) * G;
-    if (first >= n_all) return;  // the whole team; teams share no barrier
-    const uint32_t n = min(G, n_all - (uint32_t)first);
+    uint64_t first = ((uint64_t)(blockIdx.x - P.cta_begin[jid]) * (blockDim.x / T) + tib) * G;
+    if (first >= n_all && PT != kRounds) return;  // the whole team; teams share no barrier
+    uint32_t n = min(G, n_all - (uint32_t)first);
+    uint32_t rank = 0, n_blocks = 1;
+    if constexpr (PT == kRounds) {  // the last blocks of a cluster may have no copies
+        rank = cg::this_cluster().block_rank();
+        n_blocks = cg::this_cluster().num_blocks();
+        const uint32_t lo = min(ng, (rank * (blockDim.x / T) + tib) * G);
+        first = (uint64_t)(blockIdx.x / n_blocks) * ng + lo;
+        n = min(G, ng - lo);
+    }
     const StreamShape g = stream_shape<DIM>(J.L, J.N);
     // shared memory of the team: planes [colour][group][word][copy], then per
     // group [instance, first replica, active copies] and per copy [U, D], the
@@ -274,6 +294,20 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
     int* const acc = reinterpret_cast<int*>(meta + 3u * G);
     uint32_t* const sfrom = meta + 3u * G + 2u * G * C;
     uint32_t* const sthr = sfrom + G * C;
+    // rounds of tempering: the instance's maps, accepted swaps and (by round parity) energies
+    uint32_t* const srep = smw + (blockDim.x / T) * smem_words;
+    uint32_t* const stmp = srep + J.R;
+    uint32_t* const sacc = stmp + J.R;
+    int* const sE = reinterpret_cast<int*>(sacc + J.R);
+    if constexpr (PT == kRounds) {
+        const uint64_t base = (uint64_t)(blockIdx.x / n_blocks) * J.R;
+        for (uint32_t k = threadIdx.x; k < J.R; k += blockDim.x) {
+            srep[k] = X.rep_of[base + k];
+            stmp[k] = X.temp_of[base + k];
+            sacc[k] = 0u;
+        }
+        cg::this_cluster().barrier_arrive();
+    }
     uint32_t any = 0;
     for (uint32_t gi = tl; gi < n; gi += T) {
         const uint32_t grp = (uint32_t)first + gi, inst = grp / ng, r0 = (grp - inst * ng) * C;
@@ -295,7 +329,11 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
             }
         }
     }
-    if (warp ? !__any_sync(0xFFFFFFFFu, any != 0u) : !__syncthreads_or(any != 0u)) return;
+    if constexpr (PT == kRounds) {
+        cg::this_cluster().barrier_wait();  // all have started, and read the maps
+    } else if (warp ? !__any_sync(0xFFFFFFFFu, any != 0u) : !__syncthreads_or(any != 0u)) {
+        return;
+    }
     team_sync(warp);
 
     const uint32_t* mask = J.smask;
@@ -355,7 +393,17 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
     // item is -> group, copies and place; worked out once where a thread has one
     // item at most (small populations, where the chain of a half-sweep is what counts)
     uint32_t gi = 0, part = 0, inst = 0, r0 = 0;
-    Place<DIM, S == 4> at;
+    constexpr bool kEager = S == 4 || (C == 1 && PT == kRounds);
+    Place<DIM, kEager> at;
+    uint32_t jkept[PT == kRounds && EA ? 2 : 1][2 * DIM];  // bond words of both colours
+    auto bonds = [&](uint32_t colour, uint32_t in, uint32_t (&j)[2 * DIM]) {
+#pragma unroll
+        for (int k = 0; k < 2 * DIM; ++k) {
+            if constexpr (!EA) j[k] = 0u;
+            else if constexpr (PT == kRounds) j[k] = colour ? jkept[1][k] : jkept[0][k];
+            else j[k] = __ldg(J.sbond + ((uint64_t)in * 2u + colour) * NB + k * g.PW + at.w);
+        }
+    };
     auto locate = [&](uint32_t is) {
         const uint32_t i = is / S;
         part = is % S;
@@ -363,8 +411,14 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
         inst = meta[3u * gi];
         r0 = meta[3u * gi + 1u];
         at.set(g, i - gi * g.PW, mask);
+        if constexpr (PT == kRounds && EA) {
+#pragma unroll
+            for (int k = 0; k < 2 * 2 * DIM; ++k)
+                jkept[k / (2 * DIM)][k % (2 * DIM)] =
+                    __ldg(J.sbond + ((uint64_t)inst * 2u + k / (2 * DIM)) * NB + (k % (2 * DIM)) * g.PW + at.w);
+        }
     };
-    const bool once = S == 4 && items * S <= T;
+    const bool once = kEager && items * S <= T;
     if (once && tl < items * S) locate(tl);
     // adds an item's unsatisfied bonds (of colour-0 sites, d) and down spins to its
     // copies' sums: at once, or in registers first where all items are one group's
@@ -407,9 +461,46 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
             if (i < n * C) acc[2u * i] = acc[2u * i + 1u] = 0;
         }
     };
+    // Exchanges of a round of tempering, from the copies' sums
+    auto exchange = [&](uint32_t round) {
+        cg::cluster_group cluster = cg::this_cluster();
+        int* E = sE + (round & 1u) * J.R;
+        const uint32_t in = blockIdx.x / n_blocks;
+        for (uint32_t i = tl; i < n * C; i += T) {
+            const uint32_t gr = i / C, c = i % C, slot = meta[3u * gr + 1u] + c;
+            if (c < meta[3u * gr + 2u]) {
+                const int e = 2 * acc[2u * i] - DIM * (int)J.N;
+                for (uint32_t b = 0; b < n_blocks; ++b) *cluster.map_shared_rank(E + slot, b) = e;
+                if (round + 1u == X.rounds) {
+                    J.E[(uint64_t)in * J.R + slot] = e;
+                    J.M[(uint64_t)in * J.R + slot] = (int)J.N - 2 * acc[2u * i + 1u];
+                }
+            }
+            acc[2u * i] = acc[2u * i + 1u] = 0;
+        }
+        cluster.sync();
+        for (uint32_t k = 2u * threadIdx.x + ((X.round + round) & 1u); k + 1u < J.R; k += 2u * blockDim.x) {
+            const uint32_t a = srep[k], b = srep[k + 1u];
+            if (pt_accept(X, in, k, E[a], E[b], X.round + round)) {
+                srep[k] = b;
+                srep[k + 1u] = a;
+                stmp[b] = k;
+                stmp[a] = k + 1u;
+                sacc[k] += 1u;
+            }
+        }
+        __syncthreads();
+        for (uint32_t i = tl; i < n * C; i += T) {
+            const uint32_t gr = i / C, c = i % C;
+            if (c >= meta[3u * gr + 2u]) continue;
+            const uint32_t* th = J.thr_temp + 3ull * stmp[meta[3u * gr + 1u] + c];
+            for (uint32_t k = 0; k < 3u; ++k) sthr[3u * i + k] = th[k];
+        }
+    };
 #pragma unroll
     for (int c = 0; c < C; ++c) U[c] = D[c] = 0;
-    const bool series = J.Eser || J.Mser;
+    const bool series = PT != kRounds && (J.Eser || J.Mser);
+    for (uint32_t round = 0; round < (PT == kRounds ? X.rounds : 1u); ++round)
     for (uint32_t s = 0; s <= nsw; ++s) {
         if (s == nsw && nsw != 0) break;  // s == nsw: measurement-only pass when nothing is swept
         const bool sweep = s < nsw;
@@ -426,10 +517,10 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
                 Words<C> nw = own[w];
                 uint32_t ge[C], ea[C], eb[C];  // dE <= 0; dE = 4; dE = 8 (3D)
                 {
-                    uint32_t d[2 * DIM][C];
+                    uint32_t d[2 * DIM][C], j[2 * DIM];
                     Words<C> same;
-                    stream_unsat<DIM, EA, C>(g, oth, nw, at, colour,
-                                             EA ? J.sbond + ((uint64_t)inst * 2u + colour) * NB : nullptr, d, same);
+                    bonds(colour, inst, j);
+                    stream_unsat<DIM, C>(g, oth, nw, at, colour, j, d, same);
                     if (measure) tally(d, nw, same, S == 4 ? 0xFFu << (8u * part) : 0xFFFFFFFFu);
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
@@ -456,7 +547,7 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
                 for (int c = 0; c < C; ++c) {
                     uint32_t hi, lo, uh, ul;
                     mulhilo_wide(kPhiloxM1, r0 + c, hi, lo);
-                    mulhilo_wide(kPhiloxM0, hi ^ (J.t0 + s) ^ k0, uh, ul);
+                    mulhilo_wide(kPhiloxM0, hi ^ (PT == kRounds ? J.t0 + round * nsw + s : J.t0 + s) ^ k0, uh, ul);
                     ck[c].b1 = lo ^ (k0 + kPhiloxW0);
                     ck[c].u1 = uh ^ (k1 + kPhiloxW1);
                     ck[c].v1 = ul;
@@ -552,25 +643,43 @@ __global__ void __launch_bounds__(stream_max_threads(C, S), stream_min_blocks(C)
         }
         const bool last = sweep ? s + 1u == nsw : true;
         if ((last && want_final) || (series && sweep && (last || C > 1))) {
-            for (uint32_t i = tl; i < items; i += T) {
-                const uint32_t gr = G == 1u ? 0u : i / g.PW;
-                const Words<C>* p0 = reinterpret_cast<const Words<C>*>(sm + gr * g.PWX * C);
-                const Words<C>* p1 = reinterpret_cast<const Words<C>*>(sm + plane + gr * g.PWX * C);
-                gi = gr;
-                at.set(g, i - gr * g.PW, mask);
+            // (a word's four threads of S = 4 count a byte each)
+            constexpr uint32_t kParts = PT == kRounds ? S : 1;
+            for (uint32_t is = tl; is < items * kParts; is += T) {
+                if constexpr (PT == kRounds) {
+                    if (!once) locate(is);
+                } else {
+                    gi = G == 1u ? 0u : is / g.PW;
+                    inst = meta[3u * gi];
+                    at.set(g, is - gi * g.PW, mask);
+                }
+                const Words<C>* p0 = reinterpret_cast<const Words<C>*>(sm + gi * g.PWX * C);
+                const Words<C>* p1 = reinterpret_cast<const Words<C>*>(sm + plane + gi * g.PWX * C);
                 const Words<C> w0 = p0[at.w];
-                uint32_t d[2 * DIM][C];
+                uint32_t d[2 * DIM][C], j[2 * DIM];
                 Words<C> w1;
-                stream_unsat<DIM, EA, C>(g, p1, w0, at, 0u, EA ? J.sbond + (uint64_t)meta[3u * gr] * 2u * NB : nullptr, d,
-                                         w1);
-                tally(d, w0, w1, 0xFFFFFFFFu);
+                bonds(0u, inst, j);
+                stream_unsat<DIM, C>(g, p1, w0, at, 0u, j, d, w1);
+                tally(d, w0, w1, kParts == 4u ? 0xFFu << (8u * part) : 0xFFFFFFFFu);
             }
             flush();
             team_sync(warp);
-            record(s, sweep, last);
+            if constexpr (PT == kRounds) exchange(round);
+            else record(s, sweep, last);
 #pragma unroll
             for (int c = 0; c < C; ++c) U[c] = D[c] = 0;
             team_sync(warp);
+        }
+    }
+
+    if constexpr (PT == kRounds) {
+        if (rank == 0) {
+            const uint64_t in = blockIdx.x / n_blocks;
+            for (uint32_t k = threadIdx.x; k < J.R; k += blockDim.x) {
+                X.rep_of[in * J.R + k] = srep[k];
+                X.temp_of[in * J.R + k] = stmp[k];
+                if (k + 1u < J.R) X.accepted[in * (J.R - 1u) + k] += sacc[k];
+            }
         }
     }
 
@@ -673,10 +782,12 @@ struct StreamPlan {
     double cost = 1e300;
 };
 
+double stream_pass(int C, int split) { return C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 980.0 : 420.0; }
+double stream_lat(int C, int split) { return C == 4 ? 9000.0 : C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0; }
+
 StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_count) {
     // measured: 2D L = 64 with 10^5 copies (pass), L = 36 and 68 with one warp per scheduler (lat)
-    const double pass = C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 980.0 : 420.0;
-    const double lat = C == 4 ? 9000.0 : C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0;
+    const double pass = stream_pass(C, split), lat = stream_lat(C, split);
     const double by_regs = C == 4 ? 5.0 : 8.0;  // warps per scheduler the registers allow
     const double schedulers = 4.0 * sm_count;
     StreamPlan S;
@@ -719,7 +830,7 @@ StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_c
     return S;
 }
 
-template <int DIM, bool EA, int C, int SP, bool PT>
+template <int DIM, bool EA, int C, int SP, int PT>
 cudaError_t launch_stream(const SweepLaunch& P0, const StreamPlan& S, cudaStream_t st) {
     SweepLaunch P = P0;
     uint64_t total = 0;
@@ -748,21 +859,136 @@ cudaError_t launch_stream(const SweepLaunch& P0, const StreamPlan& S, cudaStream
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(uint32_t)total, S.threads, smem, st>>>(P, warp_words);
+    kern<<<(uint32_t)total, S.threads, smem, st>>>(P, PtExchange{}, warp_words);
     count_launch();
     return cudaGetLastError();
 }
 
 template <int DIM, bool EA>
 cudaError_t launch_stream_c(const SweepLaunch& P, const StreamPlan& S, bool pt, cudaStream_t st) {
-    if (S.C == 4) return pt ? launch_stream<DIM, EA, 4, 1, true>(P, S, st) : launch_stream<DIM, EA, 4, 1, false>(P, S, st);
-    if (S.C == 2) return pt ? launch_stream<DIM, EA, 2, 1, true>(P, S, st) : launch_stream<DIM, EA, 2, 1, false>(P, S, st);
+    if (S.C == 4) return pt ? launch_stream<DIM, EA, 4, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 4, 1, kOneTemp>(P, S, st);
+    if (S.C == 2) return pt ? launch_stream<DIM, EA, 2, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 2, 1, kOneTemp>(P, S, st);
     if (S.split == 4)
-        return pt ? launch_stream<DIM, EA, 1, 4, true>(P, S, st) : launch_stream<DIM, EA, 1, 4, false>(P, S, st);
-    return pt ? launch_stream<DIM, EA, 1, 1, true>(P, S, st) : launch_stream<DIM, EA, 1, 1, false>(P, S, st);
+        return pt ? launch_stream<DIM, EA, 1, 4, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 1, 4, kOneTemp>(P, S, st);
+    return pt ? launch_stream<DIM, EA, 1, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 1, 1, kOneTemp>(P, S, st);
+}
+
+// How the copies of every instance are divided for rounds of tempering: B blocks of
+// `threads` threads, in teams of T with G copies each (one copy per thread: two
+// measured 20 % slower for want of work in flight). In cycles per
+// round, by the same pass and latency as above: a block keeps its place to the
+// end, so the blocks count in whole waves.
+struct RoundsPlan {
+    int split = 1;
+    uint32_t B = 1, G = 1, T = 32, threads = 32;
+    double cost = 1e300;
+};
+
+size_t rounds_smem(const SweepJob& J, const RoundsPlan& p) {
+    return (size_t)(p.threads / p.T * stream_smem_words(J.N, p.G, 1u, true) + 5u * J.R) * 4u;
+}
+
+RoundsPlan rounds_plan(const SweepJob& J, int dim, int sm_count) {
+    RoundsPlan best;
+    const uint32_t PW = (J.N / 2u + 31u) / 32u;
+    const uint32_t ng = J.R;
+    for (const int split : {4, 1}) {
+        const uint32_t most = stream_max_threads(1, split, kRounds);
+        // (3D: four more compares of a call's sixteen)
+        const double pass = stream_pass(1, split) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, split);
+        auto consider = [&](uint32_t B, uint32_t G, uint32_t T, uint32_t threads) {
+            RoundsPlan p;
+            p.split = split, p.B = B, p.G = G, p.T = T, p.threads = threads;
+            const size_t smem = rounds_smem(J, p);
+            if (smem > 200u * 1024u) return;
+            const double passes = std::ceil(G * PW * split / (double)T), warps = threads / 32.0;
+            const double held = std::min({std::floor((double)most / threads),  // by registers
+                                          std::floor((double)kStreamSmem / (smem + 1024.0)), 16.0});
+            const double blocks = (double)J.n_inst * B, wave = held * sm_count, full = std::floor(blocks / wave);
+            auto half = [&](double per_sm) {  // a half-sweep with so many blocks on an SM
+                const double w = std::ceil(per_sm * warps / 4.0);
+                return passes * (std::max(lat, w * pass) + (w > 1.0 ? 200.0 : 0.0) + 2.0 * per_sm * warps) +
+                       (T > 32u ? 300.0 : 0.0);
+            };
+            const double rest = std::ceil((blocks - full * wave) / sm_count);
+            const double t = full * half(held) + (rest > 0.0 ? half(rest) : 0.0);
+            const double waves = full + (rest > 0.0 ? 1.0 : 0.0);
+            p.cost = (2.0 * J.nsweeps + 0.4) * t + waves * (B > 1u ? 2500.0 : 1500.0);
+            if (p.cost < best.cost) best = p;
+        };
+        for (uint32_t B = 1; B <= 8u && B <= ng; B *= 2u) {
+            // one-warp teams, with up to eight passes over their words
+            for (uint32_t G = 1; G <= ng && G * PW * split <= 256u; ++G) {
+                const uint32_t teams = (ng + G - 1u) / G, warps = (teams + B - 1u) / B;
+                if (warps * 32u <= most) consider(B, G, 32u, warps * 32u);
+            }
+            const uint32_t G = (ng + B - 1u) / B, items = G * PW * (uint32_t)split, passes = (items + most - 1u) / most;
+            const uint32_t threads = ((items + passes - 1u) / passes + 31u) & ~31u;
+            if (threads > 32u) consider(B, G, threads, threads);
+        }
+    }
+    return best;
+}
+
+template <int DIM, bool EA, int SP>
+cudaError_t launch_rounds(const SweepLaunch& P0, const PtExchange& X, const RoundsPlan& R, cudaStream_t st) {
+    SweepLaunch P = P0;
+    SweepJob& J = P.jobs[0];
+    J.ctas_per_inst = J.R;
+    J.team = R.T;
+    J.rpc = R.G;
+    P.cta_begin[0] = 0;
+    P.cta_begin[1] = P.total = J.n_inst * R.B;
+    auto kern = k_sweep_stream<DIM, EA, 1, SP, kRounds>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(P.total);
+    cfg.blockDim = dim3(R.threads);
+    cfg.dynamicSmemBytes = rounds_smem(J, R);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = R.B;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cfg.dynamicSmemBytes > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+        if (e != cudaSuccess) return e;
+    }
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P, X, stream_smem_words(J.N, R.G, 1u, true));
+    count_launch();
+    return e;
+}
+
+template <int DIM, bool EA>
+cudaError_t launch_rounds_c(const SweepLaunch& P, const PtExchange& X, const RoundsPlan& R, cudaStream_t st) {
+    return R.split == 4 ? launch_rounds<DIM, EA, 4>(P, X, R, st) : launch_rounds<DIM, EA, 1>(P, X, R, st);
 }
 
 }  // namespace
+
+// A round by itself is a sweep launch, whose copies are loaded and stored, and an
+// exchange launch, about 20 000 cycles beside the half-sweeps (3D L = 8, 250 x 40 copies, one
+// sweep per round: 15.4 us, 4.8 of them sweeping). What speaks for it is that its blocks
+// change places between rounds: 256 x 40 copies of L = 12, 10 sweeps per round, 207 us
+// each against 248 in one launch of rounds; 100 x 36 53 against 38.
+bool tempering_in_rounds(const SweepLaunch& P, int sm_count) {
+    const SweepJob& J = P.jobs[0];
+    if (!J.smask || (P.ea && !J.sbond) || J.nsweeps == 0u || J.R < 2u || J.R > 1024u) return false;
+    double alone = stream_plan(P, 1, 4, true, sm_count).cost;
+    for (int C = 4; C >= 1; C >>= 1)
+        if (C == 1 || stream_smem_words(J.N, 1u, (uint32_t)C, true) * 4u <= 36u * 1024u)
+            alone = std::min(alone, stream_plan(P, C, 1, true, sm_count).cost);
+    return rounds_plan(J, P.dim, sm_count).cost < 2.0 * J.nsweeps * alone * (P.dim == 3 ? 1.15 : 1.0) + 20000.0;
+}
+
+cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, int sm_count, cudaStream_t s) {
+    const RoundsPlan R = rounds_plan(P.jobs[0], P.dim, sm_count);
+    if (P.dim == 2 && !P.ea) return launch_rounds_c<2, false>(P, X, R, s);
+    if (P.dim == 3 && !P.ea) return launch_rounds_c<3, false>(P, X, R, s);
+    if (P.dim == 3 && P.ea) return launch_rounds_c<3, true>(P, X, R, s);
+    return cudaErrorInvalidValue;
+}
 
 size_t stream_mask_words(uint32_t N) { return 5ull * ((N / 2u + 31u) / 32u); }
 size_t stream_bond_words(uint32_t N) { return 12ull * ((N / 2u + 31u) / 32u); }
