@@ -1216,7 +1216,9 @@ gbmc_status swendsen_wang(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint32_t 
     if (n_updates == 0) return GBMC_OK;
     if ((uint64_t)l->t + n_updates > 0xFFFFFFFFull) return fail(GBMC_ERR_ARG, "update counter would wrap");
     CUDA_TRY(cudaSetDevice(ctx->device));
-    if (!l->sw_parent) {
+    const bool resident = sw_resident((uint32_t)l->d.dim, (uint32_t)l->d.L, (uint32_t)l->N, l->ncopies,
+                                      E_series || M_series, ctx->sm_count);
+    if (!resident && !l->sw_parent) {
         const bool tiled = sw_tiled((uint32_t)l->d.dim, (uint32_t)l->d.L);
         cudaError_t e = cudaMalloc(&l->sw_parent, 4 * l->N * l->ncopies);
         if (e == cudaSuccess && !tiled) e = cudaMalloc(&l->sw_bonds, l->N * l->ncopies);
@@ -1246,7 +1248,17 @@ gbmc_status swendsen_wang(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint32_t 
     P.inst_base = l->d.instance_base;
     if ((P.L & (P.L - 1)) == 0)
         while ((1u << P.lshift) < P.L) ++P.lshift;
-    for (uint32_t u = 0; u < n_updates; ++u) {
+    if (resident) {
+        P.t = l->t;
+        P.labels = labels;
+        ProfScope ps_(ctx, PK_SW);
+        CUDA_TRY(launch_sw_resident(P, l->ncopies, n_updates, E_series, M_series, ctx->stream));
+    }
+    if (!resident && (E_series || M_series)) {  // the sums of all updates are added to these
+        ProfScope ps_(ctx, PK_OBS);
+        CUDA_TRY(launch_zero2(E_series, M_series, (uint64_t)n_updates * l->ncopies, ctx->stream));
+    }
+    for (uint32_t u = 0; !resident && u < n_updates; ++u) {
         P.t = l->t + u;
         P.labels = u + 1 == n_updates ? labels : nullptr;
         {
@@ -1257,7 +1269,7 @@ gbmc_status swendsen_wang(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint32_t 
             ProfScope ps_(ctx, PK_OBS);
             CUDA_TRY(launch_observables(l->cur, l->jbits, l->d.dim, (uint32_t)l->d.L, l->d.n_instances,
                                         l->d.n_replicas, E_series ? E_series + (uint64_t)u * l->ncopies : nullptr,
-                                        M_series ? M_series + (uint64_t)u * l->ncopies : nullptr, ctx->stream));
+                                        M_series ? M_series + (uint64_t)u * l->ncopies : nullptr, ctx->stream, true));
         }
     }
     l->t += n_updates;

@@ -75,7 +75,8 @@ cudaError_t launch_split_bonds(const uint8_t* jbits, uint8_t* jsplit, uint32_t L
 cudaError_t launch_jbits_to_int8(const uint8_t* jbits, int8_t* out, uint32_t N, uint32_t n_inst,
                                  cudaStream_t s);
 cudaError_t launch_observables(const int8_t* spins, const uint8_t* jbits, int dim, uint32_t L,
-                               uint32_t n_inst, uint32_t R, int32_t* E, int32_t* M, cudaStream_t s);
+                               uint32_t n_inst, uint32_t R, int32_t* E, int32_t* M, cudaStream_t s,
+                               bool zeroed = false);
 // a[i] = b[i] = 0, i < n; either may be null.
 cudaError_t launch_zero2(int32_t* a, int32_t* b, uint64_t n, cudaStream_t s);
 
@@ -250,6 +251,11 @@ struct SwLaunch {
     uint32_t lshift;          // log2 L when L is a power of two, else 0
 };
 cudaError_t launch_sw_update(const SwLaunch& P, uint64_t copies, cudaStream_t s);
+// All updates of a call on chip, from update P.t on, with E and M after each (or null), and
+// whether that is the way to take; it needs no bonds, parent or lab.
+bool sw_resident(uint32_t dim, uint32_t L, uint32_t N, uint64_t copies, bool series, int sm_count);
+cudaError_t launch_sw_resident(const SwLaunch& P, uint64_t copies, uint32_t n_updates, int32_t* E_series,
+                               int32_t* M_series, cudaStream_t s);
 // Lattices labelled tile by tile (2D: 32 x 32 tiles, 3D: 16 x 8 x 8) need no
 // bond-flag array; the others use the global union-find over stored flags.
 inline bool sw_tiled(uint32_t dim, uint32_t L) { return (dim == 2 && L % 32 == 0) || (dim == 3 && L % 16 == 0); }

@@ -285,7 +285,7 @@ cudaError_t launch_zero2(int32_t* a, int32_t* b, uint64_t n, cudaStream_t s) {
 }
 
 cudaError_t launch_observables(const int8_t* spins, const uint8_t* jbits, int dim, uint32_t L,
-                               uint32_t n_inst, uint32_t R, int32_t* E, int32_t* M, cudaStream_t s) {
+                               uint32_t n_inst, uint32_t R, int32_t* E, int32_t* M, cudaStream_t s, bool zeroed) {
     const uint32_t N = L * L * (dim == 3 ? L : 1);
     const uint64_t copies = (uint64_t)n_inst * R;
     const bool wide = L % 16 == 0;
@@ -300,7 +300,7 @@ cudaError_t launch_observables(const int8_t* spins, const uint8_t* jbits, int di
         bx = (items + 4u * 256u - 1u) / (4u * 256u);
         if (bx > most) bx = (uint32_t)most;
     }
-    if (bx > 1) {
+    if (bx > 1 && !zeroed) {
         cudaError_t e = launch_zero2(E, M, copies, s);
         if (e != cudaSuccess) return e;
     }

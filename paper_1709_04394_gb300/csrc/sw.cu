@@ -37,21 +37,31 @@
 //
 // 2D lattices with L % 32 == 0 take 32 x 32 tiles with a scanline labelling,
 // the tile labels kept apart from the global forest:
-//  k_sw_scan2    : one warp per tile, lane x = column x, the rows in order.
-//                  Row r's x bonds cut it into runs; a run's label is the
-//                  smallest of its start and of the labels its y bonds reach in
-//                  row r - 1, and a run that reaches two components above hooks
-//                  the larger label under the smaller in the tile's label
-//                  forest (shared memory). At the end every site's label is
-//                  resolved to its component's smallest site: lab[i] = that
-//                  site's tile-local index, and parent[g] = g for each such
-//                  tile root g, the only nodes of the global forest;
+//  k_sw_scan2    : one block per tile, its warps four rows each, lane x = column x,
+//                  the rows in order. Row r's x bonds cut it into runs; a run's
+//                  label is the smallest of its start and of the labels its y
+//                  bonds reach in row r - 1, and a run that reaches two components
+//                  above hooks the larger label under the smaller in the tile's
+//                  label forest (shared memory); then the warps' seams are united.
+//                  At the end every site's label is resolved to its component's
+//                  smallest site: lab[i] = that site's tile-local index, and
+//                  parent[g] = g for each such tile root g, the only nodes of the
+//                  global forest. Bound by the chain of a warp's rows (shuffles and
+//                  label lookups, about 2000 cycles each): L = 1024 36 us with one
+//                  warp for a tile's 32 rows, 16 us with 8 rows each, 13 us with 4;
 //  k_sw_cross    : unites the tile roots of the two ends of each active
-//                  tile-crossing bond in the global forest;
+//                  tile-crossing bond in the global forest, one bond of a warp's
+//                  between the same two roots for all;
 //  k_sw_flip_lab : one CTA per tile finds the global root of each tile root
 //                  whose component touches the tile border (the others are
 //                  roots of whole clusters) and draws each tile root's coin
 //                  once; every site takes its tile root's.
+//
+// Small lattices take none of this but one launch for all updates of a call, a block per
+// copy, labels and spins in shared memory (k_sw_resident).
+#include <algorithm>
+#include <cmath>
+
 #include "bits.cuh"
 #include "check.cuh"
 #include "device.cuh"
@@ -269,7 +279,7 @@ __device__ __forceinline__ void sw_warp_push(uint32_t* q, uint32_t& n, bool has,
 
 // ---- 2D scanline tiles ----
 
-constexpr uint32_t kSwScanWarps = 4;  // tiles (warps) per block of k_sw_scan2
+constexpr uint32_t kSwRows = 4, kSwWarps = 32u / kSwRows;  // rows per warp, warps per tile of k_sw_scan2
 
 // Global index of the 32 x 32 tile-local site k (k = 32 row + column) of the
 // tile holding site i.
@@ -278,44 +288,52 @@ __device__ __forceinline__ uint32_t sw_tile_root(uint32_t k, uint32_t i, uint32_
     return ((y & ~31u) + (k >> 5)) * L + (x & ~31u) + (k & 31u);
 }
 
-__global__ void __launch_bounds__(32 * kSwScanWarps) k_sw_scan2(const __grid_constant__ SwLaunch P) {
-    __shared__ uint32_t eq[kSwScanWarps][1024];       // label forest of each warp's tile (local indices)
-    __shared__ uint16_t rowlab[kSwScanWarps][1024];   // each site's run label, resolved at the end
-    const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+__global__ void __launch_bounds__(32 * kSwWarps) k_sw_scan2(const __grid_constant__ SwLaunch P) {
+    __shared__ uint32_t f[1024];   // the tile's label forest (local indices)
+    __shared__ uint16_t rl[1024];  // each site's run label
+    constexpr uint32_t kAll = 0xffffffffu;
+    const uint32_t lane = threadIdx.x & 31u, r0 = (threadIdx.x >> 5) * kSwRows;
     const uint32_t L = P.L, ntx = L >> 5;
-    const uint32_t tile = blockIdx.x * kSwScanWarps + wib;
-    if (tile >= ntx * ntx) return;  // whole warp; no block barriers follow
     const uint64_t copy = P.copy0 + blockIdx.y;
     const int8_t* s = P.spins + copy * P.N;
     uint32_t inst, r;
     split_copy(copy, P.R, inst, r);
-    const uint32_t bx = tile % ntx, by = tile / ntx, X = bx * 32u + lane;
-    uint32_t* f = eq[wib];
-    uint16_t* rl = rowlab[wib];
+    const uint32_t bx = blockIdx.x % ntx, by = blockIdx.x / ntx, X = bx * 32u + lane, Y = by * 32u + r0;
+    const bool more = r0 + kSwRows < 32u;  // the bonds below the last strip leave the tile (k_sw_cross)
+    int sp[kSwRows + 1];
+#pragma unroll
+    for (uint32_t k = 0; k <= kSwRows; ++k)
+        sp[k] = k < kSwRows || more ? s[GBMC_IDX((uint64_t)(Y + k) * L + X, P.N)] : 0;
     // bond words: the forward bonds b = 2 i + mu of sites i = 2 q, 2 q + 1 are
-    // the four words of Philox call q (t, replica and c3 hoisted)
+    // the four words of Philox call q (t, replica and c3 hoisted). All the strip's bonds
+    // first: masks over the row of the bonds to the right and of those below
     const PhiloxFixed pf = philox_fix(P.t, r, c3_word(kPurposeSwBond, 0u, P.inst_base + inst), (uint32_t)P.seed,
                                       (uint32_t)(P.seed >> 32));
     const long long Tb = P.T_bond;
-    uint4 c = make_uint4(0u, 0u, 0u, 0u);
-    int s_prev = 0;
-    uint32_t w1_prev = 0u, lab_prev = 0u;
-    for (uint32_t rr = 0; rr < 32u; ++rr) {
-        const uint32_t y = by * 32u + rr;
-        if ((rr & 1u) == 0u)  // lane l: the call of sites 2 (l & 15), +1 of row rr + l / 16
-            c = philox_q_wide(pf, ((y + (lane >> 4)) * L + bx * 32u + 2u * (lane & 15u)) >> 1);
-        const uint32_t src = ((rr & 1u) << 4) | (lane >> 1);
-        const uint32_t a0 = __shfl_sync(0xffffffffu, c.x, src), a1 = __shfl_sync(0xffffffffu, c.y, src);
-        const uint32_t a2 = __shfl_sync(0xffffffffu, c.z, src), a3 = __shfl_sync(0xffffffffu, c.w, src);
-        const uint32_t w0 = (lane & 1u) ? a2 : a0;  // bond along x: word (2 i) & 3
-        const uint32_t w1 = (lane & 1u) ? a3 : a1;  // bond along y: word (2 i + 1) & 3
-        const int sc = s[GBMC_IDX((uint64_t)y * L + X, P.N)];
-        const int sr = __shfl_down_sync(0xffffffffu, sc, 1);
-        // the bond from lane 31 leaves the tile (k_sw_cross); so does the one into row 0
-        const bool xb = lane < 31u && sc == sr && (long long)w0 <= Tb;
-        const bool yb = rr > 0u && sc == s_prev && (long long)w1_prev <= Tb;
-        const uint32_t R = ~(__ballot_sync(0xffffffffu, xb) << 1);  // run starts
-        const uint32_t own = rr * 32u + lane;
+    uint32_t right[kSwRows], below[kSwRows];
+#pragma unroll
+    for (uint32_t k = 0; k < kSwRows; k += 2u) {
+        // lane l: the call of sites 2 (l & 15), +1 of row k + l / 16
+        const uint4 c = philox_q_wide(pf, ((Y + k + (lane >> 4)) * L + bx * 32u + 2u * (lane & 15u)) >> 1);
+#pragma unroll
+        for (uint32_t e = 0; e < 2u; ++e) {
+            const uint32_t src = (e << 4) | (lane >> 1);
+            const uint32_t a0 = __shfl_sync(kAll, c.x, src), a1 = __shfl_sync(kAll, c.y, src);
+            const uint32_t a2 = __shfl_sync(kAll, c.z, src), a3 = __shfl_sync(kAll, c.w, src);
+            const uint32_t w0 = (lane & 1u) ? a2 : a0;  // bond along x: word (2 i) & 3
+            const uint32_t w1 = (lane & 1u) ? a3 : a1;  // bond along y: word (2 i + 1) & 3
+            const int sr = __shfl_down_sync(kAll, sp[k + e], 1);
+            // the bond from lane 31 leaves the tile
+            right[k + e] = __ballot_sync(kAll, lane < 31u && sp[k + e] == sr && (long long)w0 <= Tb);
+            below[k + e] = __ballot_sync(kAll, sp[k + e] == sp[k + e + 1u] && (long long)w1 <= Tb);
+        }
+    }
+    uint32_t lab_prev = 0u;
+#pragma unroll
+    for (uint32_t k = 0; k < kSwRows; ++k) {
+        const bool yb = k > 0u && ((below[k ? k - 1u : 0u] >> lane) & 1u);
+        const uint32_t R = ~(right[k] << 1);  // run starts
+        const uint32_t own = (r0 + k) * 32u + lane;
         f[own] = own;
         const uint32_t la = yb ? sw_find<false>(f, lab_prev) : 0u;  // the component above, if reached
         // the run's label: segmented minimum over the run (lane x - d is in x's
@@ -323,24 +341,32 @@ __global__ void __launch_bounds__(32 * kSwScanWarps) k_sw_scan2(const __grid_con
         uint32_t v = yb ? la : own;
 #pragma unroll
         for (uint32_t d = 1; d < 32u; d <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, v, d);
+            const uint32_t t = __shfl_up_sync(kAll, v, d);
             if (lane >= d && ((R >> (lane - d + 1u)) & ((1u << d) - 1u)) == 0u) v = t < v ? t : v;
         }
         const uint32_t nxt = R & ~((2u << lane) - 1u);  // run starts right of this lane
-        const uint32_t m = __shfl_sync(0xffffffffu, v, nxt ? (uint32_t)__ffs(nxt) - 2u : 31u);
+        const uint32_t m = __shfl_sync(kAll, v, nxt ? (uint32_t)__ffs(nxt) - 2u : 31u);
         if (yb && la != m) sw_unite<false>(f, la, m, P.err);  // a second component above joins the run
         rl[own] = (uint16_t)m;
         lab_prev = m;
-        s_prev = sc;
-        w1_prev = w1;
         __syncwarp();
     }
+    // the strips' seams: a bond between the same two runs as the lane before is that lane's
+    __syncthreads();
+    if (more) {
+        const uint32_t under = rl[(r0 + kSwRows) * 32u + lane], up = below[kSwRows - 1u];
+        const uint32_t pu = __shfl_up_sync(kAll, under, 1), pl = __shfl_up_sync(kAll, lab_prev, 1);
+        const bool same = lane > 0u && ((up >> (lane - 1u)) & 1u) && pu == under && pl == lab_prev;
+        if (((up >> lane) & 1u) && !same) sw_unite<false>(f, lab_prev, under, P.err);
+    }
+    __syncthreads();
     // every site's label resolved to its component's smallest site: lab = its
     // tile-local index; each tile root a node of the global forest
     uint32_t* par = P.parent + copy * P.N;
     uint16_t* lab = P.lab + copy * P.N;
-    for (uint32_t rr = 0; rr < 32u; ++rr) {
-        const uint32_t own = rr * 32u + lane, i = (by * 32u + rr) * L + X;
+#pragma unroll
+    for (uint32_t k = 0; k < kSwRows; ++k) {
+        const uint32_t own = (r0 + k) * 32u + lane, i = (Y + k) * L + X;
         const uint32_t root = sw_find<false>(f, rl[own]);
         lab[GBMC_IDX(i, P.N)] = (uint16_t)root;
         if (root == own) par[GBMC_IDX(i, P.N)] = i;
@@ -357,12 +383,13 @@ __host__ __device__ __forceinline__ uint32_t sw_cross_count(uint32_t N, uint32_t
 __global__ void __launch_bounds__(256) k_sw_cross(const __grid_constant__ SwLaunch P) {
     const uint64_t copy = P.copy0 + blockIdx.y;
     uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= sw_cross_count(P.N, P.dim)) return;
+    const bool in = e < sw_cross_count(P.N, P.dim);
+    if (!in) e = 0u;
     const SwTile T = sw_tile(P.dim);
     const uint32_t L = P.L, LL = L * L;
     uint32_t i, j, mu;
-    if (e < P.N / T.tx) {  // (row, tile column) -> x = tx c + tx - 1
-        const uint32_t nc = L / T.tx, row = e / nc, x = (e - row * nc) * T.tx + T.tx - 1;
+    if (e < P.N / T.tx) {  // (tile column, row): neighbouring lanes down the same tile edge
+        const uint32_t rows = P.N / L, c = e / rows, row = e - c * rows, x = c * T.tx + T.tx - 1;
         i = row * L + x;
         j = x + 1 == L ? i - x : i + 1;
         mu = 0;
@@ -381,13 +408,24 @@ __global__ void __launch_bounds__(256) k_sw_cross(const __grid_constant__ SwLaun
     const int8_t* s = P.spins + copy * P.N;
     uint32_t inst, r;
     split_copy(copy, P.R, inst, r);
-    if (!sw_bond_active(P, s, i, j, mu, r, c3_word(kPurposeSwBond, 0u, P.inst_base + inst))) return;
-    if (P.lab) {  // 2D scanline tiles: the ends' tile roots
+    uint32_t* par = P.parent + copy * P.N;
+    // a node of the global forest for each end: its tile root (2D), or what its parent
+    // pointer holds (3D), read beside the spins
+    uint32_t a, b;
+    if (P.lab) {
         const uint16_t* lab = P.lab + copy * P.N;
-        i = sw_tile_root(lab[i], i, L);
-        j = sw_tile_root(lab[j], j, L);
+        a = sw_tile_root(lab[i], i, L);
+        b = sw_tile_root(lab[j], j, L);
+    } else {
+        a = __ldcg(par + i);
+        b = __ldcg(par + j);
     }
-    sw_unite<true>(P.parent + copy * P.N, i, j, P.err);
+    const bool active = in && sw_bond_active(P, s, i, j, mu, r, c3_word(kPurposeSwBond, 0u, P.inst_base + inst));
+    const uint32_t mask = __ballot_sync(0xffffffffu, active);
+    if (!active) return;
+    // of the warp's bonds between the same two nodes (most of a large cluster's are) one unites
+    const uint32_t same = __match_any_sync(mask, ((uint64_t)min(a, b) << 32) | max(a, b));
+    if ((threadIdx.x & 31u) + 1u == (uint32_t)__ffs(same)) sw_unite<true>(par, a, b, P.err);
 }
 
 __global__ void __launch_bounds__(256) k_sw_union(const __grid_constant__ SwLaunch P) {
@@ -563,6 +601,317 @@ __global__ void __launch_bounds__(256) k_sw_flip_lab(const __grid_constant__ SwL
     }
 }
 
+// ---- lattices that fit in one block's shared memory ----
+
+// Shared memory of k_sw_resident: every site's label, then bit masks over the sites: spins
+// (1: down; the first four again behind the last), bonds to the right within a row, around a
+// row's end, along y and z, coins.
+__host__ __device__ __forceinline__ uint32_t sw_mask_words(uint32_t N) { return N / 32u + 2u; }
+__host__ __device__ __forceinline__ uint32_t sw_resident_words(uint32_t N, uint32_t dim) {
+    return N + (3u + dim) * sw_mask_words(N);
+}
+
+// All updates of a call, one block per copy. A thread takes four consecutive sites (one
+// Philox call covers their coins, DIM their bonds); eight lanes' nibbles make a mask word.
+// Labels start at the first site of each run of bonds along x. Then in rounds: each
+// bond whose ends' labels differ lowers the larger label's own label to the smaller one,
+// and all labels follow theirs to the end of the chain, until no bond's ends differ. A link
+// that a second bond's overwrites is found again in the next round, as its bond's ends still
+// differ; every round hooks all labels but the smallest among their neighbours.
+template <uint32_t DIM>
+__global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__ SwLaunch P, uint32_t n_updates,
+                                                        uint64_t copies, int32_t* E_series, int32_t* M_series) {
+    extern __shared__ __align__(16) uint32_t f[];  // the labels
+    __shared__ int red[2];                         // unsatisfied bonds, down spins
+    constexpr uint32_t kAll = 0xffffffffu;
+    const uint32_t N = P.N, L = P.L, LL = L * L, Q = N / 4u, W = sw_mask_words(N);
+    uint32_t* const spin = f + N;
+    uint32_t* const right = spin + W;
+    uint32_t* const around = right + W;
+    uint32_t* const along = around + W;               // [DIM - 1][W]
+    uint32_t* const coin = along + (DIM - 1u) * W;
+    const uint64_t copy = P.copy0 + blockIdx.x;
+    int8_t* s = P.spins + copy * N;
+    uint32_t inst, r;
+    split_copy(copy, P.R, inst, r);
+    const uint32_t k0 = (uint32_t)P.seed, k1 = (uint32_t)(P.seed >> 32);
+    const uint32_t lane = threadIdx.x & 31u;
+    // quotients by L: exact, as the numerators times L stay below 2^32
+    const uint32_t inv = 0xFFFFFFFFu / L + 1u;
+    auto nibble_of = [&](const uint32_t* m, uint32_t q) { return (m[q >> 3] >> (4u * (q & 7u))) & 15u; };
+    // the nibbles of eight lanes to a word of m, nq quads in all (whole warps; q: the lane's)
+    auto store = [&](uint32_t* m, uint32_t q, uint32_t nq, uint32_t nibble) {
+        uint32_t v = q < nq ? nibble << (4u * (lane & 7u)) : 0u;
+#pragma unroll
+        for (uint32_t o = 1; o < 8u; o <<= 1) v |= __shfl_xor_sync(kAll, v, o);
+        if ((lane & 7u) == 0u && q < nq) m[q >> 3] = v;
+    };
+    const uint32_t T = blockDim.x, Qr = (Q + 1u + 31u) & ~31u;  // whole warps over the quads and one more
+    for (uint32_t q = threadIdx.x; q < Qr; q += T) {
+        const uint32_t w = q <= Q ? *reinterpret_cast<const uint32_t*>(s + 4u * (q < Q ? q : 0u)) : 0u;
+        const uint32_t neg = (w >> 7) & 0x01010101u;  // -1 bytes
+        store(spin, q, Q + 1u, (neg * 0x01020408u) >> 24);
+    }
+    if (threadIdx.x < 2u) red[threadIdx.x] = 0;
+    __syncthreads();
+    const bool series = E_series || M_series;
+    const uint32_t Tb = (uint32_t)P.T_bond;
+    for (uint32_t u = 0; u <= n_updates; ++u) {
+        const bool update = u < n_updates, measure = u > 0u && series;
+        if (!update && !measure) break;
+        // bonds, and E and M of the update before
+        const PhiloxFixed pb = philox_fix(P.t + u, r, c3_word(kPurposeSwBond, 0u, P.inst_base + inst), k0, k1);
+        int unsat = 0, down = 0;
+        for (uint32_t q = threadIdx.x; q < Qr; q += T) {
+            uint32_t act[DIM], ends = 0u;
+#pragma unroll
+            for (uint32_t mu = 0; mu < DIM; ++mu) act[mu] = 0u;
+            if (q < Q) {
+                const uint32_t i0 = 4u * q, row = __umulhi(i0, inv), x = i0 - row * L;
+                auto window = [&](uint32_t p) {  // four bits of the spins from site p (cyclic)
+                    p = p >= N ? p - N : p;
+                    return __funnelshift_r(spin[p >> 5], spin[(p >> 5) + 1u], p & 31u);
+                };
+                const uint32_t at = window(i0), own = at & 15u;
+                uint32_t dif[DIM];
+                dif[0] = own ^ ((at >> 1) & 15u);
+                const uint32_t e = L - 1u - x;  // the row's end, if among the four
+                if (e < 4u) {
+                    ends = 1u << e;
+                    const uint32_t first = row * L;
+                    dif[0] = (dif[0] & ~ends) | ((((own >> e) ^ (spin[first >> 5] >> (first & 31u))) & 1u) << e);
+                }
+                uint32_t below = window(i0 + L);
+                if constexpr (DIM == 3) {
+                    // sites of a layer's last row go around to its first: the whole quad, or
+                    // (L % 4 = 2) the part of it before or after a row's end
+                    const uint32_t y = row - __umulhi(row, inv) * L, head = e < 3u ? (2u << e) - 1u : 15u;
+                    const uint32_t last = (y + 1u == L ? head : 0u) | (y + 2u == L ? ~head & 15u : 0u);
+                    if (last) below = (below & ~last) | (window(i0 + L + N - LL) & last);
+                    dif[2] = own ^ (window(i0 + LL) & 15u);
+                }
+                dif[1] = own ^ (below & 15u);
+                down += __popc(own);
+#pragma unroll
+                for (uint32_t mu = 0; mu < DIM; ++mu) unsat += __popc(dif[mu]);
+                if (update && P.T_bond >= 0) {
+#pragma unroll
+                    for (uint32_t c = 0; c < DIM; ++c) {
+                        const uint4 w = philox_q_wide(pb, DIM * q + c);
+#pragma unroll
+                        for (uint32_t k = 0; k < 4u; ++k) {
+                            const uint32_t n = (4u * c + k) / DIM, mu = (4u * c + k) % DIM;
+                            const uint32_t v = k == 0u ? w.x : k == 1u ? w.y : k == 2u ? w.z : w.w;
+                            if (v <= Tb) act[mu] |= 1u << n;
+                        }
+                    }
+#pragma unroll
+                    for (uint32_t mu = 0; mu < DIM; ++mu) act[mu] &= ~dif[mu];
+                }
+            }
+            if (update) {
+                store(right, q, Q, act[0] & ~ends);
+                store(around, q, Q, act[0] & ends);
+#pragma unroll
+                for (uint32_t mu = 1; mu < DIM; ++mu) store(along + (mu - 1u) * W, q, Q, act[mu]);
+            }
+        }
+        if (measure) {
+            unsat = __reduce_add_sync(kAll, unsat);
+            down = __reduce_add_sync(kAll, down);
+            if (lane == 0u) {
+                atomicAdd(red, unsat);
+                atomicAdd(red + 1, down);
+            }
+        }
+        __syncthreads();
+        if (measure && threadIdx.x == 0u) {
+            const uint64_t to = (uint64_t)(u - 1u) * copies + copy;
+            if (E_series) E_series[to] = 2 * red[0] - (int)(DIM * N);
+            if (M_series) M_series[to] = (int)N - 2 * red[1];
+            red[0] = red[1] = 0;  // next added to after two barriers
+        }
+        if (!update) break;
+        for (uint32_t q = threadIdx.x; q < Q; q += T) {
+            const uint32_t i0 = 4u * q;
+            uint32_t w = i0 >> 5, start = 0u;
+            uint32_t open = ~right[w] & ((1u << (i0 & 31u)) - 1u);  // sites below i0 not bonded to the next
+            while (!open && w) open = ~right[--w];
+            if (open) start = 32u * w + 32u - (uint32_t)__clz(open);
+            const uint32_t joined = right[i0 >> 5] >> (i0 & 31u);
+            uint4 v;
+            v.x = start;
+            v.y = (joined & 1u) ? v.x : i0 + 1u;
+            v.z = (joined & 2u) ? v.y : i0 + 2u;
+            v.w = (joined & 4u) ? v.z : i0 + 3u;
+            *reinterpret_cast<uint4*>(f + i0) = v;
+        }
+        __syncthreads();
+        for (;;) {
+            bool differ = false;
+            for (uint32_t q = threadIdx.x; q < Qr; q += T) {
+                const uint32_t i0 = 4u * q;
+                uint32_t on[DIM], any = 0u;
+                on[0] = nibble_of(around, q);
+#pragma unroll
+                for (uint32_t mu = 1; mu < DIM; ++mu) on[mu] = nibble_of(along + (mu - 1u) * W, q);
+#pragma unroll
+                for (uint32_t mu = 0; mu < DIM; ++mu) {
+                    if (q >= Q) on[mu] = 0u;
+                    any |= on[mu];
+                }
+                if (!__any_sync(kAll, any != 0u)) continue;  // whole warps
+                uint32_t done[DIM];  // bonds whose ends have one label: out of the rounds to come
+#pragma unroll
+                for (uint32_t mu = 0; mu < DIM; ++mu) done[mu] = 0u;
+                if (any) {
+                    const uint32_t row = __umulhi(i0, inv), x = i0 - row * L;
+                    const uint32_t y = DIM == 3 ? row - __umulhi(row, inv) * L : 0u;
+                    const uint4 v = *reinterpret_cast<const uint4*>(f + i0);
+                    const uint32_t own[4] = {v.x, v.y, v.z, v.w};
+                    // one direction's bonds together: their far ends' labels, then the larger
+                    // labels' own, then the links (most of a large cluster's are made already)
+                    volatile uint32_t* vf = f;
+                    auto join = [&](uint32_t mu, const uint32_t (&far)[4]) {
+                        uint32_t lo[4], hi[4], now[4];
+#pragma unroll
+                        for (uint32_t n = 0; n < 4u; ++n) {
+                            const uint32_t b = (on[mu] >> n) & 1u ? vf[far[n]] : own[n];
+                            lo[n] = min(own[n], b);
+                            hi[n] = max(own[n], b);
+                        }
+#pragma unroll
+                        for (uint32_t n = 0; n < 4u; ++n) now[n] = vf[hi[n]];
+#pragma unroll
+                        for (uint32_t n = 0; n < 4u; ++n) {
+                            if (lo[n] == hi[n]) done[mu] |= on[mu] & (1u << n);
+                            else differ = true;
+                            if (lo[n] < now[n] && lo[n] != hi[n]) atomicMin(f + hi[n], lo[n]);
+                        }
+                    };
+                    uint32_t far[4];
+#pragma unroll
+                    for (uint32_t n = 0; n < 4u; ++n) {
+                        uint32_t j = i0 + n + L;
+                        if constexpr (DIM == 2) j -= j >= N ? N : 0u;
+                        else if ((x + n >= L ? (y + 1u == L ? 0u : y + 1u) : y) + 1u == L) j -= LL;
+                        far[n] = j;
+                    }
+                    if (on[1]) join(1u, far);
+                    if constexpr (DIM == 3) {
+#pragma unroll
+                        for (uint32_t n = 0; n < 4u; ++n) far[n] = i0 + n + LL >= N ? i0 + n + LL - N : i0 + n + LL;
+                        if (on[2]) join(2u, far);
+                    }
+                    if (on[0]) {
+#pragma unroll
+                        for (uint32_t n = 0; n < 4u; ++n) far[n] = row * L;  // (the one bond's row begins there)
+                        join(0u, far);
+                    }
+                }
+#pragma unroll
+                for (uint32_t mu = 0; mu < DIM; ++mu)
+                    if (__any_sync(kAll, done[mu] != 0u))
+                        store(mu ? along + (mu - 1u) * W : around, q, Q, on[mu] & ~done[mu]);
+            }
+            if (!__syncthreads_or(differ)) break;
+            for (uint32_t q = threadIdx.x; q < Q; q += T) {
+                volatile uint32_t* l = f + 4u * q;
+                uint32_t a0 = l[0], a1 = l[1], a2 = l[2], a3 = l[3];
+                for (;;) {  // every label follows its own, and is itself what others follow
+                    volatile uint32_t* vf = f;
+                    const uint32_t b0 = vf[a0], b1 = vf[a1], b2 = vf[a2], b3 = vf[a3];
+                    if (b0 == a0 && b1 == a1 && b2 == a2 && b3 == a3) break;
+                    l[0] = a0 = b0, l[1] = a1 = b1, l[2] = a2 = b2, l[3] = a3 = b3;
+                }
+            }
+            __syncthreads();
+        }
+        const PhiloxFixed pf = philox_fix(P.t + u, r, c3_word(kPurposeSwFlip, 0u, P.inst_base + inst), k0, k1);
+        for (uint32_t q = threadIdx.x; q < Qr; q += T) {
+            uint32_t up = 0u;
+            if (q < Q) {
+                const uint4 v = *reinterpret_cast<const uint4*>(f + 4u * q);
+                if (v.x == 4u * q || v.y == 4u * q + 1u || v.z == 4u * q + 2u || v.w == 4u * q + 3u) {
+                    const uint4 w = philox_q_wide(pf, q);
+                    up = (w.x >> 31) | (w.y >> 31) << 1 | (w.z >> 31) << 2 | (w.w >> 31) << 3;
+                }
+            }
+            store(coin, q, Q, up);
+        }
+        __syncthreads();
+        const bool named = P.labels && u + 1u == n_updates;
+        for (uint32_t q = threadIdx.x; q < Qr; q += T) {
+            uint32_t now = 0u;
+            if (q <= Q) {
+                const uint32_t from = q < Q ? q : 0u;  // (the first quad again behind the last)
+                const uint4 v = *reinterpret_cast<const uint4*>(f + 4u * from);
+                auto up = [&](uint32_t root) { return (coin[root >> 5] >> (root & 31u)) & 1u; };
+                now = up(v.x) | up(v.y) << 1 | up(v.z) << 2 | up(v.w) << 3;
+                if (named && q < Q) {
+                    int32_t* to = P.labels + copy * N + 4u * q;
+                    to[0] = (int32_t)v.x, to[1] = (int32_t)v.y, to[2] = (int32_t)v.z, to[3] = (int32_t)v.w;
+                }
+            }
+            store(right, q, Q + 1u, now);
+        }
+        __syncthreads();
+        for (uint32_t w = threadIdx.x; w < W; w += T)
+            if (w < (Q + 8u) / 8u) spin[w] ^= right[w];
+        __syncthreads();
+    }
+    for (uint32_t q = threadIdx.x; q < Q; q += T) {
+        const uint32_t b = (nibble_of(spin, q) * 0x00204081u) & 0x01010101u;  // bit n to byte n
+        *reinterpret_cast<uint32_t*>(s + 4u * q) = (b * 0xFEu) | 0x01010101u;
+    }
+}
+
+// One copy takes 5 us and 3.1 (2D) or 3.7 ns per site and update, one block after the other
+// on a multiprocessor; three kernels over the lattice and two for E and M take 25 to 40 us
+// and, per site, 13 ps (2D) or 22 in tiles, 90 or 60 without. Measured, us per update, the
+// kernels -> resident: 2D L = 16 30 -> 6, L = 64 24 -> 16 (256 copies 40 -> 32, 1000 75 ->
+// 108), L = 100 40 -> 35 (152 copies 176 -> 36), L = 128 27 -> 52, L = 150 152 copies 351 ->
+// 74; 3D L = 8 29 -> 8, L = 16 29 -> 19, L = 24 40 -> 53 (152 copies 163 -> 57).
+bool sw_resident(uint32_t dim, uint32_t L, uint32_t N, uint64_t copies, bool series, int sm_count) {
+    const uint32_t bytes = sw_resident_words(N, dim) * 4u;
+    if (L < 4u || bytes > 224u * 1024u) return false;  // a quad holds at most one row's end
+    const double held = std::min(std::floor(1024.0 / std::min(1024u, (N / 4u + 31u) & ~31u)),
+                                 std::floor(228.0 * 1024.0 / (bytes + 1024.0)));
+    const double each = (double)N * (dim == 2 ? 0.0031 : 0.0037), c = (double)copies;
+    const double chip = std::ceil(c / sm_count) * each + 5.0 * std::ceil(c / (sm_count * held));
+    const bool tiled = sw_tiled(dim, L);
+    const double grid = (tiled ? (dim == 2 ? 24.0 : 29.0) : 32.0 + N * 4e-4) - (series ? 0.0 : 8.0) +
+                        c * N * (tiled ? (dim == 2 ? 1.3e-5 : 2.2e-5) : dim == 2 ? 9e-5 : 6e-5);
+    return chip < grid;
+}
+
+cudaError_t launch_sw_resident(const SwLaunch& P0, uint64_t copies, uint32_t n_updates, int32_t* E_series,
+                               int32_t* M_series, cudaStream_t s) {
+    if (P0.N % 4 != 0) return cudaErrorInvalidValue;
+    const size_t smem = sw_resident_words(P0.N, P0.dim) * 4u;
+    auto kern = P0.dim == 2 ? k_sw_resident<2> : k_sw_resident<3>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const uint32_t threads = std::min(1024u, (P0.N / 4u + 31u) & ~31u);
+    // a launch is kept to some ten milliseconds
+    const uint32_t most = std::max(1u, (1u << 24) / P0.N);
+    for (uint32_t u = 0; u < n_updates; u += most) {
+        SwLaunch P = P0;
+        P.t = P0.t + u;
+        const uint32_t n = std::min(most, n_updates - u);
+        if (u + n < n_updates) P.labels = nullptr;
+        for (uint64_t c0 = 0; c0 < copies; c0 += 0x40000000u) {
+            P.copy0 = c0;
+            const uint32_t nc = (uint32_t)std::min<uint64_t>(copies - c0, 0x40000000u);
+            kern<<<nc, threads, smem, s>>>(P, n, copies, E_series ? E_series + (uint64_t)u * copies : nullptr,
+                                           M_series ? M_series + (uint64_t)u * copies : nullptr);
+            count_launch();
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_sw_update(const SwLaunch& P0, uint64_t copies, cudaStream_t s) {
     if (P0.N % 4 != 0) return cudaErrorInvalidValue;
     for (uint64_t c0 = 0; c0 < copies; c0 += 65535) {
@@ -575,7 +924,7 @@ cudaError_t launch_sw_update(const SwLaunch& P0, uint64_t copies, cudaStream_t s
         if (tiled && P.dim == 2) {
             if (!P.lab) return cudaErrorInvalidValue;
             const uint32_t tiles = P.N / 1024;
-            k_sw_scan2<<<dim3((tiles + kSwScanWarps - 1) / kSwScanWarps, nc), 32 * kSwScanWarps, 0, s>>>(P);
+            k_sw_scan2<<<dim3(tiles, nc), 32 * kSwWarps, 0, s>>>(P);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             k_sw_cross<<<dim3((sw_cross_count(P.N, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
