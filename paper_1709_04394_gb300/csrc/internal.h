@@ -258,7 +258,7 @@ cudaError_t launch_sw_resident(const SwLaunch& P, uint64_t copies, uint32_t n_up
                                int32_t* M_series, cudaStream_t s);
 // Lattices labelled tile by tile (2D: 32 x 32 tiles, 3D: 16 x 8 x 8) need no
 // bond-flag array; the others use the global union-find over stored flags.
-inline bool sw_tiled(uint32_t dim, uint32_t L) { return (dim == 2 && L % 32 == 0) || (dim == 3 && L % 16 == 0); }
+inline bool sw_tiled(uint32_t dim, uint32_t L) { return (dim == 2 && L >= 32) || (dim == 3 && L % 16 == 0); }
 
 // ---- population annealing resampling (Sec. 5.4, Eq. (13)) ----
 struct PaLattice {

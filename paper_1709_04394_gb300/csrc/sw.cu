@@ -35,7 +35,8 @@
 // the larger root under the smaller), so the labels and coins do not depend
 // on the order of the unions.
 //
-// 2D lattices with L % 32 == 0 take 32 x 32 tiles with a scanline labelling,
+// 2D lattices from L = 32 take 32 x 32 tiles (the last ones cut by the lattice's edge;
+// L is even) with a scanline labelling,
 // the tile labels kept apart from the global forest:
 //  k_sw_scan2    : one block per tile, its warps four rows each, lane x = column x,
 //                  the rows in order. Row r's x bonds cut it into runs; a run's
@@ -293,17 +294,17 @@ __global__ void __launch_bounds__(32 * kSwWarps) k_sw_scan2(const __grid_constan
     __shared__ uint16_t rl[1024];  // each site's run label
     constexpr uint32_t kAll = 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31u, r0 = (threadIdx.x >> 5) * kSwRows;
-    const uint32_t L = P.L, ntx = L >> 5;
+    const uint32_t L = P.L, ntx = (L + 31u) >> 5;
     const uint64_t copy = P.copy0 + blockIdx.y;
     const int8_t* s = P.spins + copy * P.N;
     uint32_t inst, r;
     split_copy(copy, P.R, inst, r);
     const uint32_t bx = blockIdx.x % ntx, by = blockIdx.x / ntx, X = bx * 32u + lane, Y = by * 32u + r0;
     const bool more = r0 + kSwRows < 32u;  // the bonds below the last strip leave the tile (k_sw_cross)
-    int sp[kSwRows + 1];
+    int sp[kSwRows + 1];  // 0 beyond the lattice's edge: no bond joins it
 #pragma unroll
     for (uint32_t k = 0; k <= kSwRows; ++k)
-        sp[k] = k < kSwRows || more ? s[GBMC_IDX((uint64_t)(Y + k) * L + X, P.N)] : 0;
+        sp[k] = (k < kSwRows || more) && X < L && Y + k < L ? s[GBMC_IDX((uint64_t)(Y + k) * L + X, P.N)] : 0;
     // bond words: the forward bonds b = 2 i + mu of sites i = 2 q, 2 q + 1 are
     // the four words of Philox call q (t, replica and c3 hoisted). All the strip's bonds
     // first: masks over the row of the bonds to the right and of those below
@@ -367,39 +368,42 @@ __global__ void __launch_bounds__(32 * kSwWarps) k_sw_scan2(const __grid_constan
 #pragma unroll
     for (uint32_t k = 0; k < kSwRows; ++k) {
         const uint32_t own = (r0 + k) * 32u + lane, i = (Y + k) * L + X;
+        if (X >= L || Y + k >= L) continue;
         const uint32_t root = sw_find<false>(f, rl[own]);
         lab[GBMC_IDX(i, P.N)] = (uint16_t)root;
         if (root == own) par[GBMC_IDX(i, P.N)] = i;
     }
 }
 
-// The bonds that leave their tile: e < N / tx are the sites with x % tx == tx - 1
-// (bond along x), then N / ty sites with y % ty == ty - 1 (along y), then in 3D
-// N / tz sites with z % tz == tz - 1 (along z).
-__host__ __device__ __forceinline__ uint32_t sw_cross_count(uint32_t N, uint32_t dim) {
-    return dim == 2 ? N / 32 + N / 32 : N / 16 + N / 8 + N / 8;
+// The bonds that leave their tile: first those of the sites at a tile's last column
+// (bond along x), then those at a tile's last row (along y), then in 3D at its last
+// layer (along z). A 2D lattice's last tiles may end with it.
+__host__ __device__ __forceinline__ uint32_t sw_cross_count(uint32_t N, uint32_t L, uint32_t dim) {
+    return dim == 2 ? 2u * L * ((L + 31u) / 32u) : N / 16 + N / 8 + N / 8;
 }
 
 __global__ void __launch_bounds__(256) k_sw_cross(const __grid_constant__ SwLaunch P) {
     const uint64_t copy = P.copy0 + blockIdx.y;
     uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = e < sw_cross_count(P.N, P.dim);
+    const bool in = e < sw_cross_count(P.N, P.L, P.dim);
     if (!in) e = 0u;
     const SwTile T = sw_tile(P.dim);
     const uint32_t L = P.L, LL = L * L;
     uint32_t i, j, mu;
-    if (e < P.N / T.tx) {  // (tile column, row): neighbouring lanes down the same tile edge
-        const uint32_t rows = P.N / L, c = e / rows, row = e - c * rows, x = c * T.tx + T.tx - 1;
+    const uint32_t rows = P.N / L, nx = rows * ((L + T.tx - 1u) / T.tx), ny = rows * ((L + T.ty - 1u) / T.ty);
+    if (e < nx) {  // (tile column, row): neighbouring lanes down the same tile edge
+        const uint32_t c = e / rows, row = e - c * rows, x = min(c * T.tx + T.tx, L) - 1u;
         i = row * L + x;
         j = x + 1 == L ? i - x : i + 1;
         mu = 0;
-    } else if ((e -= P.N / T.tx) < P.N / T.ty) {  // (z, tile row k, x) -> y = ty k + ty - 1
-        const uint32_t nk = L / T.ty, rest = e / L, x = e - rest * L, z = rest / nk, y = (rest - z * nk) * T.ty + T.ty - 1;
+    } else if ((e -= nx) < ny) {  // (z, tile row k, x)
+        const uint32_t nk = (L + T.ty - 1u) / T.ty, rest = e / L, x = e - rest * L, z = rest / nk;
+        const uint32_t y = min((rest - z * nk) * T.ty + T.ty, L) - 1u;
         i = (z * L + y) * L + x;
         j = y + 1 == L ? i - (L - 1) * L : i + L;
         mu = 1;
     } else {  // (tile layer k, y, x) -> z = tz k + tz - 1
-        e -= P.N / T.ty;
+        e -= ny;
         const uint32_t k = e / LL, z = k * T.tz + T.tz - 1;
         i = z * LL + (e - k * LL);
         j = z + 1 == L ? i - (L - 1) * LL : i + LL;
@@ -543,6 +547,9 @@ __global__ void __launch_bounds__(256) k_sw_flip_tiled(const __grid_constant__ S
     }
 }
 
+// QUADS (L % 4 = 0): a thread has four sites of a row, loaded and stored together (1 us of 10 at
+// L = 1024); else four rows' sites of a column.
+template <bool QUADS>
 __global__ void __launch_bounds__(256) k_sw_flip_lab(const __grid_constant__ SwLaunch P) {
     __shared__ uint32_t troot[1024];     // global root of each tile root (by local index)
     __shared__ uint8_t tcoin[1024];      // its coin (1: the cluster flips)
@@ -551,23 +558,47 @@ __global__ void __launch_bounds__(256) k_sw_flip_lab(const __grid_constant__ SwL
     const uint64_t copy = P.copy0 + blockIdx.y;
     uint32_t inst, r;
     split_copy(copy, P.R, inst, r);
-    const uint32_t L = P.L, ntx = L >> 5;
+    const uint32_t L = P.L, ntx = (L + 31u) >> 5;
     const uint32_t bx = blockIdx.x % ntx, by = blockIdx.x / ntx;
-    const uint32_t l0 = 4 * threadIdx.x, lx = l0 & 31u, ly = l0 >> 5;
-    const uint32_t i0 = (by * 32u + ly) * L + bx * 32u + lx;
-    // i0 % 4 == 0 and the label buffer is a cudaMalloc block: 8-byte aligned
-    const uint2 lv = *reinterpret_cast<const uint2*>(P.lab + copy * P.N + GBMC_IDX(i0, P.N));
-    // i0 % 4 == 0 and the spin buffer is 16-byte aligned: one word per thread, loaded early
-    uint32_t* sw = reinterpret_cast<uint32_t*>(P.spins + copy * P.N + i0);
-    uint32_t w = *sw;
-    const uint32_t k[4] = {lv.x & 0xFFFFu, lv.x >> 16, lv.y & 0xFFFFu, lv.y >> 16};
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t lx = QUADS ? 4u * (threadIdx.x & 7u) : lane, ly = QUADS ? threadIdx.x >> 3 : 4u * (threadIdx.x >> 5);
+    auto x = [&](uint32_t j) { return lx + (QUADS ? j : 0u); };  // of site j within the tile
+    auto y = [&](uint32_t j) { return ly + (QUADS ? 0u : j); };
+    const uint32_t X = bx * 32u + lx, Y = by * 32u + ly, i0 = Y * L + X, step = QUADS ? 1u : L;
+    const uint16_t* lab = P.lab + copy * P.N;
+    int8_t* s = P.spins + copy * P.N;
+    bool on[4];
+    uint32_t k[4], quad = 0u;
+    int8_t sp[4];
+    if constexpr (QUADS) {
+        const bool in = X < L && Y < L;
+        // i0 % 4 == 0, the label buffer is a cudaMalloc block and the spin buffer 16-byte
+        // aligned: one word each
+        const uint2 lv = in ? *reinterpret_cast<const uint2*>(lab + GBMC_IDX(i0, P.N)) : make_uint2(0u, 0u);
+        if (in) quad = *reinterpret_cast<const uint32_t*>(s + i0);
+        k[0] = lv.x & 0xFFFFu, k[1] = lv.x >> 16, k[2] = lv.y & 0xFFFFu, k[3] = lv.y >> 16;
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) {
+            on[j] = in;
+            if (!in) k[j] = 0xFFFFFFFFu;
+        }
+    } else {
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) {
+            on[j] = X < L && Y + j < L;
+            k[j] = on[j] ? lab[GBMC_IDX(i0 + j * L, P.N)] : 0xFFFFFFFFu;
+            sp[j] = on[j] ? s[i0 + j * L] : (int8_t)0;
+        }
+    }
     // the tile roots whose component has a site on the tile border: only
     // they can have been united with other tiles' components
     if (threadIdx.x < 32u) tedge[threadIdx.x] = 0u;
     __syncthreads();
 #pragma unroll
     for (uint32_t j = 0; j < 4; ++j)
-        if (ly == 0u || ly == 31u || lx + j == 0u || lx + j == 31u) atomicOr(&tedge[k[j] >> 5], 1u << (k[j] & 31u));
+        if (on[j] && (x(j) == 0u || x(j) == 31u || bx * 32u + x(j) + 1u == L || y(j) == 0u || y(j) == 31u ||
+                      by * 32u + y(j) + 1u == L))
+            atomicOr(&tedge[k[j] >> 5], 1u << (k[j] & 31u));
     __syncthreads();
     // the tile roots: their global root and coin, through a per-warp queue so
     // that every lane works on one at a time
@@ -577,9 +608,12 @@ __global__ void __launch_bounds__(256) k_sw_flip_lab(const __grid_constant__ SwL
     uint32_t* q = tqueue[threadIdx.x >> 5];
     uint32_t n = 0;
 #pragma unroll
-    for (uint32_t j = 0; j < 4; ++j) sw_warp_push(q, n, k[j] == l0 + j, l0 + j);
+    for (uint32_t j = 0; j < 4; ++j) {
+        const uint32_t l = 32u * y(j) + x(j);
+        sw_warp_push(q, n, k[j] == l, l);
+    }
     __syncwarp();
-    for (uint32_t a = threadIdx.x & 31u; a < n; a += 32u) {
+    for (uint32_t a = lane; a < n; a += 32u) {
         const uint32_t l = q[a];
         const uint32_t g = (by * 32u + (l >> 5)) * L + bx * 32u + (l & 31u);
         // a component away from the tile border is a whole cluster, rooted at g
@@ -590,15 +624,18 @@ __global__ void __launch_bounds__(256) k_sw_flip_lab(const __grid_constant__ SwL
     __syncthreads();
 #pragma unroll
     for (uint32_t j = 0; j < 4; ++j) {
-        if (!tcoin[GBMC_IDX(k[j], 1024u)]) continue;
-        const uint32_t b = (uint32_t)(uint8_t)(-(int8_t)(w >> (8 * j)));
-        w = (w & ~(0xFFu << (8 * j))) | (b << (8 * j));
+        if (!on[j]) continue;
+        if (tcoin[GBMC_IDX(k[j], 1024u)]) {
+            if constexpr (QUADS) {
+                const uint32_t b = (uint32_t)(uint8_t)(-(int8_t)(quad >> (8 * j)));
+                quad = (quad & ~(0xFFu << (8 * j))) | (b << (8 * j));
+            } else {
+                s[i0 + j * L] = (int8_t)(-sp[j]);
+            }
+        }
+        if (P.labels) P.labels[copy * P.N + i0 + j * step] = (int32_t)troot[k[j]];
     }
-    *sw = w;
-    if (P.labels) {
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) P.labels[copy * P.N + i0 + j] = (int32_t)troot[GBMC_IDX(k[j], 1024u)];
-    }
+    if (QUADS && on[0]) *reinterpret_cast<uint32_t*>(s + i0) = quad;
 }
 
 // ---- lattices that fit in one block's shared memory ----
@@ -867,11 +904,11 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
 }
 
 // One copy takes 5 us and 3.1 (2D) or 3.7 ns per site and update, one block after the other
-// on a multiprocessor; three kernels over the lattice and two for E and M take 25 to 40 us
-// and, per site, 13 ps (2D) or 22 in tiles, 90 or 60 without. Measured, us per update, the
-// kernels -> resident: 2D L = 16 30 -> 6, L = 64 24 -> 16 (256 copies 40 -> 32, 1000 75 ->
-// 108), L = 100 40 -> 35 (152 copies 176 -> 36), L = 128 27 -> 52, L = 150 152 copies 351 ->
-// 74; 3D L = 8 29 -> 8, L = 16 29 -> 19, L = 24 40 -> 53 (152 copies 163 -> 57).
+// on a multiprocessor; three kernels over the lattice and one or two for E and M take 25 to 35
+// us and, per site, 13 ps (2D, whole tiles) or 22 (3D) in tiles, 90 or 60 without. Measured, us
+// per update, the kernels -> resident: 2D L = 16 28 -> 6, L = 64 26 -> 16 (1000 copies 79 -> 108),
+// L = 100 28 -> 35 (152 copies 62 -> 36), L = 128 29 -> 52; 3D L = 8 29 -> 8, L = 16 29 -> 19 (1000
+// copies 117 -> 130), L = 24 38 -> 53 (152 copies 163 -> 57), L = 34 152 copies 446 -> 151.
 bool sw_resident(uint32_t dim, uint32_t L, uint32_t N, uint64_t copies, bool series, int sm_count) {
     const uint32_t bytes = sw_resident_words(N, dim) * 4u;
     if (L < 4u || bytes > 224u * 1024u) return false;  // a quad holds at most one row's end
@@ -880,8 +917,9 @@ bool sw_resident(uint32_t dim, uint32_t L, uint32_t N, uint64_t copies, bool ser
     const double each = (double)N * (dim == 2 ? 0.0031 : 0.0037), c = (double)copies;
     const double chip = std::ceil(c / sm_count) * each + 5.0 * std::ceil(c / (sm_count * held));
     const bool tiled = sw_tiled(dim, L);
+    const double area = dim == 2 && tiled ? 1024.0 * ((L + 31u) / 32u) * ((L + 31u) / 32u) : (double)N;
     const double grid = (tiled ? (dim == 2 ? 24.0 : 29.0) : 32.0 + N * 4e-4) - (series ? 0.0 : 8.0) +
-                        c * N * (tiled ? (dim == 2 ? 1.3e-5 : 2.2e-5) : dim == 2 ? 9e-5 : 6e-5);
+                        c * area * (tiled ? (dim == 2 ? 1.3e-5 : 2.2e-5) : dim == 2 ? 9e-5 : 6e-5);
     return chip < grid;
 }
 
@@ -923,14 +961,15 @@ cudaError_t launch_sw_update(const SwLaunch& P0, uint64_t copies, cudaStream_t s
         cudaError_t e;
         if (tiled && P.dim == 2) {
             if (!P.lab) return cudaErrorInvalidValue;
-            const uint32_t tiles = P.N / 1024;
+            const uint32_t edge = (P.L + 31u) / 32u, tiles = edge * edge;
             k_sw_scan2<<<dim3(tiles, nc), 32 * kSwWarps, 0, s>>>(P);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_cross<<<dim3((sw_cross_count(P.N, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
+            k_sw_cross<<<dim3((sw_cross_count(P.N, P.L, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_flip_lab<<<dim3(tiles, nc), 256, 0, s>>>(P);
+            if (P.L % 4 == 0) k_sw_flip_lab<true><<<dim3(tiles, nc), 256, 0, s>>>(P);
+            else k_sw_flip_lab<false><<<dim3(tiles, nc), 256, 0, s>>>(P);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             continue;
@@ -940,7 +979,7 @@ cudaError_t launch_sw_update(const SwLaunch& P0, uint64_t copies, cudaStream_t s
             k_sw_local<3><<<dim3(P.N / 1024, nc), 256, 0, s>>>(P);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_cross<<<dim3((sw_cross_count(P.N, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
+            k_sw_cross<<<dim3((sw_cross_count(P.N, P.L, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             k_sw_flip_tiled<<<dim3(P.N / 1024, nc), 256, 0, s>>>(P);

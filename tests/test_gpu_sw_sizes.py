@@ -22,8 +22,11 @@ BC2, BC3 = 0.4406868, 0.2216544
     # tiles
     (2, 64, 1200, 3, BC2, (0, 1199)), (2, 128, 1, 4, BC2, (0,)), (2, 160, 2, 3, 0.6, (1,)), (3, 32, 1, 3, BC3, (0,)),
     (3, 48, 1, 2, 0.3, (0,)), (2, 224, 1, 2, 0.0, (0,)),
+    # tiles cut by the lattice's edge
+    (2, 210, 1, 3, BC2, (0,)), (2, 250, 2, 2, 0.6, (1,)), (2, 164, 1, 3, BC2, (0,)), (2, 226, 1, 2, 1.2, (0,)),
+    (2, 34, 9000, 2, BC2, (5, 8999)), (2, 36, 9000, 2, BC2, (8999,)), (2, 254, 1, 2, 0.0, (0,)),
     # neither
-    (2, 210, 1, 3, BC2, (0,)), (2, 250, 2, 2, 0.6, (1,)), (3, 34, 1, 2, BC3, (0,)), (3, 38, 1, 2, 0.3, (0,)),
+    (3, 34, 1, 2, BC3, (0,)), (3, 38, 1, 2, 0.3, (0,)), (2, 30, 30000, 2, BC2, (29999,)),
     (2, 2, 2, 4, BC2, (0, 1)),
 ])
 def test_sw_sizes(ctx, dim, L, R, n, beta, check):
