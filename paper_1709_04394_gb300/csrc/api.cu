@@ -2610,12 +2610,31 @@ struct gbmc_pt {
     gbmc_lattice* lat;
     std::vector<double> betas;
     uint32_t T, M, theta, round;
+    bool in_rounds = false;  // whole rounds per launch are the faster way (by the sizes alone)
     uint32_t* thr_temp = nullptr;
     uint32_t *temp_of = nullptr, *rep_of = nullptr, *accepted = nullptr;
     int32_t *E = nullptr, *Mag = nullptr;
     long long* tab = nullptr;
     std::vector<void*> allocs;
 };
+
+// The sweeps of one round, from the lattice's sweep counter on.
+static SweepLaunch pt_sweeps(const gbmc_pt* pt, const Tuning& tu) {
+    SweepLaunch P;
+    std::memset(&P, 0, sizeof(P));
+    SweepJob& J = P.jobs[0];
+    J = base_job(pt->lat, tu);
+    J.nsweeps = pt->theta;
+    J.E = pt->E;
+    J.M = pt->Mag;
+    J.thr_temp = pt->thr_temp;
+    J.temp_of = pt->temp_of;
+    P.njobs = 1;
+    P.dim = pt->lat->d.dim;
+    P.ea = pt->lat->d.model == GBMC_EA_PMJ;
+    P.swar = (pt->lat->d.L % 8) == 0;
+    return P;
+}
 
 gbmc_status pt_create(gbmc_ctx* ctx, gbmc_lattice* l, const double* betas, uint32_t theta, gbmc_pt** out) {
     if (!ctx || !l || !betas || !out) return fail(GBMC_ERR_ARG, "NULL argument");
@@ -2674,6 +2693,7 @@ gbmc_status pt_create(gbmc_ctx* ctx, gbmc_lattice* l, const double* betas, uint3
         delete pt;
         return fail(GBMC_ERR_CUDA, "parallel tempering set-up: %s", cudaGetErrorString(e));
     }
+    pt->in_rounds = tempering_in_rounds(pt_sweeps(pt, tu), ctx->sm_count);
     l->run = (gbmc_pa*)pt;  // the lattice is owned by this run until pt_free
     *out = pt;
     return GBMC_OK;
@@ -2686,20 +2706,9 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
     gbmc_lattice* l = pt->lat;
     if ((uint64_t)l->t + (uint64_t)n_steps * pt->theta > 0xFFFFFFFFull) return fail(GBMC_ERR_ARG, "sweep counter would wrap");
     const Tuning tu = tune(l);
+    const bool in_rounds = pt->in_rounds && ctx->sweep_kernel == GBMC_KERNEL_AUTO && tu.bits;
     for (uint32_t n = 0; n < n_steps;) {
-        SweepJob J = base_job(l, tu);
-        J.nsweeps = pt->theta;
-        J.E = pt->E;
-        J.M = pt->Mag;
-        J.thr_temp = pt->thr_temp;
-        J.temp_of = pt->temp_of;
-        SweepLaunch P;
-        std::memset(&P, 0, sizeof(P));
-        P.jobs[0] = J;
-        P.njobs = 1;
-        P.dim = l->d.dim;
-        P.ea = l->d.model == GBMC_EA_PMJ;
-        P.swar = (l->d.L % 8) == 0;
+        const SweepLaunch P = pt_sweeps(pt, tu);
         PtExchange X;
         X.E = pt->E;
         X.rep_of = pt->rep_of;
@@ -2715,7 +2724,7 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
         // a launch of rounds is kept to some ten milliseconds: 2^34 site updates, 2^13 sweeps
         const double sweeps = std::max(1u, pt->theta), updates = (double)l->N * (double)l->ncopies * sweeps;
         X.rounds = (uint32_t)std::max(1.0, std::min({(double)(n_steps - n), 17179869184.0 / updates, 8192.0 / sweeps}));
-        if (ctx->sweep_kernel == GBMC_KERNEL_AUTO && tu.bits && tempering_in_rounds(P, ctx->sm_count)) {
+        if (in_rounds) {
             ProfScope ps_(ctx, PK_PT_ROUNDS);
             CUDA_TRY(launch_tempering_rounds(P, X, ctx->sm_count, ctx->stream));
         } else {

@@ -773,8 +773,12 @@ uint32_t stream_smem_words(uint32_t N, uint32_t G, uint32_t C, bool pt) {
 // copies each. The estimate is in cycles of a scheduler per half-sweep: a pass of
 // a warp over its words issues for `pass` cycles (the multiply and logic pipes)
 // but takes `lat` by itself, so a scheduler with w warps at work spends
-// max(pass, lat / w) per pass; on top of the average comes the longest team, for
-// what the last teams leave idle.
+// max(pass, lat / w) per pass. Where one job's teams are all held at once the fullest
+// scheduler's count; else the average and 0.6 of the longest team, for what the last
+// teams leave idle (several jobs' teams are chosen by the whole of their own: the last
+// job's are what is left at the end). Estimate : measured, thousand cycles per half-sweep,
+// C = 1, 2, 4 (* taken): 2D L = 24, 40, 96 together 64 : 56, 60* : 49, 62 : 57; 3D L = 10, 8 x
+// 5000 copies 41 : 41, 37 : 36, 33* : 34; L = 12, 4 x 1000 copies 8.7 : 9.0, 8.6* : 9.1, 9.0 : 8.3.
 struct StreamPlan {
     int C = 1, split = 1;
     uint32_t threads = kStreamThreads;
@@ -782,48 +786,63 @@ struct StreamPlan {
     double cost = 1e300;
 };
 
-double stream_pass(int C, int split) { return C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 980.0 : 420.0; }
+// measured: 2D L = 64 and 3D L = 10 with large populations (pass), L = 36 and 68 with one warp
+// per scheduler (lat)
+double stream_pass(int C, int split, int dim) {
+    return dim == 2 ? (C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 1030.0 : 430.0)
+                    : (C == 4 ? 3730.0 : C == 2 ? 2150.0 : split == 1 ? 1240.0 : 490.0);
+}
 double stream_lat(int C, int split) { return C == 4 ? 9000.0 : C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0; }
 
 StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_count) {
-    // measured: 2D L = 64 with 10^5 copies (pass), L = 36 and 68 with one warp per scheduler (lat)
-    const double pass = stream_pass(C, split), lat = stream_lat(C, split);
+    const double pass = stream_pass(C, split, P.dim), lat = stream_lat(C, split);
     const double by_regs = C == 4 ? 5.0 : 8.0;  // warps per scheduler the registers allow
     const double schedulers = 4.0 * sm_count;
     StreamPlan S;
     S.C = C;
     S.split = split;
     double total = 0.0, longest = 0.0;
-    for (int j = 0; j < P.njobs; ++j) {
-        const SweepJob& J = P.jobs[j];
-        const uint32_t PW = (J.N / 2u + 31u) / 32u * (uint32_t)split;  // items of a copy
-        const double groups = (double)J.n_inst * ((J.R + C - 1u) / C);
-        double best = 1e300, best_sum = 0.0, best_len = 0.0;
-        auto consider = [&](uint32_t T, uint32_t G) {
-            const double p = (double)((G * PW + T - 1u) / T);
-            const double share = std::ceil(groups / G) * (T / 32u) / schedulers;
-            const uint32_t warps = T == 32u ? kStreamThreads / 32u : T / 32u;
-            const size_t smem = (size_t)stream_smem_words(J.N, G, C, pt) * 4u * (T == 32u ? warps : 1u);
-            const double fit = std::floor((double)kStreamSmem / smem) * warps / 4.0;
-            const double w = std::max(1.0, std::min(share, std::min(by_regs, fit)));
-            const double step = std::max(pass, lat / w) + (T == 32u ? 0.0 : 60.0);
-            const double sum = p * share * step, len = p * step;
-            if (sum + len < best * 0.98) {
-                best = sum + len;
-                best_sum = sum;
-                best_len = len;
-                S.T[j] = T;
-                S.G[j] = G;
-            }
-        };
-        // one-warp teams; larger copies, and a single lattice with too few copies
-        // to give every scheduler work, take whole blocks
-        for (uint32_t G = 1; G <= 32u && stream_smem_words(J.N, G, C, pt) <= kStreamTeamWords; ++G) consider(32u, G);
-        if (P.njobs == 1)
-            for (uint32_t T = 64u; T <= stream_max_threads(C, split) && T < PW + 32u; T += 32u) consider(T, 1u);
-        if (S.T[j] == 0u) consider(kStreamThreads, 1u);
-        total += best_sum;
-        longest = std::max(longest, best_len);
+    // the jobs' warps share the schedulers: those of the other jobs, from the round before
+    double shares[kMaxJobs] = {}, others = 0.0;
+    for (int round = 0; round < (P.njobs > 1 ? 2 : 1); ++round) {
+        total = longest = 0.0;
+        for (int j = 0; j < P.njobs; ++j) {
+            const SweepJob& J = P.jobs[j];
+            const uint32_t PW = (J.N / 2u + 31u) / 32u * (uint32_t)split;  // items of a copy
+            const double groups = (double)J.n_inst * ((J.R + C - 1u) / C);
+            double best = 1e300, best_sum = 0.0, best_len = 0.0, best_share = 0.0;
+            others = 0.0;
+            for (int k = 0; k < P.njobs; ++k) others += k == j ? 0.0 : shares[k];
+            auto consider = [&](uint32_t T, uint32_t G) {
+                const double p = (double)((G * PW + T - 1u) / T);
+                const double share = std::ceil(groups / G) * (T / 32u) / schedulers;
+                const uint32_t warps = T == 32u ? kStreamThreads / 32u : T / 32u;
+                const size_t smem = (size_t)stream_smem_words(J.N, G, C, pt) * 4u * (T == 32u ? warps : 1u);
+                const double fit = std::floor((double)kStreamSmem / smem) * warps / 4.0;
+                const double cap = std::min(by_regs, fit), w = std::max(1.0, std::min(share + others, cap));
+                const double step = std::max(pass, lat / w) + (T == 32u ? 0.0 : 60.0), len = p * step;
+                double sum = p * share * step, cost = sum + (P.njobs > 1 ? 1.0 : 0.6) * len;
+                if (P.njobs == 1 && share <= cap)  // all teams at once
+                    cost = sum = p * (std::max(std::ceil(share) * pass, lat) + (T == 32u ? 0.0 : 60.0));
+                if (cost < best * 0.98) {
+                    best = cost;
+                    best_sum = sum;
+                    best_len = std::min(cost - sum, 0.6 * len);
+                    best_share = share;
+                    S.T[j] = T;
+                    S.G[j] = G;
+                }
+            };
+            // one-warp teams; larger copies, and a single lattice with too few copies
+            // to give every scheduler work, take whole blocks
+            for (uint32_t G = 1; G <= 32u && stream_smem_words(J.N, G, C, pt) <= kStreamTeamWords; ++G) consider(32u, G);
+            if (P.njobs == 1)
+                for (uint32_t T = 64u; T <= stream_max_threads(C, split) && T < PW + 32u; T += 32u) consider(T, 1u);
+            if (S.T[j] == 0u) consider(kStreamThreads, 1u);
+            shares[j] = best_share;
+            total += best_sum;
+            longest = std::max(longest, best_len);
+        }
     }
     if (P.njobs == 1 && S.T[0] != 32u) S.threads = S.T[0];
     S.cost = total + longest;
@@ -894,8 +913,8 @@ RoundsPlan rounds_plan(const SweepJob& J, int dim, int sm_count) {
     const uint32_t ng = J.R;
     for (const int split : {4, 1}) {
         const uint32_t most = stream_max_threads(1, split, kRounds);
-        // (3D: four more compares of a call's sixteen)
-        const double pass = stream_pass(1, split) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, split);
+        // (with places and bond words kept: less than a sweep launch's pass)
+        const double pass = (split == 4 ? 420.0 : 980.0) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, split);
         auto consider = [&](uint32_t B, uint32_t G, uint32_t T, uint32_t threads) {
             RoundsPlan p;
             p.split = split, p.B = B, p.G = G, p.T = T, p.threads = threads;
@@ -968,8 +987,8 @@ cudaError_t launch_rounds_c(const SweepLaunch& P, const PtExchange& X, const Rou
 }  // namespace
 
 // A round by itself is a sweep launch, whose copies are loaded and stored, and an
-// exchange launch, about 20 000 cycles beside the half-sweeps (3D L = 8, 250 x 40 copies, one
-// sweep per round: 15.4 us, 4.8 of them sweeping). What speaks for it is that its blocks
+// exchange launch, 20 000 to 27 000 cycles beside the half-sweeps (3D L = 8, 250 x 40 copies,
+// one sweep per round: 15.4 us, 4.8 of them sweeping; L = 12, 60 x 14: 16.4, 2). What speaks for it is that its blocks
 // change places between rounds: 256 x 40 copies of L = 12, 10 sweeps per round, 207 us
 // each against 248 in one launch of rounds; 100 x 36 53 against 38.
 bool tempering_in_rounds(const SweepLaunch& P, int sm_count) {
@@ -979,7 +998,12 @@ bool tempering_in_rounds(const SweepLaunch& P, int sm_count) {
     for (int C = 4; C >= 1; C >>= 1)
         if (C == 1 || stream_smem_words(J.N, 1u, (uint32_t)C, true) * 4u <= 36u * 1024u)
             alone = std::min(alone, stream_plan(P, C, 1, true, sm_count).cost);
-    return rounds_plan(J, P.dim, sm_count).cost < 2.0 * J.nsweeps * alone * (P.dim == 3 ? 1.15 : 1.0) + 20000.0;
+    if (bits_supported(P.dim, (int)J.L)) {  // those sweeps are bitsweep.cu's, faster where they fill the chip
+        const double copies = (double)J.n_inst * J.R, per = std::max(1.0, J.N / 2048.0);  // warps' words per lane
+        const double warps = std::ceil(copies * (J.N / 64.0) / 32.0 / per / (4.0 * sm_count));
+        alone = std::min(alone, per * std::max(warps * (P.dim == 3 ? 950.0 : 840.0), 2100.0));
+    }
+    return rounds_plan(J, P.dim, sm_count).cost < 2.0 * J.nsweeps * alone + 24000.0;
 }
 
 cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, int sm_count, cudaStream_t s) {
