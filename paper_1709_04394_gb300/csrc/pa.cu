@@ -340,14 +340,24 @@ __device__ __forceinline__ void record_population(const PaLattice& P, uint32_t i
     P.nnext[inst] = (uint32_t)total;
 }
 
-// Parent j fills the slots [S, S + n).
+// Parent j fills the slots [S, S + n); whole warps call it (n = 0: nothing to place). A
+// parent with many children -- a large step leaves a few replicas most of the
+// population -- has them written by all lanes: one thread's loop over them took 40 of
+// 53 us per step for 2D L = 96.
 __device__ __forceinline__ void place_children(const PaLattice& P, uint64_t base, uint64_t S, uint32_t n, uint32_t j) {
-    for (uint32_t m = 0; m < n; ++m) {
-        if (S + m >= P.R) {
-            atomicExch(P.overflow, 1u);
-            break;
-        }
-        P.parent[base + GBMC_IDX(S + m, P.R)] = j;
+    constexpr uint32_t kAll = 0xFFFFFFFFu, kFew = 4u;
+    if (n && S + n > P.R) {
+        atomicExch(P.overflow, 1u);
+        n = S < P.R ? (uint32_t)(P.R - S) : 0u;
+    }
+    uint32_t* to = P.parent + base;
+    if (n <= kFew)
+        for (uint32_t m = 0; m < n; ++m) to[GBMC_IDX(S + m, P.R)] = j;
+    for (uint32_t many = __ballot_sync(kAll, n > kFew); many; many &= many - 1u) {
+        const int src = __ffs(many) - 1;
+        const uint32_t nn = __shfl_sync(kAll, n, src), jj = __shfl_sync(kAll, j, src);
+        const uint64_t SS = __shfl_sync(kAll, (unsigned long long)S, src);
+        for (uint32_t m = threadIdx.x & 31u; m < nn; m += 32u) to[GBMC_IDX(SS + m, P.R)] = jj;
     }
 }
 
@@ -368,14 +378,11 @@ __device__ __forceinline__ void phase_place(const PaLattice& P, uint32_t inst, u
     if (P.nnext && threadIdx.x == 0 && chunk + 1 == P.nchunks) {
         record_population(P, inst, (uint64_t)pre + __ldcg(P.ntot + (uint64_t)inst * P.nchunks + chunk));
     }
-    for (uint32_t i = threadIdx.x; i < kScanChunk; i += blockDim.x) {
+    for (uint32_t i = threadIdx.x; i < kScanChunk; i += blockDim.x) {  // whole warps
         const uint32_t j = chunk * kScanChunk + i;
-        if (j >= live) break;
-        const uint32_t n = __ldcg(P.counts + base + j);
-        if (n) {
-            place_children(P, base, (uint64_t)pre + __ldcg(P.sloc + base + j), n, j);
-            P.counts[base + j] = 0u;
-        }
+        const uint32_t n = j < live ? __ldcg(P.counts + base + j) : 0u;
+        place_children(P, base, n ? (uint64_t)pre + __ldcg(P.sloc + base + j) : 0u, n, j);
+        if (n) P.counts[base + j] = 0u;
     }
     __syncthreads();
 }
@@ -707,9 +714,10 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
     uint32_t before = 0;
     for (uint32_t c = 0; c < rank; ++c) before += ntot[c];
     if (P.nnext && threadIdx.x == 0 && rank + 1u == K) record_population(P, inst, (uint64_t)before + total);
-    for (uint32_t i = i0; i < i1; ++i) {
-        place_children(P, base, (uint64_t)before + S32, cnt[i], j0 + i);
-        S32 += cnt[i];
+    for (uint32_t k = 0; k < per; ++k) {  // whole warps
+        const uint32_t i = i0 + k, c = i < i1 ? cnt[i] : 0u;
+        place_children(P, base, (uint64_t)before + S32, c, j0 + i);
+        S32 += c;
     }
 }
 
