@@ -778,7 +778,7 @@ uint32_t stream_smem_words(uint32_t N, uint32_t G, uint32_t C, bool pt) {
 // teams leave idle (several jobs' teams are chosen by the whole of their own: the last
 // job's are what is left at the end). Estimate : measured, thousand cycles per half-sweep,
 // C = 1, 2, 4 (* taken): 2D L = 24, 40, 96 together 64 : 56, 60* : 49, 62 : 57; 3D L = 10, 8 x
-// 5000 copies 41 : 41, 37 : 36, 33* : 34; L = 12, 4 x 1000 copies 8.7 : 9.0, 8.6* : 9.1, 9.0 : 8.3.
+// 5000 copies 41 : 41, 37 : 36, 33* : 34; L = 12, 4 x 1000 copies 8.7* : 9.0, 9.6 : 9.1, 9.0 : 8.3.
 struct StreamPlan {
     int C = 1, split = 1;
     uint32_t threads = kStreamThreads;
@@ -786,16 +786,25 @@ struct StreamPlan {
     double cost = 1e300;
 };
 
-// measured: 2D L = 64 and 3D L = 10 with large populations (pass), L = 36 and 68 with one warp
-// per scheduler (lat)
+// measured: 2D L = 64 and 3D L = 10 with large populations (pass), populations with one to
+// seven warps per scheduler (lat, stream_wave)
 double stream_pass(int C, int split, int dim) {
     return dim == 2 ? (C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 1030.0 : 430.0)
-                    : (C == 4 ? 3730.0 : C == 2 ? 2150.0 : split == 1 ? 1240.0 : 490.0);
+                    : (C == 4 ? 3730.0 : C == 2 ? 2150.0 : split == 1 ? 1240.0 : 560.0);
 }
-double stream_lat(int C, int split) { return C == 4 ? 9000.0 : C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0; }
+double stream_lat(int C, int split, int dim) {
+    return (C == 4 ? 9000.0 : (C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0) * (dim == 3 ? 1.15 : 1.0));
+}
+// A pass with w warps on every scheduler, in teams of T: two copies per thread leave gaps where
+// the warps are few, and a block's teams wait for their slowest warp.
+double stream_wave(int C, int split, int dim, double w, uint32_t T) {
+    const double lat = stream_lat(C, split, dim);
+    return std::max(w * stream_pass(C, split, dim), lat) + (w > 1.0 && C <= 2 ? (C == 2 ? 0.8 : 0.2) * lat / w : 0.0) +
+           (T == 32u ? 0.0 : 12.0 * (T / 32u));
+}
 
 StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_count) {
-    const double pass = stream_pass(C, split, P.dim), lat = stream_lat(C, split);
+    const double pass = stream_pass(C, split, P.dim), lat = stream_lat(C, split, P.dim);
     const double by_regs = C == 4 ? 5.0 : 8.0;  // warps per scheduler the registers allow
     const double schedulers = 4.0 * sm_count;
     StreamPlan S;
@@ -822,8 +831,10 @@ StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_c
                 const double cap = std::min(by_regs, fit), w = std::max(1.0, std::min(share + others, cap));
                 const double step = std::max(pass, lat / w) + (T == 32u ? 0.0 : 60.0), len = p * step;
                 double sum = p * share * step, cost = sum + (P.njobs > 1 ? 1.0 : 0.6) * len;
-                if (P.njobs == 1 && share <= cap)  // all teams at once
-                    cost = sum = p * (std::max(std::ceil(share) * pass, lat) + (T == 32u ? 0.0 : 60.0));
+                if (P.njobs == 1 && share <= cap) {  // all teams at once; a block's warps share its SM
+                    const double fullest = T == 32u ? share : std::ceil(groups / sm_count) * (T / 32u) / 4.0;
+                    cost = sum = p * stream_wave(C, split, P.dim, std::ceil(fullest), T);
+                }
                 if (cost < best * 0.98) {
                     best = cost;
                     best_sum = sum;
@@ -914,7 +925,7 @@ RoundsPlan rounds_plan(const SweepJob& J, int dim, int sm_count) {
     for (const int split : {4, 1}) {
         const uint32_t most = stream_max_threads(1, split, kRounds);
         // (with places and bond words kept: less than a sweep launch's pass)
-        const double pass = (split == 4 ? 420.0 : 980.0) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, split);
+        const double pass = (split == 4 ? 420.0 : 980.0) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, split, 2);
         auto consider = [&](uint32_t B, uint32_t G, uint32_t T, uint32_t threads) {
             RoundsPlan p;
             p.split = split, p.B = B, p.G = G, p.T = T, p.threads = threads;
