@@ -23,6 +23,9 @@
 // two ends anyway (colour 0 before its update, colour 1 as its neighbours), and
 // after the last sweep in one more pass: no launch of their own.
 //
+// Where a run is longer than its ends (2D, four threads per word) the CTA keeps it in
+// shared memory, and only the ends are written to and read from global memory.
+//
 // Bound: for small lattices the chain of a half-sweep -- words loaded from L2,
 // update, words stored --, for larger ones the integer pipes (stream.cu).
 #include "bits.cuh"
@@ -68,15 +71,23 @@ __device__ __forceinline__ void row_masks(const PlaneShape& g, uint32_t w, uint3
 }
 
 // A plane's words, the least tag seen, and the 32 bits of its stream from bit p < H
-// on, across its end.
+// on, across its end. HELD: the CTA's own run, words first .. first + count - 1, is in
+// shared memory.
+__device__ __forceinline__ uint64_t shared_word(const uint64_t* p) {
+    uint64_t x;
+    asm volatile("ld.relaxed.cta.shared.u64 %0, [%1];" : "=l"(x) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+    return x;
+}
+template <bool HELD>
 struct Plane {
-    const uint64_t* w;
-    uint32_t tag;
+    const uint64_t *w, *run;
+    uint32_t first, count, tag;
     __device__ __forceinline__ uint32_t word(uint32_t i) {
-        uint32_t v, t;
-        asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v), "=r"(t) : "l"(w + i) : "memory");
-        tag = min(tag, t);
-        return v;
+        uint64_t x;
+        if (HELD && i - first < count) x = shared_word(run + (i - first));
+        else asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(w + i) : "memory");
+        tag = min(tag, (uint32_t)(x >> 32));
+        return (uint32_t)x;
     }
     __device__ __forceinline__ void window(const PlaneShape& g, uint32_t p, uint32_t& v0, uint32_t& v1) {
         // v0: bits p .. p + 31, v1: bits p + 1 .. p + 32
@@ -99,7 +110,7 @@ struct Plane {
     }
 };
 
-template <int DIM, bool EA, int S>
+template <int DIM, bool EA, int S, bool HELD>
 __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_strips(const __grid_constant__ StreamStrips P) {
     __shared__ int acc[2][2];  // by sweep parity: unsatisfied bonds and down spins of this CTA's words
     const uint32_t tid = threadIdx.x, T = blockDim.x;
@@ -110,6 +121,13 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
     const uint32_t inst = copy / P.R, r = copy - inst * P.R, instance = P.inst_base + inst;
     const uint32_t k0 = (uint32_t)P.seed, k1 = (uint32_t)(P.seed >> 32);
     uint64_t* const planes = P.P + (uint64_t)copy * 2u * g.PW;
+    // HELD: the run's words of both planes, read by this CTA's threads without the way to L2
+    extern __shared__ __align__(16) uint64_t runs[];
+    if constexpr (HELD) {
+        for (uint32_t i = tid; i < 2u * n_words; i += T)
+            runs[i] = planes[(uint64_t)(i / n_words) * g.PW + w0 + i % n_words];
+        __syncthreads();
+    }
     // words near an end of the run come first: n_edge of them on either side
     const uint32_t n_edge = min(P.edge, (n_words + 1u) / 2u), n_first = min(2u * n_edge, n_words);
     const uint32_t items = n_words * S;
@@ -170,7 +188,8 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
             // half-sweep h - 1 (tag h) and this word's own h - 2
             uint32_t s0, same, prv, nxt, up, up1, dn1, dn, ya = 0u, yb = 0u, za = 0u, zb = 0u, tag_me, tag_oth;
             auto look = [&]() {
-                Plane me{own, 0xFFFFFFFFu}, oth{planes + (c ^ 1u) * g.PW, 0xFFFFFFFFu};
+                Plane<HELD> me{own, runs + c * n_words, w0, n_words, 0xFFFFFFFFu};
+                Plane<HELD> oth{planes + (c ^ 1u) * g.PW, runs + (c ^ 1u) * n_words, w0, n_words, 0xFFFFFFFFu};
                 s0 = me.word(w);
                 same = oth.word(w);
                 prv = oth.word(w ? w - 1u : 0u);
@@ -266,8 +285,17 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
                 v |= __shfl_xor_sync(0xFFFFFFFFu, v, 1);
                 v |= __shfl_xor_sync(0xFFFFFFFFu, v, 2);
             }
-            if (live && part == 0u)
-                asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(own + w), "r"(v), "r"(h + 1u) : "memory");
+            if (live && part == 0u) {
+                const uint64_t out = (uint64_t)(h + 1u) << 32 | v;
+                if (HELD)
+                    asm volatile("st.relaxed.cta.shared.u64 [%0], %1;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(runs + c * n_words + (w - w0))),
+                                 "l"(out)
+                                 : "memory");
+                // other CTAs read the run's ends, the caller what is there at the end
+                if (!HELD || x < n_first || h + 2u >= P.n_half)
+                    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(own + w), "l"(out) : "memory");
+            }
         }
         if (measure) {
             U = __reduce_add_sync(0xFFFFFFFFu, U);
@@ -373,11 +401,13 @@ __global__ void k_series_init(int32_t* E, int32_t* M, int32_t e, int32_t m, uint
     }
 }
 
-template <int DIM, bool EA, int S>
+template <int DIM, bool EA, int S, bool HELD>
 cudaError_t launch_strips(StreamStrips P, uint64_t copies, int sm_count, uint32_t T, cudaStream_t s) {
-    auto kern = k_stream_strips<DIM, EA, S>;
+    auto kern = k_stream_strips<DIM, EA, S, HELD>;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)T, 0);
+    const size_t smem = HELD ? 16ull * ((stream_plane_words(P.N) / 2u + P.Gc - 1u) / P.Gc) : 0u;
+    cudaError_t e = cudaSuccess;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)T, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
     const uint64_t batch = (uint64_t)sm_count / P.Gc;  // copies per launch, one CTA per SM
@@ -385,7 +415,7 @@ cudaError_t launch_strips(StreamStrips P, uint64_t copies, int sm_count, uint32_
         const uint64_t n = copies - c0 < batch ? copies - c0 : batch;
         P.copy0 = (uint32_t)c0;
         void* args[] = {&P};
-        e = cudaLaunchCooperativeKernel((const void*)kern, dim3((uint32_t)(n * P.Gc)), dim3(T), args, 0, s);
+        e = cudaLaunchCooperativeKernel((const void*)kern, dim3((uint32_t)(n * P.Gc)), dim3(T), args, smem, s);
         count_launch();
         if (e != cudaSuccess) return e;
     }
@@ -434,6 +464,10 @@ cudaError_t launch_stream_strips(const StreamStrips& P0, int dim, uint64_t copie
     // four threads per word while they make at most four warps per scheduler
     // (2100 cycles for a word per thread, 420 per warp and quarter)
     const bool split = words <= 128u;
+    // runs with more words inside than at their ends are held in shared memory, so that only
+    // the ends wait for L2 (L = 1000, 100 sweeps: 416 -> 331 us; with a word per thread the
+    // choice for every word costs more than it brings: L = 1600 456 -> 466, L = 3000 459 -> 505)
+    const bool held = dim == 2 && split && 4u * P.edge <= words;
     const uint32_t items = split ? 4u * words : words;
     const uint32_t iters = (items + kStripMaxThreads - 1u) / kStripMaxThreads;
     const uint32_t T = ((items + iters - 1u) / iters + 31u) / 32u * 32u;
@@ -447,8 +481,9 @@ cudaError_t launch_stream_strips(const StreamStrips& P0, int dim, uint64_t copie
         if (e != cudaSuccess) return e;
     }
 #define GBMC_STRIPS(D_, A_)                                                                  \
-    (split ? launch_strips<D_, A_, 4>(P, copies, sm_count, T, s)                             \
-           : launch_strips<D_, A_, 1>(P, copies, sm_count, T, s))
+    (split ? launch_strips<D_, A_, 4, false>(P, copies, sm_count, T, s)                      \
+           : launch_strips<D_, A_, 1, false>(P, copies, sm_count, T, s))
+    if (held) return launch_strips<2, false, 4, true>(P, copies, sm_count, T, s);
     if (dim == 2) return GBMC_STRIPS(2, false);
     return P.bond ? GBMC_STRIPS(3, true) : GBMC_STRIPS(3, false);
 #undef GBMC_STRIPS
