@@ -474,11 +474,13 @@ bool job_takes_bits(const SweepLaunch& P, const SweepJob& J, const Tuning& tu, i
 
 // Whether the bit-stream kernel takes a job the bit-sliced kernel does not: any
 // resident lattice, in AUTO mode only (BITS leaves what the bit-sliced kernel
-// does not support to the byte-plane kernel). One exception: up to 10^4 copies of 2D
-// L = 8 with E and M of every sweep -- a word per plane, eight byte-plane threads per
-// copy -- 100 sweeps of 53 copies 104 us there, 112 us here; of 20000 299 against 273.
-bool job_takes_stream(const SweepLaunch& P, const SweepJob& J, const Tuning& tu, int kernel) {
-    if (P.dim == 2 && J.L == 8 && (J.Eser || J.Mser) && (uint64_t)J.n_inst * J.R <= 10000u) return false;
+// does not support to the byte-plane kernel). One exception: 2D L = 8 with E and M of
+// every sweep, more copies than multiprocessors (sweeps_ahead takes fewer) and up to
+// 10^4 -- a word per plane, eight byte-plane threads per copy -- 100 sweeps of 53 copies
+// 104 us there, 112 us here; of 20000 299 against 273.
+bool job_takes_stream(const SweepLaunch& P, const SweepJob& J, const Tuning& tu, int kernel, int sm_count) {
+    const uint64_t copies = (uint64_t)J.n_inst * J.R;
+    if (P.dim == 2 && J.L == 8 && (J.Eser || J.Mser) && copies > (uint64_t)sm_count && copies <= 10000u) return false;
     return kernel == GBMC_KERNEL_AUTO && tu.bits && J.smask;
 }
 
@@ -517,7 +519,7 @@ gbmc_status launch_jobs(gbmc_ctx* ctx, const SweepLaunch& P0, const std::vector<
     for (int j = 0; j < P0.njobs; ++j) {
         if (!small && job_takes_bits(P0, P0.jobs[j], tu[j], kernel)) {
             B.jobs[B.njobs++] = P0.jobs[j];
-        } else if (job_takes_stream(P0, P0.jobs[j], tu[j], kernel)) {
+        } else if (job_takes_stream(P0, P0.jobs[j], tu[j], kernel, ctx->sm_count)) {
             S.jobs[S.njobs++] = P0.jobs[j];
         } else {
             Y.jobs[Y.njobs++] = P0.jobs[j];
@@ -530,7 +532,8 @@ gbmc_status launch_jobs(gbmc_ctx* ctx, const SweepLaunch& P0, const std::vector<
     }
     if (S.njobs) {
         ProfScope ps_(ctx, PK_SWEEP_STREAM);
-        CUDA_TRY(launch_sweep_stream(S, ctx->sm_count, ctx->stream));
+        if (sweeps_ahead(S, ctx->sm_count)) CUDA_TRY(launch_sweep_ahead(S, ctx->words + 1, ctx->stream));
+        else CUDA_TRY(launch_sweep_stream(S, ctx->sm_count, ctx->stream));
     }
     if (Y.njobs == 0) return GBMC_OK;
     return launch_bytes(ctx, Y, ty, force_persistent);

@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <utility>
 
 #include <cooperative_groups.h>
@@ -709,6 +710,254 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
     }
 }
 
+// ---- few copies: the acceptance bits drawn ahead of the sweeps ----
+//
+// A copy alone on a multiprocessor sweeps as fast as the chain of a half-sweep allows, and
+// most of that chain are the ten rounds of Philox, which do not depend on the spins. One
+// block per copy: its first warps (a thread per word) update, the other kDrawers warps draw
+// acceptance words ahead of them into a ring in shared memory, 32 words a batch,
+// whatever half-sweeps these belong to. A batch's flag says that its words are there;
+// `taken` counts the half-sweeps whose words have been read. Waits are bounded.
+//
+// Bound: the chain of a half-sweep (words and masks loaded, some 25 dependent
+// instructions, word stored, barrier); from some 64 words per plane the drawers' integer pipes.
+// Measured, 400 sweeps with E and M, threads drawing their own words -> ahead: 2D L = 8, 9 copies
+// 442 -> 237 us, L = 32, 40 copies 437 -> 267, L = 64 510 -> 394, L = 90 834 -> 526; 3D L = 4 510 ->
+// 281, L = 16 590 -> 439.
+
+constexpr uint32_t kDrawers = 12, kAheadThreads = 512;
+constexpr uint32_t kAheadWords = 32u * (kAheadThreads / 32u - kDrawers);  // words per plane, at most
+constexpr uint32_t kAheadPolls = 1u << 26;
+
+__host__ __device__ __forceinline__ uint32_t ahead_ring(uint32_t PW) {  // items, a power of two, several half-sweeps
+    uint32_t n = 1024u;
+    while (n < 8u * PW) n <<= 1;
+    return n;
+}
+
+template <int DIM, bool EA>
+__global__ void __launch_bounds__(kAheadThreads, 1) k_sweep_ahead(const __grid_constant__ SweepLaunch P, unsigned int* err) {
+    extern __shared__ __align__(16) uint32_t smw[];
+    __shared__ uint32_t taken, dead;  // dead: a wait ran out, nothing waits any more
+    __shared__ int acc[2][2];
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
+    const SweepJob& J = P.jobs[0];
+    const StreamShape g = stream_shape<DIM>(J.L, J.N);
+    const uint32_t slot = blockIdx.x, inst = slot / J.R, r = slot - inst * J.R;
+    const uint32_t tid = threadIdx.x, T = blockDim.x, lane = tid & 31u, Wc = (g.PW + 31u) / 32u;
+    const uint32_t ring = ahead_ring(g.PW), k0 = (uint32_t)J.seed, k1 = (uint32_t)(J.seed >> 32);
+    uint2* const m48 = reinterpret_cast<uint2*>(smw + 2u * g.PWX);  // [ring] acceptance bits of dE = 4, 8
+    uint32_t* const m12 = reinterpret_cast<uint32_t*>(m48 + ring);  // (3D: 12)
+    uint32_t* const flag = m12 + (DIM == 3 ? ring : 0u);
+    volatile uint32_t *const vtaken = &taken, *const vdead = &dead;
+    auto give_up = [&]() {
+        *vdead = 1u;
+        atomicExch(err, 1u);
+    };
+
+    const uint8_t* odd_b = reinterpret_cast<const uint8_t*>(J.smask);
+    const uint32_t nch = (J.N + 15u) >> 4;
+    const bool wide = (J.N & 15u) == 0u;
+    for (uint32_t ch = tid; ch < nch; ch += T) {
+        const int8_t* src = J.src + (uint64_t)slot * J.N + 16u * ch;
+        uint4 v;
+        if (wide) {
+            v = *reinterpret_cast<const uint4*>(src);
+        } else {  // copies start on 4-byte boundaries, the last chunk is short
+            const uint32_t* s4 = reinterpret_cast<const uint32_t*>(src);
+            const uint32_t left = J.N - 16u * ch;
+            v.x = s4[0];
+            v.y = left > 4u ? s4[1] : 0u;
+            v.z = left > 8u ? s4[2] : 0u;
+            v.w = left > 12u ? s4[3] : 0u;
+        }
+        uint32_t e0, o0, e1, o1;
+        pack8(v.x, v.y, e0, o0);
+        pack8(v.z, v.w, e1, o1);
+        const uint32_t ev = e0 | (e1 << 4), od = o0 | (o1 << 4), m = odd_b[ch];
+        uint8_t* p0 = reinterpret_cast<uint8_t*>(smw) + ch;
+        p0[0] = (uint8_t)sel(m, od, ev);
+        p0[4u * g.PWX] = (uint8_t)sel(m, ev, od);
+    }
+    for (uint32_t i = tid; i < ring / 32u; i += T) flag[i] = 0u;
+    if (tid == 0u) taken = dead = 0u;
+    if (tid < 4u) acc[tid >> 1][tid & 1u] = 0;
+    __syncthreads();
+    stream_extend<1>(smw, 1u, g, tid, T);
+    stream_extend<1>(smw + g.PWX, 1u, g, tid, T);
+    __syncthreads();
+
+    const uint32_t n_half = 2u * J.nsweeps;
+    // one updating warp has its scheduler (every fourth warp's) for itself: 2D L = 16, 2000 sweeps
+    // with E and M 1268 -> 1147 us
+    const uint32_t warp = tid / 32u, warps = T / 32u;
+    const bool spared = Wc == 1u && warp != 0u && (warp & 3u) == 0u;
+    if (tid >= 32u * Wc && !spared) {
+        const uint64_t items = (uint64_t)n_half * g.PW;
+        const uint32_t drawers = Wc == 1u ? warps - (warps + 3u) / 4u : warps - Wc;
+        for (uint64_t b = Wc == 1u ? warp - warp / 4u - 1u : warp - Wc; 32u * b < items; b += drawers) {
+            const uint64_t i = 32u * b + lane, last = 32u * b + 31u;  // (the last batch may end past the items)
+            // (asleep between looks: drawers far ahead would take the updaters' issue slots)
+            for (uint32_t n = 0; last >= (uint64_t)*vtaken * g.PW + ring && !*vdead; ++n) {
+                __nanosleep(200);
+                if (n == kAheadPolls / 64u) give_up();
+            }
+            const uint32_t h = (uint32_t)(i / g.PW), w = (uint32_t)(i - (uint64_t)h * g.PW);
+            const PhiloxFixed pf = philox_fix(J.t0 + (h >> 1), r, c3_word(kPurposeMetro, h & 1u, J.inst_base + inst), k0, k1);
+            uint32_t r4 = 0u, r8 = 0u, r12 = 0u;
+#pragma unroll
+            for (uint32_t k = 0; k < 8u; ++k) {
+                const uint4 v = philox_q_wide(pf, 8u * w + k);
+                if constexpr (DIM == 2) {
+                    accept_bits(r4, r8, J.thr[0], J.thr[1], v.x);
+                    accept_bits(r4, r8, J.thr[0], J.thr[1], v.y);
+                    accept_bits(r4, r8, J.thr[0], J.thr[1], v.z);
+                    accept_bits(r4, r8, J.thr[0], J.thr[1], v.w);
+                } else {
+                    accept_bits3(r4, r8, r12, J.thr[0], J.thr[1], J.thr[2], v.x);
+                    accept_bits3(r4, r8, r12, J.thr[0], J.thr[1], J.thr[2], v.y);
+                    accept_bits3(r4, r8, r12, J.thr[0], J.thr[1], J.thr[2], v.z);
+                    accept_bits3(r4, r8, r12, J.thr[0], J.thr[1], J.thr[2], v.w);
+                }
+            }
+            const uint32_t at = (uint32_t)i & (ring - 1u);
+            m48[at] = make_uint2(__brev(r4), __brev(r8));
+            if constexpr (DIM == 3) m12[at] = __brev(r12);
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0u) *(volatile uint32_t*)(flag + ((uint32_t)b & (ring / 32u - 1u))) = (uint32_t)b + 1u;
+        }
+    } else if (!spared) {
+        const uint32_t w = min(tid, g.PW - 1u);
+        const bool has = tid < g.PW;
+        Place<DIM, true> at;
+        at.set(g, w, J.smask);
+        uint32_t jb[2][2 * DIM];
+#pragma unroll
+        for (int k = 0; k < 4 * DIM; ++k)
+            jb[k / (2 * DIM)][k % (2 * DIM)] =
+                EA ? __ldg(J.sbond + (((uint64_t)inst * 2u + k / (2 * DIM)) * 2u * DIM + k % (2 * DIM)) * g.PW + w) : 0u;
+        auto sync = [&]() {
+            if (Wc == 1u) __syncwarp();
+            else asm volatile("bar.sync 1, %0;" ::"r"(32u * Wc) : "memory");
+        };
+        uint32_t a4 = 0u, a8 = 0u, a12 = 0u;
+        uint64_t known = 0;  // items below are known to be there, to this thread
+        auto fetch = [&](uint32_t h) {  // this word's acceptance bits of half-sweep h
+            const uint64_t i = (uint64_t)h * g.PW + w;
+            if (i >= known) {
+                const uint32_t b = (uint32_t)(i >> 5);
+                volatile uint32_t* f = flag + (b & (ring / 32u - 1u));
+                for (uint32_t n = 0; *f != b + 1u && !*vdead; ++n)
+                    if (n == kAheadPolls) give_up();
+                __threadfence_block();
+                known = (uint64_t)(b + 1u) << 5;
+            }
+            const uint32_t k = (uint32_t)i & (ring - 1u);
+            const uint2 m = m48[k];
+            a4 = m.x;
+            a8 = m.y;
+            if constexpr (DIM == 3) a12 = m12[k];
+        };
+        const bool series = J.Eser || J.Mser;
+        const uint64_t ncopies = (uint64_t)J.n_inst * J.R;
+        auto write = [&](uint32_t s, int U, int D) {  // every bond has one colour-0 end
+            if (J.Eser) J.Eser[s * ncopies + slot] = 2 * U - DIM * (int)J.N;
+            if (J.Mser) J.Mser[s * ncopies + slot] = (int)J.N - 2 * D;
+        };
+        if (n_half) fetch(0u);
+        auto half = [&](auto colour, uint32_t h) {
+            constexpr uint32_t c = decltype(colour)::value;
+            const bool update = h < n_half, measure = c == 0u && series && h > 0u;
+            uint32_t* const own = smw + c * g.PWX;
+            const Words<1>* oth = reinterpret_cast<const Words<1>*>(smw + (c ^ 1u) * g.PWX);
+            Words<1> nw = {{own[w]}}, same;
+            uint32_t d[2 * DIM][1], j[2 * DIM];
+#pragma unroll
+            for (int k = 0; k < 2 * DIM; ++k) j[k] = EA ? jb[c][k] : 0u;
+            stream_unsat<DIM, 1>(g, oth, nw, at, c, j, d, same);
+            if (measure) {
+                const uint32_t valid = !has ? 0u : w + 1u == g.PW ? g.mh : kAll;
+                int u = 0;
+#pragma unroll
+                for (int k = 0; k < 2 * DIM; ++k) u += __popc(d[k][0] & valid);
+                // both in one sum: a warp's down spins stay below 2^16
+                const int sum = __reduce_add_sync(kAll, u << 16 | (__popc(nw.v[0] & valid) + __popc(same.v[0] & valid)));
+                if (lane == 0u) {
+                    if (Wc == 1u) {
+                        write((h >> 1) - 1u, sum >> 16, sum & 0xFFFF);
+                    } else {
+                        atomicAdd(&acc[(h >> 1) & 1u][0], sum >> 16);
+                        atomicAdd(&acc[(h >> 1) & 1u][1], sum & 0xFFFF);
+                    }
+                }
+            }
+            if (update) {
+                uint32_t f;
+                if constexpr (DIM == 2) {
+                    const uint32_t s1 = d[0][0] ^ d[1][0], c1 = d[0][0] & d[1][0];
+                    const uint32_t s2 = d[2][0] ^ d[3][0], c2 = d[2][0] & d[3][0];
+                    const uint32_t ge = c1 | c2 | (s1 & s2), ea = (s1 ^ s2) & ~ge;
+                    f = ge | (ea & a4) | (~(ge | ea) & a8);
+                } else {
+                    const uint32_t s1 = d[0][0] ^ d[1][0] ^ d[2][0], c1 = maj3(d[0][0], d[1][0], d[2][0]);
+                    const uint32_t s2 = d[3][0] ^ d[4][0] ^ d[5][0], c2 = maj3(d[3][0], d[4][0], d[5][0]);
+                    const uint32_t a0 = s1 ^ s2, t = s1 & s2, a1 = c1 ^ c2 ^ t, a2 = maj3(c1, c2, t);
+                    const uint32_t ge = a2 | (a1 & a0), ea = a1 & ~(a0 | a2), eb = a0 & ~(a1 | a2);
+                    f = ge | (ea & a4) | (eb & a8) | (~(ge | ea | eb) & a12);
+                }
+                nw.v[0] ^= f;
+                if (g.h == 32u || Wc > 1u) {
+                    if (has) own[w] = nw.v[0];
+                    if (g.h == 32u && tid == 0u) own[g.PW] = nw.v[0];  // the extension is word 0 again
+                } else {  // the extension follows the last word's h bits
+                    const uint32_t first = __shfl_sync(kAll, nw.v[0], 0);
+                    const bool end = has && w + 1u == g.PW;
+                    const uint32_t tail = nw.v[0] & g.mh;
+                    const uint64_t e = tail | ((uint64_t)(g.PW == 1u ? tail : first) << g.h);
+                    if (has) own[w] = end ? (uint32_t)e : nw.v[0];
+                    if (end) own[g.PW] = (uint32_t)(e >> 32);
+                }
+                if (h + 1u < n_half) fetch(h + 1u);
+            }
+            sync();
+            if (tid == 0u) *vtaken = h + 2u;  // half-sweeps whose acceptance bits have been read
+            if (update && g.h != 32u && Wc > 1u) {
+                stream_extend<1>(own, 1u, g, tid, 32u * Wc);
+                sync();
+            }
+            if (measure && Wc > 1u && tid == 0u) {
+                int* a = acc[(h >> 1) & 1u];
+                write((h >> 1) - 1u, a[0], a[1]);
+                a[0] = a[1] = 0;  // next added to two sweeps later
+            }
+        };
+        for (uint32_t h = 0; h < n_half; h += 2u) {
+            half(std::integral_constant<uint32_t, 0>{}, h);
+            half(std::integral_constant<uint32_t, 1>{}, h + 1u);
+        }
+        if (series) half(std::integral_constant<uint32_t, 0>{}, n_half);
+    }
+    __syncthreads();
+    for (uint32_t ch = tid; ch < nch; ch += T) {
+        const uint8_t* p0 = reinterpret_cast<const uint8_t*>(smw) + ch;
+        const uint32_t a = p0[0], b = p0[4u * g.PWX], m = odd_b[ch];
+        const uint32_t ev = sel(m, b, a), od = sel(m, a, b);
+        const uint2 lo = unpack8(ev & 15u, od & 15u), hi = unpack8(ev >> 4, od >> 4);
+        int8_t* dst = J.dst + (uint64_t)slot * J.N + 16u * ch;
+        if (wide) {
+            *reinterpret_cast<uint4*>(dst) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+        } else {
+            uint32_t* d4 = reinterpret_cast<uint32_t*>(dst);
+            const uint32_t left = J.N - 16u * ch;
+            d4[0] = lo.x;
+            if (left > 4u) d4[1] = lo.y;
+            if (left > 8u) d4[2] = hi.x;
+            if (left > 12u) d4[3] = hi.y;
+        }
+    }
+}
+
 // Per-word masks of a lattice class, [5][PW]: the sites whose colour-0 row starts
 // at odd x; the row ends whose x neighbour wraps around, for colour 0 and for
 // colour 1; the sites with y = 0; those with y = L - 1. Bits past the stream's
@@ -996,6 +1245,26 @@ cudaError_t launch_rounds_c(const SweepLaunch& P, const PtExchange& X, const Rou
 }
 
 }  // namespace
+
+// Plain sweeps of at most one copy per multiprocessor.
+bool sweeps_ahead(const SweepLaunch& P, int sm_count) {
+    if (P.njobs != 1) return false;
+    const SweepJob& J = P.jobs[0];
+    const uint64_t copies = (uint64_t)J.n_inst * J.R;
+    return J.smask && (!P.ea || J.sbond) && (J.N / 2u + 31u) / 32u <= kAheadWords && copies <= (uint64_t)sm_count &&
+           J.nsweeps >= 2u && J.nsweeps <= 0x3FFFFFFFu && !J.parent && !J.hist && !J.temp_of && !J.nlive && !J.E && !J.M &&
+           J.src == J.dst;
+}
+
+cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, cudaStream_t s) {
+    const SweepJob& J = P.jobs[0];
+    const uint32_t PW = (J.N / 2u + 31u) / 32u, ring = ahead_ring(PW), Wc = (PW + 31u) / 32u;
+    const size_t smem = 4ull * (2u * (PW + 1u) + (P.dim == 3 ? 3u : 2u) * ring + ring / 32u);
+    auto kern = P.dim == 2 ? k_sweep_ahead<2, false> : P.ea ? k_sweep_ahead<3, true> : k_sweep_ahead<3, false>;
+    kern<<<J.n_inst * J.R, 32u * (Wc == 1u ? 12u : Wc + kDrawers), smem, s>>>(P, err);
+    count_launch();
+    return cudaGetLastError();
+}
 
 // A round by itself is a sweep launch, whose copies are loaded and stored, and an
 // exchange launch, 20 000 to 27 000 cycles beside the half-sweeps (3D L = 8, 250 x 40 copies,
