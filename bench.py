@@ -792,7 +792,7 @@ def kernel_name(w, prof):
     if w["kind"] in ("pa", "pt"):
         if w.get("msc"):
             return "sweep_msc"
-        return "sweep_bits" if "sweep_bits" in prof else "sweep_resident"
+        return next((k for k in ("sweep_bits", "pt_rounds", "sweep_stream") if k in prof), "sweep_resident")
     if w.get("layout", 0) == 1 or "bitpack_strips" in prof:
         # int8 lattices too: their strip sweeps run packed to bits
         return "bitpack_strips" if "bitpack_strips" in prof else "bitpack_halfsweep"
