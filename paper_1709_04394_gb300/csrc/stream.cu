@@ -58,7 +58,7 @@ enum { kOneTemp = 0, kPerCopy = 1, kRounds = 2 };
 // largest block, and blocks per SM the registers have to leave room for: 64 registers
 // a thread for C = 1 and 2 (128 for S = 4 and for C = 1 in rounds), 96 for C = 4
 constexpr uint32_t stream_max_threads(int C, int S, int PT = kOneTemp) {
-    return C == 4 ? 128u : C == 2 || S == 4 || PT == kRounds ? 512u : 1024u;
+    return C == 4 ? 128u : C == 2 || S > 1 || PT == kRounds ? 512u : 1024u;
 }
 constexpr uint32_t stream_min_blocks(int C) { return C == 4 ? 5u : C == 2 ? 2u : 1u; }
 
@@ -252,8 +252,8 @@ __device__ __forceinline__ void stream_extend(uint32_t* plane, uint32_t n, const
 }
 
 // A team of T threads (a warp, or the block) sweeps G groups of C copies;
-// item i of its n_groups * PW words is word i % PW of group i / PW. S = 4 (C = 1
-// only): four threads per word, each the eight sites of one byte of it (two
+// item i of its n_groups * PW words is word i % PW of group i / PW. S = 4 or 2 (C = 1
+// only): so many threads per word, each the sites of a byte or half of it (two or four
 // Philox calls), for launches too small to give every scheduler two warps.
 //
 // PT = kRounds: X.rounds rounds of parallel tempering. The copies of an instance are
@@ -388,13 +388,15 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
     const uint32_t k0 = (uint32_t)J.seed, k1 = (uint32_t)(J.seed >> 32);
     const bool want_final = J.E || J.M || J.hist;
     const uint32_t items = n * g.PW, nsw = J.nsweeps;
-    static_assert(S == 1 || (S == 4 && C == 1), "");
-    constexpr int NQ = S == 4 ? 2 : stream_calls(C);
+    static_assert(S == 1 || ((S == 2 || S == 4) && C == 1), "");
+    constexpr int NQ = S > 1 ? 8 / S : stream_calls(C);
+    constexpr uint32_t kBits = 32u / S;  // sites of a thread, and their mask in the word
+    auto my_bits = [](uint32_t part) { return S > 1 ? (0xFFFFFFFFu >> (32u - kBits)) << (kBits * part) : 0xFFFFFFFFu; };
     const uint32_t NB = 2u * DIM * g.PW;  // bond words per instance and colour
     // item is -> group, copies and place; worked out once where a thread has one
     // item at most (small populations, where the chain of a half-sweep is what counts)
     uint32_t gi = 0, part = 0, inst = 0, r0 = 0;
-    constexpr bool kEager = S == 4 || (C == 1 && PT == kRounds);
+    constexpr bool kEager = S > 1 || (C == 1 && PT == kRounds);
     Place<DIM, kEager> at;
     uint32_t jkept[PT == kRounds && EA ? 2 : 1][2 * DIM];  // bond words of both colours
     auto bonds = [&](uint32_t colour, uint32_t in, uint32_t (&j)[2 * DIM]) {
@@ -522,7 +524,7 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
                     Words<C> same;
                     bonds(colour, inst, j);
                     stream_unsat<DIM, C>(g, oth, nw, at, colour, j, d, same);
-                    if (measure) tally(d, nw, same, S == 4 ? 0xFFu << (8u * part) : 0xFFFFFFFFu);
+                    if (measure) tally(d, nw, same, my_bits(part));
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
                         if constexpr (DIM == 2) {
@@ -562,7 +564,7 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
                 for (int c = 0; c < C; ++c) r4[c] = r8[c] = r12[c] = 0u;
 #pragma unroll 2
                 for (uint32_t k = 0; k < 8u / S; k += NQ) {
-                    const uint32_t q = 8u * w + 2u * part + k;  // part: 0 unless S = 4
+                    const uint32_t q = 8u * w + (8u / S) * part + k;  // part: 0 where S = 1
                     uint4 v[NQ][C];
 #pragma unroll
                     for (int m = 0; m < NQ; ++m) {
@@ -606,15 +608,17 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
                             }
                         }
                 }
-                if constexpr (S == 4) {
-                    const uint32_t sh = 8u * part, gb = ge[0] >> sh, ab = ea[0] >> sh, bb = eb[0] >> sh;
-                    const uint32_t a4 = __brev(r4[0]) >> 24, a8 = __brev(r8[0]) >> 24, a12 = __brev(r12[0]) >> 24;
+                if constexpr (S > 1) {
+                    const uint32_t sh = kBits * part, gb = ge[0] >> sh, ab = ea[0] >> sh, bb = eb[0] >> sh;
+                    const uint32_t a4 = __brev(r4[0]) >> (32u - kBits), a8 = __brev(r8[0]) >> (32u - kBits),
+                                   a12 = __brev(r12[0]) >> (32u - kBits);
                     const uint32_t f = DIM == 2 ? gb | (ab & a4) | (~(gb | ab) & a8)
                                                 : gb | (ab & a4) | (bb & a8) | (~(gb | ab | bb) & a12);
-                    uint8_t* ob = reinterpret_cast<uint8_t*>(own) + part;
-                    const uint8_t nb = (uint8_t)((nw.v[0] >> sh) ^ f);
-                    ob[4u * w] = nb;  // the other bytes of the word belong to the neighbouring threads
-                    if (g.h == 32u && w == 0u) ob[4u * g.PW] = nb;
+                    using Part = std::conditional_t<S == 4, uint8_t, uint16_t>;
+                    Part* ob = reinterpret_cast<Part*>(own) + part;
+                    const Part nb = (Part)((nw.v[0] >> sh) ^ f);
+                    ob[S * w] = nb;  // the other parts of the word belong to the neighbouring threads
+                    if (g.h == 32u && w == 0u) ob[S * g.PW] = nb;
                 } else {
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
@@ -661,7 +665,7 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
                 Words<C> w1;
                 bonds(0u, inst, j);
                 stream_unsat<DIM, C>(g, p1, w0, at, 0u, j, d, w1);
-                tally(d, w0, w1, kParts == 4u ? 0xFFu << (8u * part) : 0xFFFFFFFFu);
+                tally(d, w0, w1, kParts > 1u ? my_bits(part) : 0xFFFFFFFFu);
             }
             flush();
             team_sync(warp);
@@ -1038,11 +1042,11 @@ struct StreamPlan {
 // measured: 2D L = 64 and 3D L = 10 with large populations (pass), populations with one to
 // seven warps per scheduler (lat, stream_wave)
 double stream_pass(int C, int split, int dim) {
-    return dim == 2 ? (C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 1030.0 : 430.0)
-                    : (C == 4 ? 3730.0 : C == 2 ? 2150.0 : split == 1 ? 1240.0 : 560.0);
+    return dim == 2 ? (C == 4 ? 3430.0 : C == 2 ? 1810.0 : split == 1 ? 1030.0 : split == 2 ? 620.0 : 430.0)
+                    : (C == 4 ? 3730.0 : C == 2 ? 2150.0 : split == 1 ? 1240.0 : split == 2 ? 750.0 : 560.0);
 }
 double stream_lat(int C, int split, int dim) {
-    return (C == 4 ? 9000.0 : (C == 2 ? 4200.0 : split == 1 ? 2100.0 : 900.0) * (dim == 3 ? 1.15 : 1.0));
+    return (C == 4 ? 9000.0 : (C == 2 ? 4200.0 : split == 1 ? 2100.0 : split == 2 ? 1300.0 : 900.0) * (dim == 3 ? 1.15 : 1.0));
 }
 // A pass with w warps on every scheduler, in teams of T: two copies per thread leave gaps where
 // the warps are few, and a block's teams wait for their slowest warp.
@@ -1147,6 +1151,8 @@ template <int DIM, bool EA>
 cudaError_t launch_stream_c(const SweepLaunch& P, const StreamPlan& S, bool pt, cudaStream_t st) {
     if (S.C == 4) return pt ? launch_stream<DIM, EA, 4, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 4, 1, kOneTemp>(P, S, st);
     if (S.C == 2) return pt ? launch_stream<DIM, EA, 2, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 2, 1, kOneTemp>(P, S, st);
+    if (S.split == 2)
+        return pt ? launch_stream<DIM, EA, 1, 2, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 1, 2, kOneTemp>(P, S, st);
     if (S.split == 4)
         return pt ? launch_stream<DIM, EA, 1, 4, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 1, 4, kOneTemp>(P, S, st);
     return pt ? launch_stream<DIM, EA, 1, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 1, 1, kOneTemp>(P, S, st);
@@ -1274,7 +1280,7 @@ cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, cudaStre
 bool tempering_in_rounds(const SweepLaunch& P, int sm_count) {
     const SweepJob& J = P.jobs[0];
     if (!J.smask || (P.ea && !J.sbond) || J.nsweeps == 0u || J.R < 2u || J.R > 1024u) return false;
-    double alone = stream_plan(P, 1, 4, true, sm_count).cost;
+    double alone = std::min(stream_plan(P, 1, 4, true, sm_count).cost, stream_plan(P, 1, 2, true, sm_count).cost);
     for (int C = 4; C >= 1; C >>= 1)
         if (C == 1 || stream_smem_words(J.N, 1u, (uint32_t)C, true) * 4u <= 36u * 1024u)
             alone = std::min(alone, stream_plan(P, C, 1, true, sm_count).cost);
@@ -1329,6 +1335,8 @@ cudaError_t launch_sweep_stream(const SweepLaunch& P0, int sm_count, cudaStream_
         key.job[j][0] = P.jobs[j].N, key.job[j][1] = P.jobs[j].R, key.job[j][2] = P.jobs[j].n_inst;
     if (std::memcmp(&key, &last, sizeof(key)) != 0) {
         S = stream_plan(P, 1, 4, pt, sm_count);
+        const StreamPlan halves = stream_plan(P, 1, 2, pt, sm_count);
+        if (halves.cost < S.cost) S = halves;
         for (int C = 4; C >= 1; C >>= 1) {
             // a group's planes at most 36 KB, so that an SM holds six blocks
             if (C > 1 && stream_smem_words(P.jobs[0].N, 1u, (uint32_t)C, pt) * 4u > 36u * 1024u) continue;
