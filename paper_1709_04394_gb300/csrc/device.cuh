@@ -131,4 +131,12 @@ __device__ __forceinline__ T block_inclusive_scan(T v, T* shared, T* total) {
     return x;
 }
 
+// A kernel launched with launch_chained may start while the one before it in the stream is
+// still running: chain_begin lets the next one do so and waits for the end of the one
+// before. First in a kernel; nothing where it was launched otherwise.
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace gbmc

@@ -63,6 +63,23 @@ struct SweepLaunch {
                                        // at launch; null: one CTA per unit
 };
 
+// Launch of a kernel that calls chain_begin (device.cuh), right behind the one before it.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, uint32_t threads, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    count_launch();
+    return e;
+}
+
 // ---- launchers (return cudaError_t of the launch) ----
 cudaError_t launch_init_spins(int8_t* spins, int dim, uint32_t L, uint32_t n_inst, uint32_t R,
                               uint32_t inst_base, uint64_t seed, int random_start, cudaStream_t s);

@@ -224,6 +224,7 @@ template <int DIM, bool EA, bool WIDE>
 __global__ void __launch_bounds__(256) k_observables(const int8_t* spins, const uint8_t* jbits, uint32_t L, uint32_t N,
                                                      uint32_t R, uint32_t T, uint64_t copy0, uint64_t ncopies,
                                                      int32_t* E, int32_t* M) {
+    chain_begin();
     const uint64_t copy = copy0 + (uint64_t)blockIdx.y * (blockDim.x / T) + threadIdx.x / T;
     const uint32_t t = blockIdx.x * T + threadIdx.x % T, n = gridDim.x * T;
     int U = 0, D = 0;
@@ -309,15 +310,14 @@ cudaError_t launch_observables(const int8_t* spins, const uint8_t* jbits, int di
     for (uint64_t c0 = 0; c0 < copies; c0 += 65535ull * per) {
         const uint64_t left = (copies - c0 + per - 1u) / per;
         const dim3 grid(bx, (uint32_t)(left < 65535ull ? left : 65535ull));
+        cudaError_t e;
 #define GBMC_OBS(D, A) \
-    (wide ? k_observables<D, A, true><<<grid, 256, 0, s>>>(spins, jbits, L, N, R, T, c0, copies, E, M) \
-          : k_observables<D, A, false><<<grid, 256, 0, s>>>(spins, jbits, L, N, R, T, c0, copies, E, M))
+    e = launch_chained(wide ? k_observables<D, A, true> : k_observables<D, A, false>, grid, 256, s, spins, jbits, L, N, R, T, \
+                       c0, copies, E, M)
         if (dim == 2) GBMC_OBS(2, false);
         else if (jbits) GBMC_OBS(3, true);
         else GBMC_OBS(3, false);
 #undef GBMC_OBS
-        count_launch();
-        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

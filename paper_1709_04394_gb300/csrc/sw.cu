@@ -58,6 +58,10 @@
 //                  roots of whole clusters) and draws each tile root's coin
 //                  once; every site takes its tile root's.
 //
+// The kernels of an update, E and M's, and the next update's follow each other chained (each is
+// in place when the one before it ends): L = 1024, 10 updates with E and M 451 -> 373
+// us.
+//
 // Small lattices take none of this but one launch for all updates of a call, a block per
 // copy, labels and spins in shared memory (k_sw_resident).
 #include <algorithm>
@@ -191,6 +195,7 @@ __device__ __forceinline__ void sw_unite(uint32_t* par, uint32_t a, uint32_t b, 
 
 template <uint32_t DIM>
 __global__ void __launch_bounds__(256) k_sw_bonds(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     const uint64_t copy = P.copy0 + blockIdx.y;
     const uint32_t i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (i0 >= P.N) return;
@@ -219,6 +224,7 @@ __device__ __forceinline__ SwTile sw_tile(uint32_t dim) {
 
 template <uint32_t DIM>
 __global__ void __launch_bounds__(256) k_sw_local(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     __shared__ uint32_t lp[1024];
     const uint64_t copy = P.copy0 + blockIdx.y;
     const int8_t* s = P.spins + copy * P.N;
@@ -290,6 +296,7 @@ __device__ __forceinline__ uint32_t sw_tile_root(uint32_t k, uint32_t i, uint32_
 }
 
 __global__ void __launch_bounds__(32 * kSwWarps) k_sw_scan2(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     __shared__ uint32_t f[1024];   // the tile's label forest (local indices)
     __shared__ uint16_t rl[1024];  // each site's run label
     constexpr uint32_t kAll = 0xffffffffu;
@@ -383,6 +390,7 @@ __host__ __device__ __forceinline__ uint32_t sw_cross_count(uint32_t N, uint32_t
 }
 
 __global__ void __launch_bounds__(256) k_sw_cross(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     const uint64_t copy = P.copy0 + blockIdx.y;
     uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = e < sw_cross_count(P.N, P.L, P.dim);
@@ -433,6 +441,7 @@ __global__ void __launch_bounds__(256) k_sw_cross(const __grid_constant__ SwLaun
 }
 
 __global__ void __launch_bounds__(256) k_sw_union(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     const uint64_t copy = P.copy0 + blockIdx.y;
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.N) return;
@@ -444,6 +453,7 @@ __global__ void __launch_bounds__(256) k_sw_union(const __grid_constant__ SwLaun
 }
 
 __global__ void __launch_bounds__(256) k_sw_flip(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     const uint64_t copy = P.copy0 + blockIdx.y;
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.N) return;
@@ -465,6 +475,7 @@ __device__ __forceinline__ uint32_t sw_coin(const PhiloxFixed& pf, uint32_t root
 }
 
 __global__ void __launch_bounds__(256) k_sw_flip_tiled(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     __shared__ uint32_t tpar[1024];   // the tile's parent pointers (global site indices)
     __shared__ uint32_t troot[1024];  // root of each end node
     __shared__ uint8_t tcoin[1024];   // its coin (1: the cluster flips)
@@ -551,6 +562,7 @@ __global__ void __launch_bounds__(256) k_sw_flip_tiled(const __grid_constant__ S
 // L = 1024); else four rows' sites of a column.
 template <bool QUADS>
 __global__ void __launch_bounds__(256) k_sw_flip_lab(const __grid_constant__ SwLaunch P) {
+    chain_begin();
     __shared__ uint32_t troot[1024];     // global root of each tile root (by local index)
     __shared__ uint8_t tcoin[1024];      // its coin (1: the cluster flips)
     __shared__ uint32_t tqueue[8][128];  // per warp: its tile roots (local indices)
@@ -904,11 +916,11 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
 }
 
 // One copy takes 5 us and 3.1 (2D) or 3.7 ns per site and update, one block after the other
-// on a multiprocessor; three kernels over the lattice and one or two for E and M take 25 to 35
+// on a multiprocessor; three kernels over the lattice and one for E and M take 19 to 30
 // us and, per site, 13 ps (2D, whole tiles) or 22 (3D) in tiles, 90 or 60 without. Measured, us
-// per update, the kernels -> resident: 2D L = 16 28 -> 6, L = 64 26 -> 16 (1000 copies 79 -> 108),
-// L = 100 28 -> 35 (152 copies 62 -> 36), L = 128 29 -> 52; 3D L = 8 29 -> 8, L = 16 29 -> 19 (1000
-// copies 117 -> 130), L = 24 38 -> 53 (152 copies 163 -> 57), L = 34 152 copies 446 -> 151.
+// per update, the kernels -> resident: 2D L = 16 20 -> 6, L = 64 17 -> 16 (152 copies 32 -> 17), L =
+// 90 19 -> 27 (152 copies 40 -> 29), L = 128 20 -> 52; 3D L = 8 22 -> 8, L = 16 22 -> 19 (256 copies
+// 51 -> 39), L = 20 30 -> 33 (152 copies 102 -> 35), L = 24 30 -> 53 (152 copies 154 -> 57).
 bool sw_resident(uint32_t dim, uint32_t L, uint32_t N, uint64_t copies, bool series, int sm_count) {
     const uint32_t bytes = sw_resident_words(N, dim) * 4u;
     if (L < 4u || bytes > 224u * 1024u) return false;  // a quad holds at most one row's end
@@ -918,7 +930,7 @@ bool sw_resident(uint32_t dim, uint32_t L, uint32_t N, uint64_t copies, bool ser
     const double chip = std::ceil(c / sm_count) * each + 5.0 * std::ceil(c / (sm_count * held));
     const bool tiled = sw_tiled(dim, L);
     const double area = dim == 2 && tiled ? 1024.0 * ((L + 31u) / 32u) * ((L + 31u) / 32u) : (double)N;
-    const double grid = (tiled ? (dim == 2 ? 24.0 : 29.0) : 32.0 + N * 4e-4) - (series ? 0.0 : 8.0) +
+    const double grid = (tiled ? (dim == 2 ? 19.0 : 23.0) : 26.0 + N * 4e-4) - (series ? 0.0 : 6.0) +
                         c * area * (tiled ? (dim == 2 ? 1.3e-5 : 2.2e-5) : dim == 2 ? 9e-5 : 6e-5);
     return chip < grid;
 }
@@ -962,42 +974,33 @@ cudaError_t launch_sw_update(const SwLaunch& P0, uint64_t copies, cudaStream_t s
         if (tiled && P.dim == 2) {
             if (!P.lab) return cudaErrorInvalidValue;
             const uint32_t edge = (P.L + 31u) / 32u, tiles = edge * edge;
-            k_sw_scan2<<<dim3(tiles, nc), 32 * kSwWarps, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_cross<<<dim3((sw_cross_count(P.N, P.L, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if (P.L % 4 == 0) k_sw_flip_lab<true><<<dim3(tiles, nc), 256, 0, s>>>(P);
-            else k_sw_flip_lab<false><<<dim3(tiles, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            e = launch_chained(k_sw_scan2, dim3(tiles, nc), 32 * kSwWarps, s, P);
+            if (e != cudaSuccess) return e;
+            e = launch_chained(k_sw_cross, dim3((sw_cross_count(P.N, P.L, P.dim) + 255) / 256, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
+            if (P.L % 4 == 0) e = launch_chained(k_sw_flip_lab<true>, dim3(tiles, nc), 256, s, P);
+            else e = launch_chained(k_sw_flip_lab<false>, dim3(tiles, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
             continue;
         }
         P.lab = nullptr;
         if (tiled) {
-            k_sw_local<3><<<dim3(P.N / 1024, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_cross<<<dim3((sw_cross_count(P.N, P.L, P.dim) + 255) / 256, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_flip_tiled<<<dim3(P.N / 1024, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            e = launch_chained(k_sw_local<3>, dim3(P.N / 1024, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
+            e = launch_chained(k_sw_cross, dim3((sw_cross_count(P.N, P.L, P.dim) + 255) / 256, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
+            e = launch_chained(k_sw_flip_tiled, dim3(P.N / 1024, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
             continue;
         } else {
-            if (P.dim == 2) k_sw_bonds<2><<<dim3((quads + 255) / 256, nc), 256, 0, s>>>(P);
-            else k_sw_bonds<3><<<dim3((quads + 255) / 256, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_sw_union<<<dim3((P.N + 255) / 256, nc), 256, 0, s>>>(P);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (P.dim == 2) e = launch_chained(k_sw_bonds<2>, dim3((quads + 255) / 256, nc), 256, s, P);
+            else e = launch_chained(k_sw_bonds<3>, dim3((quads + 255) / 256, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
+            e = launch_chained(k_sw_union, dim3((P.N + 255) / 256, nc), 256, s, P);
+            if (e != cudaSuccess) return e;
         }
-        k_sw_flip<<<dim3((P.N + 255) / 256, nc), 256, 0, s>>>(P);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_chained(k_sw_flip, dim3((P.N + 255) / 256, nc), 256, s, P);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
