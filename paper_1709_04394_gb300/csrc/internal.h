@@ -63,21 +63,31 @@ struct SweepLaunch {
                                        // at launch; null: one CTA per unit
 };
 
-// Launch of a kernel that calls chain_begin (device.cuh), right behind the one before it.
+// Launch of a kernel that calls chain_begin (device.cuh), right behind the one before it;
+// cluster: blocks per cluster, 0 for none.
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, uint32_t threads, cudaStream_t s, A... args) {
+cudaError_t launch_chained_as(void (*kern)(P...), dim3 grid, uint32_t threads, size_t smem, uint32_t cluster,
+                              cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
     count_launch();
     return e;
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, uint32_t threads, cudaStream_t s, A... args) {
+    return launch_chained_as(kern, grid, threads, 0u, 0u, s, args...);
 }
 
 // ---- launchers (return cudaError_t of the launch) ----

@@ -605,6 +605,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
     __shared__ unsigned long long sh64[32];
     __shared__ uint32_t sh32[32];
     __shared__ double sd[32];
+    chain_begin();
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t rank = cluster.block_rank(), K = cluster.num_blocks() - 1u, cid = blockIdx.x / (K + 1u);
     uint32_t job = 0;
@@ -772,14 +773,13 @@ cudaError_t launch_pa_resample_clusters(const PaLattice* jobs, double* const* ln
                 continue;
             }
         }
-        e = cudaLaunchKernelEx(&cfg, k_pa_resample_clusters, A);
-        count_launch();
-        return e;
+        return launch_chained_as(k_pa_resample_clusters, cfg.gridDim, kScanThreads, bytes, blocks, s, A);
     }
 }
 
 // Record of one step for every population of a lattice, after its sweeps.
 __global__ void k_pa_record(const __grid_constant__ PaLattice P, const double* lnZ) {
+    chain_begin();
     const uint32_t inst = blockIdx.x * blockDim.x + threadIdx.x;
     if (inst >= P.n_inst) return;
     gbmc_pa_stats* st = reinterpret_cast<gbmc_pa_stats*>(P.stats) + inst;
@@ -802,9 +802,7 @@ __global__ void k_pa_record(const __grid_constant__ PaLattice P, const double* l
 }
 
 cudaError_t launch_pa_record(const PaLattice& P, const double* lnZ, double, cudaStream_t s) {
-    k_pa_record<<<(P.n_inst + 127) / 128, 128, 0, s>>>(P, lnZ);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(k_pa_record, dim3((P.n_inst + 127) / 128), 128, s, P, lnZ);
 }
 
 // Reset of the accumulators before the first measurement (step 0).

@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const __grid_constan
     __shared__ SchedWalk walk;
     __shared__ float xin[kMlpIn], h1[kMlpHidden], h2[kMlpHidden];
     __shared__ double ys;
+    chain_begin();
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t rank = cluster.block_rank(), n_blocks = cluster.num_blocks();
     const uint32_t job = (blockIdx.x / n_blocks) % (uint32_t)S.njobs;
@@ -416,9 +417,7 @@ cudaError_t launch_schedule(const SchedLaunch& S, cudaStream_t s) {
             cudaGetLastError();
             continue;
         }
-        e = cudaLaunchKernelEx(&cfg, k_schedule, S);
-        count_launch();
-        return e;
+        return launch_chained_as(k_schedule, cfg.gridDim, kSchedThreads, sizeof(SchedBins), n, s, S);
     }
     return cudaErrorInvalidConfiguration;
 }
