@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(256) k_observables(const int8_t* spins, const 
 }
 
 __global__ void k_zero2(int32_t* a, int32_t* b, uint64_t n) {
+    chain_begin();
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (a) a[i] = 0;
@@ -280,9 +281,7 @@ __global__ void k_zero2(int32_t* a, int32_t* b, uint64_t n) {
 }
 
 cudaError_t launch_zero2(int32_t* a, int32_t* b, uint64_t n, cudaStream_t s) {
-    k_zero2<<<(uint32_t)((n + 255u) / 256u), 256, 0, s>>>(a, b, n);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(k_zero2, dim3((uint32_t)((n + 255u) / 256u)), 256, s, a, b, n);
 }
 
 cudaError_t launch_observables(const int8_t* spins, const uint8_t* jbits, int dim, uint32_t L,

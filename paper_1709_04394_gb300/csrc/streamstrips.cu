@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
 template <int DIM, bool PACK>
 __global__ void __launch_bounds__(256) k_stream_convert(int8_t* spins, uint64_t* P, const uint32_t* mask, uint32_t L,
                                                         uint32_t N, uint64_t copies) {
+    chain_begin();
     const PlaneShape g = plane_shape(DIM, L, N);
     const uint32_t nch = (N + 15u) >> 4;
     const bool wide = (N & 15u) == 0u;
@@ -387,6 +388,7 @@ __global__ void __launch_bounds__(256) k_stream_convert(int8_t* spins, uint64_t*
 // The bit-packed layout's words (the same streams) <-> the words beside tags.
 template <bool PACK>
 __global__ void __launch_bounds__(256) k_stream_words(uint32_t* words, uint64_t* P, uint64_t n) {
+    chain_begin();
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         if constexpr (PACK) P[i] = words[i];  // tag 0
         else words[i] = (uint32_t)P[i];
@@ -395,6 +397,7 @@ __global__ void __launch_bounds__(256) k_stream_words(uint32_t* words, uint64_t*
 
 // Series entries start from their constant terms.
 __global__ void k_series_init(int32_t* E, int32_t* M, int32_t e, int32_t m, uint64_t n) {
+    chain_begin();
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         if (E) E[i] = e;
         if (M) M[i] = m;
@@ -434,18 +437,14 @@ cudaError_t launch_stream_convert(int8_t* spins, uint64_t* P, const uint32_t* ma
     if (blocks > 152ull * 32ull) blocks = 152ull * 32ull;
     auto kern = dim == 2 ? (pack ? k_stream_convert<2, true> : k_stream_convert<2, false>)
                          : (pack ? k_stream_convert<3, true> : k_stream_convert<3, false>);
-    kern<<<(uint32_t)blocks, 256, 0, s>>>(spins, P, mask, L, N, copies);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((uint32_t)blocks), 256, s, spins, P, mask, L, N, copies);
 }
 
 cudaError_t launch_stream_words(uint32_t* words, uint64_t* P, uint64_t n, bool pack, cudaStream_t s) {
     uint64_t blocks = (n + 255u) / 256u;
     if (blocks > 152ull * 32ull) blocks = 152ull * 32ull;
     auto kern = pack ? k_stream_words<true> : k_stream_words<false>;
-    kern<<<(uint32_t)blocks, 256, 0, s>>>(words, P, n);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((uint32_t)blocks), 256, s, words, P, n);
 }
 
 cudaError_t launch_stream_strips(const StreamStrips& P0, int dim, uint64_t copies, int sm_count, cudaStream_t s) {
