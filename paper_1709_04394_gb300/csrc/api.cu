@@ -227,8 +227,7 @@ struct gbmc_pa {
     bool msc = false;      // multi-spin-coded sweeps
     uint32_t R0 = 0;       // its initial (and expected) population
     gbmc_pa_stats* stats = nullptr;  // device [S+1][P]
-    SchedOut* sched_dev = nullptr;   // [kMaxJobs]
-    SchedOut* sched_host = nullptr;  // pinned copy
+    SchedOut* sched_host = nullptr;  // [kMaxJobs] pinned, written by the kernel itself (a copy back took 6 us a step)
     float* mlp_dev = nullptr;        // MLP parameters (GBMC_SCHED_MLP)
     std::vector<void*> allocs;
     std::vector<void*> host_allocs;
@@ -1763,15 +1762,11 @@ gbmc_status pa_create(gbmc_ctx* ctx, gbmc_lattice* const* lattices, uint32_t n_l
     }
     if (st == GBMC_OK && adaptive) {
         void* p;
-        st = dalloc(pa, &p, kMaxJobs * sizeof(SchedOut));
-        if (st == GBMC_OK) pa->sched_dev = (SchedOut*)p;
-        if (st == GBMC_OK) {
-            cudaError_t ce = cudaMallocHost(&p, kMaxJobs * sizeof(SchedOut));
-            if (ce != cudaSuccess) st = fail(GBMC_ERR_OOM, "cudaMallocHost: %s", cudaGetErrorString(ce));
-            else {
-                pa->host_allocs.push_back(p);
-                pa->sched_host = (SchedOut*)p;
-            }
+        cudaError_t ce = cudaMallocHost(&p, kMaxJobs * sizeof(SchedOut));
+        if (ce != cudaSuccess) st = fail(GBMC_ERR_OOM, "cudaMallocHost: %s", cudaGetErrorString(ce));
+        else {
+            pa->host_allocs.push_back(p);
+            pa->sched_host = (SchedOut*)p;
         }
         if (st == GBMC_OK && sched == GBMC_SCHED_MLP) {
             st = dalloc(pa, &p, kMlpParams * sizeof(float));
@@ -1920,7 +1915,7 @@ static gbmc_status pa_enqueue_adaptive(gbmc_pa* pa, const double* beta_next) {
             const double rest = pa->cfg.beta_f - J.beta;
             J.dmax = pa->cfg.dbeta_max < rest ? pa->cfg.dbeta_max : rest;
         }
-        S.out = pa->sched_dev;
+        S.out = pa->sched_host;
         S.mlp = pa->cfg.schedule == GBMC_SCHED_MLP ? pa->mlp_dev : nullptr;
         S.target = pa->cfg.target_overlap;
         S.lo = pa->cfg.overlap_lo;
@@ -1930,7 +1925,6 @@ static gbmc_status pa_enqueue_adaptive(gbmc_pa* pa, const double* beta_next) {
             ProfScope ps_(pa->ctx, PK_SCHEDULE);
             CUDA_TRY(launch_schedule(S, s));
         }
-        CUDA_TRY(cudaMemcpyAsync(pa->sched_host, pa->sched_dev, S.njobs * sizeof(SchedOut), cudaMemcpyDeviceToHost, s));
     }
     // the staging slot written below was last read two steps ago
     CUDA_TRY(cudaStreamSynchronize(s));

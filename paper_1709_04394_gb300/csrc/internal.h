@@ -397,7 +397,7 @@ struct SchedJob {
     double beta, dmax;        // current beta; largest allowed step (<= beta_f - beta)
 };
 
-struct SchedOut {             // result per lattice (device, copied to the host)
+struct SchedOut {             // result per lattice (pinned host memory, written by the kernel)
     double dbeta;             // chosen step
     double alpha;             // realised overlap of the chosen step
     double proposal;          // MLP proposal (0 in bisection mode)
