@@ -115,9 +115,10 @@ gbmc_status gbmc_set_resample_mode(gbmc_ctx *ctx, int32_t fused);
  * Other lattices too large for shared memory (any even L, 3D too), calls with
  * E/M series, and few large copies that would fit: AUTO and PERSISTENT convert
  * the configuration to tagged bit words in a library buffer (N / 4 bytes per copy,
- * kept with the lattice), run all sweeps of the call, series included, as one
- * cooperative launch with the same bounded waits, and convert it back, unless the
- * call is only a sweep or two. GRID uses the per-launch kernels (halo tiles of up
+ * kept with the lattice; where it cannot be had -- memory full, or the stream being
+ * captured before it is there -- the GRID kernels run), run all sweeps of the call,
+ * series included, as one cooperative launch with the same bounded waits, and convert
+ * it back, unless the call is only a sweep or two. GRID uses the per-launch kernels (halo tiles of up
  * to 4 sweeps, resp. one launch per half-sweep), and so does the BYTES kernel mode
  * where its strips do not apply. Double-checkerboard sweeps with bit-sliced tiles
  * (metropolis_sweeps_dcb): PERSISTENT runs every round of a call in one
@@ -157,6 +158,12 @@ gbmc_status gbmc_set_sweep_kernel(gbmc_ctx *ctx, int32_t kernel);
  * pa_step with statistics) return GBMC_ERR_TIMEOUT; the context stays usable.
  * Pass (0, 2000000000) to restore the defaults. */
 gbmc_status gbmc_test_barrier_wait(gbmc_ctx *ctx, uint32_t phantom_arrivals, uint64_t budget_cycles);
+/* Test aid for a full device: buffers of more than `bytes` that the library can do
+ * without (those of the bit-plane sweeps of large lattices, the tables of the
+ * bit-stream sweeps) count as refused; calls then take the kernels that need none,
+ * with the same results, as they do inside a stream capture and when the device's
+ * memory is full. Pass UINT64_MAX to restore the default. */
+gbmc_status gbmc_test_spare_limit(gbmc_ctx *ctx, uint64_t bytes);
 
 /* Per-kernel timing with CUDA events recorded on the context stream around
  * every launch the library enqueues (off by default). gbmc_profile(ctx, 1)

@@ -103,6 +103,7 @@ struct gbmc_ctx {
     int32_t sweep_kernel = GBMC_KERNEL_AUTO; // bit-sliced or byte-plane resident sweeps
     uint32_t phantom = 0;           // test hook: extra barrier arrivals to wait for
     long long budget = 2000000000;  // cycles a barrier wait may last (about 1 s)
+    size_t spare_limit = SIZE_MAX;  // test hook: larger spare buffers count as refused
     bool prof = false;
     struct Pending {
         int kind;
@@ -250,6 +251,20 @@ bool is_device_ptr(const void* p) {
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Device memory for a faster way of doing what can be done without it: null where it cannot
+// be had -- the allocator refuses, or the context's stream is being captured, where an
+// allocation is not allowed and its contents would not be there before the first replay.
+void* spare_alloc(const gbmc_ctx* ctx, size_t bytes) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    void* p = nullptr;
+    if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+        bytes > ctx->spare_limit || cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();  // not left for the next launch to report
+        return nullptr;
+    }
+    return p;
 }
 
 // T(dE) = ceil(exp(-beta dE) 2^32) - 1 (Eq. (8) as an integer comparison).
@@ -668,6 +683,12 @@ gbmc_status gbmc_test_barrier_wait(gbmc_ctx* ctx, uint32_t phantom_arrivals, uin
     return GBMC_OK;
 }
 
+gbmc_status gbmc_test_spare_limit(gbmc_ctx* ctx, uint64_t bytes) {
+    if (!ctx) return fail(GBMC_ERR_ARG, "ctx is NULL");
+    ctx->spare_limit = (size_t)bytes;
+    return GBMC_OK;
+}
+
 gbmc_status gbmc_destroy(gbmc_ctx* ctx) {
     if (!ctx) return GBMC_OK;
     cudaStreamSynchronize(ctx->stream);
@@ -803,14 +824,12 @@ gbmc_status lattice_init(gbmc_ctx* ctx, const gbmc_lattice_desc* d, void* spins_
         }
     }
     if (d->layout == GBMC_INT8 && (d->dim == 3 || tune(l).resident)) {
+        // (without them the lattice is swept by the byte-plane and half-sweep kernels)
         const size_t words = stream_mask_words((uint32_t)N) + (l->jbits ? stream_bond_words((uint32_t)N) * d->n_instances : 0);
-        cudaError_t e = cudaMalloc(&l->stab, words * 4);
-        if (e != cudaSuccess) {
-            lattice_free(l);
-            return fail(GBMC_ERR_OOM, "cudaMalloc(bit-stream tables): %s", cudaGetErrorString(e));
-        }
-        CUDA_TRY(launch_stream_tables(l->jbits, l->stab, l->jbits ? l->stab + stream_mask_words((uint32_t)N) : nullptr,
-                                      d->dim, (uint32_t)d->L, d->n_instances, ctx->stream));
+        l->stab = (uint32_t*)spare_alloc(ctx, words * 4);
+        if (l->stab)
+            CUDA_TRY(launch_stream_tables(l->jbits, l->stab, l->jbits ? l->stab + stream_mask_words((uint32_t)N) : nullptr,
+                                          d->dim, (uint32_t)d->L, d->n_instances, ctx->stream));
     }
     {
         ProfScope ps_(ctx, PK_INIT);
@@ -948,6 +967,13 @@ bool takes_stream_strips(const gbmc_ctx* ctx, const gbmc_lattice* l, const Tunin
     return 4 * l->ncopies <= (uint64_t)ctx->sm_count && words >= 250.0 && n_sweeps >= (words >= 512.0 ? 4u : 8u);
 }
 
+// The buffer of those sweeps, N / 4 bytes per copy, kept with the lattice; without it the
+// call takes the kernels that need none.
+bool stream_strips_buffer(const gbmc_ctx* ctx, gbmc_lattice* l) {
+    if (!l->tagged) l->tagged = (uint64_t*)spare_alloc(ctx, l->ncopies * stream_plane_words((uint32_t)l->N) * 8);
+    return l->tagged != nullptr;
+}
+
 gbmc_status stream_strips_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint32_t n_sweeps, int32_t* E_series,
                                  int32_t* M_series) {
     uint32_t thr[3];
@@ -959,10 +985,6 @@ gbmc_status stream_strips_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, ui
         S.bond = l->jbits ? l->stab + stream_mask_words((uint32_t)l->N) : nullptr;
     }
     const uint64_t words = l->ncopies * stream_plane_words((uint32_t)l->N);
-    if (!l->tagged) {
-        cudaError_t e = cudaMalloc(&l->tagged, words * 8);
-        if (e != cudaSuccess) return fail(GBMC_ERR_OOM, "cudaMalloc(packed copy): %s", cudaGetErrorString(e));
-    }
     auto convert = [&](bool pack) -> cudaError_t {
         ProfScope ps_(ctx, PK_BP_PACK);
         if (l->d.layout == GBMC_BITPACK) return launch_stream_words((uint32_t*)l->cur, l->tagged, words, pack, ctx->stream);
@@ -1039,7 +1061,7 @@ gbmc_status metropolis_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint3
             l->t += n_sweeps;
             return GBMC_OK;
         }
-        if (takes_stream_strips(ctx, l, Tuning{}, n_sweeps, E_series || M_series))
+        if (takes_stream_strips(ctx, l, Tuning{}, n_sweeps, E_series || M_series) && stream_strips_buffer(ctx, l))
             return stream_strips_sweeps(ctx, l, beta, n_sweeps, E_series, M_series);
         for (uint32_t s = 0; s < n_sweeps; ++s) {
             for (uint32_t colour = 0; colour < 2; ++colour) {
@@ -1109,7 +1131,7 @@ gbmc_status metropolis_sweeps(gbmc_ctx* ctx, gbmc_lattice* l, double beta, uint3
             return GBMC_OK;
         }
     }
-    if (takes_stream_strips(ctx, l, tu, n_sweeps, E_series || M_series))
+    if (takes_stream_strips(ctx, l, tu, n_sweeps, E_series || M_series) && stream_strips_buffer(ctx, l))
         return stream_strips_sweeps(ctx, l, beta, n_sweeps, E_series, M_series);
     // strips of rows resident in shared memory for the whole call (large 2D ferromagnets, no E/M series)
     uint32_t sGc = 0, srmax = 0, sthreads = 0;

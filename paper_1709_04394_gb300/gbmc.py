@@ -115,6 +115,7 @@ def load():
             "pa_state_save": ([p, p, p, C.c_size_t], st),
             "pa_state_load": ([p, p, p, C.c_size_t], st),
             "gbmc_test_barrier_wait": ([p, C.c_uint32, C.c_uint64], st),
+            "gbmc_test_spare_limit": ([p, C.c_uint64], st),
             "gbmc_profile_read": ([p, p, C.c_uint32, C.POINTER(C.c_uint32)], st),
             "gbmc_kernel_launches": ([], C.c_uint64),
             "lattice_init": ([p, C.POINTER(LatticeDesc), p, C.c_size_t, C.POINTER(C.c_void_p)], st),
@@ -228,6 +229,10 @@ def gbmc_set_sweep_kernel(ctx, kernel=GBMC_KERNEL_AUTO):
 
 def gbmc_test_barrier_wait(ctx, phantom_arrivals=0, budget_cycles=2000000000):
     _check(load().gbmc_test_barrier_wait(ctx, phantom_arrivals, budget_cycles))
+
+
+def gbmc_test_spare_limit(ctx, n_bytes=2**64 - 1):
+    _check(load().gbmc_test_spare_limit(ctx, n_bytes))
 
 
 def gbmc_profile(ctx, enable=True):
