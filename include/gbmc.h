@@ -201,6 +201,22 @@ typedef struct {
     uint64_t seed;          /* Philox key */
 } gbmc_lattice_desc;
 
+/* Test aid for the way the bit-stream kernel spreads a launch over the device (no device is
+ * needed): the form it takes for the sweeps of n lattices together (dim, L, n_instances and
+ * n_replicas of each desc; tempering != 0: every copy at a temperature of its own) on
+ * sm_count multiprocessors. team and groups: largest lattice first. */
+typedef struct {
+    int32_t copies_per_thread; /* 4, 2 or 1 */
+    int32_t threads_per_word;  /* 1, 2 or 4 (one copy per thread) */
+    uint32_t block_threads;
+    uint32_t pad;
+    uint32_t team[8];          /* threads of a team: 32, or the block */
+    uint32_t groups[8];        /* groups of copies_per_thread copies a team holds */
+    double cycles;             /* estimated cycles per half-sweep */
+} gbmc_stream_form;
+gbmc_status gbmc_test_stream_form(uint32_t n, const gbmc_lattice_desc *lattices, int32_t tempering, int32_t sm_count,
+                                  gbmc_stream_form *out);
+
 typedef struct {
     int64_t n_sites;        /* N = L^dim */
     int64_t n_copies;       /* n_instances * n_replicas */

@@ -689,6 +689,34 @@ gbmc_status gbmc_test_spare_limit(gbmc_ctx* ctx, uint64_t bytes) {
     return GBMC_OK;
 }
 
+gbmc_status gbmc_test_stream_form(uint32_t n, const gbmc_lattice_desc* lattices, int32_t tempering, int32_t sm_count,
+                                  gbmc_stream_form* out) {
+    if (!lattices || !out) return fail(GBMC_ERR_ARG, "NULL argument");
+    static_assert(kMaxJobs == 8, "gbmc_stream_form");
+    if (n == 0 || n > (uint32_t)kMaxJobs || sm_count < 1) return fail(GBMC_ERR_ARG, "1 to %d lattices", kMaxJobs);
+    SweepLaunch P;
+    std::memset(&P, 0, sizeof(P));
+    P.dim = lattices[0].dim;
+    P.njobs = (int)n;
+    for (uint32_t j = 0; j < n; ++j) {
+        const gbmc_lattice_desc& d = lattices[j];
+        if (d.dim != P.dim || (d.dim != 2 && d.dim != 3) || d.L < 2 || (d.L & 1) || d.L > (d.dim == 2 ? 480 : 60) ||
+            d.n_replicas == 0 || d.n_instances == 0)
+            return fail(GBMC_ERR_ARG, "lattice %u is not one the kernel takes", j);
+        P.jobs[j].N = (uint32_t)d.L * d.L * (d.dim == 3 ? d.L : 1);
+        P.jobs[j].R = d.n_replicas;
+        P.jobs[j].n_inst = d.n_instances;
+    }
+    const StreamPlan S = stream_plan(P, tempering != 0, sm_count);
+    std::memset(out, 0, sizeof(*out));
+    out->copies_per_thread = S.C;
+    out->threads_per_word = S.split;
+    out->block_threads = S.threads;
+    out->cycles = S.cost;
+    for (uint32_t j = 0; j < n; ++j) out->team[j] = S.T[j], out->groups[j] = S.G[j];
+    return GBMC_OK;
+}
+
 gbmc_status gbmc_destroy(gbmc_ctx* ctx) {
     if (!ctx) return GBMC_OK;
     cudaStreamSynchronize(ctx->stream);

@@ -218,6 +218,16 @@ size_t stream_bond_words(uint32_t N);
 cudaError_t launch_stream_tables(const uint8_t* jbits, uint32_t* smask, uint32_t* sbond, int dim, uint32_t L,
                                  uint32_t n_inst, cudaStream_t s);
 cudaError_t launch_sweep_stream(const SweepLaunch& P, int sm_count, cudaStream_t s);
+// How a launch spreads its jobs: C copies per thread or `split` threads per word, and per job
+// teams of T threads with G groups of C copies each (largest copies first); cost: estimated
+// cycles per half-sweep. It depends on the jobs' N, R and n_inst alone.
+struct StreamPlan {
+    int C = 1, split = 1;
+    uint32_t threads = 128;
+    uint32_t T[kMaxJobs] = {}, G[kMaxJobs] = {};
+    double cost = 1e300;
+};
+StreamPlan stream_plan(const SweepLaunch& P, bool pt, int sm_count);
 
 // Large lattices, one bit per spin, every half-sweep of a call in one cooperative
 // launch (streamstrips.cu; 2D: L >= 64). P: per copy two planes of

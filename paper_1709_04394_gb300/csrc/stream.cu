@@ -1032,12 +1032,7 @@ uint32_t stream_smem_words(uint32_t N, uint32_t G, uint32_t C, bool pt) {
 // job's are what is left at the end). Estimate : measured, thousand cycles per half-sweep,
 // C = 1, 2, 4 (* taken): 2D L = 24, 40, 96 together 64 : 56, 60* : 49, 62 : 57; 3D L = 10, 8 x
 // 5000 copies 41 : 41, 37 : 36, 33* : 34; L = 12, 4 x 1000 copies 8.7* : 9.0, 9.6 : 9.1, 9.0 : 8.3.
-struct StreamPlan {
-    int C = 1, split = 1;
-    uint32_t threads = kStreamThreads;
-    uint32_t T[kMaxJobs] = {}, G[kMaxJobs] = {};
-    double cost = 1e300;
-};
+static_assert(StreamPlan{}.threads == kStreamThreads, "");
 
 // measured: 2D L = 64 and 3D L = 10 with large populations (pass), populations with one to
 // seven warps per scheduler (lat, stream_wave)
@@ -1097,12 +1092,17 @@ StreamPlan stream_plan(const SweepLaunch& P, int C, int split, bool pt, int sm_c
                     S.G[j] = G;
                 }
             };
-            // one-warp teams; larger copies, and a single lattice with too few copies
-            // to give every scheduler work, take whole blocks
+            // one-warp teams; a single lattice with too few copies to give every scheduler
+            // work takes whole blocks
             for (uint32_t G = 1; G <= 32u && stream_smem_words(J.N, G, C, pt) <= kStreamTeamWords; ++G) consider(32u, G);
             if (P.njobs == 1)
                 for (uint32_t T = 64u; T <= stream_max_threads(C, split) && T < PW + 32u; T += 32u) consider(T, 1u);
-            if (S.T[j] == 0u) consider(kStreamThreads, 1u);
+            // Copies too large for that take whole blocks; beside other lattices' teams so may
+            // all from 24 500 sites, where four copies pass a one-warp team's share (annealing
+            // 200 copies of 2D L = 160 with 2000 of L = 24, 10 steps: 2480 us without, 1150 with;
+            // 1000 of L = 180 with 5000 of L = 40: 4700 and 3780)
+            if (best == 1e300 || (P.njobs > 1 && stream_smem_words(J.N, 1u, 4u, pt) > kStreamTeamWords))
+                consider(kStreamThreads, 1u);
             shares[j] = best_share;
             total += best_sum;
             longest = std::max(longest, best_len);
@@ -1313,11 +1313,30 @@ cudaError_t launch_stream_tables(const uint8_t* jbits, uint32_t* smask, uint32_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_stream(const SweepLaunch& P0, int sm_count, cudaStream_t s) {
-    SweepLaunch P = P0;
-    // largest copies first: their blocks are dispatched first, shortening the tail
+// Largest copies first: their blocks are dispatched first, shortening the tail.
+static void largest_first(SweepLaunch& P) {
     for (int a = 1; a < P.njobs; ++a)
         for (int b = a; b > 0 && P.jobs[b].N > P.jobs[b - 1].N; --b) std::swap(P.jobs[b], P.jobs[b - 1]);
+}
+
+StreamPlan stream_plan(const SweepLaunch& P0, bool pt, int sm_count) {
+    SweepLaunch P = P0;
+    largest_first(P);
+    StreamPlan S = stream_plan(P, 1, 4, pt, sm_count);
+    const StreamPlan halves = stream_plan(P, 1, 2, pt, sm_count);
+    if (halves.cost < S.cost) S = halves;
+    for (int C = 4; C >= 1; C >>= 1) {
+        // a group's planes at most 36 KB, so that an SM holds six blocks
+        if (C > 1 && stream_smem_words(P.jobs[0].N, 1u, (uint32_t)C, pt) * 4u > 36u * 1024u) continue;
+        const StreamPlan t = stream_plan(P, C, 1, pt, sm_count);
+        if (t.cost < S.cost) S = t;
+    }
+    return S;
+}
+
+cudaError_t launch_sweep_stream(const SweepLaunch& P0, int sm_count, cudaStream_t s) {
+    SweepLaunch P = P0;
+    largest_first(P);
     bool pt = false;
     for (int j = 0; j < P.njobs; ++j) {
         if (!P.jobs[j].smask || (P.ea && !P.jobs[j].sbond)) return cudaErrorInvalidValue;
@@ -1334,15 +1353,7 @@ cudaError_t launch_sweep_stream(const SweepLaunch& P0, int sm_count, cudaStream_
     for (int j = 0; j < P.njobs; ++j)
         key.job[j][0] = P.jobs[j].N, key.job[j][1] = P.jobs[j].R, key.job[j][2] = P.jobs[j].n_inst;
     if (std::memcmp(&key, &last, sizeof(key)) != 0) {
-        S = stream_plan(P, 1, 4, pt, sm_count);
-        const StreamPlan halves = stream_plan(P, 1, 2, pt, sm_count);
-        if (halves.cost < S.cost) S = halves;
-        for (int C = 4; C >= 1; C >>= 1) {
-            // a group's planes at most 36 KB, so that an SM holds six blocks
-            if (C > 1 && stream_smem_words(P.jobs[0].N, 1u, (uint32_t)C, pt) * 4u > 36u * 1024u) continue;
-            const StreamPlan t = stream_plan(P, C, 1, pt, sm_count);
-            if (t.cost < S.cost) S = t;
-        }
+        S = stream_plan(P, pt, sm_count);
         last = key;
     }
     if (P.dim == 2 && !P.ea) return launch_stream_c<2, false>(P, S, pt, s);

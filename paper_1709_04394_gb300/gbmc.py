@@ -64,6 +64,11 @@ class LatticeInfo(C.Structure):
                 ("sweep_counter", C.c_uint32), ("pad", C.c_uint32), ("spins_dev", C.c_void_p)]
 
 
+class StreamForm(C.Structure):
+    _fields_ = [("copies_per_thread", C.c_int32), ("threads_per_word", C.c_int32), ("block_threads", C.c_uint32),
+                ("pad", C.c_uint32), ("team", C.c_uint32 * 8), ("groups", C.c_uint32 * 8), ("cycles", C.c_double)]
+
+
 class PaConfig(C.Structure):
     _fields_ = [("theta", C.c_uint32), ("n_steps", C.c_uint32), ("schedule", C.c_int32), ("init", C.c_int32),
                 ("beta_f", C.c_double), ("betas", C.c_void_p), ("target_overlap", C.c_double),
@@ -116,6 +121,7 @@ def load():
             "pa_state_load": ([p, p, p, C.c_size_t], st),
             "gbmc_test_barrier_wait": ([p, C.c_uint32, C.c_uint64], st),
             "gbmc_test_spare_limit": ([p, C.c_uint64], st),
+            "gbmc_test_stream_form": ([C.c_uint32, p, C.c_int32, C.c_int32, C.POINTER(StreamForm)], st),
             "gbmc_profile_read": ([p, p, C.c_uint32, C.POINTER(C.c_uint32)], st),
             "gbmc_kernel_launches": ([], C.c_uint64),
             "lattice_init": ([p, C.POINTER(LatticeDesc), p, C.c_size_t, C.POINTER(C.c_void_p)], st),
@@ -233,6 +239,15 @@ def gbmc_test_barrier_wait(ctx, phantom_arrivals=0, budget_cycles=2000000000):
 
 def gbmc_test_spare_limit(ctx, n_bytes=2**64 - 1):
     _check(load().gbmc_test_spare_limit(ctx, n_bytes))
+
+
+def gbmc_test_stream_form(lattices, tempering=False, sm_count=152) -> StreamForm:
+    """lattices: (dim, L, n_instances, n_replicas) each."""
+    descs = (LatticeDesc * len(lattices))(*[LatticeDesc(d, L, 0, 0, 0, i, r, 0, 0) for d, L, i, r in lattices])
+    out = StreamForm()
+    _check(load().gbmc_test_stream_form(len(lattices), C.cast(descs, C.c_void_p), int(bool(tempering)), sm_count,
+                                        C.byref(out)))
+    return out
 
 
 def gbmc_profile(ctx, enable=True):
