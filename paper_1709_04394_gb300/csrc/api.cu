@@ -982,13 +982,24 @@ namespace {
 // 17.0 -> 19.3, n = 50 412 -> 208, with E and M of every sweep 4894 -> 197; L = 4000
 // n = 2 90.6 -> 49.7, n = 50 2256 -> 754; 3D +-J L = 48 n = 50 412 -> 260; one copy of
 // L = 256 (a block: 79 us per 10 sweeps) n = 10 79 -> 35, of L = 128 n = 50 154 -> 123;
-// bit-packed L = 448 n = 2 17.0 -> 16.5, n = 50 412 -> 162.
+// bit-packed L = 448 n = 2 17.0 -> 16.5, n = 50 412 -> 162. More copies, n = 4, 60, 77, 90, 100 and
+// 153 of them (two blocks each; one each on 77, 90 and 100 of 152 multiprocessors; two batches),
+// L = 1152 in halo tiles 505, 655, 749, 840, 1265 -> here 410, 744, 755, 761, 1478 (with series 1169,
+// 1820, 1971, 2098, 3127 -> 431, 779, 789, 795, 1543); sizes without tiles, launches per half-sweep,
+// n = 10: L = 520 77 copies 575 -> 380, 153 1033 -> 750; 3D L = 64 698 -> 459, 1299 -> 910.
 bool takes_stream_strips(const gbmc_ctx* ctx, const gbmc_lattice* l, const Tuning& tu, uint32_t n_sweeps, bool series) {
     if (ctx->launch_mode == GBMC_LAUNCH_GRID || !ctx->coop || n_sweeps > 0x3FFFFFFFu) return false;
     if (n_sweeps < 2 || (l->d.dim == 2 && l->d.L < 64)) return false;
     if (l->d.layout == GBMC_BITPACK) return l->ncopies <= (uint64_t)ctx->sm_count / 8;
     if (ctx->sweep_kernel == GBMC_KERNEL_BYTES || (l->d.dim == 3 && !l->stab)) return false;
-    if (!tu.resident) return series || n_sweeps >= 3 || l->N * l->ncopies >= 1u << 21;
+    if (!tu.resident) {
+        // Copies have whole multiprocessors to themselves here, and a batch of one per
+        // multiprocessor goes at a time; the halo tiles fill the device with any number.
+        const uint64_t c = l->ncopies, sms = (uint64_t)ctx->sm_count;
+        const double busy = (double)(c < sms ? sms / c * c : c) / (double)((c + sms - 1) / sms * sms);
+        if (l->d.dim == 2 && l->d.L % (int)kTile == 0 && !series && busy < 0.6) return false;
+        return series || n_sweeps >= 3 || l->N * l->ncopies >= 1u << 21;
+    }
     if (ctx->sweep_kernel != GBMC_KERNEL_AUTO || !tu.bits) return false;
     // words per plane, less where other copies keep their multiprocessors busy
     const double words = l->N / 64.0 * (1.0 - (double)l->ncopies / ctx->sm_count);
