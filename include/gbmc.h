@@ -89,8 +89,10 @@ gbmc_status gbmc_destroy(gbmc_ctx *ctx);
  * supports cooperative launches) runs the weights, ln Q / prefix sums,
  * multinomial draws and child placement in ONE launch: populations of up to
  * some ten thousand copies of all lattices together, a cluster of blocks each;
- * larger ones a cooperative launch with grid-wide barriers per lattice.
- * fused = 0 uses one launch per phase. All give identical results. */
+ * lattices with larger ones, or with more than some hundred, a cooperative launch
+ * with grid-wide barriers each. fused = 0 uses one launch per phase. All give the
+ * same populations and configurations; ln Q adds the same terms in another order
+ * (1e-12). */
 gbmc_status gbmc_set_resample_mode(gbmc_ctx *ctx, int32_t fused);
 
 /* Launch form of the shared-memory sweep kernel (Sec. 3.1 checkerboard sweeps

@@ -722,12 +722,17 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
     }
 }
 
-// The largest populations that a cluster resamples faster than the grid-wide kernel, whose
-// blocks are all of the chip's (us, one population, clusters : grid). Multinomial 20 000
-// copies 22 : 29, 40 000 33 : 30. Nearest integer 80 000 24 : 28. Poisson, bound by fp64 in a
-// cluster's few multiprocessors, 5000 27 : 49, 10 000 44 : 52, 20 000 77 : 54.
+// The populations that clusters resample faster than the grid-wide kernel, whose blocks are all
+// of the chip's (us, clusters : grid). One population: multinomial 20 000 copies 22 : 29, 40 000
+// 33 : 30. Nearest integer 80 000 24 : 28. Poisson, bound by fp64 in a cluster's few
+// multiprocessors, 5000 27 : 49, 10 000 44 : 52, 20 000 77 : 54. Many populations: some 34
+// clusters run at a time, 5 us for the smallest, where the grid-wide kernel has a block per
+// population: multinomial, 100 copies, 96, 128, 256, 1024 populations 20 : 26, 25 : 26, 45 : 26,
+// 155 : 48; 2000 copies, 128, 200, 256 34 : 39, 48 : 45, 59 : 50; 5000 copies, 256 90 : 99. Nearest
+// integer, 1000 copies, 96, 128 25 : 27, 31 : 27; 5000 copies, 200, 256 52 : 53, 65 : 61. Poisson,
+// 100 copies, 128, 256 47 : 54, 84 : 55; 2000 copies, 128, 200 137 : 138, 201 : 188.
 bool resample_in_clusters(const PaLattice& P) {
-    return P.R <= (P.nearest == 2 ? 8192u : P.nearest ? 65536u : 24576u);
+    return P.R <= (P.nearest == 2 ? 8192u : P.nearest ? 65536u : 24576u) && P.n_inst <= 100u + P.R / 40u;
 }
 
 cudaError_t launch_pa_resample_clusters(const PaLattice* jobs, double* const* lnZ, uint32_t njobs, cudaStream_t s) {
