@@ -109,8 +109,11 @@ __device__ __forceinline__ void nb2_rows(const uint32_t* oth, uint32_t w, uint32
     q0 = 8u * w;
 }
 
-// ROWS: every job has L <= 32 (words of several rows), else every job has L >= 64.
-template <bool ROWS>
+// ROWS: every job has L <= 32 (words of several rows), else every job has L >= 64. SUMS (several
+// copies per warp): annealing, whose populations' sums are reduced over the warp (record_copies); plain
+// sweeps and tempering go without that code (3D L = 8 tempering, 512 x 32 copies, 10 sweeps per round
+// 80.1 -> 78.1 us, 4096 x 16, one sweep 45.3 -> 43.3; annealing without it 1.05 -> 2.9 ms).
+template <bool ROWS, bool SUMS>
 __global__ void __launch_bounds__(128) k_sweep_bits2(const __grid_constant__ SweepLaunch P, uint32_t wpb,
                                                      uint32_t words_per_warp) {
     extern __shared__ __align__(16) uint32_t smw[];
@@ -219,8 +222,9 @@ __global__ void __launch_bounds__(128) k_sweep_bits2(const __grid_constant__ Swe
                 U += __shfl_xor_sync(0xffffffffu, U, o);
                 D += __shfl_xor_sync(0xffffffffu, D, o);
             }
-            if (ROWS) record_copies(J, active && li == 0, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
-            else if (li == 0) record_copy(J, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
+            if (SUMS) record_copies(J, active && li == 0, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
+            else if (active && li == 0)
+                record_copy(J, slot, inst, s, sweep, last, 2 * U - 2 * (int)N, (int)N - 2 * D);
         }
     }
 
@@ -264,7 +268,7 @@ __device__ __forceinline__ void nb3(uint32_t oth, uint32_t z, uint32_t colour, u
     nb[5] = __shfl_sync(0xffffffffu, oth, gbase | ((z + 1u) & 7u));
 }
 
-template <bool EA>
+template <bool EA, bool SUMS>
 __global__ void __launch_bounds__(128) k_sweep_bits3(const __grid_constant__ SweepLaunch P, uint32_t wpb) {
     __shared__ __align__(16) uint32_t stage[kBitsWarps][4][16];  // [warp][copy][plane * 8 + z]
     const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
@@ -351,7 +355,8 @@ __global__ void __launch_bounds__(128) k_sweep_bits3(const __grid_constant__ Swe
                 D += __shfl_xor_sync(0xffffffffu, D, o);
             }
             // E = 2 (unsatisfied bonds of the colour-0 sites) - 3 N
-            record_copies(J, active && z == 0, slot, inst, s, sweep, last, 2 * U - 3 * (int)N, (int)N - 2 * D);
+            if (SUMS) record_copies(J, active && z == 0, slot, inst, s, sweep, last, 2 * U - 3 * (int)N, (int)N - 2 * D);
+            else if (active && z == 0) record_copy(J, slot, inst, s, sweep, last, 2 * U - 3 * (int)N, (int)N - 2 * D);
         }
     }
 
@@ -621,8 +626,10 @@ static cudaError_t launch_bits_group(const SweepLaunch& P0, bool rows, cudaStrea
             P.jobs[b - 1] = t;
         }
     uint32_t total = 0, words = 0;
+    bool sums = false;
     for (int j = 0; j < P.njobs; ++j) {
         const SweepJob& J = P.jobs[j];
+        sums = sums || J.hist;
         if (!bits_supported(P.dim, (int)J.L)) return cudaErrorInvalidValue;
         P.cta_begin[j] = total;
         // 2D: one copy per warp, or 32 / (N / 64) copies when a plane has fewer
@@ -640,7 +647,7 @@ static cudaError_t launch_bits_group(const SweepLaunch& P0, bool rows, cudaStrea
     if (total == 0) return cudaSuccess;
     if (P.dim == 2) {
         const size_t smem = (size_t)kWarps * words * 4u;
-        auto kern = rows ? k_sweep_bits2<true> : k_sweep_bits2<false>;
+        auto kern = !rows ? k_sweep_bits2<false, false> : sums ? k_sweep_bits2<true, true> : k_sweep_bits2<true, false>;
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
@@ -649,10 +656,10 @@ static cudaError_t launch_bits_group(const SweepLaunch& P0, bool rows, cudaStrea
     } else if (P.jobs[0].L == 16) {
         if (P.ea) k_sweep_bits3w<true><<<total, 32u * kWarps, 0, s>>>(P, kWarps);
         else k_sweep_bits3w<false><<<total, 32u * kWarps, 0, s>>>(P, kWarps);
-    } else if (P.ea) {
-        k_sweep_bits3<true><<<total, 32u * kWarps, 0, s>>>(P, kWarps);
     } else {
-        k_sweep_bits3<false><<<total, 32u * kWarps, 0, s>>>(P, kWarps);
+        auto kern = P.ea ? (sums ? k_sweep_bits3<true, true> : k_sweep_bits3<true, false>)
+                         : (sums ? k_sweep_bits3<false, true> : k_sweep_bits3<false, false>);
+        kern<<<total, 32u * kWarps, 0, s>>>(P, kWarps);
     }
     count_launch();
     return cudaGetLastError();
