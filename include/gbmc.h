@@ -152,12 +152,14 @@ gbmc_status gbmc_set_sweep_launch(gbmc_ctx *ctx, int32_t mode);
 enum { GBMC_KERNEL_AUTO = 0, GBMC_KERNEL_BYTES = 1, GBMC_KERNEL_BITS = 2 };
 gbmc_status gbmc_set_sweep_kernel(gbmc_ctx *ctx, int32_t kernel);
 /* Test aid for the bounded waits: each grid barrier of the fused resampling
- * (with phantom arrivals, every population's resampling takes that form) waits for `phantom_arrivals` CTAs more than the launch has, and each
- * neighbour wait of the strip-resident sweeps for that many half-sweeps more
- * (so with 1 a wait can only end by running out of its budget); waits give up
+ * (with phantom arrivals, every population's resampling takes that form) waits for
+ * `phantom_arrivals` CTAs more than the launch has, each neighbour wait of the
+ * strip-resident sweeps for that many half-sweeps more, and the sweeps of few small
+ * copies, whose acceptance bits other warps draw ahead, for that many batches of bits
+ * more (so with 1 a wait can only end by running out of its budget); waits give up
  * after `budget_cycles` SM cycles (default 2e9). A wait that runs out makes the
- * kernel return early and the next synchronising call (gbmc_sync, pa_run,
- * pa_step with statistics) return GBMC_ERR_TIMEOUT; the context stays usable.
+ * kernel end early or with unset bits and the next synchronising call (gbmc_sync,
+ * pa_run, pa_step with statistics) return GBMC_ERR_TIMEOUT; the context stays usable.
  * Pass (0, 2000000000) to restore the defaults. */
 gbmc_status gbmc_test_barrier_wait(gbmc_ctx *ctx, uint32_t phantom_arrivals, uint64_t budget_cycles);
 /* Test aid for a full device: buffers of more than `bytes` that the library can do

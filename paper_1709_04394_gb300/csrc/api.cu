@@ -546,8 +546,10 @@ gbmc_status launch_jobs(gbmc_ctx* ctx, const SweepLaunch& P0, const std::vector<
     }
     if (S.njobs) {
         ProfScope ps_(ctx, PK_SWEEP_STREAM);
-        if (sweeps_ahead(S, ctx->sm_count)) CUDA_TRY(launch_sweep_ahead(S, ctx->words + 1, ctx->stream));
-        else CUDA_TRY(launch_sweep_stream(S, ctx->sm_count, ctx->stream));
+        if (sweeps_ahead(S, ctx->sm_count))
+            CUDA_TRY(launch_sweep_ahead(S, ctx->words + 1, ctx->budget, ctx->phantom, ctx->stream));
+        else
+            CUDA_TRY(launch_sweep_stream(S, ctx->sm_count, ctx->stream));
     }
     if (Y.njobs == 0) return GBMC_OK;
     return launch_bytes(ctx, Y, ty, force_persistent);

@@ -369,7 +369,8 @@ struct PtExchange {
 cudaError_t launch_pt_exchange(const PtExchange& X, cudaStream_t s);
 // Plain sweeps (series included) of few small copies, acceptance bits drawn ahead (stream.cu).
 bool sweeps_ahead(const SweepLaunch& P, int sm_count);
-cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, cudaStream_t s);
+cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, long long budget, uint32_t phantom,
+                               cudaStream_t s);
 // Rounds of sweeps (J.nsweeps each) and exchanges in one launch (stream.cu), and whether
 // that is the faster way for P's one job.
 bool tempering_in_rounds(const SweepLaunch& P, int sm_count);

@@ -721,7 +721,12 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
 // block per copy: its first warps (a thread per word) update, the other kDrawers warps draw
 // acceptance words ahead of them into a ring in shared memory, 32 words a batch,
 // whatever half-sweeps these belong to. A batch's flag says that its words are there;
-// `taken` counts the half-sweeps whose words have been read. Waits are bounded.
+// `taken` counts the half-sweeps whose words have been read. Drawers wait for room in the ring
+// `naps` times at most (the caller's budget of cycles), and an updater's batch comes once its
+// drawer has stopped waiting: a wait that runs out raises *err and ends all others. Test aid:
+// with `phantom` the flags are that many batches behind, and the drawers see to it at the end that
+// nobody waits for what will not come. (Bounds in the updaters' own loop cost the chain: by the
+// clock 2D L = 16 1148 -> 1171 us, L = 64 966 -> 1041; theirs is a count far above any budget.)
 //
 // Bound: the chain of a half-sweep (words and masks loaded, some 25 dependent
 // instructions, word stored, barrier); from some 64 words per plane the drawers' integer pipes.
@@ -732,15 +737,19 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
 constexpr uint32_t kDrawers = 12, kAheadThreads = 512;
 constexpr uint32_t kAheadWords = 32u * (kAheadThreads / 32u - kDrawers);  // words per plane, at most
 constexpr uint32_t kAheadPolls = 1u << 26;
+constexpr uint32_t kNapCycles = 512u;  // a look at `taken` and a sleep of 200 ns, about
 
-__host__ __device__ __forceinline__ uint32_t ahead_ring(uint32_t PW) {  // items, a power of two, several half-sweeps
+// items, a power of two, several half-sweeps: 1024 for all sizes taken (as a constant in the
+// kernel 1 to 6 % slower)
+__host__ __device__ __forceinline__ uint32_t ahead_ring(uint32_t PW) {
     uint32_t n = 1024u;
     while (n < 8u * PW) n <<= 1;
     return n;
 }
 
 template <int DIM, bool EA>
-__global__ void __launch_bounds__(kAheadThreads, 1) k_sweep_ahead(const __grid_constant__ SweepLaunch P, unsigned int* err) {
+__global__ void __launch_bounds__(kAheadThreads, 1)
+    k_sweep_ahead(const __grid_constant__ SweepLaunch P, unsigned int* err, uint32_t naps, uint32_t phantom) {
     extern __shared__ __align__(16) uint32_t smw[];
     __shared__ uint32_t taken, dead;  // dead: a wait ran out, nothing waits any more
     __shared__ int acc[2][2];
@@ -804,7 +813,7 @@ __global__ void __launch_bounds__(kAheadThreads, 1) k_sweep_ahead(const __grid_c
             // (asleep between looks: drawers far ahead would take the updaters' issue slots)
             for (uint32_t n = 0; last >= (uint64_t)*vtaken * g.PW + ring && !*vdead; ++n) {
                 __nanosleep(200);
-                if (n == kAheadPolls / 64u) give_up();
+                if (n == naps) give_up();
             }
             const uint32_t h = (uint32_t)(i / g.PW), w = (uint32_t)(i - (uint64_t)h * g.PW);
             const PhiloxFixed pf = philox_fix(J.t0 + (h >> 1), r, c3_word(kPurposeMetro, h & 1u, J.inst_base + inst), k0, k1);
@@ -829,8 +838,14 @@ __global__ void __launch_bounds__(kAheadThreads, 1) k_sweep_ahead(const __grid_c
             if constexpr (DIM == 3) m12[at] = __brev(r12);
             __threadfence_block();
             __syncwarp();
-            if (lane == 0u) *(volatile uint32_t*)(flag + ((uint32_t)b & (ring / 32u - 1u))) = (uint32_t)b + 1u;
+            if (lane == 0u) *(volatile uint32_t*)(flag + ((uint32_t)b & (ring / 32u - 1u))) = (uint32_t)b + 1u - phantom;
         }
+        if (phantom && lane == 0u)  // no more batches: what the updaters still wait for will not come
+            for (uint32_t n = 0; *vtaken <= n_half && !*vdead; ++n) {
+                __nanosleep(200);
+                if (n == naps) give_up();
+            }
+        __syncwarp();
     } else if (!spared) {
         const uint32_t w = min(tid, g.PW - 1u);
         const bool has = tid < g.PW;
@@ -1262,12 +1277,14 @@ bool sweeps_ahead(const SweepLaunch& P, int sm_count) {
            J.src == J.dst;
 }
 
-cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, cudaStream_t s) {
+cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, long long budget, uint32_t phantom,
+                               cudaStream_t s) {
     const SweepJob& J = P.jobs[0];
     const uint32_t PW = (J.N / 2u + 31u) / 32u, ring = ahead_ring(PW), Wc = (PW + 31u) / 32u;
     const size_t smem = 4ull * (2u * (PW + 1u) + (P.dim == 3 ? 3u : 2u) * ring + ring / 32u);
     auto kern = P.dim == 2 ? k_sweep_ahead<2, false> : P.ea ? k_sweep_ahead<3, true> : k_sweep_ahead<3, false>;
-    kern<<<J.n_inst * J.R, 32u * (Wc == 1u ? 12u : Wc + kDrawers), smem, s>>>(P, err);
+    const uint32_t naps = (uint32_t)std::min<long long>(budget / kNapCycles, 0x7FFFFFFF);
+    kern<<<J.n_inst * J.R, 32u * (Wc == 1u ? 12u : Wc + kDrawers), smem, s>>>(P, err, naps, phantom);
     count_launch();
     return cudaGetLastError();
 }
