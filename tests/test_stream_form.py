@@ -24,3 +24,19 @@ def test_a_large_copys_job_counts_among_others(big, small):
     assert many.cycles > 20 * few.cycles
     # no form is taken whose estimate leaves the job out: together they cost what the large one alone does
     assert few.cycles > 0.6 * form((*big, 200)).cycles
+
+
+@pytest.mark.parametrize("copies,expected", [
+    ((2, 40, 1, 201), (1, 4, 128)), ((2, 24, 1, 1513), (1, 2, 32)), ((2, 24, 1, 9001), (1, 1, 32)),
+    ((2, 96, 1, 2161), (2, 1, 160)), ((2, 12, 1, 70001), (4, 1, 32)), ((3, 10, 3, 6603), (4, 1, 32)),
+    ((3, 4, 7, 44491), (2, 1, 32)), ((3, 14, 1, 201), (1, 2, 96)), ((2, 204, 1, 481), (1, 1, 672)),
+])
+def test_one_lattice_from_few_copies_to_many(copies, expected):
+    f = form(copies)
+    assert (f.copies_per_thread, f.threads_per_word, f.team[0]) == expected
+
+
+def test_sizes_annealed_together_share_the_device():
+    # teams of one warp for all, two copies per thread, largest lattice first
+    f = form((2, 24, 1, 20000), (2, 40, 1, 10000), (2, 96, 1, 4000))
+    assert (f.copies_per_thread, f.threads_per_word, list(f.team[:3]), list(f.groups[:3])) == (2, 1, [32] * 3, [1, 1, 3])
