@@ -426,11 +426,11 @@ __global__ void __launch_bounds__(256) k_sw_cross(const __grid_constant__ SwLaun
     uint32_t a, b;
     if (P.lab) {
         const uint16_t* lab = P.lab + copy * P.N;
-        a = sw_tile_root(lab[i], i, L);
-        b = sw_tile_root(lab[j], j, L);
+        a = sw_tile_root(lab[GBMC_IDX(i, P.N)], i, L);
+        b = sw_tile_root(lab[GBMC_IDX(j, P.N)], j, L);
     } else {
-        a = __ldcg(par + i);
-        b = __ldcg(par + j);
+        a = __ldcg(par + GBMC_IDX(i, P.N));
+        b = __ldcg(par + GBMC_IDX(j, P.N));
     }
     const bool active = in && sw_bond_active(P, s, i, j, mu, r, c3_word(kPurposeSwBond, 0u, P.inst_base + inst));
     const uint32_t mask = __ballot_sync(0xffffffffu, active);
@@ -687,13 +687,13 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
     const uint32_t lane = threadIdx.x & 31u;
     // quotients by L: exact, as the numerators times L stay below 2^32
     const uint32_t inv = 0xFFFFFFFFu / L + 1u;
-    auto nibble_of = [&](const uint32_t* m, uint32_t q) { return (m[q >> 3] >> (4u * (q & 7u))) & 15u; };
+    auto nibble_of = [&](const uint32_t* m, uint32_t q) { return (m[GBMC_IDX(q >> 3, W)] >> (4u * (q & 7u))) & 15u; };
     // the nibbles of eight lanes to a word of m, nq quads in all (whole warps; q: the lane's)
     auto store = [&](uint32_t* m, uint32_t q, uint32_t nq, uint32_t nibble) {
         uint32_t v = q < nq ? nibble << (4u * (lane & 7u)) : 0u;
 #pragma unroll
         for (uint32_t o = 1; o < 8u; o <<= 1) v |= __shfl_xor_sync(kAll, v, o);
-        if ((lane & 7u) == 0u && q < nq) m[q >> 3] = v;
+        if ((lane & 7u) == 0u && q < nq) m[GBMC_IDX(q >> 3, W)] = v;
     };
     const uint32_t T = blockDim.x, Qr = (Q + 1u + 31u) & ~31u;  // whole warps over the quads and one more
     for (uint32_t q = threadIdx.x; q < Qr; q += T) {
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
                 const uint32_t i0 = 4u * q, row = __umulhi(i0, inv), x = i0 - row * L;
                 auto window = [&](uint32_t p) {  // four bits of the spins from site p (cyclic)
                     p = p >= N ? p - N : p;
-                    return __funnelshift_r(spin[p >> 5], spin[(p >> 5) + 1u], p & 31u);
+                    return __funnelshift_r(spin[GBMC_IDX(p >> 5, W)], spin[GBMC_IDX((p >> 5) + 1u, W)], p & 31u);
                 };
                 const uint32_t at = window(i0), own = at & 15u;
                 uint32_t dif[DIM];
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
         }
         __syncthreads();
         if (measure && threadIdx.x == 0u) {
-            const uint64_t to = (uint64_t)(u - 1u) * copies + copy;
+            const uint64_t to = GBMC_IDX((uint64_t)(u - 1u) * copies + copy, n_updates * copies);
             if (E_series) E_series[to] = 2 * red[0] - (int)(DIM * N);
             if (M_series) M_series[to] = (int)N - 2 * red[1];
             red[0] = red[1] = 0;  // next added to after two barriers
@@ -793,7 +793,7 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
             v.y = (joined & 1u) ? v.x : i0 + 1u;
             v.z = (joined & 2u) ? v.y : i0 + 2u;
             v.w = (joined & 4u) ? v.z : i0 + 3u;
-            *reinterpret_cast<uint4*>(f + i0) = v;
+            *reinterpret_cast<uint4*>(f + GBMC_IDX(i0, N - 3u)) = v;
         }
         __syncthreads();
         for (;;) {
@@ -801,9 +801,10 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
             for (uint32_t q = threadIdx.x; q < Qr; q += T) {
                 const uint32_t i0 = 4u * q;
                 uint32_t on[DIM], any = 0u;
-                on[0] = nibble_of(around, q);
+                const uint32_t qm = min(q, Q);  // (the masks end there)
+                on[0] = nibble_of(around, qm);
 #pragma unroll
-                for (uint32_t mu = 1; mu < DIM; ++mu) on[mu] = nibble_of(along + (mu - 1u) * W, q);
+                for (uint32_t mu = 1; mu < DIM; ++mu) on[mu] = nibble_of(along + (mu - 1u) * W, qm);
 #pragma unroll
                 for (uint32_t mu = 0; mu < DIM; ++mu) {
                     if (q >= Q) on[mu] = 0u;
@@ -825,12 +826,12 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
                         uint32_t lo[4], hi[4], now[4];
 #pragma unroll
                         for (uint32_t n = 0; n < 4u; ++n) {
-                            const uint32_t b = (on[mu] >> n) & 1u ? vf[far[n]] : own[n];
+                            const uint32_t b = (on[mu] >> n) & 1u ? vf[GBMC_IDX(far[n], N)] : own[n];
                             lo[n] = min(own[n], b);
                             hi[n] = max(own[n], b);
                         }
 #pragma unroll
-                        for (uint32_t n = 0; n < 4u; ++n) now[n] = vf[hi[n]];
+                        for (uint32_t n = 0; n < 4u; ++n) now[n] = vf[GBMC_IDX(hi[n], N)];
 #pragma unroll
                         for (uint32_t n = 0; n < 4u; ++n) {
                             if (lo[n] == hi[n]) done[mu] |= on[mu] & (1u << n);
@@ -869,7 +870,8 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
                 uint32_t a0 = l[0], a1 = l[1], a2 = l[2], a3 = l[3];
                 for (;;) {  // every label follows its own, and is itself what others follow
                     volatile uint32_t* vf = f;
-                    const uint32_t b0 = vf[a0], b1 = vf[a1], b2 = vf[a2], b3 = vf[a3];
+                    const uint32_t b0 = vf[GBMC_IDX(a0, N)], b1 = vf[GBMC_IDX(a1, N)], b2 = vf[GBMC_IDX(a2, N)],
+                                   b3 = vf[GBMC_IDX(a3, N)];
                     if (b0 == a0 && b1 == a1 && b2 == a2 && b3 == a3) break;
                     l[0] = a0 = b0, l[1] = a1 = b1, l[2] = a2 = b2, l[3] = a3 = b3;
                 }
@@ -895,7 +897,7 @@ __global__ void __launch_bounds__(1024, 1) k_sw_resident(const __grid_constant__
             if (q <= Q) {
                 const uint32_t from = q < Q ? q : 0u;  // (the first quad again behind the last)
                 const uint4 v = *reinterpret_cast<const uint4*>(f + 4u * from);
-                auto up = [&](uint32_t root) { return (coin[root >> 5] >> (root & 31u)) & 1u; };
+                auto up = [&](uint32_t root) { return (coin[GBMC_IDX(root >> 5, W)] >> (root & 31u)) & 1u; };
                 now = up(v.x) | up(v.y) << 1 | up(v.z) << 2 | up(v.w) << 3;
                 if (named && q < Q) {
                     int32_t* to = P.labels + copy * N + 4u * q;
