@@ -5,6 +5,7 @@
 #include <climits>
 #include <cstdint>
 
+#include "check.cuh"
 #include "device.cuh"
 #include "internal.h"
 
@@ -34,7 +35,7 @@ __device__ __forceinline__ void record_copy(const SweepJob& J, uint64_t slot, ui
     if (J.E) J.E[slot] = E;
     if (J.M) J.M[slot] = M;
     if (J.hist) {
-        atomicAdd(&J.hist[(uint64_t)inst * J.nbins + (uint32_t)((E - J.e_lo) >> 2)], 1u);
+        atomicAdd(&J.hist[(uint64_t)inst * J.nbins + GBMC_IDX((uint32_t)((E - J.e_lo) >> 2), J.nbins)], 1u);
         atomicMin(&J.emin[inst], E);
         atomicMax(&J.emax[inst], E);
         unsigned long long* su = J.sums + (uint64_t)inst * 4;
@@ -73,7 +74,7 @@ __device__ __forceinline__ void record_copies(const SweepJob& J, bool has, uint6
         if (J.Mser && sweep) J.Mser[(uint64_t)s * ncopies + slot] = M;
         if (J.E) J.E[slot] = E;
         if (J.M) J.M[slot] = M;
-        atomicAdd(&J.hist[(uint64_t)inst * J.nbins + (uint32_t)((E - J.e_lo) >> 2)], 1u);
+        atomicAdd(&J.hist[(uint64_t)inst * J.nbins + GBMC_IDX((uint32_t)((E - J.e_lo) >> 2), J.nbins)], 1u);
     }
     const int mn = __reduce_min_sync(kAll, has ? E : INT_MAX), mx = __reduce_max_sync(kAll, has ? E : INT_MIN);
     // copies held on chip have fewer than 2^18 sites: |E| < 2^20, squares below

@@ -636,14 +636,14 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
             uint32_t bin[4];
             unsigned long long w[4];
 #pragma unroll
-            for (uint32_t k = 0; k < 4u; ++k) bin[k] = (uint32_t)(E[min(i + k, i1 - 1u)] - emin) >> 2;
+            for (uint32_t k = 0; k < 4u; ++k) bin[k] = (uint32_t)(E[GBMC_IDX(min(i + k, i1 - 1u), n)] - emin) >> 2;
 #pragma unroll
             for (uint32_t k = 0; k < 4u; ++k) w[k] = P.wint[GBMC_IDX(bin[k], P.nbins)];
 #pragma unroll
             for (uint32_t k = 0; k < 4u; ++k)
                 if (i + k < i1) {
                     run += w[k];
-                    cum[i + k] = run;
+                    cum[GBMC_IDX(i + k, A.slice)] = run;
                     cnt[i + k] = 0u;
                 }
         }
@@ -673,11 +673,11 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
         auto look_up = [&](uint32_t first, uint32_t count) {
             __syncwarp();
             if (lane < count) {
-                const unsigned long long xr = mine[first + lane];
+                const unsigned long long xr = mine[GBMC_IDX(first + lane, 64u)];
                 uint32_t pos = 0;  // the sums that do not exceed x
                 for (uint32_t step = top; step; step >>= 1)
                     if (pos + step <= n && cum[pos + step - 1u] <= xr) pos += step;
-                atomicAdd(cnt + pos, 1u);
+                atomicAdd(cnt + GBMC_IDX(pos, n), 1u);
             }
             __syncwarp();
         };
@@ -689,7 +689,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
                 const unsigned long long xr = __umul64hi(U[e], C) - lo;
                 const bool hit = 2u * (p0 + lane) + e < live && xr < span;
                 const uint32_t hits = __ballot_sync(~0u, hit);
-                if (hit) mine[kept + __popc(hits & below)] = xr;
+                if (hit) mine[GBMC_IDX(kept + __popc(hits & below), 64u)] = xr;
                 kept += __popc(hits);
                 if (kept >= 32u) {
                     kept -= 32u;
@@ -702,7 +702,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) k_pa_resample_clusters(const 
     } else {
         for (uint32_t i = threadIdx.x; i < n; i += kScanThreads) {
             const unsigned long long W = cum[i] - (i ? cum[i - 1u] : 0ull);
-            cnt[i] = P.nearest == 2 ? poisson_copies(P, inst, j0 + i, W, C) : nearest_copies(P, inst, j0 + i, W, C);
+            cnt[GBMC_IDX(i, A.slice)] = P.nearest == 2 ? poisson_copies(P, inst, j0 + i, W, C) : nearest_copies(P, inst, j0 + i, W, C);
         }
         __syncthreads();
     }

@@ -24,6 +24,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include "check.cuh"
 #include "device.cuh"
 #include "internal.h"
 
@@ -155,7 +156,7 @@ __device__ double overlap_fast(SchedBins* S, uint32_t n, double d, float2* sf) {
     __syncthreads();
     // a thread's bins as in overlap_eval; the weights are worked out again in the second
     // pass, for less than keeping them would take
-    auto weight = [&](uint32_t i) { return pair_mul(S->hf[i], pair_mul(S->coarse[i >> 5], S->fine[i & 31u])); };
+    auto weight = [&](uint32_t i) { return pair_mul(S->hf[i], pair_mul(S->coarse[GBMC_IDX(i >> 5, kSchedBins / 32u)], S->fine[i & 31u])); };
     float2 w = make_float2(0.0f, 0.0f);
     for (uint32_t i = t; i < n; i += kSchedThreads) w = pair_add(w, weight(i));
     w = pair_warp_sum(w);
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const __grid_constan
     if (reporter || propose) {
         double s1 = 0.0;
         for (uint32_t b = bmin + threadIdx.x; b <= bmax; b += blockDim.x)
-            s1 += (double)J.hist[b] * 4.0 * (double)(b - bmin);
+            s1 += (double)J.hist[GBMC_IDX(b, J.nbins)] * 4.0 * (double)(b - bmin);
         const double m1 = block_sum_d(s1, sh) / R;
         double s2 = 0.0, s3 = 0.0;
         for (uint32_t b = bmin + threadIdx.x; b <= bmax; b += blockDim.x) {
@@ -265,8 +266,8 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const __grid_constan
     SchedBins* bins = bmax - bmin < kSchedBins ? reinterpret_cast<SchedBins*>(raw) : nullptr;
     if (bins)  // each thread reads back only its own bins
         for (uint32_t b = bmin + threadIdx.x; b <= bmax; b += blockDim.x) {
-            const double hb = (double)J.hist[b], p0 = hb / R;
-            bins->h[b - bmin] = hb;
+            const double hb = (double)J.hist[GBMC_IDX(b, J.nbins)], p0 = hb / R;
+            bins->h[GBMC_IDX(b - bmin, kSchedBins)] = hb;
             bins->p0[b - bmin] = p0;
             bins->hf[b - bmin] = pair_of(hb);
             bins->pf[b - bmin] = pair_of(p0);

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(stream_max_threads(C, S, PT), stream_min_block
                 const uint32_t w = at.w;
                 Words<C>* own = reinterpret_cast<Words<C>*>(sm + colour * plane + gi * g.PWX * C);
                 const Words<C>* oth = reinterpret_cast<const Words<C>*>(sm + (colour ^ 1u) * plane + gi * g.PWX * C);
-                Words<C> nw = own[w];
+                Words<C> nw = own[GBMC_IDX(w, g.PWX)];
                 uint32_t ge[C], ea[C], eb[C];  // dE <= 0; dE = 4; dE = 8 (3D)
                 {
                     uint32_t d[2 * DIM][C], j[2 * DIM];
@@ -788,7 +788,7 @@ __global__ void __launch_bounds__(kAheadThreads, 1)
         pack8(v.x, v.y, e0, o0);
         pack8(v.z, v.w, e1, o1);
         const uint32_t ev = e0 | (e1 << 4), od = o0 | (o1 << 4), m = odd_b[ch];
-        uint8_t* p0 = reinterpret_cast<uint8_t*>(smw) + ch;
+        uint8_t* p0 = reinterpret_cast<uint8_t*>(smw) + GBMC_IDX(ch, 4u * g.PWX);
         p0[0] = (uint8_t)sel(m, od, ev);
         p0[4u * g.PWX] = (uint8_t)sel(m, ev, od);
     }
@@ -833,12 +833,12 @@ __global__ void __launch_bounds__(kAheadThreads, 1)
                     accept_bits3(r4, r8, r12, J.thr[0], J.thr[1], J.thr[2], v.w);
                 }
             }
-            const uint32_t at = (uint32_t)i & (ring - 1u);
+            const uint32_t at = (uint32_t)GBMC_IDX((uint32_t)i & (ring - 1u), ring);
             m48[at] = make_uint2(__brev(r4), __brev(r8));
             if constexpr (DIM == 3) m12[at] = __brev(r12);
             __threadfence_block();
             __syncwarp();
-            if (lane == 0u) *(volatile uint32_t*)(flag + ((uint32_t)b & (ring / 32u - 1u))) = (uint32_t)b + 1u - phantom;
+            if (lane == 0u) *(volatile uint32_t*)(flag + GBMC_IDX((uint32_t)b & (ring / 32u - 1u), ring / 32u)) = (uint32_t)b + 1u - phantom;
         }
         if (phantom && lane == 0u)  // no more batches: what the updaters still wait for will not come
             for (uint32_t n = 0; *vtaken <= n_half && !*vdead; ++n) {
@@ -866,13 +866,13 @@ __global__ void __launch_bounds__(kAheadThreads, 1)
             const uint64_t i = (uint64_t)h * g.PW + w;
             if (i >= known) {
                 const uint32_t b = (uint32_t)(i >> 5);
-                volatile uint32_t* f = flag + (b & (ring / 32u - 1u));
+                volatile uint32_t* f = flag + GBMC_IDX(b & (ring / 32u - 1u), ring / 32u);
                 for (uint32_t n = 0; *f != b + 1u && !*vdead; ++n)
                     if (n == kAheadPolls) give_up();
                 __threadfence_block();
                 known = (uint64_t)(b + 1u) << 5;
             }
-            const uint32_t k = (uint32_t)i & (ring - 1u);
+            const uint32_t k = (uint32_t)GBMC_IDX((uint32_t)i & (ring - 1u), ring);
             const uint2 m = m48[k];
             a4 = m.x;
             a8 = m.y;
@@ -881,8 +881,8 @@ __global__ void __launch_bounds__(kAheadThreads, 1)
         const bool series = J.Eser || J.Mser;
         const uint64_t ncopies = (uint64_t)J.n_inst * J.R;
         auto write = [&](uint32_t s, int U, int D) {  // every bond has one colour-0 end
-            if (J.Eser) J.Eser[s * ncopies + slot] = 2 * U - DIM * (int)J.N;
-            if (J.Mser) J.Mser[s * ncopies + slot] = (int)J.N - 2 * D;
+            if (J.Eser) J.Eser[GBMC_IDX(s * ncopies + slot, J.nsweeps * ncopies)] = 2 * U - DIM * (int)J.N;
+            if (J.Mser) J.Mser[GBMC_IDX(s * ncopies + slot, J.nsweeps * ncopies)] = (int)J.N - 2 * D;
         };
         if (n_half) fetch(0u);
         auto half = [&](auto colour, uint32_t h) {
@@ -890,7 +890,7 @@ __global__ void __launch_bounds__(kAheadThreads, 1)
             const bool update = h < n_half, measure = c == 0u && series && h > 0u;
             uint32_t* const own = smw + c * g.PWX;
             const Words<1>* oth = reinterpret_cast<const Words<1>*>(smw + (c ^ 1u) * g.PWX);
-            Words<1> nw = {{own[w]}}, same;
+            Words<1> nw = {{own[GBMC_IDX(w, g.PWX)]}}, same;
             uint32_t d[2 * DIM][1], j[2 * DIM];
 #pragma unroll
             for (int k = 0; k < 2 * DIM; ++k) j[k] = EA ? jb[c][k] : 0u;
@@ -959,7 +959,7 @@ __global__ void __launch_bounds__(kAheadThreads, 1)
     }
     __syncthreads();
     for (uint32_t ch = tid; ch < nch; ch += T) {
-        const uint8_t* p0 = reinterpret_cast<const uint8_t*>(smw) + ch;
+        const uint8_t* p0 = reinterpret_cast<const uint8_t*>(smw) + GBMC_IDX(ch, 4u * g.PWX);
         const uint32_t a = p0[0], b = p0[4u * g.PWX], m = odd_b[ch];
         const uint32_t ev = sel(m, b, a), od = sel(m, a, b);
         const uint2 lo = unpack8(ev & 15u, od & 15u), hi = unpack8(ev >> 4, od >> 4);

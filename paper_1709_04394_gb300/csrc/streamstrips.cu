@@ -29,6 +29,7 @@
 // Bound: for small lattices the chain of a half-sweep -- words loaded from L2,
 // update, words stored --, for larger ones the integer pipes (stream.cu).
 #include "bits.cuh"
+#include "check.cuh"
 #include "device.cuh"
 #include "internal.h"
 
@@ -81,11 +82,11 @@ __device__ __forceinline__ uint64_t shared_word(const uint64_t* p) {
 template <bool HELD>
 struct Plane {
     const uint64_t *w, *run;
-    uint32_t first, count, tag;
+    uint32_t first, count, words, tag;
     __device__ __forceinline__ uint32_t word(uint32_t i) {
         uint64_t x;
         if (HELD && i - first < count) x = shared_word(run + (i - first));
-        else asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(w + i) : "memory");
+        else asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(w + GBMC_IDX(i, words)) : "memory");
         tag = min(tag, (uint32_t)(x >> 32));
         return (uint32_t)x;
     }
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
     extern __shared__ __align__(16) uint64_t runs[];
     if constexpr (HELD) {
         for (uint32_t i = tid; i < 2u * n_words; i += T)
-            runs[i] = planes[(uint64_t)(i / n_words) * g.PW + w0 + i % n_words];
+            runs[i] = planes[GBMC_IDX((uint64_t)(i / n_words) * g.PW + w0 + i % n_words, 2u * g.PW)];
         __syncthreads();
     }
     // words near an end of the run come first: n_edge of them on either side
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
             if constexpr (DIM == 2) {
                 row_masks(g, w, c, odd, edge);
             } else {
-                odd = __ldg(P.mask + w) ^ (c ? 0xFFFFFFFFu : 0u);
+                odd = __ldg(P.mask + GBMC_IDX(w, g.PW)) ^ (c ? 0xFFFFFFFFu : 0u);
                 edge = __ldg(P.mask + (1u + c) * g.PW + w);
                 y0 = __ldg(P.mask + 3u * g.PW + w);
                 yl = __ldg(P.mask + 4u * g.PW + w);
@@ -188,8 +189,8 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
             // half-sweep h - 1 (tag h) and this word's own h - 2
             uint32_t s0, same, prv, nxt, up, up1, dn1, dn, ya = 0u, yb = 0u, za = 0u, zb = 0u, tag_me, tag_oth;
             auto look = [&]() {
-                Plane<HELD> me{own, runs + c * n_words, w0, n_words, 0xFFFFFFFFu};
-                Plane<HELD> oth{planes + (c ^ 1u) * g.PW, runs + (c ^ 1u) * n_words, w0, n_words, 0xFFFFFFFFu};
+                Plane<HELD> me{own, runs + c * n_words, w0, n_words, g.PW, 0xFFFFFFFFu};
+                Plane<HELD> oth{planes + (c ^ 1u) * g.PW, runs + (c ^ 1u) * n_words, w0, n_words, g.PW, 0xFFFFFFFFu};
                 s0 = me.word(w);
                 same = oth.word(w);
                 prv = oth.word(w ? w - 1u : 0u);
@@ -289,12 +290,13 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
                 const uint64_t out = (uint64_t)(h + 1u) << 32 | v;
                 if (HELD)
                     asm volatile("st.relaxed.cta.shared.u64 [%0], %1;" ::"r"(
-                                     (uint32_t)__cvta_generic_to_shared(runs + c * n_words + (w - w0))),
+                                     (uint32_t)__cvta_generic_to_shared(runs + GBMC_IDX(c * n_words + (w - w0), 2u * n_words))),
                                  "l"(out)
                                  : "memory");
                 // other CTAs read the run's ends, the caller what is there at the end
                 if (!HELD || x < n_first || h + 2u >= P.n_half)
-                    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(own + w), "l"(out) : "memory");
+                    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(own + GBMC_IDX(w, g.PW)), "l"(out)
+                                 : "memory");
             }
         }
         if (measure) {
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(S == 4 ? 512 : kStripMaxThreads, 1) k_stream_s
             }
             if (__syncthreads_or(dead)) return;
             if (tid == 0) {  // E = 2 U - DIM N, M = N - 2 D: the constants are there already
-                const uint64_t at = (uint64_t)((h >> 1) - 1u) * P.ncopies + copy;
+                const uint64_t at = GBMC_IDX((uint64_t)((h >> 1) - 1u) * P.ncopies + copy, P.n_half / 2u * P.ncopies);
                 if (P.Eser) atomicAdd(P.Eser + at, 2 * a[0]);
                 if (P.Mser) atomicAdd(P.Mser + at, -2 * a[1]);
                 a[0] = a[1] = 0;  // next added to two sweeps later, a block barrier in between
@@ -340,11 +342,11 @@ __global__ void __launch_bounds__(256) k_stream_convert(int8_t* spins, uint64_t*
         } else {
             m = reinterpret_cast<const uint8_t*>(mask)[ch];
         }
-        uint64_t* const w0 = P + copy * 2u * g.PW + (ch >> 2);
+        uint64_t* const w0 = P + GBMC_IDX(copy * 2u * g.PW + (ch >> 2), copies * 2u * g.PW - g.PW);
         uint64_t* const w1 = w0 + g.PW;
         uint8_t* p0 = reinterpret_cast<uint8_t*>(w0) + (ch & 3u);
         uint8_t* p1 = reinterpret_cast<uint8_t*>(w1) + (ch & 3u);
-        int8_t* site = spins + copy * N + 16ull * ch;
+        int8_t* site = spins + GBMC_IDX(copy * N + 16ull * ch, copies * N);
         uint32_t* s4 = reinterpret_cast<uint32_t*>(site);
         if constexpr (PACK) {
             uint4 v;
