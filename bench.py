@@ -793,6 +793,8 @@ def kernel_name(w, prof):
         if w.get("msc"):
             return "sweep_msc"
         return next((k for k in ("sweep_bits", "pt_rounds", "sweep_stream") if k in prof), "sweep_resident")
+    if "stream_strips" in prof:  # either layout
+        return "stream_strips"
     if w.get("layout", 0) == 1 or "bitpack_strips" in prof:
         # int8 lattices too: their strip sweeps run packed to bits
         return "bitpack_strips" if "bitpack_strips" in prof else "bitpack_halfsweep"
@@ -833,7 +835,13 @@ def alg_bytes_per_update(w, kname):
         tot_bytes = sum(copies(l) * (2 * l[1] ** l[0] + 12) for l in lat)
         return tot_bytes / (tot_upd * w["theta"])
     if w["kind"] == "pt":
-        return 2.0 / w["theta"]
+        # the copies read and written once per launch: of a round, or of the rounds of one
+        # launch (at most 2^13 sweeps and 2^34 updates)
+        rounds = 1
+        if kname == "pt_rounds":
+            per_round = site_updates_per_step(w) // w["rounds"]
+            rounds = max(1, min(w["rounds"], 2 ** 34 // per_round, 8192 // w["theta"]))
+        return 2.0 / (w["theta"] * rounds)
     if w.get("sw"):
         return float(SW_BYTES_PER_SITE)
     if "dcb" in w:
@@ -847,6 +855,8 @@ def alg_bytes_per_update(w, kname):
         return ((tile + 16) ** 2 + tile ** 2) / tile ** 2 / k   # window in, tile out, per k sweeps
     if kname == "sweep_strips":
         return 2.0 / w["sweeps"]                               # the int8 lattice read and written once per call
+    if kname == "stream_strips":
+        return 0.5 / w["sweeps"]                               # bit words and tags, read and written once per call
     if kname == "bitpack_strips":
         return 0.25 / w["sweeps"]                              # the packed lattice read and written once per call
     if kname == "bitpack_halfsweep":
