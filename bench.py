@@ -14,7 +14,8 @@ double-checkerboard rounds with k = 10 sweeps per 64 x 64 tile load),
 pa-ea3d-L8 (3D +-J spin glass, 32 instances), pa-mixed-2d (four lattice sizes
 in one launch) and pa-learned (time to |dF| <= 1e-4 with the learned schedule).
 
-Prints one JSON line (rank 0). --impl reference times the CPU oracle on a
+Prints one JSON line of about 2 KB (rank 0); --record PATH writes the whole record, with
+per-kernel times and the secondary records, to a file. --impl reference times the CPU oracle on a
 bounded sample of the same workload instead.
 """
 from __future__ import annotations
@@ -676,6 +677,9 @@ def main():
     ap.add_argument("--no-secondary", action="store_true",
                     help="default workload only: skip the secondary records (configs 2, 4 and the single-seed "
                          "learned-schedule comparison)")
+    ap.add_argument("--record", default=None, metavar="PATH",
+                    help="write the whole record (per-kernel times, secondary records, clocks) to this file; the "
+                         "printed line holds its main numbers")
     ap.add_argument("--learned-seeds", type=int, default=3)
     ap.add_argument("--mlp-band", type=float, nargs=2, default=None,
                     help="pa-learned: overlap band [lo, hi] in which an MLP proposal is kept (default 0.80 0.90)")
@@ -764,7 +768,29 @@ def main():
                               "independent runs)" % (na, na)}
             except Exception as ex:  # a host without working process pools still gets its line
                 line["cpu_baseline"]["all_cores"] = {"unavailable": "%s: %s" % (type(ex).__name__, ex)}
-    print(json.dumps(line))
+    if args.record:
+        with open(args.record, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(printed_line(line)))
+
+
+def printed_line(line):
+    """What is printed of a record: the contract's keys and one number of each part, about 2 KB, as
+    readers of the output may keep only its end. --record writes all of it to a file."""
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "gpu_launches", "config")}
+    out["e2e"] = {k: line["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")}
+    out["clocks"] = {k: line["clocks"].get(k) for k in ("sm_mhz", "sm_max_mhz", "reasons")}
+    out["roofline"] = {k: line["roofline"][k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                                                        "hbm_frac", "kernel_share")}
+    if "cpu_baseline" in line:
+        c = line["cpu_baseline"]
+        out["cpu_baseline"] = {k: c[k] for k in ("value", "unit", "cores", "kind")}
+        if "value" in c.get("all_cores", {}):
+            out["cpu_baseline"]["all_cores"] = {k: c["all_cores"][k] for k in ("value", "cores")}
+    if "secondary" in line:  # spin-flips/ns; the learned schedule: seconds to the target accuracy
+        out["secondary"] = {k: float("%.5g" % r["value"]) for k, r in line["secondary"].items()}
+    return out
 
 
 # Secondary records of the default run: the other configurations of the path
