@@ -47,6 +47,9 @@ __device__ __forceinline__ void record_copy(const SweepJob& J, uint64_t slot, ui
     }
 }
 
+// Sites of a copy held on chip, at most: as many as bytes of shared memory.
+constexpr uint32_t kCopySites = 1u << 18;
+
 // The same for the copies of a warp (has: this lane holds one), called by all 32
 // lanes: the population's range and sums are reduced over the warp first when
 // its copies belong to one instance, one set of atomics per warp. (Atomics on one
@@ -77,7 +80,7 @@ __device__ __forceinline__ void record_copies(const SweepJob& J, bool has, uint6
         atomicAdd(&J.hist[(uint64_t)inst * J.nbins + GBMC_IDX((uint32_t)((E - J.e_lo) >> 2), J.nbins)], 1u);
     }
     const int mn = __reduce_min_sync(kAll, has ? E : INT_MAX), mx = __reduce_max_sync(kAll, has ? E : INT_MIN);
-    // copies held on chip have fewer than 2^18 sites: |E| < 2^20, squares below
+    // copies held on chip have fewer than kCopySites sites: |E| < 2^20, squares below
     // 2^40 summed as two 20-bit halves
     const int e = has ? E : 0, m = has ? (M < 0 ? -M : M) : 0;
     const uint64_t e2 = (uint64_t)((long long)e * e), m2 = (uint64_t)((long long)m * m);

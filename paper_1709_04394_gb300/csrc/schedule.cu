@@ -44,12 +44,14 @@ struct SchedBins {
     float2 hf[kSchedBins], pf[kSchedBins];  // h and p0 as pairs of floats
     float2 coarse[kSchedBins / 32], fine[32];  // overlap_fast's exponentials
 };
-// Error bound of overlap_fast against overlap_eval: with u = 2^-24, three products of at
-// most 5 u^2, and per sum at most 16 + 8 additions of positive terms of 3 u^2 each (Joldes,
-// Muller, Popescu 2017) on the way from a weight to the overlap, that is below 7e-13; the
-// exponentials' arguments add less than 2e-14 where a bin's weight matters.
+// Error bound of overlap_fast against overlap_eval, u = 2^-24: a product is within 5 u^2, an
+// addition of positive terms within 3 u^2 (Joldes, Muller, Popescu 2017), and on the way from a
+// bin to a sum lie at most 15 additions of the thread's own, 5 in the warp and 7 over the warps: 81
+// u^2. A weight is within 12 u^2 (two products, three conversions), their sum W 93, 1 / W 102, p1
+// 119, the overlap 200 u^2 = 7.1e-13; the exponentials' arguments add less than 2e-14 where a
+// bin's weight matters. (Measured: 5e-15.)
 constexpr double kFastError = 1e-12;
-static_assert(kSchedBins / kSchedThreads <= 16, "overlap_fast's error bound");
+static_assert(kSchedBins / kSchedThreads <= 16 && kSchedThreads <= 256, "overlap_fast's error bound");
 
 __device__ __forceinline__ float bfr(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 

@@ -25,9 +25,9 @@
 // threshold compares, about 95 to 105 cycles; the kernel runs at 107 to 109 (2D).
 // Replacing the carry compares by predicates, or moving them to the float adder,
 // left that unchanged. Site updates per ns before (byte planes; per-site loop where
-// L % 8 != 0) and after, theta = 10 sweeps per load: 2D L = 24 610 -> 1399, L = 96
-// 843 -> 1363, L = 10 286 -> 1090; 3D +-J L = 4 240 -> 1299, L = 10 248 -> 1268, L = 12
-// 240 -> 1194, L = 32 540 -> 1291. (L = 16, 32, 64 in 2D and L = 8, 16 in 3D stay on
+// L % 8 != 0) and after, theta = 10 sweeps per load: 2D L = 24 610 -> 1392, L = 96
+// 843 -> 1366, L = 10 286 -> 1110; 3D +-J L = 4 240 -> 1306, L = 10 248 -> 1272, L = 12
+// 240 -> 1215, L = 32 540 -> 1319. (L = 16, 32, 64 in 2D and L = 8, 16 in 3D stay on
 // bitsweep.cu, whose fixed sizes need no windows: 1475 / 1512 and 1323 / 1337 there
 // against 1437 / 1486 and 1317 / 1328 here.)
 #include <algorithm>
@@ -52,6 +52,7 @@ namespace {
 
 constexpr uint32_t kStreamThreads = 128;      // threads per block with one-warp teams
 constexpr size_t kStreamSmem = 227 * 1024;   // shared memory of an SM
+static_assert(kStreamSmem < kCopySites, "record_copies: a copy that runs have is one that would fit as bytes");
 constexpr uint32_t kStreamTeamWords = 3072;  // a one-warp team's share of shared memory, at most
 // temperatures of the copies of a launch (kRounds: exchanged, too, round after round)
 enum { kOneTemp = 0, kPerCopy = 1, kRounds = 2 };
