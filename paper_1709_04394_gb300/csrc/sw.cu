@@ -947,16 +947,16 @@ cudaError_t launch_sw_resident(const SwLaunch& P0, uint64_t copies, uint32_t n_u
     const uint32_t threads = std::min(1024u, (P0.N / 4u + 31u) & ~31u);
     // a launch is kept to some ten milliseconds
     const uint32_t most = std::max(1u, (1u << 24) / P0.N);
-    for (uint32_t u = 0; u < n_updates; u += most) {
+    for (uint64_t u = 0; u < n_updates; u += most) {  // (64 bits: u does not wrap past the last launch)
         SwLaunch P = P0;
-        P.t = P0.t + u;
-        const uint32_t n = std::min(most, n_updates - u);
+        P.t = P0.t + (uint32_t)u;
+        const uint32_t n = (uint32_t)std::min<uint64_t>(most, n_updates - u);
         if (u + n < n_updates) P.labels = nullptr;
         for (uint64_t c0 = 0; c0 < copies; c0 += 0x40000000u) {
             P.copy0 = c0;
             const uint32_t nc = (uint32_t)std::min<uint64_t>(copies - c0, 0x40000000u);
-            kern<<<nc, threads, smem, s>>>(P, n, copies, E_series ? E_series + (uint64_t)u * copies : nullptr,
-                                           M_series ? M_series + (uint64_t)u * copies : nullptr);
+            kern<<<nc, threads, smem, s>>>(P, n, copies, E_series ? E_series + u * copies : nullptr,
+                                           M_series ? M_series + u * copies : nullptr);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
