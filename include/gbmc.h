@@ -120,7 +120,8 @@ gbmc_status gbmc_set_resample_mode(gbmc_ctx *ctx, int32_t fused);
  * kept with the lattice; where it cannot be had -- memory full, or the stream being
  * captured before it is there -- the GRID kernels run), run all sweeps of the call,
  * series included, as one cooperative launch with the same bounded waits, and convert
- * it back, unless the call is only a sweep or two. GRID uses the per-launch kernels (halo tiles of up
+ * it back, unless the launches of a call -- a sweep or two, or bit-packed lattices of
+ * tens of millions of sites -- cost less than that. GRID uses the per-launch kernels (halo tiles of up
  * to 4 sweeps, resp. one launch per half-sweep), and so does the BYTES kernel mode
  * where its strips do not apply. Double-checkerboard sweeps with bit-sliced tiles
  * (metropolis_sweeps_dcb): PERSISTENT runs every round of a call in one

@@ -989,10 +989,19 @@ namespace {
 // L = 1152 in halo tiles 505, 655, 749, 840, 1265 -> here 410, 744, 755, 761, 1478 (with series 1169,
 // 1820, 1971, 2098, 3127 -> 431, 779, 789, 795, 1543); sizes without tiles, launches per half-sweep,
 // n = 10: L = 520 77 copies 575 -> 380, 153 1033 -> 750; 3D L = 64 698 -> 459, 1299 -> 910.
+// Bit-packed without series, n = 2, 4, 20, launches per half-sweep : strips: L = 4032 (16 M sites)
+// 43 : 42, 84 : 71, 412 : 302; 8 x L = 1984 (31 M) 68 : 74, 133 : 131, 658 : 589; 4 x L = 4032 (65 M)
+// 117 : 133, 232 : 248, 1151 : 1156; 8 x L = 3008 (72 M) 127 : 149, 249 : 280, 1240 : 1319.
 bool takes_stream_strips(const gbmc_ctx* ctx, const gbmc_lattice* l, const Tuning& tu, uint32_t n_sweeps, bool series) {
     if (ctx->launch_mode == GBMC_LAUNCH_GRID || !ctx->coop || n_sweeps > 0x3FFFFFFFu) return false;
     if (n_sweeps < 2 || (l->d.dim == 2 && l->d.L < 64)) return false;
-    if (l->d.layout == GBMC_BITPACK) return l->ncopies <= (uint64_t)ctx->sm_count / 8;
+    if (l->d.layout == GBMC_BITPACK) {
+        // The launches per half-sweep read these bits as they are; what the strips save of
+        // launches and gaps has to pay for the words' way beside their tags and back.
+        const uint64_t sites = l->N * l->ncopies;
+        const bool pays = sites <= 1u << 24 || (sites <= 5u << 23 && n_sweeps >= 5) || (sites <= 1u << 26 && n_sweeps >= 20);
+        return l->ncopies <= (uint64_t)ctx->sm_count / 8 && (series || pays);
+    }
     if (ctx->sweep_kernel == GBMC_KERNEL_BYTES || (l->d.dim == 3 && !l->stab)) return false;
     if (!tu.resident) {
         // Copies have whole multiprocessors to themselves here, and a batch of one per

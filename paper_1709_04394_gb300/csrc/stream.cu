@@ -22,7 +22,7 @@
 // takes 2.1 cycles of a scheduler, a wide 32 x 32 -> 64-bit multiply 4.3, and a mix
 // of both 2.1 per logic instruction + 2.2 per multiply: the two do not overlap. A
 // Philox call (4 sites) is 18 xors, 16.5 to 18 multiplies and 8 (2D) or 12 (3D)
-// threshold compares, about 95 to 105 cycles; the kernel runs at 107 to 109 (2D).
+// threshold compares, 92 to 95 cycles in 2D and 100 to 104 in 3D; the kernel runs at 107 to 109 (2D).
 // Replacing the carry compares by predicates, or moving them to the float adder,
 // left that unchanged. Site updates per ns before (byte planes; per-site loop where
 // L % 8 != 0) and after, theta = 10 sweeps per load: 2D L = 24 610 -> 1392, L = 96
