@@ -242,7 +242,7 @@ __device__ __forceinline__ void resident_unit(const SweepLaunch& P, uint32_t uni
         // s == nsw is a measurement-only pass when nothing was swept
         if (s == nsw && nsw != 0) break;
         const bool sweep = s < nsw;
-        const bool measure = (J.Eser != nullptr && sweep) || ((sweep ? s + 1 == nsw : true) && want_final);
+        const bool measure = ((J.Eser || J.Mser) && sweep) || ((sweep ? s + 1 == nsw : true) && want_final);
         const uint32_t t = J.t0 + s;
         int e = 0, m = 0;
         for (uint32_t colour = 0; colour < 2; ++colour) {
