@@ -488,13 +488,16 @@ bool job_takes_bits(const SweepLaunch& P, const SweepJob& J, const Tuning& tu, i
 
 // Whether the bit-stream kernel takes a job the bit-sliced kernel does not: any
 // resident lattice, in AUTO mode only (BITS leaves what the bit-sliced kernel
-// does not support to the byte-plane kernel). One exception: 2D L = 8 with E and M of
+// does not support to the byte-plane kernel). Exceptions, where a plane is at most one
+// word and the byte planes' shorter way in and out counts: 2D L = 8 with E and M of
 // every sweep, more copies than multiprocessors (sweeps_ahead takes fewer) and up to
-// 10^4 -- a word per plane, eight byte-plane threads per copy -- 100 sweeps of 53 copies
-// 104 us there, 112 us here; of 20000 299 against 273.
+// 10^4, 100 sweeps of 53 copies 104 us there, 112 us here, of 20000 299 against 273; one
+// sweep of up to 5000 copies of 2D L <= 8, 4.1 us a call there, 6.2 here (L = 2 and 8;
+// L = 4 and 6 alike; L = 10 8.2 and 6.2).
 bool job_takes_stream(const SweepLaunch& P, const SweepJob& J, const Tuning& tu, int kernel, int sm_count) {
     const uint64_t copies = (uint64_t)J.n_inst * J.R;
     if (P.dim == 2 && J.L == 8 && (J.Eser || J.Mser) && copies > (uint64_t)sm_count && copies <= 10000u) return false;
+    if (P.dim == 2 && J.N <= 64u && J.nsweeps == 1u && !J.hist && !J.temp_of && copies <= 5000u) return false;
     return kernel == GBMC_KERNEL_AUTO && tu.bits && J.smask;
 }
 
