@@ -509,7 +509,10 @@ bool job_takes_stream(const SweepLaunch& P, const SweepJob& J, const Tuning& tu,
 // (bit-sliced -> bit-stream): 2D L = 16 R = 1200 15.2 -> 10.8, R = 5000 19.9 -> 22.2;
 // L = 64 R = 1 31.5 -> 10.7, R = 600 31.6 -> 25.9, R = 1200 47.1 -> 51.2; L = 128 R = 1
 // 119 -> 31, R = 1200 168 -> 145; L = 256 R = 1 471 -> 79; 3D L = 8 R = 1200 18.1 ->
-// 15.1, R = 2500 23.6 -> 29.5; L = 16 R = 600 37.2 -> 30.1, R = 1200 53.3 -> 59.4.
+// 15.1, R = 2500 23.6 -> 29.5; L = 16 R = 600 37.2 -> 30.1, R = 1200 53.3 -> 59.4. The fewer
+// sweeps, the more the bit-stream kernel's longer way in and out counts: one sweep, L = 64 R =
+// 300 8.5 -> 6.7, R = 640 8.8 -> 10.7; L = 128 R = 600 19.0 -> 16.8, R = 2500 45.7 -> 49.8; L = 256 R =
+// 1300 109 -> 103, R = 3000 189 -> 225, R = 6000 354 -> 431, three sweeps of those 885 -> 913.
 bool bits_jobs_small(const SweepLaunch& P, const std::vector<Tuning>& tu, int kernel, int sm_count) {
     if (kernel != GBMC_KERNEL_AUTO) return false;
     double warps = 0.0;
@@ -517,7 +520,9 @@ bool bits_jobs_small(const SweepLaunch& P, const std::vector<Tuning>& tu, int ke
         const SweepJob& J = P.jobs[j];
         if (!job_takes_bits(P, J, tu[j], kernel)) continue;
         if (!J.smask) return false;
-        warps += (double)J.n_inst * J.R * (J.N / 64u) / 32.0 / std::max(1.0, J.N / 2048.0 * (J.N / 2048.0));
+        const double copies = (double)J.n_inst * J.R, lane = J.N / 2048.0;  // words of a lane
+        if (copies > 1250.0 * std::max(2u, J.nsweeps)) return false;
+        warps += copies * lane / std::max(1.0, J.nsweeps == 1u ? lane * std::sqrt(lane) : lane * lane);
     }
     return warps <= 0.53 * 4.0 * sm_count;
 }
