@@ -2687,7 +2687,7 @@ struct gbmc_pt {
     gbmc_lattice* lat;
     std::vector<double> betas;
     uint32_t T, M, theta, round;
-    bool in_rounds = false;  // whole rounds per launch are the faster way (by the sizes alone)
+    TemperingCost cost;  // of rounds in one launch and apart (by the sizes alone)
     uint32_t* thr_temp = nullptr;
     uint32_t *temp_of = nullptr, *rep_of = nullptr, *accepted = nullptr;
     int32_t *E = nullptr, *Mag = nullptr;
@@ -2770,7 +2770,7 @@ gbmc_status pt_create(gbmc_ctx* ctx, gbmc_lattice* l, const double* betas, uint3
         delete pt;
         return fail(GBMC_ERR_CUDA, "parallel tempering set-up: %s", cudaGetErrorString(e));
     }
-    pt->in_rounds = tempering_in_rounds(pt_sweeps(pt, tu), ctx->sm_count);
+    pt->cost = tempering_cost(pt_sweeps(pt, tu), ctx->sm_count);
     l->run = (gbmc_pa*)pt;  // the lattice is owned by this run until pt_free
     *out = pt;
     return GBMC_OK;
@@ -2783,7 +2783,7 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
     gbmc_lattice* l = pt->lat;
     if ((uint64_t)l->t + (uint64_t)n_steps * pt->theta > 0xFFFFFFFFull) return fail(GBMC_ERR_ARG, "sweep counter would wrap");
     const Tuning tu = tune(l);
-    const bool in_rounds = pt->in_rounds && ctx->sweep_kernel == GBMC_KERNEL_AUTO && tu.bits;
+    const bool may = ctx->sweep_kernel == GBMC_KERNEL_AUTO && tu.bits;
     for (uint32_t n = 0; n < n_steps;) {
         const SweepLaunch P = pt_sweeps(pt, tu);
         PtExchange X;
@@ -2801,9 +2801,9 @@ gbmc_status pt_step(gbmc_ctx* ctx, gbmc_pt* pt, uint32_t n_steps) {
         // a launch of rounds is kept to some ten milliseconds: 2^34 site updates, 2^13 sweeps
         const double sweeps = std::max(1u, pt->theta), updates = (double)l->N * (double)l->ncopies * sweeps;
         X.rounds = (uint32_t)std::max(1.0, std::min({(double)(n_steps - n), 17179869184.0 / updates, 8192.0 / sweeps}));
-        if (in_rounds) {
+        if (may && pt->cost.together(X.rounds)) {
             ProfScope ps_(ctx, PK_PT_ROUNDS);
-            CUDA_TRY(launch_tempering_rounds(P, X, ctx->sm_count, ctx->stream));
+            CUDA_TRY(launch_tempering_rounds(P, X, pt->cost.plan, ctx->stream));
         } else {
             X.rounds = 1;
             gbmc_status st = launch_jobs(ctx, P, std::vector<Tuning>{tu});

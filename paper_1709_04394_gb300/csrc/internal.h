@@ -364,17 +364,30 @@ struct PtExchange {
     const long long* tab;      // [T-1][M+1] threshold of pair k at energy gap 4m (-1: never)
     uint64_t seed;
     uint32_t T, M, n_inst, inst_base, round;
-    uint32_t rounds;           // tempering_in_rounds: rounds of the launch, from `round`
+    uint32_t rounds;           // launch_tempering_rounds: rounds of the launch, from `round`
 };
 cudaError_t launch_pt_exchange(const PtExchange& X, cudaStream_t s);
 // Plain sweeps (series included) of few small copies, acceptance bits drawn ahead (stream.cu).
 bool sweeps_ahead(const SweepLaunch& P, int sm_count);
 cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, long long budget, uint32_t phantom,
                                cudaStream_t s);
-// Rounds of sweeps (J.nsweeps each) and exchanges in one launch (stream.cu), and whether
-// that is the faster way for P's one job.
-bool tempering_in_rounds(const SweepLaunch& P, int sm_count);
-cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, int sm_count, cudaStream_t s);
+// Rounds of sweeps (J.nsweeps each) and exchanges in one launch (stream.cu): every instance in B
+// blocks of `threads` threads, in teams of T with G copies each; cost: estimated cycles of a round.
+struct RoundsPlan {
+    int split = 1;
+    uint32_t B = 1, G = 1, T = 32, threads = 32;
+    double cost = 1e300;
+};
+// Whether that is the faster way for P's one job: estimated cycles of a round within such a
+// launch, of the launch besides, and of a round as two launches. The estimates are good to a
+// quarter or so; several rounds are kept together unless that is clearly the slower way.
+struct TemperingCost {
+    RoundsPlan plan;
+    double round = 1e300, launch = 0.0, apart = 0.0;
+    bool together(uint32_t n) const { return n * apart * (n > 1u ? 1.25 : 1.1) > launch + n * round; }
+};
+TemperingCost tempering_cost(const SweepLaunch& P, int sm_count);
+cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, const RoundsPlan& R, cudaStream_t s);
 
 // ---- schedule MLP (6 -> 64 -> 64 -> 1) ----
 constexpr int kMlpIn = 6;

@@ -9,7 +9,7 @@
 // configurations, as the paper recommends for shared memory.
 //
 // One launch per round, after the round's sweep launch; where that is faster, whole
-// rounds run in one launch instead (stream.cu, tempering_in_rounds).
+// rounds run in one launch instead (stream.cu, tempering_cost).
 #include "copies.cuh"
 #include "device.cuh"
 #include "internal.h"

@@ -1174,19 +1174,35 @@ cudaError_t launch_stream_c(const SweepLaunch& P, const StreamPlan& S, bool pt, 
     return pt ? launch_stream<DIM, EA, 1, 1, kPerCopy>(P, S, st) : launch_stream<DIM, EA, 1, 1, kOneTemp>(P, S, st);
 }
 
-// How the copies of every instance are divided for rounds of tempering: B blocks of
-// `threads` threads, in teams of T with G copies each (one copy per thread: two
-// measured 20 % slower for want of work in flight). In cycles per
+// How the copies of every instance are divided for rounds of tempering (one copy per thread:
+// two measured 20 % slower for want of work in flight). In cycles per
 // round, by the same pass and latency as above: a block keeps its place to the
 // end, so the blocks count in whole waves.
-struct RoundsPlan {
-    int split = 1;
-    uint32_t B = 1, G = 1, T = 32, threads = 32;
-    double cost = 1e300;
-};
-
 size_t rounds_smem(const SweepJob& J, const RoundsPlan& p) {
     return (size_t)(p.threads / p.T * stream_smem_words(J.N, p.G, 1u, true) + 5u * J.R) * 4u;
+}
+
+// A plan's cycles per round, its blocks on so many multiprocessors, and how often these fill up.
+struct RoundsCost {
+    double cycles, waves;
+};
+RoundsCost rounds_cost(const SweepJob& J, int dim, const RoundsPlan& p, double sms) {
+    const uint32_t PW = (J.N / 2u + 31u) / 32u;
+    // (with places and bond words kept: less than a sweep launch's pass)
+    const double pass = (p.split == 4 ? 420.0 : 980.0) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, p.split, 2);
+    const double passes = std::ceil(p.G * PW * p.split / (double)p.T), warps = p.threads / 32.0;
+    const double held = std::min({std::floor((double)stream_max_threads(1, p.split, kRounds) / p.threads),  // by registers
+                                  std::floor((double)kStreamSmem / (rounds_smem(J, p) + 1024.0)), 16.0});
+    const double blocks = (double)J.n_inst * p.B, wave = held * sms, full = std::floor(blocks / wave);
+    auto half = [&](double per_sm) {  // a half-sweep with so many blocks on an SM
+        const double w = std::ceil(per_sm * warps / 4.0);
+        return passes * (std::max(lat, w * pass) + (w > 1.0 ? 200.0 : 0.0) + 2.0 * per_sm * warps) +
+               (p.T > 32u ? 300.0 : 0.0);
+    };
+    const double rest = std::ceil((blocks - full * wave) / sms);
+    const double t = full * half(held) + (rest > 0.0 ? half(rest) : 0.0);
+    const double waves = full + (rest > 0.0 ? 1.0 : 0.0);
+    return {(2.0 * J.nsweeps + 0.4) * t + waves * (p.B > 1u ? 2500.0 : 1500.0), waves};
 }
 
 RoundsPlan rounds_plan(const SweepJob& J, int dim, int sm_count) {
@@ -1195,26 +1211,11 @@ RoundsPlan rounds_plan(const SweepJob& J, int dim, int sm_count) {
     const uint32_t ng = J.R;
     for (const int split : {4, 1}) {
         const uint32_t most = stream_max_threads(1, split, kRounds);
-        // (with places and bond words kept: less than a sweep launch's pass)
-        const double pass = (split == 4 ? 420.0 : 980.0) * (dim == 3 ? 1.15 : 1.0), lat = stream_lat(1, split, 2);
         auto consider = [&](uint32_t B, uint32_t G, uint32_t T, uint32_t threads) {
             RoundsPlan p;
             p.split = split, p.B = B, p.G = G, p.T = T, p.threads = threads;
-            const size_t smem = rounds_smem(J, p);
-            if (smem > 200u * 1024u) return;
-            const double passes = std::ceil(G * PW * split / (double)T), warps = threads / 32.0;
-            const double held = std::min({std::floor((double)most / threads),  // by registers
-                                          std::floor((double)kStreamSmem / (smem + 1024.0)), 16.0});
-            const double blocks = (double)J.n_inst * B, wave = held * sm_count, full = std::floor(blocks / wave);
-            auto half = [&](double per_sm) {  // a half-sweep with so many blocks on an SM
-                const double w = std::ceil(per_sm * warps / 4.0);
-                return passes * (std::max(lat, w * pass) + (w > 1.0 ? 200.0 : 0.0) + 2.0 * per_sm * warps) +
-                       (T > 32u ? 300.0 : 0.0);
-            };
-            const double rest = std::ceil((blocks - full * wave) / sm_count);
-            const double t = full * half(held) + (rest > 0.0 ? half(rest) : 0.0);
-            const double waves = full + (rest > 0.0 ? 1.0 : 0.0);
-            p.cost = (2.0 * J.nsweeps + 0.4) * t + waves * (B > 1u ? 2500.0 : 1500.0);
+            if (rounds_smem(J, p) > 200u * 1024u) return;
+            p.cost = rounds_cost(J, dim, p, sm_count).cycles;
             if (p.cost < best.cost) best = p;
         };
         for (uint32_t B = 1; B <= 8u && B <= ng; B *= 2u) {
@@ -1294,10 +1295,13 @@ cudaError_t launch_sweep_ahead(const SweepLaunch& P, unsigned int* err, long lon
 // exchange launch, 20 000 to 27 000 cycles beside the half-sweeps (3D L = 8, 250 x 40 copies,
 // one sweep per round: 15.4 us, 4.8 of them sweeping; L = 12, 60 x 14: 16.4, 2). What speaks for it is that its blocks
 // change places between rounds: 256 x 40 copies of L = 12, 10 sweeps per round, 207 us
-// each against 248 in one launch of rounds; 100 x 36 53 against 38.
-bool tempering_in_rounds(const SweepLaunch& P, int sm_count) {
+// each against 248 in one launch of rounds; 100 x 36 53 against 38. A launch of rounds loads
+// the maps and the copies once, so it has to have rounds enough: 2000 x 4 copies of 3D L = 8, one
+// sweep per round, 1, 2 and 20 rounds per call 20.7, 13.6 and 8.0 us per round in one launch, 12.6
+// apart; 200 x 8 14.6, 9.9, 5.6 and 10.4.
+TemperingCost tempering_cost(const SweepLaunch& P, int sm_count) {
     const SweepJob& J = P.jobs[0];
-    if (!J.smask || (P.ea && !J.sbond) || J.nsweeps == 0u || J.R < 2u || J.R > 1024u) return false;
+    if (!J.smask || (P.ea && !J.sbond) || J.nsweeps == 0u || J.R < 2u || J.R > 1024u) return {};
     double alone = std::min(stream_plan(P, 1, 4, true, sm_count).cost, stream_plan(P, 1, 2, true, sm_count).cost);
     for (int C = 4; C >= 1; C >>= 1)
         if (C == 1 || stream_smem_words(J.N, 1u, (uint32_t)C, true) * 4u <= 36u * 1024u)
@@ -1307,11 +1311,23 @@ bool tempering_in_rounds(const SweepLaunch& P, int sm_count) {
         const double warps = std::ceil(copies * (J.N / 64.0) / 32.0 / per / (4.0 * sm_count));
         alone = std::min(alone, per * std::max(warps * (P.dim == 3 ? 950.0 : 840.0), 2100.0));
     }
-    return rounds_plan(J, P.dim, sm_count).cost < 2.0 * J.nsweeps * alone + 24000.0;
+    const RoundsPlan p = rounds_plan(J, P.dim, sm_count);
+    if (!(p.cost < 2.0 * J.nsweeps * alone + 24000.0)) return {};
+    // A cluster's blocks lie within one group of the device's multiprocessors, of which some are
+    // left over: 16 clusters of eight blocks that fill a multiprocessor each run as two waves
+    const double sms = J.n_inst == 1u || p.B == 1u ? 1.0 : p.B == 8u ? 0.74 : p.B == 4u ? 0.9 : 0.97;
+    const RoundsCost c = rounds_cost(J, P.dim, p, std::floor(sms * sm_count));
+    const double copies = (double)J.n_inst * J.R, kb = J.N / 1024.0, blocks = (double)J.n_inst * p.B;
+    TemperingCost t;
+    t.plan = p;
+    t.round = c.cycles;
+    t.launch = 12000.0 + 830.0 * blocks / sm_count +
+               std::max(c.waves * std::ceil((double)J.R / p.B), copies / sm_count) * (100.0 + 110.0 * kb);
+    t.apart = 2.0 * J.nsweeps * alone + 22800.0 + 0.35 * copies * kb;
+    return t;
 }
 
-cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, int sm_count, cudaStream_t s) {
-    const RoundsPlan R = rounds_plan(P.jobs[0], P.dim, sm_count);
+cudaError_t launch_tempering_rounds(const SweepLaunch& P, const PtExchange& X, const RoundsPlan& R, cudaStream_t s) {
     if (P.dim == 2 && !P.ea) return launch_rounds_c<2, false>(P, X, R, s);
     if (P.dim == 3 && !P.ea) return launch_rounds_c<3, false>(P, X, R, s);
     if (P.dim == 3 && P.ea) return launch_rounds_c<3, true>(P, X, R, s);
